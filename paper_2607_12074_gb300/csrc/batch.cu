@@ -5,6 +5,7 @@
 // graphs of uneven size share one persistent launch per kernel.  The whole sequence - union build,
 // orientation, anchors, reductions, per-graph closure, and the copy of the counts to pinned host
 // memory - is captured once into a CUDA graph and replayed on every count.
+#include <algorithm>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -253,6 +254,7 @@ harp_status batch_prepare(harp_batch* b, const harp_plan& plan) {
     b->u.ws.gid = b->d_gid;
     b->u.ws.accG = b->d_accG;
     b->u.ws.G = b->G;
+    b->u.ws.max_member_m = b->G > 0 ? *std::max_element(b->m_of.begin(), b->m_of.end()) : 0;
     b->u.ws.gbase = b->d_gbase;
     b->u.ws.ginfo = b->d_ginfo;
     const bool use_graph = !(plan.flags & HARP_PLAN_NO_GRAPH);

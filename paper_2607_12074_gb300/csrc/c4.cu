@@ -72,7 +72,7 @@ constexpr int kChunk = 1024;                 // elements per split chunk
 // ends where band b + 1 starts, the last band at GI_HI).  GI_N1 = GI_BAND: the first band starts at n1.
 constexpr int kBands = 7;
 enum : int { GI_HI = 0, GI_NWIN = 1, GI_BAND = 2, GI_N1 = GI_BAND };
-static_assert(GI_BAND + kBands <= kGInfo && kBands < 32, "ginfo slots; one search per lane");
+static_assert(GI_BAND + kBands <= GI_CORE && kBands < 32, "ginfo slots; one search per lane");
 
 // counter bits of band b and the largest degree the band holds
 __host__ __device__ constexpr int band_width(int b) {
@@ -154,21 +154,70 @@ __device__ __forceinline__ int64_t merged_windows(const int64_t* st, unsigned ma
 
 constexpr int kMergeMasks = 1 << (kBands - 1);
 constexpr int kMergeSamples = 64;
+constexpr int kGinfoThreads = 128;
+constexpr int kGinfoWarps = kGinfoThreads / 32;
 
-// One warp per graph.  The x-range of a graph's grid is [n1, hi) intersected with [x_lo, x_hi) (a
+// The graph's wedge core (c4core.cu), by one warp: ranks [lo, gend), arcs [alo, ahi) of the rank-order CSR.
+// The core is the largest K = 2^10 .. 2^14 (at most half the graph) with
+//   * deg >= K / 64 at the core's first rank: a core row's words then hold enough bits to beat walking
+//     its list (R-MAT scale 15: 728 us a count at K / 64, 746 at K / 128; Chung-Lu with 500,000 vertices:
+//     5.08 ms against 5.23 at K / 256; R-MAT 16 to 20 choose the same K with each),
+//   * an eighth of the graph's arcs at core vertices, else the wedges are elsewhere (Barabasi-Albert,
+//     100,000 vertices: 637 us with its core of 17 % of the arcs, 710 without; random geometric graphs
+//     have about 0.1 %),
+//   * K * K bits in the graph's share of the region (4 bytes an arc and 64 a vertex).
+__device__ __forceinline__ void choose_core(const int32_t* __restrict__ deg, const int64_t* __restrict__ off,
+                                            int64_t lo, int64_t gend, int64_t* gi, uint64_t* acc) {
+    const int l = lane_id();
+    int64_t c0 = INT64_MAX, K = 0, base = 0;
+    if (off) {  // uniform: a kernel argument
+        const int64_t alo = off[lo], ahi = off[gend], ng = gend - lo;
+        const int64_t b0 = (4 * alo + 64 * lo + 15) & ~(int64_t)15;
+        const int64_t cap = 4 * ahi + 64 * gend - b0;
+        bool ok = false;
+        const int64_t k = (int64_t)1024 << l;
+        if (l < 5 && ahi - alo >= 2 * kCoreMinM && 2 * k <= ng && k * k / 8 <= cap &&
+            deg[gend - 1] >= kCoreMinMaxDeg)
+            ok = (int64_t)deg[gend - k] >= k / 64 && 8 * (ahi - off[gend - k]) >= ahi - alo;
+        const uint32_t m = __ballot_sync(kFull, ok);
+        if (m) {
+            K = (int64_t)1024 << (31 - __clz(m));
+            c0 = gend - K;
+            base = b0 / 4;
+        }
+    }
+    if (l == 0) {
+        gi[GI_CORE] = c0;
+        gi[GI_CORE_K] = K;
+        gi[GI_CORE_BASE] = base;
+        if (K > 0) atomicAdd((unsigned long long*)&acc[A_CORE_ANY], 1ull);
+    }
+}
+
+// One block per graph.  The x-range of a graph's grid is [n1, hi) intersected with [x_lo, x_hi) (a
 // partitioned wedge block owns only the opposite vertices in that slice; a whole graph passes
 // [0, INT64_MAX)).  A narrow band holding few vertices costs a partly filled window for every root
-// that reaches past it, so bands may merge into the next wider one: each lane scores merge masks by
+// that reaches past it, so bands may merge into the next wider one: each lane scores two merge masks by
 // the windows of kMergeSamples roots spread evenly over the graph's ranks of degree >= 64 (the roots
 // that take the windowed mode), each weighted by its degree; the cheapest mask (lowest on a tie) wins.
-// merge = false keeps every band separate (mask 0).
+// The samples are dealt to the block's warps and the scores are integers: by one warp in FP64 the scoring
+// took 55 us, a fifth of a whole count of a graph of 8,000 edges.
+// merge = false keeps every band separate (mask 0).  off (nullptr: no core): see choose_core.
 template <int WORDS>
-__global__ void k_c4_ginfo(const int32_t* __restrict__ deg, int64_t n, const int64_t* __restrict__ gbase,
-                           int64_t G, int64_t x_lo, int64_t x_hi, bool merge, int64_t* __restrict__ ginfo) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < G; g += warps) {
+__global__ void __launch_bounds__(kGinfoThreads) k_c4_ginfo(const int32_t* __restrict__ deg, int64_t n,
+                                                            const int64_t* __restrict__ gbase, int64_t G, int64_t x_lo,
+                                                            int64_t x_hi, bool merge, const int64_t* __restrict__ off,
+                                                            int64_t* __restrict__ ginfo, uint64_t* __restrict__ acc) {
+    __shared__ uint64_t s_score[kGinfoWarps][kMergeMasks];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t g = blockIdx.x; g < G; g += gridDim.x) {
         const int64_t lo = gbase ? gbase[g] : 0, gend = gbase ? gbase[g + 1] : n;
+        int64_t* gi = ginfo + g * kGInfo;
+        if (warp == kGinfoWarps - 1 && gend > lo) choose_core(deg, off, lo, gend, gi, acc);
+        if (warp == kGinfoWarps - 1 && gend <= lo && lane == 0) {
+            gi[GI_CORE] = INT64_MAX;
+            gi[GI_CORE_K] = gi[GI_CORE_BASE] = 0;
+        }
         auto clamp = [&](int64_t v) { return v < x_lo ? x_lo : (v > x_hi ? x_hi : v); };
         const int64_t hi = gend < x_hi ? gend : x_hi;
         // lane 0: n1 (first rank of degree >= 2); lane b < kBands: the first rank above band b - 1's
@@ -185,47 +234,54 @@ __global__ void k_c4_ginfo(const int32_t* __restrict__ deg, int64_t n, const int
             const int64_t r = clamp(__shfl_sync(0xffffffffu, r_lane, b));
             st[b] = r > n1 ? (r < hi ? r : hi) : n1;
         }
-        int64_t s0 = __shfl_sync(0xffffffffu, r_lane, kBands);
-        if (s0 >= gend) s0 = lo;
-        const int64_t span = gend - s0;  // samples u lie in [s0, gend); none for an empty graph
-        static_assert(kMergeSamples == 64 && kMergeMasks == 64, "two samples and two masks per lane");
-        int64_t us[2];
-        double ws[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {  // lane holds samples lane and lane + 32 (loads issued together)
-            us[h] = s0 + (span * (2 * (lane + 32 * h) + 1)) / (2 * kMergeSamples);
-            ws[h] = span > 0 ? (double)deg[us[h]] : 0.0;
-        }
         unsigned best_mask = 0;  // mask 0: every band separate
-        if (merge) {             // uniform over the warp (a kernel argument)
-            double best = 0.0;
-            for (int m = lane; m < kMergeMasks; m += 32) {
-                double c = 0.0;
-                for (int k = 0; k < kMergeSamples; ++k) {  // uniform over the warp: every lane shuffles
-                    const int64_t u = __shfl_sync(0xffffffffu, k < 32 ? us[0] : us[1], k & 31);
-                    const double w = __shfl_sync(0xffffffffu, k < 32 ? ws[0] : ws[1], k & 31);
-                    c += w * (double)merged_windows<WORDS>(st, (unsigned)m, u);
-                }
-                if (m == lane || c < best) {
-                    best = c;
-                    best_mask = (unsigned)m;
-                }
-            }
+        if (merge) {             // uniform over the block (a kernel argument)
+            int64_t s0 = __shfl_sync(0xffffffffu, r_lane, kBands);
+            if (s0 >= gend) s0 = lo;
+            const int64_t span = gend - s0;  // samples u lie in [s0, gend); none for an empty graph
+            constexpr int kPer = kMergeSamples / kGinfoWarps;  // this warp's samples, one per lane
+            static_assert(kPer <= 32 && kMergeMasks == 64, "a sample and two masks per lane");
+            const int64_t u_l = s0 + (span * (2 * (warp * kPer + lane) + 1)) / (2 * kMergeSamples);
+            const uint32_t w_l = span > 0 && lane < kPer ? (uint32_t)deg[u_l] : 0u;
+            uint64_t c[2] = {0, 0};
+            for (int k = 0; k < kPer; ++k) {  // uniform over the warp: every lane shuffles
+                const int64_t u = __shfl_sync(0xffffffffu, u_l, k);
+                const uint32_t w = __shfl_sync(0xffffffffu, w_l, k);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const double oc = __shfl_xor_sync(0xffffffffu, best, o);
-                const unsigned om = __shfl_xor_sync(0xffffffffu, best_mask, o);
-                if (oc < best || (oc == best && om < best_mask)) {
-                    best = oc;
-                    best_mask = om;
+                for (int h = 0; h < 2; ++h)
+                    c[h] += (uint64_t)w * (uint64_t)merged_windows<WORDS>(st, (unsigned)(lane + 32 * h), u);
+            }
+            s_score[warp][lane] = c[0];
+            s_score[warp][lane + 32] = c[1];
+            __syncthreads();
+            if (warp == 0) {
+                uint64_t best = 0;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint64_t v = 0;
+#pragma unroll
+                    for (int k = 0; k < kGinfoWarps; ++k) v += s_score[k][lane + 32 * h];
+                    if (h == 0 || v < best) {
+                        best = v;
+                        best_mask = (unsigned)(lane + 32 * h);
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const uint64_t oc = __shfl_xor_sync(0xffffffffu, best, o);
+                    const unsigned om = __shfl_xor_sync(0xffffffffu, best_mask, o);
+                    if (oc < best || (oc == best && om < best_mask)) {
+                        best = oc;
+                        best_mask = om;
+                    }
                 }
             }
+            __syncthreads();  // the scores are read before the next graph's are written
         }
-        if (lane == 0) {
+        if (threadIdx.x == 0) {
 #pragma unroll
             for (int b = 0; b + 1 < kBands; ++b)
                 if ((best_mask >> b) & 1u) st[b + 1] = st[b];  // band b becomes empty, b + 1 starts at its start
-            int64_t* gi = ginfo + g * kGInfo;
             gi[GI_HI] = hi;
 #pragma unroll
             for (int b = 0; b < kBands; ++b) gi[GI_BAND + b] = st[b];
@@ -247,6 +303,7 @@ template <bool ROWS>
 __global__ void __launch_bounds__(256) k_c4_rev(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
                                                 const int64_t* __restrict__ offp, const int32_t* __restrict__ colsp,
                                                 const int32_t* __restrict__ deg, const int32_t* __restrict__ dplus,
+                                                const int32_t* __restrict__ gid, const int64_t* __restrict__ ginfo,
                                                 int64_t n, int64_t arcs, int32_t* __restrict__ rev) {
     const int64_t runs = (arcs + kRevRun - 1) / kRevRun;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < runs; r += (int64_t)gridDim.x * blockDim.x) {
@@ -258,16 +315,34 @@ __global__ void __launch_bounds__(256) k_c4_rev(const int64_t* __restrict__ off,
             if (off[mid] <= a0) lo = mid;
             else hi = mid;
         }
+        // the end of u's lower arcs; core roots are counted elsewhere and need none
+        auto row_lower_end = [&](int64_t v, int64_t vb) {
+            if (!ROWS && v >= ginfo[(gid ? (int64_t)gid[v] : 0) * kGInfo + GI_CORE]) return vb;
+            return vb + ((int64_t)deg[v] - dplus[v]);
+        };
         int64_t u = lo;
         int64_t ub = off[u], ue = off[u + 1];
-        int64_t lower_end = ub + ((int64_t)deg[u] - dplus[u]);
+        int64_t lower_end = row_lower_end(u, ub);
         for (int64_t a = a0; a < a1; ++a) {
-            while (a >= ue) {  // next non-empty row
+            if (a >= ue) {  // the row of arc a: last u with off[u] <= a, searched outward from u + 1 (the
+                            // empty rows of a graph's isolated vertices come in runs of up to its whole size)
                 if (u + 1 >= n) return;  // only if arcs > off[n]
-                ++u;
-                ub = ue;
+                int64_t p = u + 1, step = 1;
+                while (p + step < n && off[p + step] <= a) {
+                    p += step;
+                    step <<= 1;
+                }
+                int64_t q = p + step < n ? p + step : n;  // off[p] <= a < off[q], or q = n
+                while (q - p > 1) {
+                    const int64_t mid = (p + q) >> 1;
+                    if (off[mid] <= a) p = mid;
+                    else q = mid;
+                }
+                u = p;
+                ub = off[u];
                 ue = off[u + 1];
-                lower_end = ub + ((int64_t)deg[u] - dplus[u]);
+                if (a >= ue) return;  // only if arcs > off[n]
+                lower_end = row_lower_end(u, ub);
             }
             if (a >= lower_end || lower_end - ub < 2) continue;  // only lower arcs of roots with d- >= 2
             const int32_t w = cols[a];
@@ -478,7 +553,9 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
         const int64_t k = k0 + (int64_t)l * nw;
         const int32_t u = (int32_t)(n - 1 - k);
         int64_t dm = 0;
-        if (k < n && u >= own_lo && u < own_hi) dm = (int64_t)deg[u] - dplus[u];  // the owner rule
+        if (k < n && u >= own_lo && u < own_hi &&                       // the owner rule
+            u < ginfo[(gid ? (int64_t)gid[u] : 0) * kGInfo + GI_CORE])  // core roots are counted by the core pass
+            dm = (int64_t)deg[u] - dplus[u];
         const int64_t ub = dm >= 2 ? loff[u] : 0;
         uint64_t W = 0;
         if (dm >= 2 && dm <= 32) {
@@ -872,10 +949,12 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     const Sink sink{ws.acc, ws.gid, ws.accG};
     const int sms = num_sms();
     int32_t* wcount = ws.q_win + n;
-    HARP_CK(cudaMemsetAsync(wcount, 0, (size_t)n * sizeof(int32_t), s));
-    k_c4_ginfo<WORDS><<<grid_cap(G * 32, 128, 1024), 128, 0, s>>>(ws.deg, n, ws.gbase, G, ws.x_lo, ws.x_hi, merge,
-                                                                  ws.ginfo);
+    const bool core = wedge_core_applies(g, ws);
+    k_c4_ginfo<WORDS><<<(unsigned)(G < 8192 ? G : 8192), kGinfoThreads, 0, s>>>(
+        ws.deg, n, ws.gbase, G, ws.x_lo, ws.x_hi, merge, core ? ws.off : nullptr, ws.ginfo, ws.acc);
     HARP_LAUNCHED();
+    if (core) HARP_TRY(count_wedge_core(g, ws, s));  // uses rev, bpos and the queues before they are filled below
+    HARP_CK(cudaMemsetAsync(wcount, 0, (size_t)n * sizeof(int32_t), s));
     // the roots' lower lists: row prefixes of a whole graph, or their own CSR in a partitioned block
     const bool lists = ws.loff != nullptr;
     const int64_t* loff = lists ? ws.loff : ws.off;
@@ -883,11 +962,11 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     if (lists) {
         const int64_t la = ws.lower_arcs;  // == loff[n]
         k_c4_rev<true><<<grid_cap((la + kRevRun - 1) / kRevRun, 256, (int64_t)sms * 64), 256, 0, s>>>(
-            ws.loff, ws.lcols, ws.off, ws.cols, ws.deg, ws.dplus, n, la, ws.rev);
+            ws.loff, ws.lcols, ws.off, ws.cols, ws.deg, ws.dplus, ws.gid, ws.ginfo, n, la, ws.rev);
     } else {
         const int64_t arcs = ws.arcs >= 0 ? ws.arcs : 2 * g->m;  // must equal off[n]
         k_c4_rev<false><<<grid_cap((arcs + kRevRun - 1) / kRevRun, 256, (int64_t)sms * 64), 256, 0, s>>>(
-            ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.dplus, n, arcs, ws.rev);
+            ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.dplus, ws.gid, ws.ginfo, n, arcs, ws.rev);
     }
     HARP_LAUNCHED();
     k_c4_bpos<WORDS><<<grid_cap(n * kGridCap, 256, (int64_t)sms * 64), 256, 0, s>>>(ws.off, ws.cols, ws.gid, ws.ginfo, n,
