@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(256) k_c4_rev(const int64_t* __restrict__ off,
         }
         // the end of u's lower arcs; core roots are counted elsewhere and need none
         auto row_lower_end = [&](int64_t v, int64_t vb) {
-            if (!ROWS && v >= ginfo[(gid ? (int64_t)gid[v] : 0) * kGInfo + GI_CORE]) return vb;
+            if (!ROWS && ginfo && v >= ginfo[(gid ? (int64_t)gid[v] : 0) * kGInfo + GI_CORE]) return vb;
             return vb + ((int64_t)deg[v] - dplus[v]);
         };
         int64_t u = lo;
@@ -344,7 +344,8 @@ __global__ void __launch_bounds__(256) k_c4_rev(const int64_t* __restrict__ off,
                 if (a >= ue) return;  // only if arcs > off[n]
                 lower_end = row_lower_end(u, ub);
             }
-            if (a >= lower_end || lower_end - ub < 2) continue;  // only lower arcs of roots with d- >= 2
+            // only lower arcs of roots with d- >= 2 (of every row without ginfo)
+            if (a >= lower_end || (ginfo && lower_end - ub < 2)) continue;
             const int32_t w = cols[a];
             const int64_t pb = offp[w];
             if (ROWS) rev[a] = (int32_t)lower_bound_i32(colsp + pb, offp[w + 1] - pb, (int32_t)u);
@@ -1005,6 +1006,14 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
 }
 
 }  // namespace
+
+harp_status wedge_positions(const harp_csr* g, Workspace& ws, cudaStream_t s) {
+    const int64_t arcs = 2 * g->m;
+    k_c4_rev<false><<<grid_cap((arcs + kRevRun - 1) / kRevRun, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(
+        ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.dplus, nullptr, nullptr, g->n, arcs, ws.rev);
+    HARP_LAUNCHED();
+    return HARP_OK;
+}
 
 harp_status count_wedge_c4(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s) {
     if (g->n == 0 || g->m == 0) return HARP_OK;

@@ -231,6 +231,21 @@ harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s);
 // tri.cu: triangle + per-edge t_e + 4-clique anchor (steps a3, a4)
 harp_status count_triangles_k4(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s);
 
+// the largest possible out-degree: bounded by sqrt(2m) and by the maximum degree
+int64_t max_out_degree(const harp_csr* g);
+
+// tri.cu: the orbit outputs' triangle and 4-clique statistics, after count_triangles_k4 under the default plan
+// (its queues and t_e), over anchors of out-degree 2 .. 1024.  Per vertex (n9; tau6, six times the 4-cliques) or
+// per out-arc (e5, e8; e9, twice the 4-cliques; n9 is nullptr); all start at zero.
+struct OrbTri {
+    unsigned long long *n9, *tau6;
+    unsigned long long *e5, *e8, *e9;
+};
+harp_status orbit_triangles(const harp_csr* g, Workspace& ws, const OrbTri& o, cudaStream_t s);
+
+// c4.cu: the position of u in w's row for every lower arc (u -> w) of a whole graph (ws.rev)
+harp_status wedge_positions(const harp_csr* g, Workspace& ws, cudaStream_t s);
+
 // c4.cu: wedge anchor, non-induced 4-cycles (step a5)
 harp_status count_wedge_c4(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s);
 

@@ -489,6 +489,125 @@ struct CtaSmem {
 };
 
 
+// The anchor a block works on: its list L = N+(u) of d members; direct: membership by the table indexed by
+// y - L0 (where L's span fits: dense anchors, high ranks close together) instead of the hash.
+struct CtaAnchor {
+    int d;
+    int32_t L0;
+    uint32_t span;
+    bool direct;
+};
+
+// Stages L, the membership structure and the rows' probe ranges; clears own and the bitmap (d rows of WS
+// words).  Ends with a block barrier.
+template <int DMAX, int THREADS, bool BS>
+__device__ __forceinline__ CtaAnchor stage_anchor(CtaSmem<DMAX>& s, const int64_t* __restrict__ offp,
+                                                  const int32_t* __restrict__ colsp, int64_t ub, int d, int WS) {
+    using S = CtaSmem<DMAX>;
+    CtaAnchor A;
+    A.d = d;
+    A.L0 = colsp[ub];
+    A.span = (uint32_t)(colsp[ub + d - 1] - A.L0) + 1u;
+    A.direct = !BS && A.span <= (uint32_t)S::TAB;
+    for (int i = threadIdx.x; i < d; i += THREADS) {
+        s.L[i] = colsp[ub + i];
+        s.own[i] = 0;
+    }
+    for (int i = threadIdx.x; i < d * WS; i += THREADS) s.R[i] = 0;
+    if (A.direct) {
+        for (int i = threadIdx.x; i < (int)A.span; i += THREADS) s.m.tab[i] = 0;
+    } else {
+        for (int i = threadIdx.x; i < (1 << S::HB); i += THREADS) s.m.h.hk[i] = kNoKey;
+        for (int i = threadIdx.x; i < (1 << S::FB) / 32; i += THREADS) s.filt[i] = 0;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < d; i += THREADS) {
+        if (A.direct) {
+            s.m.tab[s.L[i] - A.L0] = (uint16_t)(i + 1);
+        } else {
+            if (!BS) hash_put(s.m.h.hk, s.m.h.hv, S::HB, s.L[i], i);
+            const uint32_t h = hash32((uint32_t)s.L[i]) >> (32 - S::FB);
+            atomicOr(&s.filt[h >> 5], 1u << (h & 31));
+        }
+        if (!S::PRE && A.direct && i < d - 1) {  // as offsets into N+(L[i]) (rows are short)
+            const int32_t v = s.L[i];
+            const int64_t b = offp[v], e = offp[v + 1];
+            const int32_t lo = (int32_t)lower_bound_i32(colsp + b, e - b, s.L[i + 1]);
+            s.rel[i] = lo;
+            s.rel[DMAX + i] = lo + (int32_t)lower_bound_i32(colsp + b + lo, e - b - lo, s.L[d - 1] + 1);
+        }
+        if (S::PRE && i < d - 1) {  // every row's probe range at once: dependent loads overlap across rows
+            const int32_t v = s.L[i];
+            const int64_t b = offp[v], e = offp[v + 1];
+            const int64_t lo = b + lower_bound_i32(colsp + b, e - b, s.L[i + 1]);
+            s.rb[i] = lo;
+            s.re[i] = lo + lower_bound_i32(colsp + lo, e - lo, s.L[d - 1] + 1);  // elements <= max L
+        }
+    }
+    __syncthreads();
+    return A;
+}
+
+// index of y in the staged list, or -1
+template <int DMAX, bool BS>
+__device__ __forceinline__ int anchor_find(const CtaSmem<DMAX>& s, const CtaAnchor& A, int32_t y) {
+    if (A.direct) {
+        const uint32_t o = (uint32_t)(y - A.L0);
+        return o < A.span ? (int)s.m.tab[o] - 1 : -1;
+    }
+    return BS ? find_sorted(s.L, A.d, y) : hash_get(s.m.h.hk, s.m.h.hv, CtaSmem<DMAX>::HB, y);
+}
+
+// Row i by a warp: the ordered intersection of N+(L[i]) with L over the exact range of N+(L[i]) in
+// [L[i+1], max L] (no smaller element can be in L after L[i], no larger one at all).  hit(j, p) is called for
+// every j > i with L[j] at position p of colsp; returns this lane's hits summed over the warp.
+template <int DMAX, bool BS, typename Hit>
+__device__ __forceinline__ uint32_t walk_row(const CtaSmem<DMAX>& s, const CtaAnchor& A, const int64_t* __restrict__ offp,
+                                             const int32_t* __restrict__ colsp, int i, FilterChoice& fc, Hit&& hit) {
+    using S = CtaSmem<DMAX>;
+    const int d = A.d, l = lane_id();
+    int64_t b = 0, e = 0;
+    if (S::PRE) {
+        b = s.rb[i];
+        e = s.re[i];
+    } else if (A.direct) {
+        const int64_t o = offp[s.L[i]];
+        b = o + s.rel[i];
+        e = o + s.rel[DMAX + i];
+    } else {
+        const int32_t v = s.L[i];
+        const int64_t e0 = offp[v + 1];
+        b = warp_lower_bound(colsp, offp[v], e0, s.L[i + 1]);
+        e = warp_lower_bound(colsp, b, e0, s.L[d - 1] + 1);
+    }
+    uint32_t hits = 0;
+    if (row_searches(d - 1 - i, e - b)) {  // the keys after L[i] searched in the range
+        const int len = (int)(e - b);
+        for (int j = i + 1 + l; j < d; j += 32) {
+            const int64_t p = find_in_range(colsp, b, len, s.L[j]);
+            if (p >= 0) {
+                hit(j, p);
+                ++hits;
+            }
+        }
+        hits = warp_sum(hits);
+    } else {
+        // the filter is built and used only with the hash or the binary search
+        probe_filtered(colsp, b, e, !A.direct && fc.use(),
+                       [&](int32_t y) { return filter_may_hold<S::FB>(s.filt, y); },
+                       [&](int32_t y, int64_t p) {
+                           const int j = anchor_find<DMAX, BS>(s, A, y);
+                           if (j >= 0) {
+                               hit(j, p);
+                               ++hits;
+                           }
+                       });
+        hits = warp_sum(hits);
+        fc.add(e - b, hits);
+    }
+    return hits;
+}
+
 template <int DMAX, int THREADS, int MINB, bool BS>
 __global__ void __launch_bounds__(THREADS, MINB) k_tri_cta(const int64_t* __restrict__ offp,
                                                      const int32_t* __restrict__ colsp,
@@ -519,107 +638,20 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tri_cta(const int64_t* __rest
         if (tri_class(d, wmax, cmax, bmax) != cls) continue;
         const int W = (d + 31) >> 5;
         const int WS = W | 1;
-        // the direct table where L's span fits (dense anchors: high ranks, close together), the hash else
-        const int32_t L0 = colsp[ub];
-        const uint32_t span = (uint32_t)(colsp[ub + d - 1] - L0) + 1u;
-        const bool direct = !BS && span <= (uint32_t)S::TAB;
-        for (int i = threadIdx.x; i < d; i += THREADS) {
-            s.L[i] = colsp[ub + i];
-            s.own[i] = 0;
-        }
-        for (int i = threadIdx.x; i < d * WS; i += THREADS) s.R[i] = 0;
-        if (direct) {
-            for (int i = threadIdx.x; i < (int)span; i += THREADS) s.m.tab[i] = 0;
-        } else {
-            for (int i = threadIdx.x; i < (1 << S::HB); i += THREADS) s.m.h.hk[i] = kNoKey;
-            for (int i = threadIdx.x; i < (1 << S::FB) / 32; i += THREADS) s.filt[i] = 0;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < d; i += THREADS) {
-            if (direct) {
-                s.m.tab[s.L[i] - L0] = (uint16_t)(i + 1);
-            } else {
-                if (!BS) hash_put(s.m.h.hk, s.m.h.hv, S::HB, s.L[i], i);
-                const uint32_t h = hash32((uint32_t)s.L[i]) >> (32 - S::FB);
-                atomicOr(&s.filt[h >> 5], 1u << (h & 31));
-            }
-            if (!S::PRE && direct && i < d - 1) {  // the same, as offsets into N+(L[i]) (rows are short)
-                const int32_t v = s.L[i];
-                const int64_t b = offp[v], e = offp[v + 1];
-                const int32_t lo = (int32_t)lower_bound_i32(colsp + b, e - b, s.L[i + 1]);
-                s.rel[i] = lo;
-                s.rel[DMAX + i] = lo + (int32_t)lower_bound_i32(colsp + b + lo, e - b - lo, s.L[d - 1] + 1);
-            }
-            if (S::PRE && i < d - 1) {  // every row's probe range at once: dependent loads overlap across rows
-                const int32_t v = s.L[i];
-                const int64_t b = offp[v], e = offp[v + 1];
-                const int64_t lo = b + lower_bound_i32(colsp + b, e - b, s.L[i + 1]);
-                s.rb[i] = lo;
-                s.re[i] = lo + lower_bound_i32(colsp + lo, e - lo, s.L[d - 1] + 1);  // elements <= max L
-            }
-        }
-        __syncthreads();
+        const CtaAnchor A = stage_anchor<DMAX, THREADS, BS>(s, offp, colsp, ub, d, WS);
         const int32_t last = s.L[d - 1];
-        // index of y in L, or -1
-        auto find = [&](int32_t y) {
-            if (direct) {
-                const uint32_t o = (uint32_t)(y - L0);
-                return o < span ? (int)s.m.tab[o] - 1 : -1;
-            }
-            return BS ? find_sorted(s.L, d, y) : hash_get(s.m.h.hk, s.m.h.hv, S::HB, y);
-        };
         auto lookup = [&](int32_t y) {
-            if (!direct && !filter_may_hold<S::FB>(s.filt, y)) return -1;
-            return find(y);
+            if (!A.direct && !filter_may_hold<S::FB>(s.filt, y)) return -1;
+            return anchor_find<DMAX, BS>(s, A, y);
         };
-        // rows: warp per row, ordered intersection of N+(L[i]) with L over the exact range of N+(L[i]) in
-        // [L[i+1], max L] (no smaller element can be in L after L[i], no larger one at all)
-        for (int i = w; i < d - 1; i += NW) {
-            int64_t b = 0, e = 0;
-            if (S::PRE) {
-                b = s.rb[i];
-                e = s.re[i];
-            } else if (direct) {
-                const int64_t o = offp[s.L[i]];
-                b = o + s.rel[i];
-                e = o + s.rel[DMAX + i];
-            } else {
-                const int32_t v = s.L[i];
-                const int64_t e0 = offp[v + 1];
-                b = warp_lower_bound(colsp, offp[v], e0, s.L[i + 1]);
-                e = warp_lower_bound(colsp, b, e0, last + 1);
-            }
+        for (int i = w; i < d - 1; i += NW) {  // a warp per row
             uint32_t* Ri = &s.R[i * WS];
-            uint32_t hits = 0;
-            if (row_searches(d - 1 - i, e - b)) {  // the keys after L[i] searched in the range
-                const int len = (int)(e - b);
-                for (int j = i + 1 + l; j < d; j += 32) {
-                    const int64_t p = find_in_range(colsp, b, len, s.L[j]);
-                    if (p >= 0) {
-                        atomicAdd(&te[p], 1u);  // arc (L[i], L[j]): top edge of triangle (u, L[i], L[j])
-                        atomicOr(&Ri[j >> 5], 1u << (j & 31));
-                        atomicAdd(&s.own[j], 1u);
-                        ++hits;
-                    }
-                }
-                hits = warp_sum(hits);
-            } else {
-                // the filter is built and used only with the hash or the binary search
-                probe_filtered(colsp, b, e, !direct && fc.use(),
-                               [&](int32_t y) { return filter_may_hold<S::FB>(s.filt, y); },
-                               [&](int32_t y, int64_t p) {
-                                   const int j = find(y);
-                                   if (j >= 0) {
-                                       atomicAdd(&te[p], 1u);  // arc (L[i], y): top edge of triangle (u, L[i], y)
-                                       atomicOr(&Ri[j >> 5], 1u << (j & 31));
-                                       atomicAdd(&s.own[j], 1u);
-                                       ++hits;
-                                   }
-                               });
-                hits = warp_sum(hits);
-                fc.add(e - b, hits);
-            }
-            if (l == 0 && hits) atomicAdd(&s.own[i], hits);
+            const uint32_t row_hits = walk_row<DMAX, BS>(s, A, offp, colsp, i, fc, [&](int j, int64_t p) {
+                atomicAdd(&te[p], 1u);  // arc (L[i], L[j]): top edge of triangle (u, L[i], L[j])
+                atomicOr(&Ri[j >> 5], 1u << (j & 31));
+                atomicAdd(&s.own[j], 1u);
+            });
+            if (l == 0 && row_hits) atomicAdd(&s.own[i], row_hits);
         }
         __syncthreads();
         // triangles and 4-cliques (the X_3 extension): the bitmap's (word, row) units are dealt to all the
@@ -930,6 +962,281 @@ __global__ void __launch_bounds__(256) k_tri_fallback(const int64_t* __restrict_
     flush_block(sink, tri, k4, paw, 0, red);
 }
 
+// ---------------------------------------------------------------------------------------------
+// Orbit statistics of the triangles and 4-cliques (orbits.cu), anchored like the counts, after t_e is final.
+// With the symmetric bitmap of G[L], c_ij = |row_i n row_j| is the number of 4-cliques {u, L[i], L[j], .}, so
+// every triangle (u, a = L[i], b = L[j]) at position p of colsp gives, in one visit,
+//   per vertex: N9(u) += t_ab - 1, N9(a) += t_ub - 1, N9(b) += t_ua - 1 (t from t_e); 3 K4(u) += c_ij; and
+//               2 K4(a), 2 K4(b) += c_ij over the anchors u (the 4-cliques on a with u lowest are the
+//               triangles of G[L] through a: half of sum_j c_ij)
+//   per edge:   e5 (sum of d - 2 of the third vertex) and e8 (sum of t - 1 of the other two edges) of its three
+//               edges, e9 (twice the 4-cliques) of (a, b) += 2 c_ij and of (u, a), (u, b) += c_ij.
+// What goes to L[j] is gathered in shared memory, 16 bits of the value to each of two words (at most 1024
+// terms), and added to global memory once per anchor; only the (a, b) edge needs an atomic per triangle.
+// (A warp per edge that walked the common neighbours per triangle took 13.2 ms on R-MAT scale 15.)
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void split_add(uint32_t* lo, uint32_t* hi, int j, uint32_t v) {
+    atomicAdd(&lo[j], v & 0xffffu);
+    if (v >> 16) atomicAdd(&hi[j], v >> 16);
+}
+__device__ __forceinline__ uint64_t split_sum(const uint32_t* lo, const uint32_t* hi, int j) {
+    return (uint64_t)lo[j] + ((uint64_t)hi[j] << 16);
+}
+__device__ __forceinline__ void add_u64(unsigned long long* p, uint64_t v) {
+    if (v) atomicAdd(p, (unsigned long long)v);
+}
+
+// Warp-local anchors (2 <= d <= 32): every (row, key) pair searched once, its position kept in shared memory
+// while the bitmap is completed.
+constexpr int kOrbWarps = 8;
+
+template <bool EDGE>
+__global__ void __launch_bounds__(kOrbWarps * 32) k_orb_tri_warp(const int64_t* __restrict__ offp,
+                                                                 const int32_t* __restrict__ colsp,
+                                                                 const int32_t* __restrict__ deg,
+                                                                 const uint32_t* __restrict__ te,
+                                                                 const int32_t* __restrict__ q,
+                                                                 const unsigned long long* __restrict__ cnt, OrbTri o) {
+    __shared__ int32_t s_L[kOrbWarps][32], s_pos[kOrbWarps][32 * 31 / 2];
+    __shared__ uint32_t s_row[kOrbWarps][32], s_k[kOrbWarps][32], s_t[kOrbWarps][32], s_d[kOrbWarps][32];
+    __shared__ uint32_t s_lo[kOrbWarps][32], s_hi[kOrbWarps][32], s_lo2[kOrbWarps][32], s_hi2[kOrbWarps][32];
+    const int w = threadIdx.x >> 5, l = lane_id();
+    const int64_t nq = (int64_t)cnt[0];
+    for (int64_t k = (int64_t)blockIdx.x * kOrbWarps + w; k < nq; k += (int64_t)gridDim.x * kOrbWarps) {
+        const int32_t u = q[k];
+        const int64_t ub = offp[u];
+        const int d = (int)(offp[u + 1] - ub);
+        const int32_t x = l < d ? colsp[ub + l] : 0;
+        int64_t b = 0;
+        int len = 0;
+        if (l < d) {
+            b = offp[x];
+            len = (int)(offp[x + 1] - b);
+        }
+        s_L[w][l] = x;
+        s_row[w][l] = s_k[w][l] = s_lo[w][l] = s_hi[w][l] = s_lo2[w][l] = s_hi2[w][l] = 0;
+        s_t[w][l] = l < d ? te[ub + l] - 1u : 0u;  // used only where the edge has a triangle
+        s_d[w][l] = l < d ? (uint32_t)deg[x] - 2u : 0u;
+        __syncwarp();
+        // pairs (i, j), i < j, flattened: row i's first pair is excl(i)
+        const int npairs = l < d ? d - 1 - l : 0;
+        int incl = npairs;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const int y = __shfl_up_sync(kFull, incl, s);
+            if (l >= s) incl += y;
+        }
+        const int excl = incl - npairs;
+        const int total = d * (d - 1) / 2;
+        auto each_pair = [&](auto&& f) {
+            for (int t0 = 0; t0 < total; t0 += 32) {
+                const int t = t0 + l;
+                int i = 0;
+#pragma unroll
+                for (int s = 16; s >= 1; s >>= 1) {
+                    const int e = __shfl_sync(kFull, excl, i + s);
+                    if (i + s < d && e <= t) i += s;
+                }
+                const int64_t rb = __shfl_sync(kFull, b, i);
+                const int rl = __shfl_sync(kFull, len, i), e = __shfl_sync(kFull, excl, i);
+                if (t < total) f(t, i, i + 1 + (t - e), rb, rl);
+            }
+        };
+        each_pair([&](int t, int i, int j, int64_t rb, int rl) {
+            const int64_t p = find_in_range(colsp, rb, rl, s_L[w][j]);
+            s_pos[w][t] = p < 0 ? -1 : (int32_t)(p - rb);
+            if (p >= 0) {
+                atomicOr(&s_row[w][i], 1u << j);
+                atomicOr(&s_row[w][j], 1u << i);
+            }
+        });
+        __syncwarp();
+        uint64_t n9u = 0, k3u = 0;
+        const uint32_t du2 = (uint32_t)deg[u] - 2u;
+        each_pair([&](int t, int i, int j, int64_t rb, int) {
+            const int32_t rel = s_pos[w][t];
+            if (rel < 0) return;
+            const int64_t p = rb + rel;
+            const uint32_t c = (uint32_t)__popc(s_row[w][i] & s_row[w][j]);
+            const uint32_t ti = s_t[w][i], tj = s_t[w][j], tp = te[p] - 1u;
+            if (c) {
+                atomicAdd(&s_k[w][i], c);
+                atomicAdd(&s_k[w][j], c);
+            }
+            if (EDGE) {
+                split_add(s_lo[w], s_hi[w], i, s_d[w][j]);
+                split_add(s_lo[w], s_hi[w], j, s_d[w][i]);
+                split_add(s_lo2[w], s_hi2[w], i, tp);
+                split_add(s_lo2[w], s_hi2[w], i, tj);
+                split_add(s_lo2[w], s_hi2[w], j, tp);
+                split_add(s_lo2[w], s_hi2[w], j, ti);
+                add_u64(&o.e5[p], du2);
+                add_u64(&o.e8[p], (uint64_t)ti + tj);
+                add_u64(&o.e9[p], 2ull * c);
+            } else {
+                split_add(s_lo[w], s_hi[w], i, tj);
+                split_add(s_lo[w], s_hi[w], j, ti);
+                n9u += tp;
+                k3u += c;
+            }
+        });
+        __syncwarp();
+        if (l < d) {
+            if (EDGE) {
+                add_u64(&o.e5[ub + l], split_sum(s_lo[w], s_hi[w], l));
+                add_u64(&o.e8[ub + l], split_sum(s_lo2[w], s_hi2[w], l));
+                add_u64(&o.e9[ub + l], s_k[w][l]);
+            } else {
+                add_u64(&o.n9[x], split_sum(s_lo[w], s_hi[w], l));
+                add_u64(&o.tau6[x], 3ull * s_k[w][l]);
+            }
+        }
+        if (!EDGE) {
+            n9u = warp_sum(n9u);
+            k3u = warp_sum(k3u);
+            if (l == 0) {
+                add_u64(&o.n9[u], n9u);
+                add_u64(&o.tau6[u], 2 * k3u);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+template <int DMAX>
+struct OrbSmem {
+    CtaSmem<DMAX> c;
+    uint32_t t[DMAX], d[DMAX];                            // t_e - 1 of (u, L[i]) and deg - 2 of L[i]
+    uint32_t lo[DMAX], hi[DMAX], lo2[DMAX], hi2[DMAX];
+};
+
+template <int DMAX, int THREADS, bool EDGE>
+__global__ void __launch_bounds__(THREADS) k_orb_tri_cta(const int64_t* __restrict__ offp,
+                                                         const int32_t* __restrict__ colsp,
+                                                         const int32_t* __restrict__ deg, const uint32_t* __restrict__ te,
+                                                         const int32_t* __restrict__ q, int64_t n, int cls,
+                                                         const unsigned long long* __restrict__ cnt,
+                                                         unsigned long long* __restrict__ ticket, OrbTri o) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    OrbSmem<DMAX>& s = *reinterpret_cast<OrbSmem<DMAX>*>(smem_raw);
+    __shared__ int64_t s_item;
+    constexpr int NW = THREADS / 32;
+    const int w = threadIdx.x >> 5, l = lane_id();
+    const int64_t nq = (int64_t)cnt[1];
+    FilterChoice fc;
+    for (;;) {
+        if (threadIdx.x == 0) s_item = (int64_t)atomicAdd(ticket, 1ull);
+        __syncthreads();
+        const int64_t k = s_item;
+        __syncthreads();
+        if (k >= nq) break;
+        const int32_t u = q[n - 1 - k];
+        const int64_t ub = offp[u];
+        const int d = (int)(offp[u + 1] - ub);
+        if (tri_class(d, 32, kCtaMax, kBigMax) != cls) continue;
+        const int W = (d + 31) >> 5;
+        const int WS = W | 1;
+        for (int i = threadIdx.x; i < d; i += THREADS) {
+            s.t[i] = te[ub + i] - 1u;
+            s.d[i] = (uint32_t)deg[colsp[ub + i]] - 2u;
+            s.lo[i] = s.hi[i] = s.lo2[i] = s.hi2[i] = 0;
+        }
+        const CtaAnchor A = stage_anchor<DMAX, THREADS, false>(s.c, offp, colsp, ub, d, WS);
+        for (int i = w; i < d - 1; i += NW)
+            walk_row<DMAX, false>(s.c, A, offp, colsp, i, fc, [&](int j, int64_t) {
+                atomicOr(&s.c.R[i * WS + (j >> 5)], 1u << (j & 31));
+                atomicOr(&s.c.R[j * WS + (i >> 5)], 1u << (i & 31));
+            });
+        __syncthreads();
+        uint64_t n9u = 0, k3u = 0;
+        const uint32_t du2 = (uint32_t)deg[u] - 2u;
+        for (int i = w; i < d - 1; i += NW) {
+            const uint32_t* Ri = &s.c.R[i * WS];
+            const uint32_t ti = s.t[i];
+            uint64_t a5 = 0, a8 = 0;  // to L[i]: N9, or e5 and e8
+            uint32_t ki = 0;
+            walk_row<DMAX, false>(s.c, A, offp, colsp, i, fc, [&](int j, int64_t p) {
+                const uint32_t* Rj = &s.c.R[j * WS];
+                uint32_t c = 0;
+                for (int y = 0; y < W; ++y) c += __popc(Ri[y] & Rj[y]);
+                const uint32_t tj = s.t[j], tp = te[p] - 1u;
+                if (c) atomicAdd(&s.c.own[j], c);
+                ki += c;
+                if (EDGE) {
+                    a5 += s.d[j];
+                    a8 += (uint64_t)tp + tj;
+                    split_add(s.lo, s.hi, j, s.d[i]);
+                    split_add(s.lo2, s.hi2, j, tp);
+                    split_add(s.lo2, s.hi2, j, ti);
+                    add_u64(&o.e5[p], du2);
+                    add_u64(&o.e8[p], (uint64_t)ti + tj);
+                    add_u64(&o.e9[p], 2ull * c);
+                } else {
+                    a5 += tj;
+                    split_add(s.lo, s.hi, j, ti);
+                    n9u += tp;
+                }
+            });
+            if (!EDGE) k3u += ki;
+            ki = warp_sum(ki);
+            a5 = warp_sum(a5);
+            if (EDGE) a8 = warp_sum(a8);
+            if (l == 0) {
+                if (ki) atomicAdd(&s.c.own[i], ki);
+                if (EDGE) {
+                    add_u64(&o.e5[ub + i], a5);
+                    add_u64(&o.e8[ub + i], a8);
+                } else {
+                    add_u64(&o.n9[s.c.L[i]], a5);
+                }
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < d; i += THREADS) {
+            if (EDGE) {
+                add_u64(&o.e5[ub + i], split_sum(s.lo, s.hi, i));
+                add_u64(&o.e8[ub + i], split_sum(s.lo2, s.hi2, i));
+                add_u64(&o.e9[ub + i], s.c.own[i]);
+            } else {
+                add_u64(&o.n9[s.c.L[i]], split_sum(s.lo, s.hi, i));
+                add_u64(&o.tau6[s.c.L[i]], 3ull * s.c.own[i]);
+            }
+        }
+        if (!EDGE) {
+            n9u = block_sum_u64(n9u, s.c.red);
+            k3u = block_sum_u64(k3u, s.c.red);
+            if (threadIdx.x == 0) {
+                add_u64(&o.n9[u], n9u);
+                add_u64(&o.tau6[u], 2 * k3u);
+            }
+        }
+        __syncthreads();  // the shared arrays are read before the next anchor fills them
+    }
+}
+
+template <int DMAX, int THREADS, bool EDGE>
+harp_status launch_orb_cta(const harp_csr* g, Workspace& ws, int cls, int ticket_slot, int per_sm, const OrbTri& o,
+                           cudaStream_t s) {
+    const size_t smem = sizeof(OrbSmem<DMAX>);
+    HARP_CK(cudaFuncSetAttribute(k_orb_tri_cta<DMAX, THREADS, EDGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_orb_tri_cta<DMAX, THREADS, EDGE><<<num_sms() * per_sm, THREADS, smem, s>>>(
+        ws.offp, ws.colsp, ws.deg, ws.te, ws.q_tri, g->n, cls, (const unsigned long long*)&ws.acc[Q_TRI_WARP],
+        (unsigned long long*)&ws.acc[ticket_slot], o);
+    HARP_LAUNCHED();
+    return HARP_OK;
+}
+
+template <bool EDGE>
+harp_status orbit_tiers(const harp_csr* g, Workspace& ws, const OrbTri& o, int64_t dmax, cudaStream_t s) {
+    k_orb_tri_warp<EDGE><<<num_sms() * 8, kOrbWarps * 32, 0, s>>>(ws.offp, ws.colsp, ws.deg, ws.te, ws.q_tri,
+                                                                  (const unsigned long long*)&ws.acc[Q_TRI_WARP], o);
+    HARP_LAUNCHED();
+    if (dmax > 32) HARP_TRY((launch_orb_cta<kCta1, 256, EDGE>(g, ws, 1, T_TRI_S, 5, o, s)));
+    if (dmax > kCta1) HARP_TRY((launch_orb_cta<kCta2, 256, EDGE>(g, ws, 2, T_TRI_M, 3, o, s)));
+    if (dmax > kCta2) HARP_TRY((launch_orb_cta<kCtaMax, 512, EDGE>(g, ws, 3, T_TRI_L, 1, o, s)));
+    return HARP_OK;
+}
+
 template <int DMAX, int THREADS, int MINB, bool BS>
 harp_status launch_cta(const harp_csr* g, Workspace& ws, int cls, int ticket_slot, int wmax, int cmax, int bmax,
                        bool reuse, cudaStream_t s) {
@@ -969,6 +1276,19 @@ harp_status launch_tiers(const harp_csr* g, Workspace& ws, int wmax, int cmax, i
 
 }  // namespace
 
+int64_t max_out_degree(const harp_csr* g) {
+    int64_t dmax = 1;
+    while (dmax * dmax < 2 * g->m) ++dmax;
+    return dmax > g->max_deg ? g->max_deg : dmax;
+}
+
+harp_status orbit_triangles(const harp_csr* g, Workspace& ws, const OrbTri& o, cudaStream_t s) {
+    // the tickets of the triangle pass (slots T_TRI_S .. T_TRI_M) start again
+    HARP_CK(cudaMemsetAsync(&ws.acc[T_TRI_S], 0, sizeof(uint64_t) * (T_TRI_M - T_TRI_S + 1), s));
+    const int64_t dmax = max_out_degree(g);
+    return o.n9 ? orbit_tiers<false>(g, ws, o, dmax, s) : orbit_tiers<true>(g, ws, o, dmax, s);
+}
+
 // acc[Q_TRI_WARP], acc[Q_TRI_CTA] hold the queue lengths, acc[T_TRI_*] the CTA tickets (all cleared
 // with the accumulators before the count).
 harp_status count_triangles_k4(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s) {
@@ -989,9 +1309,7 @@ harp_status count_triangles_k4(const harp_csr* g, Workspace& ws, const harp_plan
     const Sink sink{ws.acc, ws.gid, ws.accG};
     HARP_TRY(launch_tiers(g, ws, wmax, cmax, bmax, reuse, plan.tri_probe_bin, s));
     // the largest possible out-degree is bounded by sqrt(2m) and by the maximum degree
-    int64_t dmax = 1;
-    while (dmax * dmax < 2 * g->m) ++dmax;
-    if (dmax > g->max_deg) dmax = g->max_deg;
+    const int64_t dmax = max_out_degree(g);
     if (dmax > cmax && bmax > cmax) {  // global-staged tier: one block per SM, scratch of kBigMax rows
         const size_t bytes = (size_t)num_sms() * kBigMax * kBigWords * sizeof(uint32_t);
         uint32_t* scratch = nullptr;
