@@ -100,6 +100,7 @@ struct harp_batch {
     cudaStream_t capture_stream = nullptr;
     int64_t G = 0;
     std::vector<int64_t> m_of;        // per-member m (host)
+    int64_t max_n = 0;                // most vertices of one member
     harp_csr u;                       // the union (owns off/cols + workspace)
     MemberDesc* d_desc = nullptr;
     int32_t* d_gid_in = nullptr;      // [N]
@@ -196,6 +197,7 @@ harp_status harp_batch_create(const harp_csr* const* graphs, int64_t G, harp_bat
         desc[(size_t)g] = MemberDesc{c->off, c->cols, c->n, vb, ab, blocks};
         gbase[(size_t)g] = vb;
         b->m_of[(size_t)g] = c->m;
+        if (c->n > b->max_n) b->max_n = c->n;
         vb += c->n;
         ab += 2 * c->m;
         blocks += union_blocks(c->n, 2 * c->m);
@@ -254,6 +256,7 @@ harp_status batch_prepare(harp_batch* b, const harp_plan& plan) {
     b->u.ws.gid = b->d_gid;
     b->u.ws.accG = b->d_accG;
     b->u.ws.G = b->G;
+    b->u.ws.max_member_n = b->max_n;
     b->u.ws.max_member_m = b->G > 0 ? *std::max_element(b->m_of.begin(), b->m_of.end()) : 0;
     b->u.ws.gbase = b->d_gbase;
     b->u.ws.ginfo = b->d_ginfo;

@@ -72,10 +72,10 @@ enum : int {
     Q_C4_WIN = 29,
     T_TRI_S = 30,          // work tickets of persistent kernels
     T_TRI_L = 31,
-    T_TRI_F = 32,
-    T_C4_MID = 33,
+    T_C4_MID = 32,
+    T_C4_LIGHT = 33,
     T_C4_WIN = 34,
-    W_TOTAL = 35,          // total window items of the windowed wedge kernel
+    T_TRI_W = 35,          // ticket of the warp triangle kernel
     Q_SORT_CTA = 36,       // rows for the CTA row sort (36) and the hub row sort (37)
     T_TRI_M = 38,          // ticket of the 512-wide CTA triangle kernel
     ACC_SIG_HITS = 39,     // 4-clique extensions answered by a staged signature frontier
@@ -160,7 +160,8 @@ struct Workspace {
     uint64_t* acc = nullptr;       // [kOutLen]
     // batch mode only (the union of many graphs); nullptr for a single graph
     int64_t G = 1;                    // graphs
-    int64_t max_member_m = 0;         // most edges of one graph
+    int64_t max_member_m = 0;         // most edges and vertices of one graph
+    int64_t max_member_n = 0;
     const int64_t* gbase = nullptr;   // [G+1] first vertex of each graph (ranks and input ids alike)
     const int32_t* gid_in = nullptr;  // [n] graph of each input (union) vertex
     int32_t* gid = nullptr;           // [n] graph of each rank-order vertex
