@@ -102,7 +102,9 @@ enum : int {
     T_CORE_L = 61,
     T_CORE_XL = 62,
     A_CORE_ANY = 63,       // graphs that have a wedge core
-    kOutLen = 64
+    ACC_LIT_CORR = 64,     // 64 lo, 65 hi: what the staged edge pass counts too much (literal.cu)
+    T_LIT_EDGE = 66,       // its ticket
+    kOutLen = 72
 };
 
 // Bits of acc[ACC_ERR].  Any set bit makes a blocking count return HARP_EDEVICE; the asynchronous
