@@ -85,13 +85,19 @@ __host__ __device__ constexpr int32_t band_max_degree(int b) {
     return band_width(b) >= 31 ? INT32_MAX : (int32_t)((1u << band_width(b)) - 1u);
 }
 
-__device__ __forceinline__ int64_t first_above_in(const int32_t* __restrict__ deg, int64_t lo, int64_t hi, int32_t t) {
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (deg[mid] <= t) lo = mid + 1;
-        else hi = mid;
+// first position in [lo, hi) of the ascending deg above t, by a whole warp (32 probes a round)
+__device__ __forceinline__ int64_t warp_first_above(const int32_t* __restrict__ deg, int64_t lo, int64_t hi, int32_t t) {
+    const int l = lane_id();
+    while (hi - lo > 32) {
+        const int64_t step = (hi - lo + 31) >> 5;
+        const int64_t i = lo + (int64_t)(l + 1) * step - 1;
+        const uint32_t m = __ballot_sync(kFull, i >= hi || deg[i] > t);
+        if (!m) return hi;
+        lo += (int64_t)(__ffs(m) - 1) * step;
+        hi = lo + step < hi ? lo + step : hi;
     }
-    return lo;
+    const uint32_t m = __ballot_sync(kFull, lo + l < hi && deg[lo + l] > t);
+    return m ? lo + __ffs(m) - 1 : hi;
 }
 
 // x-values one window of band b covers: the window's words times counters per word
@@ -211,6 +217,7 @@ __global__ void __launch_bounds__(kGinfoThreads) k_c4_ginfo(const int32_t* __res
                                                             int64_t x_hi, bool merge, const int64_t* __restrict__ off,
                                                             int64_t* __restrict__ ginfo, uint64_t* __restrict__ acc) {
     __shared__ uint64_t s_score[kGinfoWarps][kMergeMasks];
+    __shared__ int64_t s_rank[kBands + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t g = blockIdx.x; g < G; g += gridDim.x) {
         const int64_t lo = gbase ? gbase[g] : 0, gend = gbase ? gbase[g + 1] : n;
@@ -222,23 +229,28 @@ __global__ void __launch_bounds__(kGinfoThreads) k_c4_ginfo(const int32_t* __res
         }
         auto clamp = [&](int64_t v) { return v < x_lo ? x_lo : (v > x_hi ? x_hi : v); };
         const int64_t hi = gend < x_hi ? gend : x_hi;
-        // lane 0: n1 (first rank of degree >= 2); lane b < kBands: the first rank above band b - 1's
-        // degrees (band b's start); lane kBands: the first rank of degree >= 64.  One search each.
-        const int32_t t = lane == 0 ? 1 : (lane < kBands ? band_max_degree(lane - 1) : 63);
-        const int64_t r_lane = lane <= kBands ? first_above_in(deg, lo, gend, t) : gend;
-        int64_t n1 = clamp(__shfl_sync(0xffffffffu, r_lane, 0));
+        // threshold 0: n1 (first rank of degree >= 2); b < kBands: the first rank above band b - 1's degrees
+        // (band b's start); kBands: the first rank of degree >= 64.  A warp-wide search each.
+        for (int b = warp; b <= kBands; b += kGinfoWarps) {
+            const int64_t r = warp_first_above(deg, lo, gend, b == 0 ? 1 : (b < kBands ? band_max_degree(b - 1) : 63));
+            if (lane == 0) s_rank[b] = r;
+        }
+        __syncthreads();
+        int64_t n1 = clamp(s_rank[0]);
         n1 = n1 < hi ? n1 : hi;
         int64_t st[kBands + 1];
         st[0] = n1;
         st[kBands] = hi;
 #pragma unroll
         for (int b = 1; b < kBands; ++b) {
-            const int64_t r = clamp(__shfl_sync(0xffffffffu, r_lane, b));
+            const int64_t r = clamp(s_rank[b]);
             st[b] = r > n1 ? (r < hi ? r : hi) : n1;
         }
         unsigned best_mask = 0;  // mask 0: every band separate
-        if (merge) {             // uniform over the block (a kernel argument)
-            int64_t s0 = __shfl_sync(0xffffffffu, r_lane, kBands);
+        if (merge && hi - n1 <= WORDS) {
+            best_mask = kMergeMasks - 1;  // all in one window of 32-bit counters
+        } else if (merge) {               // uniform over the block
+            int64_t s0 = s_rank[kBands];
             if (s0 >= gend) s0 = lo;
             const int64_t span = gend - s0;  // samples u lie in [s0, gend); none for an empty graph
             constexpr int kPer = kMergeSamples / kGinfoWarps;  // this warp's samples, one per lane
@@ -278,8 +290,8 @@ __global__ void __launch_bounds__(kGinfoThreads) k_c4_ginfo(const int32_t* __res
                     }
                 }
             }
-            __syncthreads();  // the scores are read before the next graph's are written
         }
+        __syncthreads();  // the scores and ranks are read before the next graph's are written
         if (threadIdx.x == 0) {
 #pragma unroll
             for (int b = 0; b + 1 < kBands; ++b)

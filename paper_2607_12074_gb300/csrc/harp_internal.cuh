@@ -76,7 +76,7 @@ enum : int {
     T_C4_LIGHT = 33,
     T_C4_WIN = 34,
     T_TRI_W = 35,          // ticket of the warp triangle kernel
-    Q_SORT_CTA = 36,       // rows for the CTA row sort (36) and the hub row sort (37)
+    Q_SORT_WARP = 36,      // rows for the warp (36) and the hub (37) row sort; Q_SORT_BLOCK
     T_TRI_M = 38,          // ticket of the 512-wide CTA triangle kernel
     ACC_SIG_HITS = 39,     // 4-clique extensions answered by a staged signature frontier
     Q_TRI_FB = 40,         // length of the unstaged-fallback triangle queue
@@ -104,6 +104,7 @@ enum : int {
     A_CORE_ANY = 63,       // graphs that have a wedge core
     ACC_LIT_CORR = 64,     // 64 lo, 65 hi: what the staged edge pass counts too much (literal.cu)
     T_LIT_EDGE = 66,       // its ticket
+    Q_SORT_BLOCK = 67,     // rows for the block row sort
     kOutLen = 72
 };
 
@@ -325,6 +326,21 @@ struct Sink {
 __device__ __forceinline__ void sink_add(const Sink& s, int32_t anchor, int gslot, uint64_t v) {
     if (v) atomicAdd((unsigned long long*)&s.accG[(int64_t)s.gid[anchor] * kGStride + gslot],
                      (unsigned long long)v);
+}
+
+// Lane values v of graphs g (any lanes may hold v = 0), by a whole warp: one atomic per graph present among the
+// lanes that hold a value.  One per lane would serialise on the slot of a large graph.
+__device__ __forceinline__ void warp_add_by_graph(uint64_t* accG, int gslot, int32_t g, uint64_t v) {
+    uint32_t left = __ballot_sync(kFull, v != 0);
+    while (left) {  // one graph per round: the first lane still holding a value names it
+        const int src = __ffs(left) - 1;
+        const int32_t gs = __shfl_sync(kFull, g, src);
+        const bool mine = ((left >> lane_id()) & 1u) && g == gs;
+        const uint64_t sum = warp_sum(mine ? v : (uint64_t)0);
+        if (lane_id() == src)
+            atomicAdd((unsigned long long*)&accG[(int64_t)gs * kGStride + gslot], (unsigned long long)sum);
+        left &= ~__ballot_sync(kFull, mine);
+    }
 }
 
 // lower_bound in a sorted int32 array a[0..len): first index with a[i] >= key

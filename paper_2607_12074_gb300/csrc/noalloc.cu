@@ -122,9 +122,10 @@ extern "C" harp_status harp_count4_noalloc(int64_t n, int64_t m, const int64_t* 
     if (carve(base, kNoAllocBytes, n, m, ws) == 0) return HARP_ENOMEM;
     harp_plan plan;
     normalise_plan(nullptr, &plan);
-    // every accumulator, queue counter and ticket starts at zero; the kernels clear t_e and the
-    // window counts themselves
+    // every accumulator, queue counter and ticket starts at zero; t_e too: the kernels clear it by out-arcs, and
+    // a CSR that fails its check has none
     HARP_CK(cudaMemsetAsync(ws.acc, 0, sizeof(uint64_t) * kOutLen, s));
+    HARP_CK(cudaMemsetAsync(ws.te, 0, sizeof(uint32_t) * (size_t)(m > 0 ? m : 1), s));
     k_check_offsets<<<check_grid(n + 1), 256, 0, s>>>(d_offsets, n, m, ws.acc);
     HARP_LAUNCHED();
     if (m > 0) {

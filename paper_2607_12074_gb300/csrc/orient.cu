@@ -10,17 +10,17 @@
 // every row sorted), dplus, offp/colsp (out-CSR: only N+), te zeroed, S = sum_v C(d_v, 3).
 //
 // Rows are sorted by four kernels chosen by degree: for d <= 32 a lane's bitonic network in registers
-// (d <= 16) or the warp's over its lanes (every row is visited), a warp bitonic sort in the warp's
-// shared buffer for d <= 256, a block bitonic sort in shared memory for d <= 4096 and a per-row LSD
-// radix sort through global memory for hubs (the last three from queues filled by the relabel pass;
-// the warp and block sorts share one).
+// (d <= 16) or the warp's over its lanes (every row is visited), a warp's bitonic network over up to 32
+// registers a lane for d <= 1024, a block's for d <= 4096 (16 warps' networks joined through shared memory),
+// and for hubs a bitmap of the ranks, or a per-row LSD radix sort through global memory where the graph
+// has too many ranks for one (the last three from queues filled by the relabel pass).
 #include "harp_internal.cuh"
 
 namespace harp {
 namespace {
 
 constexpr int kTierA = 32;
-constexpr int kTierB1 = 256;
+constexpr int kTierB1 = 1024;
 constexpr int kTierB = 4096;
 
 int bits_for(int64_t x) {
@@ -44,29 +44,32 @@ __global__ void k_vertex_keys(const int64_t* __restrict__ off, int64_t n, int b,
     // a caller-built CSR that failed its check (harp_count4_noalloc) is counted as edgeless: every
     // later kernel then stays inside the arrays sized for its (n, m)
     const bool bad_csr = (acc[ACC_ERR] & kErrBadCsr) != 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t d = bad_csr ? 0 : (uint64_t)(off[v + 1] - off[v]);
-        const uint64_t g = gid_in ? (uint64_t)gid_in[v] : 0;
-        keys[v] = (g << (bd + b)) | (d << b) | (uint64_t)v;
-        const uint64_t c3 = choose3_u64(d);
-        if (gid_in) {
-            if (c3) atomicAdd((unsigned long long*)&accG[(int64_t)gid_in[v] * kGStride + G_S], (unsigned long long)c3);
-        } else {
-            s3 += c3;
+    const int l = lane_id();
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - l; base < n;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = base + l;
+        uint64_t c3 = 0;
+        int32_t g = 0;
+        if (v < n) {
+            const uint64_t d = bad_csr ? 0 : (uint64_t)(off[v + 1] - off[v]);
+            if (gid_in) g = gid_in[v];
+            keys[v] = ((uint64_t)g << (bd + b)) | (d << b) | (uint64_t)v;
+            c3 = choose3_u64(d);
         }
+        if (gid_in) warp_add_by_graph(accG, G_S, g, c3);
+        else s3 += c3;
     }
     __shared__ uint64_t red[32];
     uint64_t t = block_sum_u64(s3, red);
     if (threadIdx.x == 0 && t) atomicAdd((unsigned long long*)&acc[ACC_S], (unsigned long long)t);
 }
 
-// New ids = sorted key order.  Rows that need the CTA or hub sort are queued (q: CTA rows from the
-// front, hub rows from the back); the warp sort takes every other row directly.
+// New ids = sorted key order.  Rows of more than kTierA neighbours are queued: q holds the warp sort's rows from
+// the front and hub rows from the back, q_block the block sort's.
 __global__ void k_relabel(const uint64_t* __restrict__ keys, int64_t n, int b, int bd, int32_t* __restrict__ order,
                           int32_t* __restrict__ perm, int32_t* __restrict__ deg,
                           const int32_t* __restrict__ gid_in, int32_t* __restrict__ gid,
-                          int32_t* __restrict__ q, unsigned long long* __restrict__ qcnt) {
+                          int32_t* __restrict__ q, int32_t* __restrict__ q_block, uint64_t* __restrict__ acc) {
     const uint64_t mask = ((uint64_t)1 << b) - 1;
     const uint64_t dmask = ((uint64_t)1 << bd) - 1;
     const int l = lane_id();
@@ -82,20 +85,22 @@ __global__ void k_relabel(const uint64_t* __restrict__ keys, int64_t n, int b, i
             perm[old] = (int32_t)i;
             deg[i] = d;
             if (gid_in) gid[i] = gid_in[old];
-            cls = d > kTierB ? 1 : (d > kTierA ? 0 : -1);
+            cls = d > kTierB ? 1 : (d > kTierB1 ? 2 : (d > kTierA ? 0 : -1));
         }
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
+        for (int c = 0; c < 3; ++c) {
             const uint32_t m = __ballot_sync(kFull, cls == c);
             if (!m) continue;
             unsigned long long start = 0;
             const int leader = __ffs(m) - 1;
-            if (l == leader) start = atomicAdd(&qcnt[c], (unsigned long long)__popc(m));
+            unsigned long long* ctr = (unsigned long long*)&acc[c == 2 ? Q_SORT_BLOCK : Q_SORT_WARP + c];
+            if (l == leader) start = atomicAdd(ctr, (unsigned long long)__popc(m));
             start = __shfl_sync(kFull, start, leader);
             if (cls == c) {
                 const unsigned long long k = start + __popc(m & lanemask_lt());
                 if (c == 0) q[k] = (int32_t)i;
-                else q[n - 1 - (int64_t)k] = (int32_t)i;
+                else if (c == 1) q[n - 1 - (int64_t)k] = (int32_t)i;
+                else q_block[k] = (int32_t)i;
             }
         }
     }
@@ -164,139 +169,307 @@ __global__ void __launch_bounds__(256) k_sort_rows_warp(const int64_t* __restric
         if (d == 0) dplus[i] = 0;
         else if (d >= 1 && d <= 8) lane_sort_row<8>(i, d, goff, gcols, order, perm, off, cols, dplus);
         else if (d > 8 && d <= 16) lane_sort_row<16>(i, d, goff, gcols, order, perm, off, cols, dplus);
-        uint32_t rest = __ballot_sync(kFull, d > 16 && d <= kTierA);
-        while (rest) {
-            const int src = __ffs(rest) - 1;
-            rest &= rest - 1;
-            const int64_t r = i0 + src;
-            const int dr = __shfl_sync(kFull, d, src);
-            const int64_t rsrc = goff[order[r]];
-            int32_t v = (l < dr) ? perm[gcols[rsrc + l]] : 0x7fffffff;
+        const bool wide = d > 16 && d <= kTierA;
+        uint32_t rest = __ballot_sync(kFull, wide);
+        if (!rest) continue;
+        const int64_t mysrc = wide ? goff[order[i]] : 0, myoff = wide ? off[i] : 0;
+        while (rest) {  // four rows at a time: their loads overlap
+            int row[4], dr[4];
+            int32_t v[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                row[t] = rest ? __ffs(rest) - 1 : -1;
+                rest &= rest - 1;
+                dr[t] = row[t] >= 0 ? __shfl_sync(kFull, d, row[t] & 31) : 0;
+                const int64_t rsrc = __shfl_sync(kFull, mysrc, row[t] & 31);
+                v[t] = l < dr[t] ? gcols[rsrc + l] : -1;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) v[t] = v[t] >= 0 ? perm[v[t]] : 0x7fffffff;
 #pragma unroll
             for (int k = 2; k <= 32; k <<= 1) {
 #pragma unroll
                 for (int j = k >> 1; j > 0; j >>= 1) {
-                    int32_t o = __shfl_xor_sync(kFull, v, j);
-                    bool up = (l & k) == 0;
-                    bool lower = (l & j) == 0;
-                    v = (lower == up) ? min(v, o) : max(v, o);
+                    const bool keep_min = ((l & j) == 0) == ((l & k) == 0);
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const int32_t o = __shfl_xor_sync(kFull, v[t], j);
+                        v[t] = keep_min ? min(v[t], o) : max(v[t], o);
+                    }
                 }
             }
-            if (l < dr) cols[off[r] + l] = v;
-            uint32_t above = __ballot_sync(kFull, l < dr && v > (int32_t)r);
-            if (l == 0) dplus[r] = __popc(above);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                if (row[t] < 0) continue;  // uniform
+                const int64_t r = i0 + row[t];
+                const int64_t ob = __shfl_sync(kFull, myoff, row[t]);
+                if (l < dr[t]) cols[ob + l] = v[t];
+                const uint32_t above = __ballot_sync(kFull, l < dr[t] && v[t] > (int32_t)r);
+                if (l == 0) dplus[r] = __popc(above);
+            }
         }
     }
 }
 
-// Tier B1: 32 < d <= 256, one warp per row, bitonic sort in the warp's shared buffer (a block per
-// row would leave most of its warps idle behind a block barrier at every stage).
-constexpr int kMidWarps = 8;
+// Bitonic network over 32 * E keys held by a warp, key lane * E + e in register e: steps of stride below E stay in
+// a lane's registers, the others exchange over the lanes.  Sorts blocks of 2, 4, .. up to 32 * E; up: the final
+// order of the whole (descending where false, for a larger network's alternate halves).
+template <int E>
+__device__ __forceinline__ void bitonic_step(int32_t (&v)[E], int j, bool up_all, int k) {
+    const int l = lane_id();
+    if (j >= E) {
+        const int jl = j / E;
+        const bool lower = (l & jl) == 0;
+        const bool up = k >= 32 * E ? up_all : ((l * E) & k) == 0;  // k > j >= E: a bit of the lane
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int32_t o = __shfl_xor_sync(kFull, v[e], jl);
+            v[e] = lower == up ? min(v[e], o) : max(v[e], o);
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int p = e ^ j;
+            if (p > e && p < E) {
+                const bool up = k >= 32 * E ? up_all : ((l * E + e) & k) == 0;
+                const int32_t lo = min(v[e], v[p]), hi = max(v[e], v[p]);
+                v[e] = up ? lo : hi;
+                v[p] = up ? hi : lo;
+            }
+        }
+    }
+}
+
+template <int E>
+__device__ __forceinline__ void warp_bitonic_sort(int32_t (&v)[E], bool up) {
+#pragma unroll
+    for (int k = 2; k <= 32 * E; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) bitonic_step<E>(v, j, up, k);
+}
+
+// The last merge steps of a larger network: strides 16 * E .. 1, all in one direction.
+template <int E>
+__device__ __forceinline__ void warp_bitonic_merge(int32_t (&v)[E], bool up) {
+#pragma unroll
+    for (int j = 16 * E; j > 0; j >>= 1) bitonic_step<E>(v, j, up, 32 * E);
+}
+
+// Tier B1: 32 < d <= 1024, a warp per row, E registers a lane.  (Through shared memory, a warp barrier per
+// stage up to 256 and a block barrier per stage above: 0.23 + 0.87 ms on R-MAT scale 20.)
+constexpr int kMidWarps = 4;
+
+template <int E>
+__device__ __forceinline__ void warp_sort_row(int64_t i, int d, int64_t src, int64_t dst,
+                                              const int32_t* __restrict__ gcols, const int32_t* __restrict__ perm,
+                                              int32_t* __restrict__ cols, int32_t* __restrict__ dplus) {
+    const int l = lane_id();
+    int32_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = e * 32 + l < d ? gcols[src + e * 32 + l] : -1;  // any order will do
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = v[e] >= 0 ? perm[v[e]] : 0x7fffffff;
+    warp_bitonic_sort<E>(v, true);
+    int above = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        if (l * E + e < d) {
+            cols[dst + l * E + e] = v[e];
+            above += v[e] > (int32_t)i;
+        }
+    }
+    above = warp_sum(above);
+    if (l == 0) dplus[i] = above;
+}
 
 __global__ void __launch_bounds__(kMidWarps * 32) k_sort_rows_mid(const int64_t* __restrict__ goff,
                                                                    const int32_t* __restrict__ gcols,
                                                                    const int32_t* __restrict__ order,
                                                                    const int32_t* __restrict__ perm,
                                                                    const int32_t* __restrict__ deg,
-                                                                   const int64_t* __restrict__ off, int64_t n,
+                                                                   const int64_t* __restrict__ off,
                                                                    int32_t* __restrict__ cols,
                                                                    int32_t* __restrict__ dplus,
                                                                    const int32_t* __restrict__ q,
-                                                                   const unsigned long long* __restrict__ qcnt) {
-    __shared__ int32_t sbuf[kMidWarps][kTierB1];
-    const int w = threadIdx.x >> 5, l = lane_id();
-    int32_t* buf = sbuf[w];
-    const int64_t nq = (int64_t)qcnt[0];
-    for (int64_t qi = (int64_t)blockIdx.x * kMidWarps + w; qi < nq; qi += (int64_t)gridDim.x * kMidWarps) {
+                                                                   const uint64_t* __restrict__ acc) {
+    const int64_t nq = (int64_t)acc[Q_SORT_WARP];
+    for (int64_t qi = (int64_t)blockIdx.x * kMidWarps + (threadIdx.x >> 5); qi < nq; qi += (int64_t)gridDim.x * kMidWarps) {
         const int64_t i = q[qi];
         const int d = deg[i];
-        if (d > kTierB1) continue;  // the block sort's row
-        int P = 64;
-        while (P < d) P <<= 1;
-        const int64_t src = goff[order[i]];
-        for (int k = l; k < P; k += 32) buf[k] = (k < d) ? perm[gcols[src + k]] : 0x7fffffff;
-        __syncwarp();
-        for (int k = 2; k <= P; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int t = l; t < (P >> 1); t += 32) {
-                    const int a = 2 * t - (t & (j - 1));  // index with bit j clear
-                    const int c = a + j;
-                    const bool up = (a & k) == 0;
-                    const int32_t x = buf[a], y = buf[c];
-                    if ((x > y) == up) {
-                        buf[a] = y;
-                        buf[c] = x;
-                    }
-                }
-                __syncwarp();
-            }
-        }
-        int below = 0;
-        for (int k = l; k < d; k += 32) {
-            const int32_t x = buf[k];
-            cols[off[i] + k] = x;
-            below += x < (int32_t)i;
-        }
-        below = warp_sum(below);
-        if (l == 0) dplus[i] = d - below;
-        __syncwarp();  // every lane has read the buffer before the next row fills it
+        const int64_t src = goff[order[i]], dst = off[i];
+        if (d <= 64) warp_sort_row<2>(i, d, src, dst, gcols, perm, cols, dplus);
+        else if (d <= 128) warp_sort_row<4>(i, d, src, dst, gcols, perm, cols, dplus);
+        else if (d <= 256) warp_sort_row<8>(i, d, src, dst, gcols, perm, cols, dplus);
+        else if (d <= 512) warp_sort_row<16>(i, d, src, dst, gcols, perm, cols, dplus);
+        else warp_sort_row<32>(i, d, src, dst, gcols, perm, cols, dplus);
     }
 }
 
-// Tier B: 256 < d <= 4096, one block per row, bitonic sort in shared memory.
-__global__ void __launch_bounds__(512) k_sort_rows_block(const int64_t* __restrict__ goff,
-                                                         const int32_t* __restrict__ gcols,
-                                                         const int32_t* __restrict__ order,
-                                                         const int32_t* __restrict__ perm,
-                                                         const int32_t* __restrict__ deg,
-                                                         const int64_t* __restrict__ off, int64_t n,
-                                                         int32_t* __restrict__ cols,
-                                                         int32_t* __restrict__ dplus,
-                                                         const int32_t* __restrict__ q,
-                                                         const unsigned long long* __restrict__ qcnt) {
+// Tier B: 1024 < d <= 4096, one block per row: 16 warps sort 256 keys each (in alternate directions), then the
+// merges of 512, 1024, 2048 and 4096 keys exchange through shared memory for strides of 256 and more (10
+// barriers instead of one per stage of the whole network) and finish in registers.
+constexpr int kBlockE = 8;
+constexpr int kBlockWarps = kTierB / (32 * kBlockE);
+
+__global__ void __launch_bounds__(kBlockWarps * 32) k_sort_rows_block(const int64_t* __restrict__ goff,
+                                                                      const int32_t* __restrict__ gcols,
+                                                                      const int32_t* __restrict__ order,
+                                                                      const int32_t* __restrict__ perm,
+                                                                      const int32_t* __restrict__ deg,
+                                                                      const int64_t* __restrict__ off,
+                                                                      int32_t* __restrict__ cols,
+                                                                      int32_t* __restrict__ dplus,
+                                                                      const int32_t* __restrict__ q,
+                                                                      const uint64_t* __restrict__ acc) {
+    constexpr int E = kBlockE, RUN = 32 * E;
     __shared__ int32_t buf[kTierB];
-    __shared__ int cnt_below;
-    const int64_t nq = (int64_t)qcnt[0];
+    __shared__ int s_above[kBlockWarps];
+    const int w = threadIdx.x >> 5, l = lane_id();
+    const int64_t nq = (int64_t)acc[Q_SORT_BLOCK];
     for (int64_t qi = blockIdx.x; qi < nq; qi += gridDim.x) {
         const int64_t i = q[qi];
         const int d = deg[i];
-        if (d <= kTierB1) continue;  // the warp sort's row (the same value in every thread)
-        int P = 64;
-        while (P < d) P <<= 1;
-        const int64_t src = goff[order[i]];
-        for (int k = threadIdx.x; k < P; k += blockDim.x) buf[k] = (k < d) ? perm[gcols[src + k]] : 0x7fffffff;
-        if (threadIdx.x == 0) cnt_below = 0;
-        __syncthreads();
-        for (int k = 2; k <= P; k <<= 1) {
+        const int64_t src = goff[order[i]], dst = off[i];
+        int32_t v[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int k = w * RUN + e * 32 + l;
+            v[e] = k < d ? gcols[src + k] : -1;
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = v[e] >= 0 ? perm[v[e]] : 0x7fffffff;
+        warp_bitonic_sort<E>(v, (w & 1) == 0);
+        // buf holds key x of warp w's run at w * RUN + (x mod E) * 32 + x / E: register e of lane l, conflict-free;
+        // exchanges of stride >= RUN keep x, so they only change the run
+        for (int k = 2; k <= kBlockWarps; k <<= 1) {  // merge runs of k warps
+            const bool up = (w & k) == 0;             // k = kBlockWarps: every warp
             for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int t = threadIdx.x; t < (P >> 1); t += blockDim.x) {
-                    int a = 2 * t - (t & (j - 1));  // index with bit j clear
-                    int c = a + j;
-                    bool up = (a & k) == 0;
-                    int32_t x = buf[a], y = buf[c];
-                    if ((x > y) == up) {
-                        buf[a] = y;
-                        buf[c] = x;
-                    }
-                }
+                __syncthreads();  // the previous exchange is read
+#pragma unroll
+                for (int e = 0; e < E; ++e) buf[w * RUN + e * 32 + l] = v[e];
                 __syncthreads();
+                const bool lower = (w & j) == 0;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int32_t o = buf[(w ^ j) * RUN + e * 32 + l];
+                    v[e] = lower == up ? min(v[e], o) : max(v[e], o);
+                }
+            }
+            warp_bitonic_merge<E>(v, up);
+        }
+        int above = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int k = w * RUN + l * E + e;
+            if (k < d) {
+                cols[dst + k] = v[e];
+                above += v[e] > (int32_t)i;
             }
         }
-        int below = 0;
-        for (int k = threadIdx.x; k < d; k += blockDim.x) {
-            int32_t x = buf[k];
-            cols[off[i] + k] = x;
-            below += x < (int32_t)i;
-        }
-        below = warp_sum(below);
-        if (lane_id() == 0 && below) atomicAdd(&cnt_below, below);
+        above = warp_sum(above);
+        if (l == 0) s_above[w] = above;
         __syncthreads();
-        if (threadIdx.x == 0) dplus[i] = d - cnt_below;
+        if (threadIdx.x == 0) {
+            int t = 0;
+            for (int x = 0; x < kBlockWarps; ++x) t += s_above[x];
+            dplus[i] = t;
+        }
         __syncthreads();
     }
 }
 
-// Tier C: hubs (d > 4096), one block per row, LSD radix sort (8-bit digits) through global memory.
+// Tier C: hubs (d > 4096) of graphs of at most kBitmapRanks ranks: a block per row sets the row's ranks in a bitmap
+// in shared memory and writes them out in order, a window of ranks at a time (one for up to 1.6 M ranks).
+constexpr int kBitmapThreads = 1024;
+constexpr int kBitmapWarps = kBitmapThreads / 32;
+constexpr int kBitmapWords = 50176;  // 196 KiB; a multiple of 32 * kBitmapWarps
+constexpr int64_t kBitmapRanks = 4 * 32 * (int64_t)kBitmapWords;
+static_assert(kBitmapWords % (32 * kBitmapWarps) == 0, "every warp takes whole groups of 32 words");
+
+__global__ void __launch_bounds__(kBitmapThreads) k_sort_rows_bitmap(const int64_t* __restrict__ goff,
+                                                                     const int32_t* __restrict__ gcols,
+                                                                     const int32_t* __restrict__ order,
+                                                                     const int32_t* __restrict__ perm,
+                                                                     const int32_t* __restrict__ deg,
+                                                                     const int64_t* __restrict__ off, int64_t n,
+                                                                     const int32_t* __restrict__ gid,
+                                                                     const int64_t* __restrict__ gbase,
+                                                                     int32_t* __restrict__ cols,
+                                                                     int32_t* __restrict__ dplus,
+                                                                     const int32_t* __restrict__ q,
+                                                                     const uint64_t* __restrict__ acc) {
+    extern __shared__ uint32_t bm[];
+    __shared__ int s_count[kBitmapWarps];
+    __shared__ int s_above;
+    const int w = threadIdx.x >> 5, l = lane_id();
+    const int64_t nq = (int64_t)acc[Q_SORT_WARP + 1];
+    for (int64_t qi = blockIdx.x; qi < nq; qi += gridDim.x) {
+        const int64_t i = q[n - 1 - qi];
+        const int64_t d = deg[i], src = goff[order[i]];
+        const int64_t r0 = gid ? gbase[gid[i]] : 0, r1 = gid ? gbase[gid[i] + 1] : n;  // the graph's ranks
+        int64_t dst = off[i];
+        if (threadIdx.x == 0) s_above = 0;
+        int above = 0;
+        for (int64_t lo = r0; lo < r1; lo += 32 * (int64_t)kBitmapWords) {
+            const int64_t hi = lo + 32 * (int64_t)kBitmapWords < r1 ? lo + 32 * (int64_t)kBitmapWords : r1;
+            // each warp's share of the words: whole groups of 32
+            const int groups = (int)((hi - lo + 1023) / 1024), per = (groups + kBitmapWarps - 1) / kBitmapWarps;
+            for (int k = threadIdx.x; k < per * kBitmapThreads; k += kBitmapThreads) bm[k] = 0;
+            __syncthreads();
+            for (int64_t k0 = threadIdx.x; k0 < d; k0 += 4 * kBitmapThreads) {
+                int32_t x[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) x[t] = k0 + t * kBitmapThreads < d ? gcols[src + k0 + t * kBitmapThreads] : -1;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) x[t] = x[t] >= 0 ? perm[x[t]] : -1;
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (x[t] >= lo && x[t] < hi) {
+                        const uint32_t b = (uint32_t)(x[t] - lo);
+                        atomicOr(&bm[b >> 5], 1u << (b & 31));
+                    }
+            }
+            __syncthreads();
+            int count = 0;
+            for (int g = 0; g < per; ++g) count += __popc(bm[(w * per + g) * 32 + l]);
+            count = warp_sum(count);
+            if (l == 0) s_count[w] = count;
+            __syncthreads();
+            const int before_me = l < w ? s_count[l] : 0;  // kBitmapWarps == 32
+            int64_t out = dst + warp_sum(before_me);
+            const int all = warp_sum(s_count[l]);
+            for (int g = 0; g < per; ++g) {
+                const int word = (w * per + g) * 32 + l;
+                uint32_t bits = bm[word];
+                const int c = __popc(bits);
+                int incl = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(kFull, incl, o);
+                    if (l >= o) incl += y;
+                }
+                int64_t p = out + incl - c;
+                while (bits) {
+                    const int32_t x = (int32_t)(lo + (int64_t)word * 32 + __ffs(bits) - 1);
+                    bits &= bits - 1;
+                    cols[p++] = x;
+                    above += x > (int32_t)i;
+                }
+                out += __shfl_sync(kFull, incl, 31);
+            }
+            dst += all;
+            __syncthreads();  // the bitmap is read before the next window clears it
+        }
+        above = warp_sum(above);
+        if (l == 0 && above) atomicAdd(&s_above, above);
+        __syncthreads();
+        if (threadIdx.x == 0) dplus[i] = s_above;
+        __syncthreads();
+    }
+}
+static_assert(kBitmapWarps == 32, "a lane per warp in the block's prefix");
+
+// Tier C, graphs of more ranks: one block per hub row, LSD radix sort (8-bit digits) through global memory.
 // Pass p reads the previous pass's output; pass 0 reads the old row through perm.  The pass count
 // decides which buffer each pass writes so that the last one lands in `cols`.
 constexpr int kHubThreads = 512;
@@ -396,13 +569,13 @@ __global__ void __launch_bounds__(kHubThreads) k_sort_rows_hub(const int64_t* __
 
 // colsp[offp[i] + k] = the k-th neighbour of i ranked above i (the row suffix), 32 consecutive rows
 // per warp: a lane copies its own row when the suffix has at most 32 entries, the warp copies the
-// longer ones together.  The same pass accumulates sum over edges of (d_u - 1)(d_v - 1) (3-edge paths
-// + 3T).
+// longer ones together.  The same pass clears t_e and accumulates sum over edges of (d_u - 1)(d_v - 1)
+// (3-edge paths + 3T).
 __global__ void __launch_bounds__(256) k_out_csr(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
                                                  const int32_t* __restrict__ dplus,
                                                  const int32_t* __restrict__ deg,
                                                  const int64_t* __restrict__ offp, int64_t n,
-                                                 int32_t* __restrict__ colsp, Sink sink) {
+                                                 int32_t* __restrict__ colsp, uint32_t* __restrict__ te, Sink sink) {
     __shared__ uint64_t red[32];
     const int l = lane_id();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -411,6 +584,7 @@ __global__ void __launch_bounds__(256) k_out_csr(const int64_t* __restrict__ off
     for (int64_t i0 = wid * 32; i0 < n; i0 += nw * 32) {
         const int64_t i = i0 + l;
         const int64_t dp = i < n ? dplus[i] : 0;
+        uint64_t lane_pw = 0;  // the lane's own row's part
         if (dp > 0 && dp <= 32) {
             const int64_t srcb = off[i + 1] - dp;
             const int64_t dstb = offp[i];
@@ -419,10 +593,10 @@ __global__ void __launch_bounds__(256) k_out_csr(const int64_t* __restrict__ off
             for (int64_t k = 0; k < dp; ++k) {
                 const int32_t v = cols[srcb + k];
                 colsp[dstb + k] = v;
+                te[dstb + k] = 0;
                 row_pw += di1 * ((uint64_t)deg[v] - 1);
             }
-            if (sink.batch()) sink_add(sink, (int32_t)i, G_PW, row_pw);
-            else pw += row_pw;
+            lane_pw = row_pw;
         }
         uint32_t rest = __ballot_sync(kFull, dp > 32);
         while (rest) {
@@ -434,18 +608,30 @@ __global__ void __launch_bounds__(256) k_out_csr(const int64_t* __restrict__ off
             const int64_t dstb = offp[r];
             const uint64_t di1 = (uint64_t)deg[r] - 1;
             uint64_t row_pw = 0;
-            for (int64_t k = l; k < rdp; k += 32) {
-                const int32_t v = cols[srcb + k];
-                colsp[dstb + k] = v;
-                row_pw += di1 * ((uint64_t)deg[v] - 1);
+            for (int64_t k0 = l; k0 < rdp; k0 += 128) {  // four loads in flight: the hubs' rows come together
+                int32_t v[4];
+                uint64_t dv[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) v[t] = k0 + 32 * t < rdp ? cols[srcb + k0 + 32 * t] : -1;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) dv[t] = v[t] >= 0 ? (uint64_t)deg[v[t]] : 1;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    if (v[t] < 0) continue;
+                    colsp[dstb + k0 + 32 * t] = v[t];
+                    te[dstb + k0 + 32 * t] = 0;
+                    row_pw += di1 * (dv[t] - 1);
+                }
             }
             if (sink.batch()) {
                 row_pw = warp_sum(row_pw);
-                if (l == 0) sink_add(sink, (int32_t)r, G_PW, row_pw);
+                if (l == src) lane_pw = row_pw;
             } else {
                 pw += row_pw;
             }
         }
+        if (sink.batch()) warp_add_by_graph(sink.accG, G_PW, i < n ? sink.gid[i] : -1, lane_pw);
+        else pw += lane_pw;
     }
     pw = block_sum_u64(pw, red);
     if (threadIdx.x == 0 && pw) atomicAdd((unsigned long long*)&sink.acc[ACC_PW], (unsigned long long)pw);
@@ -470,9 +656,8 @@ harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     // the keys are written in id order and every pass is stable, so only the graph and degree bits
     // need sorting: equal (graph, degree) keep ascending ids
     HARP_TRY(radix_sort_u64(&k0, &k1, n, b, b + bd + bg, ws.hist, ws.scan_tmp, ws.scan_tmp_len, s));
-    unsigned long long* qsort = (unsigned long long*)&ws.acc[Q_SORT_CTA];
     k_relabel<<<grid_for(n, 256), 256, 0, s>>>(k0, n, b, bd, ws.order, ws.perm, ws.deg, ws.gid_in, ws.gid, ws.q_tri,
-                                               qsort);
+                                               ws.q_mid, ws.acc);
     HARP_LAUNCHED();
     HARP_TRY(exclusive_scan_i32_to_i64(ws.deg, ws.off, n, ws.scan_tmp, ws.scan_tmp_len, s));
     if (m > 0) {
@@ -480,16 +665,31 @@ harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s) {
         k_sort_rows_warp<<<grid_for(n, 256), 256, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg,
                                                                 ws.off, n, ws.cols, ws.dplus);
         HARP_LAUNCHED();
-        k_sort_rows_mid<<<num_sms() * 8, kMidWarps * 32, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg,
-                                                                 ws.off, n, ws.cols, ws.dplus, ws.q_tri, qsort);
-        HARP_LAUNCHED();
-        k_sort_rows_block<<<num_sms() * 4, 512, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off, n,
-                                                   ws.cols, ws.dplus, ws.q_tri, qsort);
-        HARP_LAUNCHED();
-        // the out-CSR columns + t_e region (2m int32) is free until k_out_csr: hub sort ping-pong
-        k_sort_rows_hub<<<num_sms(), kHubThreads, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off, n, b,
-                                                     ws.cols, ws.colsp, ws.dplus, ws.q_tri, qsort);
-        HARP_LAUNCHED();
+        if (g->max_deg > kTierA) {
+            k_sort_rows_mid<<<num_sms() * 8, kMidWarps * 32, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off,
+                                                                     ws.cols, ws.dplus, ws.q_tri, ws.acc);
+            HARP_LAUNCHED();
+        }
+        if (g->max_deg > kTierB1) {
+            k_sort_rows_block<<<num_sms() * 4, kBlockWarps * 32, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg,
+                                                                         ws.off, ws.cols, ws.dplus, ws.q_mid, ws.acc);
+            HARP_LAUNCHED();
+        }
+        const int64_t most_n = ws.G > 1 ? ws.max_member_n : n;  // ranks of the largest graph
+        if (g->max_deg > kTierB && most_n <= kBitmapRanks) {
+            const size_t smem = sizeof(uint32_t) * (size_t)kBitmapWords;
+            HARP_CK(cudaFuncSetAttribute(k_sort_rows_bitmap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k_sort_rows_bitmap<<<num_sms(), kBitmapThreads, smem, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off,
+                                                                       n, ws.G > 1 ? ws.gid : nullptr, ws.gbase, ws.cols,
+                                                                       ws.dplus, ws.q_tri, ws.acc);
+            HARP_LAUNCHED();
+        } else if (g->max_deg > kTierB) {
+            // the out-CSR columns + t_e region (2m int32) is free until k_out_csr: hub sort ping-pong
+            k_sort_rows_hub<<<num_sms(), kHubThreads, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off, n, b,
+                                                              ws.cols, ws.colsp, ws.dplus, ws.q_tri,
+                                                              (const unsigned long long*)&ws.acc[Q_SORT_WARP]);
+            HARP_LAUNCHED();
+        }
     } else {
         HARP_CK(cudaMemsetAsync(ws.dplus, 0, (size_t)n * sizeof(int32_t), s));
     }
@@ -498,9 +698,8 @@ harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s) {
         const Sink sink{ws.acc, ws.gid, ws.accG};
         // 32 rows per warp
         k_out_csr<<<grid_for(n, 256), 256, 0, s>>>(ws.off, ws.cols, ws.dplus, ws.deg, ws.offp, n, ws.colsp,
-                                                         sink);
+                                                   ws.te, sink);
         HARP_LAUNCHED();
-        HARP_CK(cudaMemsetAsync(ws.te, 0, (size_t)m * sizeof(uint32_t), s));
     }
     return HARP_OK;
 }

@@ -93,16 +93,7 @@ __global__ void __launch_bounds__(256) k_reduce_rows_batch(const int64_t* __rest
             rd = warp_sum(rd);
             if (l == src) d = rd;
         }
-        uint32_t left = __ballot_sync(kFull, d != 0);
-        while (left) {  // one graph per round: the first lane still holding a sum names it
-            const int src = __ffs(left) - 1;
-            const int32_t gs = __shfl_sync(kFull, g, src);
-            const bool mine = ((left >> l) & 1u) && g == gs;
-            const uint64_t sum = warp_sum(mine ? d : (uint64_t)0);
-            if (l == src)
-                atomicAdd((unsigned long long*)&sink.accG[(int64_t)gs * kGStride + G_D], (unsigned long long)sum);
-            left &= ~__ballot_sync(kFull, mine);
-        }
+        warp_add_by_graph(sink.accG, G_D, g, d);
     }
 }
 

@@ -1338,7 +1338,7 @@ harp_status launch_cta(const harp_csr* g, Workspace& ws, int cls, int ticket_slo
 
 // The four staged tiers, each with its bin's membership probe (plan.tri_probe_bin[k]: bsearch or hash).
 harp_status launch_tiers(const harp_csr* g, Workspace& ws, int wmax, int cmax, int bmax, bool reuse,
-                         const uint8_t* probe_bin, cudaStream_t s) {
+                         const uint8_t* probe_bin, int64_t dmax, cudaStream_t s) {
     const Sink sink{ws.acc, ws.gid, ws.accG};
     const bool bs0 = probe_bin[0] == HARP_PROBE_BSEARCH, bs1 = probe_bin[1] == HARP_PROBE_BSEARCH;
     const bool bs2 = probe_bin[2] == HARP_PROBE_BSEARCH, bs3 = probe_bin[3] == HARP_PROBE_BSEARCH;
@@ -1348,13 +1348,20 @@ harp_status launch_tiers(const harp_csr* g, Workspace& ws, int wmax, int cmax, i
     else k_tri_warp<false><<<wgrid, kWarpThreads, 0, s>>>(ws.offp, ws.colsp, ws.deg, ws.q_tri, qcnt, reuse, ws.te, sink);
     HARP_LAUNCHED();
     HARP_CK(prof_mark(s, SEG_TRI_WARP));
-    if (bs1) HARP_TRY((launch_cta<kCta1, kCta1Threads, kCta1Blocks, true>(g, ws, 1, T_TRI_S, wmax, cmax, bmax, reuse, s)));
-    else HARP_TRY((launch_cta<kCta1, kCta1Threads, kCta1Blocks, false>(g, ws, 1, T_TRI_S, wmax, cmax, bmax, reuse, s)));
+    // tiers that the largest possible out-degree does not reach have no anchors
+    if (dmax > wmax) {
+        if (bs1) HARP_TRY((launch_cta<kCta1, kCta1Threads, kCta1Blocks, true>(g, ws, 1, T_TRI_S, wmax, cmax, bmax, reuse, s)));
+        else HARP_TRY((launch_cta<kCta1, kCta1Threads, kCta1Blocks, false>(g, ws, 1, T_TRI_S, wmax, cmax, bmax, reuse, s)));
+    }
     HARP_CK(prof_mark(s, SEG_TRI_CTA_S));
-    if (bs2) HARP_TRY((launch_cta<kCta2, 256, 4, true>(g, ws, 2, T_TRI_M, wmax, cmax, bmax, reuse, s)));
-    else HARP_TRY((launch_cta<kCta2, 256, 4, false>(g, ws, 2, T_TRI_M, wmax, cmax, bmax, reuse, s)));
-    if (bs3) HARP_TRY((launch_cta<kCtaMax, 1024, 1, true>(g, ws, 3, T_TRI_L, wmax, cmax, bmax, reuse, s)));
-    else HARP_TRY((launch_cta<kCtaMax, 1024, 1, false>(g, ws, 3, T_TRI_L, wmax, cmax, bmax, reuse, s)));
+    if (dmax > kCta1) {
+        if (bs2) HARP_TRY((launch_cta<kCta2, 256, 4, true>(g, ws, 2, T_TRI_M, wmax, cmax, bmax, reuse, s)));
+        else HARP_TRY((launch_cta<kCta2, 256, 4, false>(g, ws, 2, T_TRI_M, wmax, cmax, bmax, reuse, s)));
+    }
+    if (dmax > kCta2) {
+        if (bs3) HARP_TRY((launch_cta<kCtaMax, 1024, 1, true>(g, ws, 3, T_TRI_L, wmax, cmax, bmax, reuse, s)));
+        else HARP_TRY((launch_cta<kCtaMax, 1024, 1, false>(g, ws, 3, T_TRI_L, wmax, cmax, bmax, reuse, s)));
+    }
     HARP_CK(prof_mark(s, SEG_TRI_CTA_L));
     return HARP_OK;
 }
@@ -1392,9 +1399,9 @@ harp_status count_triangles_k4(const harp_csr* g, Workspace& ws, const harp_plan
                                                     ws.q_mid, cnt, cnt_fb, cnt_big);
     HARP_LAUNCHED();
     const Sink sink{ws.acc, ws.gid, ws.accG};
-    HARP_TRY(launch_tiers(g, ws, wmax, cmax, bmax, reuse, plan.tri_probe_bin, s));
-    // the largest possible out-degree is bounded by sqrt(2m) and by the maximum degree
     const int64_t dmax = max_out_degree(g);
+    HARP_TRY(launch_tiers(g, ws, wmax, cmax, bmax, reuse, plan.tri_probe_bin, dmax, s));
+    // the largest possible out-degree is bounded by sqrt(2m) and by the maximum degree
     if (dmax > cmax && bmax > cmax) {  // global-staged tier: one block per SM, scratch of kBigMax rows
         const size_t bytes = (size_t)num_sms() * kBigMax * kBigWords * sizeof(uint32_t);
         uint32_t* scratch = nullptr;
