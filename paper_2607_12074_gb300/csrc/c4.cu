@@ -16,7 +16,7 @@
 //     counters packed floor(32 / bits) to a word.  The bands cut into windows of 48-100 KiB of
 //     counters form a fixed grid per graph, so the row position of every grid boundary is computed
 //     once per row (bpos) instead of being searched for every (root, lower neighbour, window).
-// pos_w(u) itself is computed once per lower arc (rev) by a fully parallel pass.
+// pos_w(u) itself is computed once per lower arc (rev, as the segment length) by a fully parallel pass.
 //
 // The frontier (the set of x) is not an induced class: whether u ~ x or w1 ~ w2 holds decides
 // whether the cycle is induced, a diamond or part of a 4-clique; the closure resolves that mix
@@ -56,8 +56,6 @@ constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallSlots = 1024;            // per-warp hash table of the light roots (W <= 512)
 constexpr int kMidSlots = 4096;              // hash table of the middle tier (W <= 2048)
 constexpr int kMidWarps = 4;                 // warps of the block that takes a middle root
-constexpr int64_t kTableMinN = 65536;        // no boundary table up to here: its 16 entries a row cost more than
-                                             // the few windowed roots' searches (batch of 4,096: 2.1 ms)
 constexpr int kLong = 32;                    // segments this long are read warp-coalesced
 constexpr int kSplit = 2048;                 // segments this long are split across the block
 constexpr int kSplitQ = 128;                 // split-queue capacity per window item
@@ -304,66 +302,150 @@ __global__ void __launch_bounds__(kGinfoThreads) k_c4_ginfo(const int32_t* __res
     }
 }
 
-// rev[a] = pos_w(u) for every lower arc (u -> w) at position a of u's list.  Each thread takes a run
-// of kRevRun consecutive arcs (one search for the run's first row, then it walks forward), so hub
-// rows are spread over many threads.  arcs must equal off[n]; the walk never passes row n - 1.
-// Whole graph (ROWS = false): the lists are the row prefixes of (off, cols) and the position comes
-// from N+(w) (offp, colsp): d-(w) + rank of u in N+(w).  Partitioned (ROWS = true): the lists are
-// the roots' lower lists (off = loff, cols = lcols) and the position is searched in w's row of the
-// halo (offp = off, colsp = cols of the rows).
+// fpos[w] = row position of w's first neighbour of degree >= 2 (the graph's n1 boundary); vinfo[w] (whole graphs) =
+// what a lower arc to w needs, side by side: the start and length of N+(w), d-(w) - fpos[w], and the start of
+// w's segments in cols.  Positions fit 32 bits.  Without ginfo every segment starts at its row (fpos = 0).
+__global__ void __launch_bounds__(256) k_c4_fpos(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
+                                                 const int64_t* __restrict__ offp, const int32_t* __restrict__ gid,
+                                                 const int64_t* __restrict__ ginfo, int64_t n,
+                                                 int32_t* __restrict__ fpos, uint4* __restrict__ vinfo) {
+    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t wb = off[w], we = off[w + 1];
+        int32_t f = 0;
+        if (ginfo) {
+            const int64_t n1 = ginfo[(gid ? (int64_t)gid[w] : 0) * kGInfo + GI_N1];
+            f = (int32_t)lower_bound_i32(cols + wb, we - wb, (int32_t)n1);
+            fpos[w] = f;
+        }
+        if (vinfo) {
+            const int64_t pb = offp[w];
+            const int32_t dp = (int32_t)(offp[w + 1] - pb);
+            vinfo[w] = make_uint4((uint32_t)pb, (uint32_t)dp, (uint32_t)((int32_t)(we - wb) - dp - f), (uint32_t)(wb + f));
+        }
+    }
+}
+
+// rev[a] = the wedge segment's length for every lower arc (u -> w) at position a of u's list: the position of u in
+// w's row less fpos[w] (0 where u stands before it).
+// Whole graph: the lower arcs of all rows are numbered through, row u's from off[u] - offp[u] on.  A warp takes a run
+// of steps, a step being a lower arc or a row's end (runs of rows without lower arcs are as long as the graph's
+// isolated vertices), a lane per arc: the rows are held by the lanes, 32 at a time, and an arc finds its row by a
+// search over the lanes.  The position comes from N+(w): d-(w) + rank of u in N+(w).  (A thread per 16 arcs that
+// walked its rows and gathered four arrays per arc: 2.59 ms on the batch of 4,096 graphs, 0.25 ms on the random
+// geometric graph with 1,000,003 vertices.)  Core roots and roots of one lower neighbour need no length.
+__device__ __forceinline__ int64_t lower_start(const int64_t* __restrict__ off, const int64_t* __restrict__ offp, int64_t u) {
+    return off[u] - offp[u];
+}
+
+__global__ void __launch_bounds__(256) k_c4_seglen(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
+                                                   const int64_t* __restrict__ offp, const int32_t* __restrict__ colsp,
+                                                   const uint4* __restrict__ vinfo, const int32_t* __restrict__ gid,
+                                                   const int64_t* __restrict__ ginfo, int64_t n, int run,
+                                                   int32_t* __restrict__ rev) {
+    const int l = lane_id();
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    // one graph: the arcs of its core rows come last and are left out
+    int64_t rows = n;
+    if (ginfo && !gid && ginfo[GI_CORE] < n) rows = ginfo[GI_CORE];
+    // first row u in [lo, hi) whose place lower_start(u) + u lies past t, less one: the row of step t; 32 probes a round
+    auto row_of = [&](int64_t lo, int64_t hi, int64_t t) {
+        while (hi - lo > 1) {
+            const int64_t step = (hi - lo + 31) >> 5;
+            const int64_t p = lo + (int64_t)(l + 1) * step;
+            const uint32_t m = __ballot_sync(kFull, p >= hi || lower_start(off, offp, p) + p > t);
+            const int k = __ffs(m) - 1;  // lane 31 probes at or past hi
+            lo += (int64_t)k * step;
+            hi = lo + step < hi ? lo + step : hi;
+        }
+        return lo;
+    };
+    const int64_t steps = lower_start(off, offp, rows) + rows;  // row u: its lower arcs, then one step
+    for (int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * run; t0 < steps; t0 += nw * run) {
+        const int64_t t1 = t0 + run < steps ? t0 + run : steps;
+        int64_t r0 = row_of(0, rows, t0);
+        const int64_t a1 = t1 - (t1 < steps ? row_of(r0, r0 + run + 1 < rows ? r0 + run + 1 : rows, t1) : rows);
+        int64_t s = 0, e = 0, ob = 0;  // the lanes hold rows r0 .. r0 + 31
+        uint32_t valid = 0;
+        for (int64_t cur = t0 - r0; cur < a1; r0 += 32) {
+            {
+                const int64_t r = r0 + l;
+                s = lower_start(off, offp, r < rows ? r : rows);
+                e = lower_start(off, offp, r + 1 < rows ? r + 1 : rows);
+                if (__shfl_sync(kFull, e, 31) <= cur) continue;  // no arc left in these rows
+            }
+            {
+                const int64_t r = r0 + l;
+                ob = r < rows ? off[r] : 0;
+                bool want = r < rows && e - s >= (ginfo ? 2 : 1);
+                if (want && gid) want = r < ginfo[(int64_t)gid[r] * kGInfo + GI_CORE];
+                valid = __ballot_sync(kFull, want);
+            }
+            const int64_t end0 = __shfl_sync(kFull, e, 31);
+            const int64_t end = end0 < a1 ? end0 : a1;
+            for (int64_t b = cur; b < end; b += 32) {
+                const int64_t a = b + l;
+                int k = 0;  // last row with s <= a
+#pragma unroll
+                for (int sft = 16; sft >= 1; sft >>= 1) {
+                    const int64_t v = __shfl_sync(kFull, s, k + sft);
+                    if (v <= a) k += sft;
+                }
+                const int64_t pos = __shfl_sync(kFull, ob, k) + (a - __shfl_sync(kFull, s, k));
+                if (a < end && ((valid >> k) & 1u)) {
+                    const uint4 vi = __ldg(vinfo + cols[pos]);
+                    const int32_t len = (int32_t)vi.z + (int32_t)lower_bound_i32(colsp + vi.x, vi.y, (int32_t)(r0 + k));
+                    rev[pos] = len > 0 ? len : 0;
+                }
+            }
+            cur = end;
+        }
+    }
+}
+
+// Partitioned blocks: the lists are the roots' lower lists (loff, lcols), the position is searched in w's row of
+// the halo.  Each thread takes a run of kRevRun consecutive arcs.  arcs must equal loff[n].
 constexpr int kRevRun = 16;
 
-template <bool ROWS>
-__global__ void __launch_bounds__(256) k_c4_rev(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
-                                                const int64_t* __restrict__ offp, const int32_t* __restrict__ colsp,
-                                                const int32_t* __restrict__ deg, const int32_t* __restrict__ dplus,
-                                                const int32_t* __restrict__ gid, const int64_t* __restrict__ ginfo,
-                                                int64_t n, int64_t arcs, int32_t* __restrict__ rev) {
+__global__ void __launch_bounds__(256) k_c4_seglen_rows(const int64_t* __restrict__ loff, const int32_t* __restrict__ lcols,
+                                                        const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
+                                                        const int32_t* __restrict__ fpos, int64_t n, int64_t arcs,
+                                                        int32_t* __restrict__ rev) {
     const int64_t runs = (arcs + kRevRun - 1) / kRevRun;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < runs; r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t a0 = r * kRevRun;
         const int64_t a1 = a0 + kRevRun < arcs ? a0 + kRevRun : arcs;
-        int64_t lo = 0, hi = n;  // row of arc a0: last u with off[u] <= a0
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (off[mid] <= a0) lo = mid;
+        int64_t u = 0, hi = n;  // row of arc a0: last u with loff[u] <= a0
+        while (hi - u > 1) {
+            const int64_t mid = (u + hi) >> 1;
+            if (loff[mid] <= a0) u = mid;
             else hi = mid;
         }
-        // the end of u's lower arcs; core roots are counted elsewhere and need none
-        auto row_lower_end = [&](int64_t v, int64_t vb) {
-            if (!ROWS && ginfo && v >= ginfo[(gid ? (int64_t)gid[v] : 0) * kGInfo + GI_CORE]) return vb;
-            return vb + ((int64_t)deg[v] - dplus[v]);
-        };
-        int64_t u = lo;
-        int64_t ub = off[u], ue = off[u + 1];
-        int64_t lower_end = row_lower_end(u, ub);
+        int64_t ub = loff[u], ue = loff[u + 1];
         for (int64_t a = a0; a < a1; ++a) {
-            if (a >= ue) {  // the row of arc a: last u with off[u] <= a, searched outward from u + 1 (the
-                            // empty rows of a graph's isolated vertices come in runs of up to its whole size)
-                if (u + 1 >= n) return;  // only if arcs > off[n]
+            if (a >= ue) {  // the row of arc a: last u with loff[u] <= a, searched outward from u + 1 (rows that the
+                            // block does not own are empty and come in long runs)
+                if (u + 1 >= n) return;  // only if arcs > loff[n]
                 int64_t p = u + 1, step = 1;
-                while (p + step < n && off[p + step] <= a) {
+                while (p + step < n && loff[p + step] <= a) {
                     p += step;
                     step <<= 1;
                 }
-                int64_t q = p + step < n ? p + step : n;  // off[p] <= a < off[q], or q = n
+                int64_t q = p + step < n ? p + step : n;  // loff[p] <= a < loff[q], or q = n
                 while (q - p > 1) {
                     const int64_t mid = (p + q) >> 1;
-                    if (off[mid] <= a) p = mid;
+                    if (loff[mid] <= a) p = mid;
                     else q = mid;
                 }
                 u = p;
-                ub = off[u];
-                ue = off[u + 1];
-                if (a >= ue) return;  // only if arcs > off[n]
-                lower_end = row_lower_end(u, ub);
+                ub = loff[u];
+                ue = loff[u + 1];
+                if (a >= ue) return;  // only if arcs > loff[n]
             }
-            // only lower arcs of roots with d- >= 2 (of every row without ginfo)
-            if (a >= lower_end || (ginfo && lower_end - ub < 2)) continue;
-            const int32_t w = cols[a];
-            const int64_t pb = offp[w];
-            if (ROWS) rev[a] = (int32_t)lower_bound_i32(colsp + pb, offp[w + 1] - pb, (int32_t)u);
-            else rev[a] = (deg[w] - dplus[w]) + (int32_t)lower_bound_i32(colsp + pb, offp[w + 1] - pb, (int32_t)u);
+            if (ue - ub < 2) continue;  // only roots with d- >= 2
+            const int32_t w = lcols[a];
+            const int64_t pb = off[w];
+            const int32_t len = (int32_t)lower_bound_i32(cols + pb, off[w + 1] - pb, (int32_t)u) - fpos[w];
+            rev[a] = len > 0 ? len : 0;
         }
     }
 }
@@ -397,27 +479,32 @@ __device__ __forceinline__ int64_t gallop_i32(const int32_t* __restrict__ a, int
     return l;
 }
 
-// fpos[w] = row position of w's first neighbour of degree >= 2 (the graph's n1 boundary), and
+// The table pays for its 16 searches a row only where the windowed roots make many visits: it is built and used
+// from kTableVisits visits per row on.  (R-MAT scale 20, whose core leaves few windowed roots: 0.20 ms to build,
+// 0.15 ms saved; a random geometric graph has none; Chung-Lu with 2,000,000 vertices needs it.)
+constexpr uint64_t kTableVisits = 8;
+__device__ __forceinline__ bool table_pays(const uint64_t* acc, int64_t n) {
+    return acc[C4_VISITS] >= kTableVisits * (uint64_t)n;
+}
+
 // bpos[w * kGridCap + k] = row position of grid boundary k << s (see table_shift)
 template <int WORDS>
 __global__ void k_c4_bpos(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
                           const int32_t* __restrict__ gid, const int64_t* __restrict__ ginfo, int64_t n,
-                          int32_t* __restrict__ fpos, int32_t* __restrict__ bpos) {
-    const int64_t total = bpos ? n * kGridCap : n;
+                          const int32_t* __restrict__ fpos, const uint64_t* __restrict__ acc, int32_t* __restrict__ bpos) {
+    if (!table_pays(acc, n)) return;
+    const int64_t total = n * kGridCap;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t w = bpos ? t / kGridCap : t;
-        const int k = bpos ? (int)(t % kGridCap) : 0;
-        const int64_t* gi = ginfo + (gid ? (int64_t)gid[w] : 0) * kGInfo;
-        const int64_t nwin = gi[GI_NWIN];
+        const int64_t w = t / kGridCap;
+        const int k = (int)(t % kGridCap);
         if (k == 0) {
-            const int64_t wb = off[w];
-            const int32_t f = (int32_t)lower_bound_i32(cols + wb, off[w + 1] - wb, (int32_t)gi[GI_N1]);
-            fpos[w] = f;
-            if (bpos) bpos[t] = f;
+            bpos[t] = fpos[w];
             continue;
         }
+        const int64_t* gi = ginfo + (gid ? (int64_t)gid[w] : 0) * kGInfo;
+        const int64_t nwin = gi[GI_NWIN];
         const int64_t i = (int64_t)k << table_shift(nwin);
-        if (!bpos || i > nwin) continue;
+        if (i > nwin) continue;
         int64_t bound = gi[GI_HI];
         if (i < nwin) {
             int64_t xhi;
@@ -544,10 +631,8 @@ __device__ __forceinline__ uint32_t hash_add(int32_t* keys, uint32_t* cnt, uint3
 // Classification: every root (a lane per root, descending rank so heavy roots are queued first).
 // ---------------------------------------------------------------------------------------------
 template <int WORDS>
-__global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__ loff, const int32_t* __restrict__ lcols,
-                                                     const int32_t* __restrict__ deg,
+__global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__ loff, const int32_t* __restrict__ deg,
                                                      const int32_t* __restrict__ dplus,
-                                                     const int32_t* __restrict__ fpos,
                                                      const int32_t* __restrict__ rev,
                                                      const int32_t* __restrict__ gid,
                                                      const int64_t* __restrict__ ginfo, int64_t n, int64_t own_lo,
@@ -564,6 +649,7 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
     // ranks fall to different warps): a lane sums W(u) itself when u has at most 32 lower neighbours,
     // the warp sums the larger roots together; queue slots are taken in lane order (descending rank).
     // A warp per root left most lanes idle on the many small roots of a batch of small graphs.
+    uint64_t visits = 0;
     for (int64_t k0 = wid; k0 < n; k0 += nw * 32) {
         const int64_t k = k0 + (int64_t)l * nw;
         const int32_t u = (int32_t)(n - 1 - k);
@@ -574,11 +660,7 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
         const int64_t ub = dm >= 2 ? loff[u] : 0;
         uint64_t W = 0;
         if (dm >= 2 && dm <= 32) {
-            for (int64_t a = 0; a < dm; ++a) {
-                const int32_t f = fpos[lcols[ub + a]];
-                const int32_t p = rev[ub + a];
-                W += p > f ? (uint64_t)(p - f) : 0;
-            }
+            for (int64_t a = 0; a < dm; ++a) W += (uint64_t)rev[ub + a];
         }
         uint32_t big = __ballot_sync(kFull, dm > 32);
         while (big) {
@@ -586,11 +668,7 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
             big &= big - 1;
             const int64_t bdm = __shfl_sync(kFull, dm, src), bub = __shfl_sync(kFull, ub, src);
             uint64_t bw = 0;
-            for (int64_t a = l; a < bdm; a += 32) {
-                const int32_t f = fpos[lcols[bub + a]];
-                const int32_t p = rev[bub + a];
-                bw += p > f ? (uint64_t)(p - f) : 0;
-            }
+            for (int64_t a = l; a < bdm; a += 32) bw += (uint64_t)rev[bub + a];
             bw = warp_sum(bw);
             if (l == src) W = bw;
         }
@@ -614,12 +692,16 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
                     q_small[2 * n - 1 - slot] = (int32_t)W;
                 } else {
                     const int64_t* gi = ginfo + (gid ? (int64_t)gid[u] : 0) * kGInfo;
+                    const int64_t windows = windows_below<WORDS>(gi, u);
                     q_win[slot] = u;
-                    wcount[slot] = (int32_t)windows_below<WORDS>(gi, u);
+                    wcount[slot] = (int32_t)windows;
+                    visits += (uint64_t)(windows * dm);
                 }
             }
         }
     }
+    visits = warp_sum(visits);
+    if (l == 0 && visits) atomicAdd((unsigned long long*)&acc[C4_VISITS], (unsigned long long)visits);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -732,6 +814,7 @@ __global__ void __launch_bounds__(kSmallThreads, PACKED ? 5 : 3) k_c4_light(cons
                                                                             const int32_t* __restrict__ dplus,
                                                                             const int32_t* __restrict__ fpos,
                                                                             const int32_t* __restrict__ rev,
+                                                                            const uint4* __restrict__ vinfo,
                                                                             const int64_t* __restrict__ ginfo,
                                                                             const int32_t* __restrict__ q_small,
                                                                             int64_t n, uint64_t* __restrict__ acc,
@@ -799,9 +882,8 @@ __global__ void __launch_bounds__(kSmallThreads, PACKED ? 5 : 3) k_c4_light(cons
                 uint32_t base = 0;
                 int len = 0;
                 if (a0 + l < dm) {
-                    const int32_t f = fpos[wv];
-                    base = (uint32_t)(off[wv] + f);
-                    len = rv > f ? rv - f : 0;
+                    base = vinfo ? __ldg(&vinfo[wv].w) : (uint32_t)(off[wv] + fpos[wv]);
+                    len = rv;
                 }
                 if (tabled) {
                     uint32_t part = 0;
@@ -841,7 +923,7 @@ __global__ void __launch_bounds__(kMidThreads) k_c4_mid(const int64_t* __restric
                                                         const int32_t* __restrict__ lcols,
                                                         const int32_t* __restrict__ deg, const int32_t* __restrict__ dplus,
                                                         const int32_t* __restrict__ fpos, const int32_t* __restrict__ rev,
-                                                        const int64_t* __restrict__ ginfo,
+                                                        const uint4* __restrict__ vinfo, const int64_t* __restrict__ ginfo,
                                                         const int32_t* __restrict__ q_small, int64_t n,
                                                         uint64_t* __restrict__ acc, Sink sink) {
     using Table = HashTable<kMidSlots, kMidBits, PACKED>;
@@ -880,9 +962,8 @@ __global__ void __launch_bounds__(kMidThreads) k_c4_mid(const int64_t* __restric
             int len = 0;
             if (a < dm) {
                 const int32_t wv = lcols[ub + a];
-                const int32_t f = fpos[wv], r = rev[ub + a];
-                base = (uint32_t)(off[wv] + f);
-                len = r > f ? r - f : 0;
+                base = vinfo ? __ldg(&vinfo[wv].w) : (uint32_t)(off[wv] + fpos[wv]);
+                len = rev[ub + a];
             }
             warp_flat_rel(cols, base, len, s_rel[w], [&](int32_t x, bool in) {
                 if (in) part += table.add(x);
@@ -979,7 +1060,7 @@ __device__ __forceinline__ void window_pass(const int64_t* __restrict__ off, con
             else if (table && (j & mask) == 0) p0 = bpos[(int64_t)wv * kGridCap + (j >> sl)];
             else if (table) p0 = gallop_i32(cols + wb, bpos[(int64_t)wv * kGridCap + (j >> sl)], rowlen, xlo);
             else p0 = lower_bound_i32(cols + wb, rowlen, xlo);
-            if (last) p1 = rev[ub + a];
+            if (last) p1 = (int64_t)(first ? p0 : fpos[wv]) + rev[ub + a];
             else if (table && ((j + 1) & mask) == 0 && j + 1 <= nwin) p1 = bpos[(int64_t)wv * kGridCap + ((j + 1) >> sl)];
             else if (table) p1 = gallop_i32(cols + wb, p0 < 0 ? 0 : p0, rowlen, xhi);
             else p1 = lower_bound_i32(cols + wb, rowlen, xhi);
@@ -1088,7 +1169,7 @@ __global__ void __launch_bounds__(win_threads(MINB), MINB) k_c4_window(const int
                                                               const int32_t* __restrict__ gid,
                                                               const int64_t* __restrict__ ginfo,
                                                               const int32_t* __restrict__ q_win,
-                                                              const int64_t* __restrict__ win_prefix,
+                                                              const int64_t* __restrict__ win_prefix, int64_t n,
                                                               uint64_t* __restrict__ acc, Sink sink) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t* cw = reinterpret_cast<uint32_t*>(smem_raw);
@@ -1099,7 +1180,7 @@ __global__ void __launch_bounds__(win_threads(MINB), MINB) k_c4_window(const int
     const int64_t nroots = (int64_t)acc[Q_C4_WIN];
     const int64_t total = win_prefix[nroots];
     unsigned long long* ticket = (unsigned long long*)&acc[T_C4_WIN];
-    const bool table = bpos != nullptr;
+    const bool table = bpos != nullptr && table_pays(acc, n);
     uint64_t c4 = 0;
     if (threadIdx.x == 0)
         resolve_item<WORDS>(s_next, (int64_t)atomicAdd(ticket, 1ull), total, nroots, win_prefix, q_win, gid, ginfo,
@@ -1166,6 +1247,18 @@ unsigned grid_cap(int64_t work, int threads, int64_t cap) {
     return (unsigned)b;
 }
 
+// k_c4_seglen over a whole graph's lower arcs; runs long enough to pay for finding their rows, short enough to give
+// every warp one.
+harp_status segment_lengths(const harp_csr* g, Workspace& ws, const uint4* vinfo, const int64_t* ginfo, cudaStream_t s) {
+    const int64_t warps = (int64_t)num_sms() * 64;
+    int64_t run = ((g->m + g->n) / warps + 31) / 32 * 32;
+    run = run < 32 ? 32 : (run > 256 ? 256 : run);
+    k_c4_seglen<<<grid_cap((g->m + g->n + run - 1) / run * 32, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(
+        ws.off, ws.cols, ws.offp, ws.colsp, vinfo, ginfo ? ws.gid : nullptr, ginfo, g->n, (int)run, ws.rev);
+    HARP_LAUNCHED();
+    return HARP_OK;
+}
+
 // The whole wedge pass for one window size (MINB resident window blocks per SM).
 template <int MINB>
 harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint32_t mid_max, bool merge,
@@ -1182,28 +1275,25 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
         ws.deg, n, ws.gbase, G, ws.x_lo, ws.x_hi, merge, core ? ws.off : nullptr, ws.ginfo, ws.acc);
     HARP_LAUNCHED();
     if (core) HARP_TRY(count_wedge_core(g, ws, s));  // uses rev, bpos and the queues before they are filled below
-    HARP_CK(cudaMemsetAsync(wcount, 0, (size_t)n * sizeof(int32_t), s));
     // the roots' lower lists: row prefixes of a whole graph, or their own CSR in a partitioned block
     const bool lists = ws.loff != nullptr;
     const int64_t* loff = lists ? ws.loff : ws.off;
     const int32_t* lcols = lists ? ws.lcols : ws.cols;
+    uint4* vinfo = lists ? nullptr : reinterpret_cast<uint4*>(ws.vkeys);  // the sort keys' two arrays are done with
+    k_c4_fpos<<<grid_cap(n, 256, (int64_t)sms * 64), 256, 0, s>>>(ws.off, ws.cols, ws.offp, ws.gid, ws.ginfo, n, ws.fpos,
+                                                                 vinfo);
+    HARP_LAUNCHED();
     if (lists) {
         const int64_t la = ws.lower_arcs;  // == loff[n]
-        k_c4_rev<true><<<grid_cap((la + kRevRun - 1) / kRevRun, 256, (int64_t)sms * 64), 256, 0, s>>>(
-            ws.loff, ws.lcols, ws.off, ws.cols, ws.deg, ws.dplus, ws.gid, ws.ginfo, n, la, ws.rev);
+        k_c4_seglen_rows<<<grid_cap((la + kRevRun - 1) / kRevRun, 256, (int64_t)sms * 64), 256, 0, s>>>(
+            ws.loff, ws.lcols, ws.off, ws.cols, ws.fpos, n, la, ws.rev);
+        HARP_LAUNCHED();
     } else {
-        const int64_t arcs = ws.arcs >= 0 ? ws.arcs : 2 * g->m;  // must equal off[n]
-        k_c4_rev<false><<<grid_cap((arcs + kRevRun - 1) / kRevRun, 256, (int64_t)sms * 64), 256, 0, s>>>(
-            ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.dplus, ws.gid, ws.ginfo, n, arcs, ws.rev);
+        HARP_TRY(segment_lengths(g, ws, vinfo, ws.ginfo, s));
     }
-    HARP_LAUNCHED();
-    int32_t* bpos = most_n <= kTableMinN ? nullptr : ws.bpos;
-    k_c4_bpos<WORDS><<<grid_cap(bpos ? n * kGridCap : n, 256, (int64_t)sms * 64), 256, 0, s>>>(ws.off, ws.cols, ws.gid,
-                                                                                           ws.ginfo, n, ws.fpos, bpos);
-    HARP_LAUNCHED();
     k_c4_classify<WORDS><<<grid_cap(n, 256, (int64_t)sms * 32), 256, 0, s>>>(  // a lane per root
-        loff, lcols, ws.deg, ws.dplus, ws.fpos, ws.rev, ws.gid, ws.ginfo, n, ws.own_lo, ws.own_hi, warp_max,
-        mid_max, ws.q_mid, ws.q_win, wcount, ws.acc);
+        loff, ws.deg, ws.dplus, ws.rev, ws.gid, ws.ginfo, n, ws.own_lo, ws.own_hi, warp_max, mid_max, ws.q_mid, ws.q_win,
+        wcount, ws.acc);
     HARP_LAUNCHED();
     // one word per hash slot where every graph's ranks fit beside the count
     const bool packed_light = most_n < ((int64_t)1 << (32 - kLightBits)) - 1;
@@ -1212,7 +1302,7 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     auto light = packed_light ? k_c4_light<true> : k_c4_light<false>;
     HARP_CK(cudaFuncSetAttribute(light, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)light_smem));
     light<<<sms * (packed_light ? 5 : 3), kSmallThreads, light_smem, s>>>(ws.off, ws.cols, loff, lcols, ws.deg, ws.dplus,
-                                                                          ws.fpos, ws.rev, ws.ginfo, ws.q_mid, n, ws.acc,
+                                                                          ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc,
                                                                           sink);
     HARP_LAUNCHED();
     HARP_CK(prof_mark(s, SEG_C4_SMALL));
@@ -1221,17 +1311,23 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
         auto mid = packed_mid ? k_c4_mid<true> : k_c4_mid<false>;
         HARP_CK(cudaFuncSetAttribute(mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem));
         mid<<<sms * (packed_mid ? 12 : 6), kMidThreads, mid_smem, s>>>(ws.off, ws.cols, loff, lcols, ws.deg, ws.dplus,
-                                                                       ws.fpos, ws.rev, ws.ginfo, ws.q_mid, n, ws.acc,
+                                                                       ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc,
                                                                        sink);
         HARP_LAUNCHED();
     }
     HARP_CK(prof_mark(s, SEG_C4_MID));
+    // only the queued roots' counts matter (and are set); what follows them in the scan is never read
     HARP_TRY(exclusive_scan_i32_to_i64(wcount, ws.win_prefix, n, ws.scan_tmp, ws.scan_tmp_len, s));
+    if (ws.bpos) {
+        k_c4_bpos<WORDS><<<grid_cap(n * kGridCap, 256, (int64_t)sms * 64), 256, 0, s>>>(ws.off, ws.cols, ws.gid, ws.ginfo,
+                                                                                       n, ws.fpos, ws.acc, ws.bpos);
+        HARP_LAUNCHED();
+    }
     const size_t win_smem = (size_t)WORDS * sizeof(uint32_t);
     HARP_CK(cudaFuncSetAttribute(k_c4_window<MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_smem));
     k_c4_window<MINB><<<sms * MINB, win_threads(MINB), win_smem, s>>>(ws.off, ws.cols, loff, lcols, ws.deg, ws.dplus,
                                                                 ws.fpos, ws.rev,
-                                                                bpos, ws.gid, ws.ginfo, ws.q_win, ws.win_prefix,
+                                                                ws.bpos, ws.gid, ws.ginfo, ws.q_win, ws.win_prefix, n,
                                                                 ws.acc, sink);
     HARP_LAUNCHED();
     HARP_CK(prof_mark(s, SEG_C4_WINDOW));
@@ -1241,11 +1337,11 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
 }  // namespace
 
 harp_status wedge_positions(const harp_csr* g, Workspace& ws, cudaStream_t s) {
-    const int64_t arcs = 2 * g->m;
-    k_c4_rev<false><<<grid_cap((arcs + kRevRun - 1) / kRevRun, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(
-        ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.dplus, nullptr, nullptr, g->n, arcs, ws.rev);
+    uint4* vinfo = reinterpret_cast<uint4*>(ws.vkeys);
+    k_c4_fpos<<<grid_cap(g->n, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(ws.off, ws.cols, ws.offp, nullptr, nullptr, g->n,
+                                                                          nullptr, vinfo);
     HARP_LAUNCHED();
-    return HARP_OK;
+    return segment_lengths(g, ws, vinfo, nullptr, s);
 }
 
 harp_status count_wedge_c4(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s) {

@@ -105,6 +105,7 @@ enum : int {
     ACC_LIT_CORR = 64,     // 64 lo, 65 hi: what the staged edge pass counts too much (literal.cu)
     T_LIT_EDGE = 66,       // its ticket
     Q_SORT_BLOCK = 67,     // rows for the block row sort
+    C4_VISITS = 68,        // (root, lower neighbour, window) visits of the windowed wedge mode
     kOutLen = 72
 };
 
@@ -148,7 +149,7 @@ struct Workspace {
     int32_t* cols = nullptr;       // [2m]  rank-order CSR columns, rows ascending
     int32_t* dplus = nullptr;      // [n]   out-degree (neighbours with larger rank)
     int32_t* fpos = nullptr;       // [n]   first row position holding a neighbour of degree >= 2
-    int32_t* rev = nullptr;        // [2m]  pos_w(u) for every lower arc (u -> w), at u's row position
+    int32_t* rev = nullptr;        // [2m]  wedge segment length of every lower arc (u -> w), at u's row position
     int32_t* bpos = nullptr;       // [n * kGridCap] row positions of the wedge-window grid boundaries
     int64_t* ginfo = nullptr;      // [G * kGInfo] per-graph bands of the wedge-window grid
     int64_t* offp = nullptr;       // [n+1] out-CSR offsets
@@ -247,7 +248,7 @@ struct OrbTri {
 };
 harp_status orbit_triangles(const harp_csr* g, Workspace& ws, const OrbTri& o, cudaStream_t s);
 
-// c4.cu: the position of u in w's row for every lower arc (u -> w) of a whole graph (ws.rev)
+// c4.cu: the position of u in w's row for every lower arc (u -> w) of a whole graph (ws.rev); uses ws.vkeys
 harp_status wedge_positions(const harp_csr* g, Workspace& ws, cudaStream_t s);
 
 // c4.cu: wedge anchor, non-induced 4-cycles (step a5)
