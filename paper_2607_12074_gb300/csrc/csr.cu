@@ -1,86 +1,346 @@
-// harp_build_csr on the device: canonical arc keys -> radix sort -> dedupe -> CSR.
+// harp_build_csr on the device: degrees -> offsets -> scatter -> rows sorted and deduplicated -> CSR.
 //
-// Every input pair (u, v), u != v, yields the arcs u->v and v->u as 64-bit keys (u << b) | v with
-// b = bits(n).  Self-loops and out-of-range ids become a sentinel that sorts last (out-of-range ids
-// also raise a flag that turns into HARP_EINVAL).  After the sort, the first copy of every key is
-// kept; row offsets are the positions where the source id changes.
+// Every input pair (u, v), u != v, counts towards both degrees and is scattered into both rows at slots taken by
+// atomics (equal endpoints within a warp take theirs together: edge lists often run along one vertex).  Self-loops
+// are skipped; out-of-range ids are skipped and raise a flag that turns into HARP_EINVAL.  Rows are then sorted by
+// the tiers of rowsort.cuh, equal neighbours dropped while they are written, and, where any were, the rows
+// closed up.  The rows' order makes the result independent of the order in which slots were taken.
+// (A radix sort of all arcs as 64-bit keys moved every arc 2 * bits(n) / 8 times: R-MAT scale 18, 4.1 M pairs:
+// 0.66 ms of kernels against 0.22.)
 #include "harp_internal.cuh"
+#include "rowsort.cuh"
 
 namespace harp {
 namespace {
 
-__global__ void k_make_arc_keys(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                                int64_t m_in, int64_t n, int b, uint64_t sentinel,
-                                uint64_t* __restrict__ keys, unsigned int* __restrict__ bad) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m_in;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        int32_t u = src[e], v = dst[e];
-        bool ok = u >= 0 && v >= 0 && (int64_t)u < n && (int64_t)v < n;
-        if (!ok) atomicOr(bad, 1u);
-        if (!ok || u == v) {
-            keys[2 * e] = sentinel;
-            keys[2 * e + 1] = sentinel;
-        } else {
-            keys[2 * e] = ((uint64_t)u << b) | (uint64_t)v;
-            keys[2 * e + 1] = ((uint64_t)v << b) | (uint64_t)u;
-        }
+// Words of the build's summary, read back by the host.
+enum : int { B_BAD = 0, B_MAXDEG, B_ARCS, B_RAW, B_Q_WARP, B_Q_BLOCK, B_Q_HUB, B_WORDS = 8 };
+
+// An input pair's endpoints; valid: in range and not a self-loop.
+struct Pair {
+    int32_t u, v;
+    bool valid;
+};
+
+__device__ __forceinline__ Pair load_pair(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t e,
+                                          int64_t m_in, int64_t n, bool& bad) {
+    Pair p{-1, -1, false};
+    if (e < m_in) {
+        p.u = src[e];
+        p.v = dst[e];
+        const bool ok = p.u >= 0 && p.v >= 0 && (int64_t)p.u < n && (int64_t)p.v < n;
+        bad |= !ok;
+        p.valid = ok && p.u != p.v;
     }
+    return p;
 }
 
-__global__ void k_unique_flags(const uint64_t* __restrict__ keys, int64_t len, uint64_t sentinel,
-                               int32_t* __restrict__ flag) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t k = keys[i];
-        flag[i] = (k != sentinel && (i == 0 || keys[i - 1] != k)) ? 1 : 0;
-    }
-}
-
-__global__ void k_compact_cols(const uint64_t* __restrict__ keys, const int32_t* __restrict__ flag,
-                               const int64_t* __restrict__ pos, int64_t len, uint64_t low_mask,
-                               int32_t* __restrict__ cols, uint64_t* __restrict__ ckeys) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (flag[i]) {
-            int64_t p = pos[i];
-            cols[p] = (int32_t)(keys[i] & low_mask);
-            ckeys[p] = keys[i];
-        }
-    }
-}
-
-// off[x] = first position whose source id is >= x (positions of the compacted, sorted arcs).
-__global__ void k_row_offsets(const uint64_t* __restrict__ ckeys, int64_t M, int64_t n, int b,
-                              int64_t* __restrict__ off) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < M;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        int64_t u = (int64_t)(ckeys[p] >> b);
-        int64_t up = p > 0 ? (int64_t)(ckeys[p - 1] >> b) : -1;
-        for (int64_t x = up + 1; x <= u; ++x) off[x] = p;
-        if (p == M - 1)
-            for (int64_t x = u + 1; x <= n; ++x) off[x] = M;
-    }
-}
-
-__global__ void k_fill_i64(int64_t* __restrict__ a, int64_t len, int64_t v) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len;
-         i += (int64_t)gridDim.x * blockDim.x)
-        a[i] = v;
-}
-
-__global__ void k_max_degree(const int64_t* __restrict__ off, int64_t n, unsigned long long* __restrict__ out) {
-    int64_t best = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        int64_t d = off[v + 1] - off[v];
-        best = d > best ? d : best;
-    }
+__global__ void __launch_bounds__(256) k_build_degrees(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                                       int64_t m_in, int64_t n, int32_t* __restrict__ deg,
+                                                       unsigned long long* __restrict__ summary) {
+    const int l = lane_id();
+    bool bad = false;
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - l; base < m_in;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const Pair p = load_pair(src, dst, base + l, m_in, n, bad);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        int64_t other = __shfl_xor_sync(kFull, best, o);
-        best = other > best ? other : best;
+        for (int h = 0; h < 2; ++h) {
+            const int32_t x = p.valid ? (h ? p.v : p.u) : -1 - l;
+            const uint32_t same = __match_any_sync(kFull, x);
+            if (p.valid && l == __ffs(same) - 1) atomicAdd(&deg[x], __popc(same));
+        }
     }
-    if (lane_id() == 0) atomicMax(out, (unsigned long long)best);
+    if (__any_sync(kFull, bad) && l == 0) atomicOr(&summary[B_BAD], 1ull);
+}
+
+// deg counts down to zero: each pair's slot is the value before.
+__global__ void __launch_bounds__(256) k_build_scatter(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                                       int64_t m_in, int64_t n, const int64_t* __restrict__ roff,
+                                                       int32_t* __restrict__ deg, int32_t* __restrict__ out) {
+    const int l = lane_id();
+    bool bad = false;
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - l; base < m_in;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const Pair p = load_pair(src, dst, base + l, m_in, n, bad);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int32_t x = p.valid ? (h ? p.v : p.u) : -1 - l, y = h ? p.u : p.v;
+            const uint32_t same = __match_any_sync(kFull, x);
+            const int leader = __ffs(same) - 1;
+            int left = 0;
+            if (p.valid && l == leader) left = atomicSub(&deg[x], __popc(same));
+            left = __shfl_sync(kFull, left, leader);
+            if (p.valid) out[roff[x] + left - 1 - __popc(same & lanemask_lt())] = y;
+        }
+    }
+}
+
+// Rows of at most kTierA entries, 32 consecutive rows per warp (a lane's network up to 16, the warp's above); longer
+// ones are queued: the warp sort's from the front of q, hubs from its back, the block sort's in q_block.
+template <int P>
+__device__ __forceinline__ int lane_unique_row(const int32_t* __restrict__ in, int32_t* __restrict__ out, int d) {
+    int32_t a[P];
+#pragma unroll
+    for (int r = 0; r < P; ++r) a[r] = r < d ? in[r] : kPadKey;
+    sort_regs<P>(a);
+    int k = 0;
+#pragma unroll
+    for (int r = 0; r < P; ++r)
+        if (r < d && (r == 0 || a[r] != a[r - 1])) out[k++] = a[r];
+    return k;
+}
+
+__global__ void __launch_bounds__(256) k_build_rows_small(const int64_t* __restrict__ roff, int64_t n,
+                                                          const int32_t* __restrict__ in, int32_t* __restrict__ out,
+                                                          int32_t* __restrict__ ndeg, int32_t* __restrict__ q,
+                                                          int32_t* __restrict__ q_block,
+                                                          unsigned long long* __restrict__ summary) {
+    const int l = lane_id();
+    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i0 = wid * 32; i0 < n; i0 += nw * 32) {
+        const int64_t i = i0 + l;
+        const int64_t b = i < n ? roff[i] : 0;
+        const int d = i < n ? (int)(roff[i + 1] - b) : -1;
+        if (d == 0) ndeg[i] = 0;
+        else if (d >= 1 && d <= 8) ndeg[i] = lane_unique_row<8>(in + b, out + b, d);
+        else if (d > 8 && d <= 16) ndeg[i] = lane_unique_row<16>(in + b, out + b, d);
+        const int cls = d > kTierB ? 2 : (d > kTierB1 ? 1 : (d > kTierA ? 0 : -1));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const uint32_t m = __ballot_sync(kFull, cls == c);
+            if (!m) continue;
+            unsigned long long start = 0;
+            const int leader = __ffs(m) - 1;
+            if (l == leader) start = atomicAdd(&summary[B_Q_WARP + c], (unsigned long long)__popc(m));
+            start = __shfl_sync(kFull, start, leader);
+            if (cls != c) continue;
+            const int64_t k = (int64_t)start + __popc(m & lanemask_lt());
+            if (c == 0) q[k] = (int32_t)i;
+            else if (c == 1) q_block[k] = (int32_t)i;
+            else q[n - 1 - k] = (int32_t)i;
+        }
+        uint32_t rest = __ballot_sync(kFull, d > 16 && d <= kTierA);
+        while (rest) {  // four rows at a time: their loads overlap
+            int row[4], dr[4];
+            int64_t rb[4];
+            int32_t v[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                row[t] = rest ? __ffs(rest) - 1 : -1;
+                rest &= rest - 1;
+                dr[t] = __shfl_sync(kFull, d, row[t] & 31);
+                if (row[t] < 0) dr[t] = 0;
+                rb[t] = __shfl_sync(kFull, b, row[t] & 31);
+                v[t] = l < dr[t] ? in[rb[t] + l] : kPadKey;
+            }
+#pragma unroll
+            for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+                for (int j = k >> 1; j > 0; j >>= 1) {
+                    const bool keep_min = ((l & j) == 0) == ((l & k) == 0);
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const int32_t o = __shfl_xor_sync(kFull, v[t], j);
+                        v[t] = keep_min ? min(v[t], o) : max(v[t], o);
+                    }
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int32_t before = __shfl_up_sync(kFull, v[t], 1);
+                const bool first = l < dr[t] && (l == 0 || v[t] != before);
+                const uint32_t kept = __ballot_sync(kFull, first);
+                if (first) out[rb[t] + __popc(kept & lanemask_lt())] = v[t];
+                if (l == 0 && row[t] >= 0) ndeg[i0 + row[t]] = __popc(kept);
+            }
+        }
+    }
+}
+
+// Unique members of a sorted run held lane * E + e in v (d of them count); before: the key ahead of the run's
+// first (kPadKey: none).  Writes them from out on and returns their number (in every lane).
+template <int E>
+__device__ __forceinline__ int warp_write_unique(const int32_t (&v)[E], int d, int32_t before, int32_t* __restrict__ out) {
+    const int l = lane_id();
+    const int32_t up = __shfl_up_sync(kFull, v[E - 1], 1);
+    uint32_t keep = 0;  // bit e: register e is the first of its value
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int32_t prev = e > 0 ? v[e > 0 ? e - 1 : 0] : (l > 0 ? up : before);
+        if (l * E + e < d && v[e] != prev) keep |= 1u << e;
+    }
+    const int c = __popc(keep);
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (l >= o) incl += y;
+    }
+    int at = incl - c;
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if ((keep >> e) & 1u) out[at++] = v[e];
+    return __shfl_sync(kFull, incl, 31);
+}
+
+constexpr int kMidWarps = 4;
+
+template <int E>
+__device__ __forceinline__ int warp_unique_row(const int32_t* __restrict__ in, int32_t* __restrict__ out, int d) {
+    const int l = lane_id();
+    int32_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = e * 32 + l < d ? in[e * 32 + l] : kPadKey;  // any order will do
+    warp_bitonic_sort<E>(v, true);
+    return warp_write_unique<E>(v, d, kPadKey, out);
+}
+
+__global__ void __launch_bounds__(kMidWarps * 32) k_build_rows_mid(const int64_t* __restrict__ roff,
+                                                                    const int32_t* __restrict__ in,
+                                                                    int32_t* __restrict__ out, int32_t* __restrict__ ndeg,
+                                                                    const int32_t* __restrict__ q,
+                                                                    const unsigned long long* __restrict__ summary) {
+    const int64_t nq = (int64_t)summary[B_Q_WARP];
+    for (int64_t k = (int64_t)blockIdx.x * kMidWarps + (threadIdx.x >> 5); k < nq; k += (int64_t)gridDim.x * kMidWarps) {
+        const int64_t i = q[k], b = roff[i];
+        const int d = (int)(roff[i + 1] - b);
+        int u;
+        if (d <= 64) u = warp_unique_row<2>(in + b, out + b, d);
+        else if (d <= 128) u = warp_unique_row<4>(in + b, out + b, d);
+        else if (d <= 256) u = warp_unique_row<8>(in + b, out + b, d);
+        else if (d <= 512) u = warp_unique_row<16>(in + b, out + b, d);
+        else u = warp_unique_row<32>(in + b, out + b, d);
+        if (lane_id() == 0) ndeg[i] = u;
+    }
+}
+
+__global__ void __launch_bounds__(kBlockWarps * 32) k_build_rows_block(const int64_t* __restrict__ roff,
+                                                                       const int32_t* __restrict__ in,
+                                                                       int32_t* __restrict__ out,
+                                                                       int32_t* __restrict__ ndeg,
+                                                                       const int32_t* __restrict__ q_block,
+                                                                       const unsigned long long* __restrict__ summary) {
+    constexpr int E = kBlockE, RUN = 32 * E;
+    __shared__ int32_t buf[kTierB];
+    __shared__ int32_t s_last[kBlockWarps];
+    __shared__ int s_kept[kBlockWarps];
+    const int w = threadIdx.x >> 5, l = lane_id();
+    const int64_t nq = (int64_t)summary[B_Q_BLOCK];
+    for (int64_t k = blockIdx.x; k < nq; k += gridDim.x) {
+        const int64_t i = q_block[k], b = roff[i];
+        const int d = (int)(roff[i + 1] - b);
+        int32_t v[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int x = w * RUN + e * 32 + l;
+            v[e] = x < d ? in[b + x] : kPadKey;
+        }
+        block_bitonic_sort(v, buf);
+        if (l == 31) s_last[w] = v[E - 1];
+        __syncthreads();
+        const int32_t before = w > 0 ? s_last[w - 1] : kPadKey;
+        const int mine = d - w * RUN < 0 ? 0 : (d - w * RUN < RUN ? d - w * RUN : RUN);
+        // the warp's unique keys go to its own part of buf, then behind those of the warps before it
+        const int kept = warp_write_unique<E>(v, mine, before, buf + w * RUN);
+        if (l == 0) s_kept[w] = kept;
+        __syncthreads();
+        int at = 0, all = 0;
+        for (int x = 0; x < kBlockWarps; ++x) {
+            if (x < w) at += s_kept[x];
+            all += s_kept[x];
+        }
+        for (int x = l; x < kept; x += 32) out[b + at + x] = buf[w * RUN + x];
+        if (threadIdx.x == 0) ndeg[i] = all;
+        __syncthreads();  // buf and the shared words are read before the next row
+    }
+}
+
+__global__ void __launch_bounds__(kBitmapThreads) k_build_rows_bitmap(const int64_t* __restrict__ roff, int64_t n,
+                                                                      const int32_t* __restrict__ in,
+                                                                      int32_t* __restrict__ out,
+                                                                      int32_t* __restrict__ ndeg,
+                                                                      const int32_t* __restrict__ q,
+                                                                      const unsigned long long* __restrict__ summary) {
+    extern __shared__ uint32_t bm[];
+    __shared__ int s_count[kBitmapWarps];
+    const int64_t nq = (int64_t)summary[B_Q_HUB];
+    for (int64_t k = blockIdx.x; k < nq; k += gridDim.x) {
+        const int64_t i = q[n - 1 - k], b = roff[i], e = roff[i + 1];
+        int64_t dst = b;
+        for (int64_t lo = 0; lo < n; lo += 32 * (int64_t)kBitmapWords) {
+            const int64_t hi = lo + 32 * (int64_t)kBitmapWords < n ? lo + 32 * (int64_t)kBitmapWords : n;
+            const int groups = (int)((hi - lo + 1023) / 1024), per = (groups + kBitmapWarps - 1) / kBitmapWarps;
+            for (int x = threadIdx.x; x < per * kBitmapThreads; x += kBitmapThreads) bm[x] = 0;
+            __syncthreads();
+            for (int64_t p = b + threadIdx.x; p < e; p += 4 * kBitmapThreads) {
+                int32_t x[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) x[t] = p + t * kBitmapThreads < e ? in[p + t * kBitmapThreads] : -1;
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (x[t] >= lo && x[t] < hi) {
+                        const uint32_t y = (uint32_t)(x[t] - lo);
+                        atomicOr(&bm[y >> 5], 1u << (y & 31));
+                    }
+            }
+            __syncthreads();
+            dst += bitmap_write(bm, per, lo, out + dst, s_count, [](int32_t) {});
+            __syncthreads();  // the bitmap is read before the next window clears it
+        }
+        if (threadIdx.x == 0) ndeg[i] = (int32_t)(dst - b);
+    }
+}
+
+// Largest degree, and the arc counts before and after dropping repeats.
+__global__ void __launch_bounds__(256) k_build_summary(const int32_t* __restrict__ ndeg, const int64_t* __restrict__ off,
+                                                       const int64_t* __restrict__ roff, int64_t n,
+                                                       unsigned long long* __restrict__ summary) {
+    int32_t best = 0;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+        best = max(best, ndeg[v]);
+    best = __reduce_max_sync(kFull, best);
+    if (lane_id() == 0 && best > 0) atomicMax(&summary[B_MAXDEG], (unsigned long long)best);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        summary[B_ARCS] = (unsigned long long)off[n];
+        summary[B_RAW] = (unsigned long long)roff[n];
+    }
+}
+
+// Closes up the rows: cols[off[i] + k] = in[roff[i] + k], 32 consecutive rows per warp (a lane copies a short row).
+__global__ void __launch_bounds__(256) k_build_compact(const int64_t* __restrict__ roff, const int64_t* __restrict__ off,
+                                                       int64_t n, const int32_t* __restrict__ in,
+                                                       int32_t* __restrict__ cols) {
+    const int l = lane_id();
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; i0 < n; i0 += nw * 32) {
+        const int64_t i = i0 + l;
+        const int64_t s = i < n ? roff[i] : 0, o = i < n ? off[i] : 0;
+        const int d = i < n ? (int)(off[i + 1] - o) : 0;
+        if (d <= 16) {  // all loads first
+            int32_t x[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) x[k] = k < d ? in[s + k] : 0;
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if (k < d) cols[o + k] = x[k];
+        }
+        uint32_t rest = __ballot_sync(kFull, d > 16);
+        while (rest) {
+            const int src = __ffs(rest) - 1;
+            rest &= rest - 1;
+            const int64_t rs = __shfl_sync(kFull, s, src), ro = __shfl_sync(kFull, o, src);
+            const int rd = __shfl_sync(kFull, d, src);
+            for (int k = l; k < rd; k += 128) {
+                int32_t x[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) x[t] = k + 32 * t < rd ? in[rs + k + 32 * t] : 0;
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (k + 32 * t < rd) cols[ro + k + 32 * t] = x[t];
+            }
+        }
+    }
 }
 
 unsigned grid_for(int64_t work, int threads) {
@@ -90,38 +350,20 @@ unsigned grid_for(int64_t work, int threads) {
     return (unsigned)b;
 }
 
-int bits_for(int64_t x) {  // number of bits to represent x (x >= 0)
-    int b = 0;
-    while (b < 63 && ((int64_t)1 << b) <= x) ++b;
-    return b < 1 ? 1 : b;
-}
+size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
 
 harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t* d_src,
                              const int32_t* d_dst, cudaStream_t s) {
-    const int b = bits_for(n);
-    const uint64_t sentinel = ((uint64_t)n << b) | (uint64_t)n;
-    const int64_t len = 2 * m_in;
     harp_status st = HARP_OK;
-
-    uint64_t *keys = nullptr, *alt = nullptr;
-    int32_t* flag = nullptr;
-    int64_t* pos = nullptr;
-    uint32_t* hist = nullptr;
-    int64_t* tmp = nullptr;
-    unsigned long long* small = nullptr;  // [0] bad flag, [1] max degree
-    const size_t tmp_len = scan_tmp_needed(len > 0 ? len : 1) + scan_tmp_needed((int64_t)radix_hist_len(len));
-    const size_t hist_len = radix_hist_len(len);
-
+    const int64_t nn = n > 0 ? n : 1;
+    int32_t *raw = nullptr, *sorted = nullptr;  // [2 m_in] scattered and sorted rows, at roff
+    unsigned char* slab = nullptr;              // everything else
     auto cleanup = [&]() {
-        if (keys) cudaFreeAsync(keys, s);
-        if (alt) cudaFreeAsync(alt, s);
-        if (flag) cudaFreeAsync(flag, s);
-        if (pos) cudaFreeAsync(pos, s);
-        if (hist) cudaFreeAsync(hist, s);
-        if (tmp) cudaFreeAsync(tmp, s);
-        if (small) cudaFreeAsync(small, s);
+        if (raw) cudaFreeAsync(raw, s);
+        if (sorted) cudaFreeAsync(sorted, s);
+        if (slab) cudaFreeAsync(slab, s);
     };
 #define BCK(call)                                              \
     do {                                                       \
@@ -137,65 +379,88 @@ harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t
         st = (call);                                           \
         if (st != HARP_OK) { cleanup(); return st; }           \
     } while (0)
+#define BLAUNCHED()                                            \
+    do {                                                       \
+        note_launch();                                         \
+        BCK(cudaGetLastError());                               \
+    } while (0)
 
-    BCK(cudaMallocAsync((void**)&small, 2 * sizeof(unsigned long long), s));
-    BCK(cudaMemsetAsync(small, 0, 2 * sizeof(unsigned long long), s));
     BCK(cudaMallocAsync((void**)&g->off, (size_t)(n + 1) * sizeof(int64_t), s));
-    int64_t M = 0;
-    if (len > 0) {
-        BCK(cudaMallocAsync((void**)&keys, (size_t)len * sizeof(uint64_t), s));
-        BCK(cudaMallocAsync((void**)&alt, (size_t)len * sizeof(uint64_t), s));
-        BCK(cudaMallocAsync((void**)&flag, (size_t)len * sizeof(int32_t), s));
-        BCK(cudaMallocAsync((void**)&pos, (size_t)(len + 1) * sizeof(int64_t), s));
-        BCK(cudaMallocAsync((void**)&hist, hist_len * sizeof(uint32_t), s));
-        BCK(cudaMallocAsync((void**)&tmp, tmp_len * sizeof(int64_t), s));
-        k_make_arc_keys<<<grid_for(m_in, 256), 256, 0, s>>>(d_src, d_dst, m_in, n, b, sentinel, keys,
-                                                             (unsigned int*)small);
-        note_launch();
-        BCK(cudaGetLastError());
-        BTRY(radix_sort_u64(&keys, &alt, len, 0, 2 * b, hist, tmp, tmp_len, s));
-        k_unique_flags<<<grid_for(len, 256), 256, 0, s>>>(keys, len, sentinel, flag);
-        note_launch();
-        BCK(cudaGetLastError());
-        BTRY(exclusive_scan_i32_to_i64(flag, pos, len, tmp, tmp_len, s));
-        BCK(cudaMemcpyAsync(&M, pos + len, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    if (m_in == 0) {
+        BCK(cudaMemsetAsync(g->off, 0, (size_t)(n + 1) * sizeof(int64_t), s));
+        BCK(cudaMallocAsync((void**)&g->cols, sizeof(int32_t), s));
+        g->n = n;
+        g->csr_bytes = (size_t)(n + 1) * sizeof(int64_t) + sizeof(int32_t);
+        BCK(cudaStreamSynchronize(s));
+        return HARP_OK;
     }
-    unsigned long long bad = 0;
-    BCK(cudaMemcpyAsync(&bad, small, sizeof(bad), cudaMemcpyDeviceToHost, s));
+    const size_t tmp_len = scan_tmp_needed(nn) + 64;
+    const size_t head = align256(B_WORDS * sizeof(unsigned long long)), per_n = align256((size_t)nn * sizeof(int32_t));
+    const size_t offs = align256((size_t)(nn + 1) * sizeof(int64_t));
+    BCK(cudaMallocAsync((void**)&slab, head + 4 * per_n + offs + tmp_len * sizeof(int64_t), s));
+    unsigned long long* summary = reinterpret_cast<unsigned long long*>(slab);
+    int32_t* deg = reinterpret_cast<int32_t*>(slab + head);
+    int32_t* ndeg = reinterpret_cast<int32_t*>(slab + head + per_n);
+    int32_t* q = reinterpret_cast<int32_t*>(slab + head + 2 * per_n);
+    int32_t* q_block = reinterpret_cast<int32_t*>(slab + head + 3 * per_n);
+    int64_t* roff = reinterpret_cast<int64_t*>(slab + head + 4 * per_n);
+    int64_t* tmp = reinterpret_cast<int64_t*>(slab + head + 4 * per_n + offs);
+    BCK(cudaMallocAsync((void**)&raw, 2 * (size_t)m_in * sizeof(int32_t), s));
+    BCK(cudaMallocAsync((void**)&sorted, 2 * (size_t)m_in * sizeof(int32_t), s));
+    BCK(cudaMemsetAsync(slab, 0, head + per_n, s));  // summary and degrees
+    k_build_degrees<<<grid_for(m_in, 256), 256, 0, s>>>(d_src, d_dst, m_in, n, deg, summary);
+    BLAUNCHED();
+    BTRY(exclusive_scan_i32_to_i64(deg, roff, n, tmp, tmp_len, s));
+    k_build_scatter<<<grid_for(m_in, 256), 256, 0, s>>>(d_src, d_dst, m_in, n, roff, deg, raw);
+    BLAUNCHED();
+    k_build_rows_small<<<grid_for(n, 256), 256, 0, s>>>(roff, n, raw, sorted, ndeg, q, q_block, summary);
+    BLAUNCHED();
+    // a row has at most m_in entries: tiers above that are empty
+    if (m_in > kTierA) {
+        k_build_rows_mid<<<num_sms() * 8, kMidWarps * 32, 0, s>>>(roff, raw, sorted, ndeg, q, summary);
+        BLAUNCHED();
+    }
+    if (m_in > kTierB1) {
+        k_build_rows_block<<<num_sms() * 4, kBlockWarps * 32, 0, s>>>(roff, raw, sorted, ndeg, q_block, summary);
+        BLAUNCHED();
+    }
+    if (m_in > kTierB) {
+        const size_t smem = sizeof(uint32_t) * (size_t)kBitmapWords;
+        BCK(cudaFuncSetAttribute(k_build_rows_bitmap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_build_rows_bitmap<<<num_sms(), kBitmapThreads, smem, s>>>(roff, n, raw, sorted, ndeg, q, summary);
+        BLAUNCHED();
+    }
+    BTRY(exclusive_scan_i32_to_i64(ndeg, g->off, n, tmp, tmp_len, s));
+    k_build_summary<<<grid_for(n, 256), 256, 0, s>>>(ndeg, g->off, roff, n, summary);
+    BLAUNCHED();
+    unsigned long long host[B_WORDS] = {0};
+    BCK(cudaMemcpyAsync(host, summary, sizeof(host), cudaMemcpyDeviceToHost, s));
     BCK(cudaStreamSynchronize(s));
-    if (bad) {
+    if (host[B_BAD]) {
         cleanup();
         return HARP_EINVAL;
     }
+    const int64_t M = (int64_t)host[B_ARCS];
     g->n = n;
     g->m = M / 2;
-    BCK(cudaMallocAsync((void**)&g->cols, (size_t)(M > 0 ? M : 1) * sizeof(int32_t), s));
+    g->max_deg = (int64_t)host[B_MAXDEG];
     g->csr_bytes = (size_t)(n + 1) * sizeof(int64_t) + (size_t)(M > 0 ? M : 1) * sizeof(int32_t);
-    if (M > 0) {
-        // reuse `alt` for the compacted keys
-        k_compact_cols<<<grid_for(len, 256), 256, 0, s>>>(keys, flag, pos, len, ((uint64_t)1 << b) - 1,
-                                                           g->cols, alt);
-        note_launch();
-        BCK(cudaGetLastError());
-        k_row_offsets<<<grid_for(M, 256), 256, 0, s>>>(alt, M, n, b, g->off);
-        note_launch();
-        BCK(cudaGetLastError());
-        k_max_degree<<<grid_for(n, 256), 256, 0, s>>>(g->off, n, small + 1);
-        note_launch();
-        BCK(cudaGetLastError());
+    if (M == 2 * m_in) {  // nothing was dropped: the sorted rows are the columns
+        g->cols = sorted;
+        sorted = nullptr;
     } else {
-        k_fill_i64<<<grid_for(n + 1, 256), 256, 0, s>>>(g->off, n + 1, 0);
-        note_launch();
-        BCK(cudaGetLastError());
+        BCK(cudaMallocAsync((void**)&g->cols, (size_t)(M > 0 ? M : 1) * sizeof(int32_t), s));
+        if (M > 0) {
+            k_build_compact<<<grid_for(n, 256), 256, 0, s>>>(roff, g->off, n, sorted, g->cols);
+            BLAUNCHED();
+        }
+        BCK(cudaStreamSynchronize(s));
     }
-    unsigned long long md = 0;
-    BCK(cudaMemcpyAsync(&md, small + 1, sizeof(md), cudaMemcpyDeviceToHost, s));
-    BCK(cudaStreamSynchronize(s));
-    g->max_deg = (int64_t)md;
     cleanup();
     return HARP_OK;
 #undef BCK
 #undef BTRY
+#undef BLAUNCHED
 }
 
 }  // namespace harp

@@ -15,13 +15,11 @@
 // and for hubs a bitmap of the ranks, or a per-row LSD radix sort through global memory where the graph
 // has too many ranks for one (the last three from queues filled by the relabel pass).
 #include "harp_internal.cuh"
+#include "rowsort.cuh"
 
 namespace harp {
 namespace {
 
-constexpr int kTierA = 32;
-constexpr int kTierB1 = 1024;
-constexpr int kTierB = 4096;
 
 int bits_for(int64_t x) {
     int b = 0;
@@ -111,26 +109,6 @@ __global__ void k_relabel(const uint64_t* __restrict__ keys, int64_t n, int b, i
 // registers padded with +inf; the warp then sorts its rows of 17..32 together, a bitonic network over
 // the lanes.  A warp per row left most lanes idle on the many short rows of sparse graphs.
 template <int P>
-__device__ __forceinline__ void sort_regs(int32_t (&a)[P]) {
-#pragma unroll
-    for (int k = 2; k <= P; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-#pragma unroll
-            for (int i = 0; i < P; ++i) {
-                const int p = i ^ j;
-                if (p > i) {
-                    const int32_t lo = min(a[i], a[p]), hi = max(a[i], a[p]);
-                    const bool up = (i & k) == 0;
-                    a[i] = up ? lo : hi;
-                    a[p] = up ? hi : lo;
-                }
-            }
-        }
-    }
-}
-
-template <int P>
 __device__ __forceinline__ void lane_sort_row(int64_t i, int d, const int64_t* __restrict__ goff,
                                               const int32_t* __restrict__ gcols, const int32_t* __restrict__ order,
                                               const int32_t* __restrict__ perm, const int64_t* __restrict__ off,
@@ -211,50 +189,6 @@ __global__ void __launch_bounds__(256) k_sort_rows_warp(const int64_t* __restric
     }
 }
 
-// Bitonic network over 32 * E keys held by a warp, key lane * E + e in register e: steps of stride below E stay in
-// a lane's registers, the others exchange over the lanes.  Sorts blocks of 2, 4, .. up to 32 * E; up: the final
-// order of the whole (descending where false, for a larger network's alternate halves).
-template <int E>
-__device__ __forceinline__ void bitonic_step(int32_t (&v)[E], int j, bool up_all, int k) {
-    const int l = lane_id();
-    if (j >= E) {
-        const int jl = j / E;
-        const bool lower = (l & jl) == 0;
-        const bool up = k >= 32 * E ? up_all : ((l * E) & k) == 0;  // k > j >= E: a bit of the lane
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int32_t o = __shfl_xor_sync(kFull, v[e], jl);
-            v[e] = lower == up ? min(v[e], o) : max(v[e], o);
-        }
-    } else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int p = e ^ j;
-            if (p > e && p < E) {
-                const bool up = k >= 32 * E ? up_all : ((l * E + e) & k) == 0;
-                const int32_t lo = min(v[e], v[p]), hi = max(v[e], v[p]);
-                v[e] = up ? lo : hi;
-                v[p] = up ? hi : lo;
-            }
-        }
-    }
-}
-
-template <int E>
-__device__ __forceinline__ void warp_bitonic_sort(int32_t (&v)[E], bool up) {
-#pragma unroll
-    for (int k = 2; k <= 32 * E; k <<= 1)
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) bitonic_step<E>(v, j, up, k);
-}
-
-// The last merge steps of a larger network: strides 16 * E .. 1, all in one direction.
-template <int E>
-__device__ __forceinline__ void warp_bitonic_merge(int32_t (&v)[E], bool up) {
-#pragma unroll
-    for (int j = 16 * E; j > 0; j >>= 1) bitonic_step<E>(v, j, up, 32 * E);
-}
-
 // Tier B1: 32 < d <= 1024, a warp per row, E registers a lane.  (Through shared memory, a warp barrier per
 // stage up to 256 and a block barrier per stage above: 0.23 + 0.87 ms on R-MAT scale 20.)
 constexpr int kMidWarps = 4;
@@ -305,11 +239,7 @@ __global__ void __launch_bounds__(kMidWarps * 32) k_sort_rows_mid(const int64_t*
     }
 }
 
-// Tier B: 1024 < d <= 4096, one block per row: 16 warps sort 256 keys each (in alternate directions), then the
-// merges of 512, 1024, 2048 and 4096 keys exchange through shared memory for strides of 256 and more (10
-// barriers instead of one per stage of the whole network) and finish in registers.
-constexpr int kBlockE = 8;
-constexpr int kBlockWarps = kTierB / (32 * kBlockE);
+// Tier B: 1024 < d <= 4096, one block per row (block_bitonic_sort).
 
 __global__ void __launch_bounds__(kBlockWarps * 32) k_sort_rows_block(const int64_t* __restrict__ goff,
                                                                       const int32_t* __restrict__ gcols,
@@ -338,25 +268,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32) k_sort_rows_block(const int6
         }
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = v[e] >= 0 ? perm[v[e]] : 0x7fffffff;
-        warp_bitonic_sort<E>(v, (w & 1) == 0);
-        // buf holds key x of warp w's run at w * RUN + (x mod E) * 32 + x / E: register e of lane l, conflict-free;
-        // exchanges of stride >= RUN keep x, so they only change the run
-        for (int k = 2; k <= kBlockWarps; k <<= 1) {  // merge runs of k warps
-            const bool up = (w & k) == 0;             // k = kBlockWarps: every warp
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                __syncthreads();  // the previous exchange is read
-#pragma unroll
-                for (int e = 0; e < E; ++e) buf[w * RUN + e * 32 + l] = v[e];
-                __syncthreads();
-                const bool lower = (w & j) == 0;
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const int32_t o = buf[(w ^ j) * RUN + e * 32 + l];
-                    v[e] = lower == up ? min(v[e], o) : max(v[e], o);
-                }
-            }
-            warp_bitonic_merge<E>(v, up);
-        }
+        block_bitonic_sort(v, buf);
         int above = 0;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -380,12 +292,6 @@ __global__ void __launch_bounds__(kBlockWarps * 32) k_sort_rows_block(const int6
 
 // Tier C: hubs (d > 4096) of graphs of at most kBitmapRanks ranks: a block per row sets the row's ranks in a bitmap
 // in shared memory and writes them out in order, a window of ranks at a time (one for up to 1.6 M ranks).
-constexpr int kBitmapThreads = 1024;
-constexpr int kBitmapWarps = kBitmapThreads / 32;
-constexpr int kBitmapWords = 50176;  // 196 KiB; a multiple of 32 * kBitmapWarps
-constexpr int64_t kBitmapRanks = 4 * 32 * (int64_t)kBitmapWords;
-static_assert(kBitmapWords % (32 * kBitmapWarps) == 0, "every warp takes whole groups of 32 words");
-
 __global__ void __launch_bounds__(kBitmapThreads) k_sort_rows_bitmap(const int64_t* __restrict__ goff,
                                                                      const int32_t* __restrict__ gcols,
                                                                      const int32_t* __restrict__ order,
@@ -430,34 +336,7 @@ __global__ void __launch_bounds__(kBitmapThreads) k_sort_rows_bitmap(const int64
                     }
             }
             __syncthreads();
-            int count = 0;
-            for (int g = 0; g < per; ++g) count += __popc(bm[(w * per + g) * 32 + l]);
-            count = warp_sum(count);
-            if (l == 0) s_count[w] = count;
-            __syncthreads();
-            const int before_me = l < w ? s_count[l] : 0;  // kBitmapWarps == 32
-            int64_t out = dst + warp_sum(before_me);
-            const int all = warp_sum(s_count[l]);
-            for (int g = 0; g < per; ++g) {
-                const int word = (w * per + g) * 32 + l;
-                uint32_t bits = bm[word];
-                const int c = __popc(bits);
-                int incl = c;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(kFull, incl, o);
-                    if (l >= o) incl += y;
-                }
-                int64_t p = out + incl - c;
-                while (bits) {
-                    const int32_t x = (int32_t)(lo + (int64_t)word * 32 + __ffs(bits) - 1);
-                    bits &= bits - 1;
-                    cols[p++] = x;
-                    above += x > (int32_t)i;
-                }
-                out += __shfl_sync(kFull, incl, 31);
-            }
-            dst += all;
+            dst += bitmap_write(bm, per, lo, cols + dst, s_count, [&](int32_t x) { above += x > (int32_t)i; });
             __syncthreads();  // the bitmap is read before the next window clears it
         }
         above = warp_sum(above);
@@ -467,8 +346,6 @@ __global__ void __launch_bounds__(kBitmapThreads) k_sort_rows_bitmap(const int64
         __syncthreads();
     }
 }
-static_assert(kBitmapWarps == 32, "a lane per warp in the block's prefix");
-
 // Tier C, graphs of more ranks: one block per hub row, LSD radix sort (8-bit digits) through global memory.
 // Pass p reads the previous pass's output; pass 0 reads the old row through perm.  The pass count
 // decides which buffer each pass writes so that the last one lands in `cols`.
@@ -590,11 +467,20 @@ __global__ void __launch_bounds__(256) k_out_csr(const int64_t* __restrict__ off
             const int64_t dstb = offp[i];
             const uint64_t di1 = (uint64_t)deg[i] - 1;
             uint64_t row_pw = 0;
-            for (int64_t k = 0; k < dp; ++k) {
-                const int32_t v = cols[srcb + k];
-                colsp[dstb + k] = v;
-                te[dstb + k] = 0;
-                row_pw += di1 * ((uint64_t)deg[v] - 1);
+            for (int64_t k = 0; k < dp; k += 8) {  // eight loads in flight
+                int32_t v[8];
+                uint64_t dv[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) v[t] = k + t < dp ? cols[srcb + k + t] : -1;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) dv[t] = v[t] >= 0 ? (uint64_t)deg[v[t]] : 1;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    if (v[t] < 0) continue;
+                    colsp[dstb + k + t] = v[t];
+                    te[dstb + k + t] = 0;
+                    row_pw += di1 * (dv[t] - 1);
+                }
             }
             lane_pw = row_pw;
         }
