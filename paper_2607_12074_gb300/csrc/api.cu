@@ -158,6 +158,7 @@ harp_status enqueue_count(harp_csr* g, const harp_plan* user_plan, cudaStream_t 
     if (plan.basis == HARP_BASIS_LITERAL) {
         if (st == HARP_OK) st = count_literal(g, ws, plan, s);
     } else {
+        if (st == HARP_OK) st = wedge_geometry(g, ws, plan, s);
         if (st == HARP_OK) st = count_triangles_k4(g, ws, plan, s);
         if (st == HARP_OK) st = count_wedge_c4(g, ws, plan, s);
         if (st == HARP_OK) st = reduce_and_close(g, ws, s);
@@ -216,6 +217,7 @@ harp_status orbit_output(harp_csr* g, uint64_t* orbits_out, uint32_t flags, size
     uint64_t* d_out = orbits_out;
     if (flags == HARP_PTR_HOST) HARP_CK(cudaMallocAsync((void**)&d_out, out_bytes, s));
     harp_status st = orient(g, ws, s);
+    if (st == HARP_OK && wedge_core_applies(g, ws)) st = wedge_geometry(g, ws, plan, s);  // core bitmaps for the triangles
     if (st == HARP_OK) st = count_triangles_k4(g, ws, plan, s);
     if (st == HARP_OK) st = run(ws, d_out, s);
     uint64_t err = 0;

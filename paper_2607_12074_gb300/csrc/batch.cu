@@ -148,6 +148,7 @@ harp_status enqueue_batch(harp_batch* b, const harp_plan& plan, cudaStream_t s) 
     HARP_CK(cudaMemsetAsync(ws.acc, 0, sizeof(uint64_t) * kOutLen, s));
     HARP_CK(cudaMemsetAsync(b->d_accG, 0, sizeof(uint64_t) * kGStride * (size_t)b->G, s));
     HARP_TRY(orient(&b->u, ws, s));
+    HARP_TRY(wedge_geometry(&b->u, ws, plan, s));
     HARP_TRY(count_triangles_k4(&b->u, ws, plan, s));
     HARP_TRY(count_wedge_c4(&b->u, ws, plan, s));
     HARP_TRY(reduce_and_close_batch(&b->u, ws, b->G, b->d_out, s));

@@ -171,7 +171,7 @@ constexpr int kGinfoWarps = kGinfoThreads / 32;
 //   * an eighth of the graph's arcs at core vertices, else the wedges are elsewhere (Barabasi-Albert,
 //     100,000 vertices: 637 us with its core of 17 % of the arcs, 710 without; random geometric graphs
 //     have about 0.1 %),
-//   * K * K bits in the graph's share of the region (4 bytes an arc and 64 a vertex).
+//   * K * K bits and K * K / 32 prefix counts in the graph's share of the region (4 bytes an arc and 64 a vertex).
 __device__ __forceinline__ void choose_core(const int32_t* __restrict__ deg, const int64_t* __restrict__ off,
                                             int64_t lo, int64_t gend, int64_t* gi, uint64_t* acc) {
     const int l = lane_id();
@@ -182,7 +182,7 @@ __device__ __forceinline__ void choose_core(const int32_t* __restrict__ deg, con
         const int64_t cap = 4 * ahi + 64 * gend - b0;
         bool ok = false;
         const int64_t k = (int64_t)1024 << l;
-        if (l < 5 && ahi - alo >= 2 * kCoreMinM && 2 * k <= ng && k * k / 8 <= cap &&
+        if (l < 5 && ahi - alo >= 2 * kCoreMinM && 2 * k <= ng && 3 * k * k / 16 <= cap &&
             deg[gend - 1] >= kCoreMinMaxDeg)
             ok = (int64_t)deg[gend - k] >= k / 64 && 8 * (ahi - off[gend - k]) >= ahi - alo;
         const uint32_t m = __ballot_sync(kFull, ok);
@@ -1261,20 +1261,14 @@ harp_status segment_lengths(const harp_csr* g, Workspace& ws, const uint4* vinfo
 
 // The whole wedge pass for one window size (MINB resident window blocks per SM).
 template <int MINB>
-harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint32_t mid_max, bool merge,
-                       cudaStream_t s) {
+harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint32_t mid_max, cudaStream_t s) {
     constexpr int WORDS = win_words(MINB);
     const int64_t n = g->n;
-    const int64_t G = ws.G > 0 ? ws.G : 1;
     const Sink sink{ws.acc, ws.gid, ws.accG};
     const int sms = num_sms();
     const int64_t most_n = ws.G > 1 ? ws.max_member_n : n;  // vertices of the largest graph
     int32_t* wcount = ws.q_win + n;
-    const bool core = wedge_core_applies(g, ws);
-    k_c4_ginfo<WORDS><<<(unsigned)(G < 8192 ? G : 8192), kGinfoThreads, 0, s>>>(
-        ws.deg, n, ws.gbase, G, ws.x_lo, ws.x_hi, merge, core ? ws.off : nullptr, ws.ginfo, ws.acc);
-    HARP_LAUNCHED();
-    if (core) HARP_TRY(count_wedge_core(g, ws, s));  // uses rev, bpos and the queues before they are filled below
+    if (ws.core) HARP_TRY(count_wedge_core(g, ws, s));  // uses rev, bpos and the queues before they are filled below
     // the roots' lower lists: row prefixes of a whole graph, or their own CSR in a partitioned block
     const bool lists = ws.loff != nullptr;
     const int64_t* loff = lists ? ws.loff : ws.off;
@@ -1344,6 +1338,48 @@ harp_status wedge_positions(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     return segment_lengths(g, ws, vinfo, nullptr, s);
 }
 
+namespace {
+
+// Resident window blocks per SM (MINB) for this plan and workspace, which fixes the window size: the largest of the
+// four that fits plan.c4_window_bytes (at least the smallest).
+// 0 = by graph: a single graph of more than 2^22 vertices takes 200 KiB (its x-range spans tens to
+// hundreds of 100 KiB windows, and halving the (root, window) visits measured 37.7 -> 26.1 s on
+// the 5e7-vertex Chung-Lu graph), anything smaller and every batch 100 KiB (R-MAT scale 20: 13.2
+// ms at 100 KiB against 15.7 ms at 200 KiB)
+int window_blocks(const harp_csr* g, const Workspace& ws, const harp_plan& plan) {
+    uint32_t wbytes = plan.c4_window_bytes;
+    if (wbytes == 0) wbytes = (ws.G <= 1 && g->n > ((int64_t)1 << 22)) ? (uint32_t)kWinWords1 * 4 : (uint32_t)kWinWords2 * 4;
+    if (wbytes >= (uint32_t)kWinWords1 * 4) return 1;
+    if (wbytes >= (uint32_t)kWinWords2 * 4) return 2;
+    return wbytes >= (uint32_t)kWinWords3 * 4 ? 3 : 4;
+}
+
+template <int MINB>
+harp_status launch_ginfo(const harp_csr* g, Workspace& ws, bool merge, bool core, cudaStream_t s) {
+    const int64_t G = ws.G > 0 ? ws.G : 1;
+    k_c4_ginfo<win_words(MINB)><<<(unsigned)(G < 8192 ? G : 8192), kGinfoThreads, 0, s>>>(
+        ws.deg, g->n, ws.gbase, G, ws.x_lo, ws.x_hi, merge, core ? ws.off : nullptr, ws.ginfo, ws.acc);
+    HARP_LAUNCHED();
+    return HARP_OK;
+}
+
+}  // namespace
+
+harp_status wedge_geometry(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s) {
+    ws.core = false;
+    if (g->n == 0 || g->m == 0) return HARP_OK;
+    const bool merge = !(plan.flags & HARP_PLAN_NO_BAND_MERGE), core = wedge_core_applies(g, ws);
+    switch (window_blocks(g, ws, plan)) {
+        case 1: HARP_TRY(launch_ginfo<1>(g, ws, merge, core, s)); break;
+        case 2: HARP_TRY(launch_ginfo<2>(g, ws, merge, core, s)); break;
+        case 3: HARP_TRY(launch_ginfo<3>(g, ws, merge, core, s)); break;
+        default: HARP_TRY(launch_ginfo<4>(g, ws, merge, core, s));
+    }
+    if (core) HARP_TRY(build_core_bits(ws, s));
+    ws.core = core;
+    return HARP_OK;
+}
+
 harp_status count_wedge_c4(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s) {
     if (g->n == 0 || g->m == 0) return HARP_OK;
     uint32_t warp_max = plan.c4_warp_max_work ? plan.c4_warp_max_work : 512;
@@ -1352,18 +1388,12 @@ harp_status count_wedge_c4(const harp_csr* g, Workspace& ws, const harp_plan& pl
     uint32_t mid_max = plan.c4_cta_max_work;
     if (mid_max > kMidSlots / 2) mid_max = kMidSlots / 2;
     if (mid_max < warp_max) mid_max = warp_max;
-    // window size: the largest of the four that fits plan.c4_window_bytes (at least the smallest).
-    // 0 = by graph: a single graph of more than 2^22 vertices takes 200 KiB (its x-range spans tens to
-    // hundreds of 100 KiB windows, and halving the (root, window) visits measured 37.7 -> 26.1 s on
-    // the 5e7-vertex Chung-Lu graph), anything smaller and every batch 100 KiB (R-MAT scale 20: 13.2
-    // ms at 100 KiB against 15.7 ms at 200 KiB)
-    const bool merge = !(plan.flags & HARP_PLAN_NO_BAND_MERGE);
-    uint32_t wbytes = plan.c4_window_bytes;
-    if (wbytes == 0) wbytes = (ws.G <= 1 && g->n > ((int64_t)1 << 22)) ? (uint32_t)kWinWords1 * 4 : (uint32_t)kWinWords2 * 4;
-    if (wbytes >= (uint32_t)kWinWords1 * 4) return wedge_pass<1>(g, ws, warp_max, mid_max, merge, s);
-    if (wbytes >= (uint32_t)kWinWords2 * 4) return wedge_pass<2>(g, ws, warp_max, mid_max, merge, s);
-    if (wbytes >= (uint32_t)kWinWords3 * 4) return wedge_pass<3>(g, ws, warp_max, mid_max, merge, s);
-    return wedge_pass<4>(g, ws, warp_max, mid_max, merge, s);
+    switch (window_blocks(g, ws, plan)) {
+        case 1: return wedge_pass<1>(g, ws, warp_max, mid_max, s);
+        case 2: return wedge_pass<2>(g, ws, warp_max, mid_max, s);
+        case 3: return wedge_pass<3>(g, ws, warp_max, mid_max, s);
+        default: return wedge_pass<4>(g, ws, warp_max, mid_max, s);
+    }
 }
 
 }  // namespace harp

@@ -11,9 +11,8 @@
 // word, in registers) and rows are added through carry-save adders, about 4 instructions for each word
 // of 32 counters, where a counter per element costs about 28 thread instructions.
 //
-//   * core rows: K x K bits, bit j of row r set iff core vertex j is in N+ of core vertex r (j > r), in the
-//     bytes of ws.rev and ws.bpos (which the walk from the top vertex fills afterwards).  32 MiB for
-//     K = 16384: the table stays in L2.
+//   * core rows: K x K bits (CoreTable), in the bytes of ws.rev and ws.bpos (which the walk from the top vertex fills
+//     afterwards).  32 MiB for K = 16384: the table stays in L2.  The triangle pass reads it too (tri.cu).
 //   * w outside the core: the part of N+(w) inside the core, element by element, in packed counters in
 //     shared memory.  A bit transpose turns the counters into planes, the starting value of the register
 //     planes, so both kinds of w meet in one exact count.  (Counting these elements in planes as well, by
@@ -39,36 +38,32 @@ constexpr int kBitsS = 4, kBitsM = 8, kBitsL = 16, kBitsXL = 32;
 constexpr int kWarpsS = 4;  // x per block in class S
 
 // One thread per vertex, highest rank first.  Outside the core: cseg[v] = (start, length) of the part of
-// N+(v) inside the core.  Inside: the vertex joins the queue of core rows.  Every vertex x of a graph with a
-// core joins its degree class (fewer than two neighbours close no cycle); below[x] = its neighbours below the
-// core.
+// N+(v) inside the core.  Every vertex x of a graph with a core joins its degree class (fewer than two neighbours
+// close no cycle); below[x] = its neighbours below the core.
 __global__ void __launch_bounds__(256) k_core_queue(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
                                                     const int64_t* __restrict__ offp, const int32_t* __restrict__ colsp,
                                                     const int32_t* __restrict__ deg, const int32_t* __restrict__ gid,
                                                     const int64_t* __restrict__ ginfo, int64_t n,
                                                     uint2* __restrict__ cseg, int32_t* __restrict__ below,
-                                                    int32_t* __restrict__ q_s,
-                                                    int32_t* __restrict__ q_m, int32_t* __restrict__ q_l,
-                                                    int32_t* __restrict__ q_row, uint64_t* __restrict__ acc) {
+                                                    int32_t* __restrict__ q_s, int32_t* __restrict__ q_m,
+                                                    int32_t* __restrict__ q_l, uint64_t* __restrict__ acc) {
     if (acc[A_CORE_ANY] == 0) return;
     const int l = lane_id();
     for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - l; base < n;
          base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = n - 1 - (base + l);
         int cls = -1;
-        bool row = false;
         if (v >= 0) {
             const int64_t* gi = ginfo + (gid ? (int64_t)gid[v] : 0) * kGInfo;
             const int64_t c0 = gi[GI_CORE];
             if (gi[GI_CORE_K] > 0) {
                 const int32_t d = deg[v];
-                if (d >= 2) cls = d < (1 << kBitsS) ? 0 : (d < (1 << kBitsM) ? 1 : (d < (1 << kBitsL) ? 2 : 3));
                 if (d >= 2) {
+                    cls = d < (1 << kBitsS) ? 0 : (d < (1 << kBitsM) ? 1 : (d < (1 << kBitsL) ? 2 : 3));
                     const int64_t rb = off[v];
                     below[v] = (int32_t)lower_bound_i32(cols + rb, d, (int32_t)c0);
                 }
-                row = v >= c0;
-                if (!row) {
+                if (v < c0) {
                     const int64_t b = offp[v], len = offp[v + 1] - b;
                     const int64_t p = lower_bound_i32(colsp + b, len, (int32_t)c0);
                     cseg[v] = make_uint2((uint32_t)(b + p), (uint32_t)(len - p));
@@ -76,57 +71,71 @@ __global__ void __launch_bounds__(256) k_core_queue(const int64_t* __restrict__ 
             }
         }
 #pragma unroll
-        for (int c = 0; c < 5; ++c) {
-            const bool in = c < 4 ? cls == c : row;
-            const uint32_t mask = __ballot_sync(kFull, in);
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t mask = __ballot_sync(kFull, cls == c);
             if (!mask) continue;
             unsigned long long start = 0;
             const int leader = __ffs(mask) - 1;
-            unsigned long long* ctr = (unsigned long long*)&acc[c < 4 ? Q_CORE_S + c : Q_CORE_ROW];
-            if (l == leader) start = atomicAdd(ctr, (unsigned long long)__popc(mask));
+            if (l == leader) start = atomicAdd((unsigned long long*)&acc[Q_CORE_S + c], (unsigned long long)__popc(mask));
             start = __shfl_sync(kFull, start, leader);
             const int64_t slot = (int64_t)(start + __popc(mask & lanemask_lt()));
-            if (!in) continue;
+            if (cls != c) continue;
             if (c < 3) (c == 0 ? q_s : (c == 1 ? q_m : q_l))[slot] = (int32_t)v;
-            else if (c == 3) q_l[n - 1 - slot] = (int32_t)v;
-            else q_row[slot] = (int32_t)v;
+            else q_l[n - 1 - slot] = (int32_t)v;
         }
     }
 }
 
-// A warp per core row: the row's bits built in shared memory, written with 16-byte stores.  Words before
-// the row's own 4-word group hold no bit and are never read (core_rows).
+// A warp per core row: the row's bits built in shared memory and written with 16-byte stores, with the number of bits
+// before each word beside them.  Words before the row's own 4-word group hold no bit and are never read.
+// The graphs with a core are found 32 at a time.
 constexpr int kRowWarps = 8;
 
 __global__ void __launch_bounds__(kRowWarps * 32) k_core_bits(const int64_t* __restrict__ offp,
-                                                              const int32_t* __restrict__ colsp,
-                                                              const int32_t* __restrict__ gid,
+                                                              const int32_t* __restrict__ colsp, int64_t G,
                                                               const int64_t* __restrict__ ginfo,
-                                                              const int32_t* __restrict__ q_row,
                                                               const uint64_t* __restrict__ acc,
-                                                              uint32_t* __restrict__ bits) {
+                                                              uint32_t* __restrict__ region) {
     __shared__ __align__(16) uint32_t sbuf[kRowWarps][kKWordsMax];
+    if (acc[A_CORE_ANY] == 0) return;
     uint32_t* buf = sbuf[threadIdx.x >> 5];
     const int l = lane_id();
-    const int64_t nq = (int64_t)acc[Q_CORE_ROW];
-    for (int64_t k = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5); k < nq; k += (int64_t)gridDim.x * kRowWarps) {
-        const int32_t w = q_row[k];
-        const int64_t* gi = ginfo + (gid ? (int64_t)gid[w] : 0) * kGInfo;
-        const int64_t c0 = gi[GI_CORE];
-        const int KW = (int)(gi[GI_CORE_K] >> 5);
-        const int r = (int)(w - c0);
-        const int first = (r >> 5) & ~3;
-        for (int i = first + l; i < KW; i += 32) buf[i] = 0;
-        __syncwarp();
-        for (int64_t p = offp[w] + l, e = offp[w + 1]; p < e; p += 32) {
-            const int j = (int)(colsp[p] - c0);
-            atomicOr(&buf[j >> 5], 1u << (j & 31));
+    const int64_t wid = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5), nw = (int64_t)gridDim.x * kRowWarps;
+    for (int64_t g0 = 0; g0 < G; g0 += 32) {
+        uint32_t with_core = __ballot_sync(kFull, g0 + l < G && ginfo[(g0 + l) * kGInfo + GI_CORE_K] > 0);
+        while (with_core) {
+            const CoreTable t = core_table(ginfo, g0 + __ffs(with_core) - 1, region);
+            with_core &= with_core - 1;
+            const int KW = t.KW;
+            for (int64_t r = wid; r < 32 * (int64_t)KW; r += nw) {
+                const int64_t w = t.c0 + r;
+                const int first = (int)(r >> 5) & ~3;
+                for (int i = first + l; i < KW; i += 32) buf[i] = 0;
+                __syncwarp();
+                for (int64_t p = offp[w] + l, e = offp[w + 1]; p < e; p += 32) {
+                    const int j = (int)(colsp[p] - t.c0);
+                    atomicOr(&buf[j >> 5], 1u << (j & 31));
+                }
+                __syncwarp();
+                uint32_t* out = const_cast<uint32_t*>(t.bits) + r * KW;
+                for (int i = first + 4 * l; i < KW; i += 128)
+                    *reinterpret_cast<uint4*>(out + i) = *reinterpret_cast<const uint4*>(buf + i);
+                uint16_t* before = const_cast<uint16_t*>(t.before) + r * KW;
+                int run = 0;
+                for (int i = first; i < KW; i += 32) {
+                    const int c = i + l < KW ? __popc(buf[i + l]) : 0;
+                    int incl = c;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(kFull, incl, o);
+                        if (l >= o) incl += y;
+                    }
+                    if (i + l < KW) before[i + l] = (uint16_t)(run + incl - c);
+                    run += __shfl_sync(kFull, incl, 31);
+                }
+                __syncwarp();
+            }
         }
-        __syncwarp();
-        uint32_t* out = bits + gi[GI_CORE_BASE] + (int64_t)r * KW;
-        for (int i = first + 4 * l; i < KW; i += 128)
-            *reinterpret_cast<uint4*>(out + i) = *reinterpret_cast<const uint4*>(buf + i);
-        __syncwarp();
     }
 }
 
@@ -584,19 +593,24 @@ bool wedge_core_applies(const harp_csr* g, const Workspace& ws) {
     return whole && m >= kCoreMinM && g->max_deg >= kCoreMinMaxDeg;
 }
 
+harp_status build_core_bits(Workspace& ws, cudaStream_t s) {
+    k_core_bits<<<num_sms() * 4, kRowWarps * 32, 0, s>>>(ws.offp, ws.colsp, ws.G > 0 ? ws.G : 1, ws.ginfo, ws.acc,
+                                                         reinterpret_cast<uint32_t*>(ws.rev));
+    HARP_LAUNCHED();
+    return HARP_OK;
+}
+
 harp_status count_wedge_core(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     const int64_t n = g->n;
     const int sms = num_sms();
     const Sink sink{ws.acc, ws.gid, ws.accG};
     uint32_t* bits = reinterpret_cast<uint32_t*>(ws.rev);  // rev and bpos are adjacent (ws_layout) and still unused
     uint2* cseg = reinterpret_cast<uint2*>(ws.vkeys);      // the sort keys are done with
-    int32_t *q_s = ws.q_mid, *q_m = ws.q_mid + n, *q_l = ws.q_win, *q_row = ws.q_win + n;
+    int32_t *q_s = ws.q_mid, *q_m = ws.q_mid + n, *q_l = ws.q_win;
     int64_t blocks = (n + 255) / 256;
     if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
-    k_core_queue<<<(unsigned)blocks, 256, 0, s>>>(ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.gid, ws.ginfo, n, cseg, ws.fpos, q_s, q_m, q_l,
-                                                  q_row, ws.acc);
-    HARP_LAUNCHED();
-    k_core_bits<<<sms * 4, kRowWarps * 32, 0, s>>>(ws.offp, ws.colsp, ws.gid, ws.ginfo, q_row, ws.acc, bits);
+    k_core_queue<<<(unsigned)blocks, 256, 0, s>>>(ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.gid, ws.ginfo, n, cseg,
+                                                  ws.fpos, q_s, q_m, q_l, ws.acc);
     HARP_LAUNCHED();
     if (g->max_deg >= (1 << kBitsL))
         HARP_TRY((launch_block<kBitsXL, 512, 1, 1>(ws, bits, cseg, q_l + n - 1, Q_CORE_XL, T_CORE_XL, sink, s)));

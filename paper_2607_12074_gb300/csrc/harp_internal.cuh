@@ -97,7 +97,6 @@ enum : int {
     Q_CORE_M = 56,
     Q_CORE_L = 57,
     Q_CORE_XL = 58,
-    Q_CORE_ROW = 59,
     T_CORE_M = 60,         // its tickets
     T_CORE_L = 61,
     T_CORE_XL = 62,
@@ -123,6 +122,28 @@ constexpr int kGInfo = 16;     // int64 per graph of wedge-window geometry
 // The last ginfo slots describe the graph's wedge core (c4core.cu): its first rank (INT64_MAX without a
 // core), its size K (a power of two, 0 without a core) and its bitmap's first word in the bitmap region.
 enum : int { GI_CORE = 13, GI_CORE_K = 14, GI_CORE_BASE = 15 };
+// The bitmap region is ws.rev and ws.bpos.  A graph's part holds K rows of K bits (bit j of row r: core vertex j is in
+// N+ of core vertex r; j > r, words before the row's own group of four are not written) and then, per word, the
+// number of bits of its row before it (uint16).
+struct CoreTable {
+    int32_t c0 = 0x7fffffff;  // first rank of the core; none: above every rank
+    int KW = 0;               // words per row
+    const uint32_t* bits = nullptr;
+    const uint16_t* before = nullptr;
+};
+__device__ __forceinline__ CoreTable core_table(const int64_t* __restrict__ ginfo, int64_t graph, const uint32_t* region) {
+    CoreTable t;
+    if (!region) return t;
+    const int64_t* gi = ginfo + graph * kGInfo;
+    const int64_t K = gi[GI_CORE_K];
+    if (K == 0) return t;
+    t.c0 = (int32_t)gi[GI_CORE];
+    t.KW = (int)(K >> 5);
+    t.bits = region + gi[GI_CORE_BASE];
+    t.before = reinterpret_cast<const uint16_t*>(t.bits + K * t.KW);
+    return t;
+}
+
 // A graph below either bound gets no wedge core: few wedges, or none through a hub.  With 65,536 edges the
 // Barabasi-Albert members of a batch of 4,096 graphs took cores and the batch count went from 55.2 to
 // 55.7 ms; R-MAT scale 15 (440,000 edges) gains (0.99 -> 0.73 ms).
@@ -162,6 +183,7 @@ struct Workspace {
     int64_t* scan_tmp = nullptr;   // scan partials
     size_t scan_tmp_len = 0;
     uint64_t* acc = nullptr;       // [kOutLen]
+    bool core = false;             // wedge_geometry built core bitmaps (in rev and bpos)
     // batch mode only (the union of many graphs); nullptr for a single graph
     int64_t G = 1;                    // graphs
     int64_t max_member_m = 0;         // most edges and vertices of one graph
@@ -251,14 +273,18 @@ harp_status orbit_triangles(const harp_csr* g, Workspace& ws, const OrbTri& o, c
 // c4.cu: the position of u in w's row for every lower arc (u -> w) of a whole graph (ws.rev); uses ws.vkeys
 harp_status wedge_positions(const harp_csr* g, Workspace& ws, cudaStream_t s);
 
-// c4.cu: wedge anchor, non-induced 4-cycles (step a5)
+// c4.cu: the grid of the wedge windows and the graphs' cores (ginfo), and the cores' row bitmaps where one can
+// apply (ws.core); before the triangle pass, which reads the bitmaps, and the wedge pass
+harp_status wedge_geometry(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s);
+
+// c4.cu: wedge anchor, non-induced 4-cycles (step a5), after wedge_geometry
 harp_status count_wedge_c4(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s);
 
-// c4core.cu: wedges whose top vertex lies in the graph's core (the ranks from ginfo[GI_CORE] on), after
-// k_c4_ginfo; count_wedge_c4 then leaves those roots out
-harp_status count_wedge_core(const harp_csr* g, Workspace& ws, cudaStream_t s);
-// whether the core pass can apply to this workspace at all (else GI_CORE stays INT64_MAX)
+// c4core.cu: whether a core can apply to this workspace at all (else GI_CORE stays INT64_MAX); the cores' row
+// bitmaps, after k_c4_ginfo; the wedges whose top vertex lies in a core (count_wedge_c4 then leaves those roots out)
 bool wedge_core_applies(const harp_csr* g, const Workspace& ws);
+harp_status build_core_bits(Workspace& ws, cudaStream_t s);
+harp_status count_wedge_core(const harp_csr* g, Workspace& ws, cudaStream_t s);
 
 // literal.cu: the literal basis (per-triangle X_j, per-edge A_e x B_e, per-vertex H_u stars) and its
 // closure, after orient(); writes acc[OUT_COUNTS..], acc[OUT_STATS..]

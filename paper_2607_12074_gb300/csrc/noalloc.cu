@@ -134,6 +134,7 @@ extern "C" harp_status harp_count4_noalloc(int64_t n, int64_t m, const int64_t* 
     }
     if (n > 0) {
         HARP_TRY(orient(&g, ws, s));
+        HARP_TRY(wedge_geometry(&g, ws, plan, s));
         HARP_TRY(count_triangles_k4(&g, ws, plan, s));
         HARP_TRY(count_wedge_c4(&g, ws, plan, s));
     }

@@ -894,6 +894,7 @@ harp_status run_wedge_block(const RankGraph& g, const WedgeBlock& blk, int dev, 
     harp_plan plan;
     normalise_plan(nullptr, &plan);
     cudaEventRecord(sum.ev[1], s);
+    if (st == HARP_OK) st = wedge_geometry(&view, ws, plan, s);
     if (st == HARP_OK) st = count_wedge_c4(&view, ws, plan, s);
     cudaEventRecord(sum.ev[2], s);
     uint64_t acc[kOutLen] = {0};

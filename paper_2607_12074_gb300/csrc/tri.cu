@@ -14,7 +14,8 @@
 //                  per set bit (global atomic at the position where the intersection found it)
 //   * 4-cliques:   K4_u = sum over set bits (i, j) of popc(row_i & row_j)   (the X_3 extension)
 //   * paw sums:    sum over triangles of (d_a + d_b + d_c)
-// The intersection either probes the exact range of N+(L[i]) in [L[i+1], max L] (16-byte loads, a
+// Where L[i] lies in the wedge core (CoreTable), row i is read from the core's bitmap, a bit per pair (gather_rows).
+// Otherwise the intersection either probes the exact range of N+(L[i]) in [L[i+1], max L] (16-byte loads, a
 // membership filter while hits are rare, then the index j of each element in L), or, where few keys
 // of L remain after L[i], searches each of those keys in N+(L[i]) (row_searches).
 // Warp-local mode: d <= tri_warp_max (<= 32), rows are single words, one warp per anchor.
@@ -40,11 +41,11 @@ namespace harp {
 namespace {
 
 constexpr int kCta1 = 256;
-// Block shape of the 256 mode: 192 threads, 7 resident blocks per SM (48 registers a thread).  On
-// R-MAT scale 20 it measured 5.49 ms against 5.77 ms for 256 x 5 and 6.09 ms for 128 x 9: an anchor's
-// rows spread over fewer warps wait less at its block barriers, and more blocks share each SM.
-constexpr int kCta1Threads = 192;
-constexpr int kCta1Blocks = 7;
+// Block shape of the 256 mode: 128 threads, 9 resident blocks per SM.  An anchor's rows spread over fewer warps wait
+// less at its block barriers, and more blocks share each SM: Chung-Lu of 2,000,000 vertices 5.58 ms, against 6.05 ms
+// for 192 x 7 and 7.9 ms for 256 x 5; R-MAT scale 20 2.98, 3.10 and 4.0 ms.
+constexpr int kCta1Threads = 128;
+constexpr int kCta1Blocks = 9;
 constexpr int kCta2 = 512;
 constexpr int kCtaMax = 1024;
 constexpr int kInf = 0x7fffffff;
@@ -571,23 +572,26 @@ struct CtaSmem {
     int64_t rb[PRE ? DMAX : 1];
     int64_t re[PRE ? DMAX : 1];
     uint64_t red[32];
+    int walk;
 };
 
-
-// The anchor a block works on: its list L = N+(u) of d members; direct: membership by the table indexed by
+// The anchor a block works on: its list L = N+(u) of d members, of which the first `walk` have their rows walked (the
+// others are in the core and have theirs read from its bitmap); direct: membership by the table indexed by
 // y - L0 (where L's span fits: dense anchors, high ranks close together) instead of the hash.
 struct CtaAnchor {
-    int d;
+    int d, walk;
     int32_t L0;
     uint32_t span;
     bool direct;
 };
 
-// Stages L, the membership structure and the rows' probe ranges; clears own and the bitmap (d rows of WS
-// words).  Ends with a block barrier.
+// Stages L and, where rows are walked, the membership structure and these rows' probe ranges; clears own and the
+// bitmap (d rows of WS words).  c0: the core's first rank (s.walk is then INT_MAX on entry), or INT_MAX.  Ends with a
+// block barrier.
 template <int DMAX, int THREADS, bool BS>
 __device__ __forceinline__ CtaAnchor stage_anchor(CtaSmem<DMAX>& s, const int64_t* __restrict__ offp,
-                                                  const int32_t* __restrict__ colsp, int64_t ub, int d, int WS) {
+                                                  const int32_t* __restrict__ colsp, int64_t ub, int d, int WS,
+                                                  int32_t c0) {
     using S = CtaSmem<DMAX>;
     CtaAnchor A;
     A.d = d;
@@ -595,10 +599,17 @@ __device__ __forceinline__ CtaAnchor stage_anchor(CtaSmem<DMAX>& s, const int64_
     A.span = (uint32_t)(colsp[ub + d - 1] - A.L0) + 1u;
     A.direct = !BS && A.span <= (uint32_t)S::TAB;
     for (int i = threadIdx.x; i < d; i += THREADS) {
-        s.L[i] = colsp[ub + i];
+        const int32_t x = colsp[ub + i];
+        s.L[i] = x;
         s.own[i] = 0;
+        if (x >= c0 && (i == 0 || colsp[ub + i - 1] < c0)) s.walk = i;
     }
     for (int i = threadIdx.x; i < d * WS; i += THREADS) s.R[i] = 0;
+    if (A.L0 >= c0) {
+        __syncthreads();
+        A.walk = 0;
+        return A;
+    }
     if (A.direct) {
         for (int i = threadIdx.x; i < (int)A.span; i += THREADS) s.m.tab[i] = 0;
     } else {
@@ -606,6 +617,7 @@ __device__ __forceinline__ CtaAnchor stage_anchor(CtaSmem<DMAX>& s, const int64_
         for (int i = threadIdx.x; i < (1 << S::FB) / 32; i += THREADS) s.filt[i] = 0;
     }
     __syncthreads();
+    A.walk = c0 == kInf || s.walk > d - 1 ? d - 1 : s.walk;  // row d - 1 is empty
     for (int i = threadIdx.x; i < d; i += THREADS) {
         if (A.direct) {
             s.m.tab[s.L[i] - A.L0] = (uint16_t)(i + 1);
@@ -614,14 +626,14 @@ __device__ __forceinline__ CtaAnchor stage_anchor(CtaSmem<DMAX>& s, const int64_
             const uint32_t h = hash32((uint32_t)s.L[i]) >> (32 - S::FB);
             atomicOr(&s.filt[h >> 5], 1u << (h & 31));
         }
-        if (!S::PRE && A.direct && i < d - 1) {  // as offsets into N+(L[i]) (rows are short)
+        if (!S::PRE && A.direct && i < A.walk) {  // as offsets into N+(L[i]) (rows are short)
             const int32_t v = s.L[i];
             const int64_t b = offp[v], e = offp[v + 1];
             const int32_t lo = (int32_t)lower_bound_i32(colsp + b, e - b, s.L[i + 1]);
             s.rel[i] = lo;
             s.rel[DMAX + i] = lo + (int32_t)lower_bound_i32(colsp + b + lo, e - b - lo, s.L[d - 1] + 1);
         }
-        if (S::PRE && i < d - 1) {  // every row's probe range at once: dependent loads overlap across rows
+        if (S::PRE && i < A.walk) {  // every row's probe range at once: dependent loads overlap across rows
             const int32_t v = s.L[i];
             const int64_t b = offp[v], e = offp[v + 1];
             const int64_t lo = b + lower_bound_i32(colsp + b, e - b, s.L[i + 1]);
@@ -693,6 +705,52 @@ __device__ __forceinline__ uint32_t walk_row(const CtaSmem<DMAX>& s, const CtaAn
     return hits;
 }
 
+// The rows i >= walk, whose L[i] are in the core: the core's bitmap has a bit for each pair (L[i], L[j]), so they are
+// gathered, one word a pair.  A warp takes a tile of ROWS rows and the 32 keys of a word of the row: a lane keeps
+// its key, the tile's words are loaded side by side, the ballots are the words of R and the keys' counts meet in
+// registers.
+
+template <int DMAX, int ROWS>
+__device__ __forceinline__ void gather_rows(CtaSmem<DMAX>& s, const CoreTable& t, int d, int walk, int WS, int warp,
+                                            int nwarps, const int64_t* __restrict__ offp, uint32_t* __restrict__ te) {
+    const int l = lane_id();
+    int unit = warp;
+    for (int c = walk >> 5; 32 * c < d; ++c) {
+        const int end = 32 * c + 31 < d - 1 ? 32 * c + 31 : d - 1;  // rows below have keys in word c
+        const int tiles = (end - walk + ROWS - 1) / ROWS;
+        for (; unit < tiles; unit += nwarps) {
+            const int j = 32 * c + l, below = j < d ? j : 0;  // the lane's rows
+            const uint32_t o = j < d ? (uint32_t)(s.L[j] - t.c0) : 0u, bit = 1u << (o & 31);
+            const uint32_t base = (o >> 5) - (uint32_t)t.c0 * (uint32_t)t.KW;  // + L[i] * KW, modulo 2^32
+            const int r0 = walk + unit * ROWS;
+            uint32_t word[ROWS], mine = 0, mrow = 0;
+#pragma unroll
+            for (int k = 0; k < ROWS; ++k) {
+                word[k] = 0;
+                if (r0 + k < below) word[k] = __ldg(t.bits + ((uint32_t)s.L[r0 + k] * (uint32_t)t.KW + base));
+            }
+#pragma unroll
+            for (int k = 0; k < ROWS; ++k) {
+                const bool is = (word[k] & bit) != 0;
+                const uint32_t m = __ballot_sync(kFull, is);
+                if (l == k) mrow = m;
+                if (is) {  // arc (L[i], L[j]): top edge of triangle (u, L[i], L[j])
+                    const int32_t v = s.L[r0 + k];
+                    const uint32_t before = __ldg(t.before + ((uint32_t)v * (uint32_t)t.KW + base));
+                    atomicAdd(&te[offp[v] + before + __popc(word[k] & (bit - 1))], 1u);
+                    ++mine;
+                }
+            }
+            if (mrow) {
+                s.R[(r0 + l) * WS + c] = mrow;
+                atomicAdd(&s.own[r0 + l], (uint32_t)__popc(mrow));
+            }
+            if (mine) atomicAdd(&s.own[j], mine);
+        }
+        unit -= tiles;
+    }
+}
+
 template <int DMAX, int THREADS, int MINB, bool BS>
 __global__ void __launch_bounds__(THREADS, MINB) k_tri_cta(const int64_t* __restrict__ offp,
                                                      const int32_t* __restrict__ colsp,
@@ -701,6 +759,8 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tri_cta(const int64_t* __rest
                                                      int wmax, int cmax, int bmax, bool reuse,
                                                      const unsigned long long* __restrict__ cnt,
                                                      unsigned long long* __restrict__ ticket,
+                                                     const int64_t* __restrict__ ginfo,
+                                                     const uint32_t* __restrict__ region,
                                                      uint32_t* __restrict__ te, Sink sink) {
     using S = CtaSmem<DMAX>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -711,8 +771,12 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tri_cta(const int64_t* __rest
     const int64_t nq = (int64_t)cnt[1];
     uint64_t tri = 0, k4 = 0, paw = 0, hits = 0;
     FilterChoice fc;
+    CoreTable core = sink.batch() ? CoreTable{} : core_table(ginfo, 0, region);
     for (;;) {
-        if (threadIdx.x == 0) s_item = (int64_t)atomicAdd(ticket, 1ull);
+        if (threadIdx.x == 0) {
+            s_item = (int64_t)atomicAdd(ticket, 1ull);
+            s.walk = kInf;
+        }
         __syncthreads();
         const int64_t k = s_item;
         __syncthreads();
@@ -723,13 +787,14 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tri_cta(const int64_t* __rest
         if (tri_class(d, wmax, cmax, bmax) != cls) continue;
         const int W = (d + 31) >> 5;
         const int WS = W | 1;
-        const CtaAnchor A = stage_anchor<DMAX, THREADS, BS>(s, offp, colsp, ub, d, WS);
+        if (region && sink.batch()) core = core_table(ginfo, sink.gid[u], region);
+        const CtaAnchor A = stage_anchor<DMAX, THREADS, BS>(s, offp, colsp, ub, d, WS, core.c0);
         const int32_t last = s.L[d - 1];
         auto lookup = [&](int32_t y) {
             if (!A.direct && !filter_may_hold<S::FB>(s.filt, y)) return -1;
             return anchor_find<DMAX, BS>(s, A, y);
         };
-        for (int i = w; i < d - 1; i += NW) {  // a warp per row
+        for (int i = w; i < A.walk; i += NW) {  // a warp per row
             uint32_t* Ri = &s.R[i * WS];
             const uint32_t row_hits = walk_row<DMAX, BS>(s, A, offp, colsp, i, fc, [&](int j, int64_t p) {
                 atomicAdd(&te[p], 1u);  // arc (L[i], L[j]): top edge of triangle (u, L[i], L[j])
@@ -738,6 +803,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tri_cta(const int64_t* __rest
             });
             if (l == 0 && row_hits) atomicAdd(&s.own[i], row_hits);
         }
+        if (A.walk < d - 1) gather_rows<DMAX, (DMAX <= 256 ? 8 : 16)>(s, core, d, A.walk, WS, w, NW, offp, te);
         __syncthreads();
         // triangles and 4-cliques (the X_3 extension): the bitmap's (word, row) units are dealt to all the
         // block's threads.  Unit (x, i) counts the set bits j of word x of row i (the triangles (u, L[i],
@@ -1226,7 +1292,7 @@ __global__ void __launch_bounds__(THREADS) k_orb_tri_cta(const int64_t* __restri
             s.d[i] = (uint32_t)deg[colsp[ub + i]] - 2u;
             s.lo[i] = s.hi[i] = s.lo2[i] = s.hi2[i] = 0;
         }
-        const CtaAnchor A = stage_anchor<DMAX, THREADS, false>(s.c, offp, colsp, ub, d, WS);
+        const CtaAnchor A = stage_anchor<DMAX, THREADS, false>(s.c, offp, colsp, ub, d, WS, kInf);
         for (int i = w; i < d - 1; i += NW)
             walk_row<DMAX, false>(s.c, A, offp, colsp, i, fc, [&](int j, int64_t) {
                 atomicOr(&s.c.R[i * WS + (j >> 5)], 1u << (j & 31));
@@ -1330,8 +1396,8 @@ harp_status launch_cta(const harp_csr* g, Workspace& ws, int cls, int ticket_slo
                                  (int)smem));
     k_tri_cta<DMAX, THREADS, MINB, BS><<<num_sms() * MINB, THREADS, smem, s>>>(
         ws.offp, ws.colsp, ws.deg, ws.q_tri, g->n, cls, wmax, cmax, bmax, reuse,
-        (const unsigned long long*)&ws.acc[Q_TRI_WARP], (unsigned long long*)&ws.acc[ticket_slot], ws.te,
-        Sink{ws.acc, ws.gid, ws.accG});
+        (const unsigned long long*)&ws.acc[Q_TRI_WARP], (unsigned long long*)&ws.acc[ticket_slot], ws.ginfo,
+        ws.core && reuse ? reinterpret_cast<const uint32_t*>(ws.rev) : nullptr, ws.te, Sink{ws.acc, ws.gid, ws.accG});
     HARP_LAUNCHED();
     return HARP_OK;
 }
