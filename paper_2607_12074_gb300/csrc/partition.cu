@@ -77,11 +77,13 @@ struct RankGraph {
     std::vector<int32_t> deg, dplus;  // by rank
     std::vector<int64_t> offp;        // global out-arc numbering: N+(r) holds out-arcs offp[r] ..
     int64_t n1 = 0;                   // first rank of degree >= 2
+    int32_t max_dplus = 0;            // largest out-degree
     std::vector<int32_t> rank;        // rank[v] of input vertex v
 };
 
 // f(lo, hi) over chunks of [0, n) taken from a shared counter by every host thread (rows of very
 // different lengths, e.g. hubs at the start of the id range, stay balanced).
+constexpr int64_t kRowChunk = 512;  // rows of a chunk where the work is the rows' elements: hubs are neighbours in rank
 template <typename F>
 void parallel_dynamic(int64_t n, int64_t chunk, F&& f) {
     const unsigned nt = (n + chunk - 1) / chunk < 2 ? 1 : host_threads();
@@ -257,52 +259,88 @@ harp_status build_rank_graph(int64_t n, int64_t m_in, const int32_t* src, const 
     // each bucket into its rows (positions of the id-order CSR are the bucket's own range), then each
     // row's duplicates dropped in place through a small hash table (stamped by row, so it is never
     // cleared): row v keeps deg0[v] entries from off0[v], in first-seen order
-    std::vector<int64_t> off0((size_t)n + 1, 0);
+    std::vector<int64_t> off0((size_t)n, 0);
     std::vector<int32_t> deg0((size_t)n, 0);
-    parallel_dynamic(nb, 1, [&](int64_t k0, int64_t k1) {
+    // row r of c0[off0[r], end) keeps its first entry of each value
+    static std::atomic<uint64_t> builds{0};
+    const uint64_t build = ++builds;  // a thread's table is of one build: row stamps repeat in the next
+    auto dedupe = [&](int64_t r, int64_t end) {
         thread_local std::vector<uint64_t> table;
-        for (int64_t k = k0; k < k1; ++k) {
-            const int64_t r0 = k << sh, r1 = std::min<int64_t>((k + 1) << sh, n);
-            if (r0 >= r1) continue;
-            std::vector<int64_t> pos((size_t)(r1 - r0 + 1), 0);
-            for (int64_t i = bstart[(size_t)k]; i < bstart[(size_t)k + 1]; ++i)
-                pos[(size_t)((int64_t)(pairs[(size_t)i] >> 32) - r0) + 1]++;
-            for (int64_t r = 0; r < r1 - r0; ++r) pos[(size_t)r + 1] += pos[(size_t)r];
-            for (int64_t r = r0; r < r1; ++r) off0[(size_t)r] = bstart[(size_t)k] + pos[(size_t)(r - r0)];
-            for (int64_t i = bstart[(size_t)k]; i < bstart[(size_t)k + 1]; ++i) {
-                const uint64_t pr = pairs[(size_t)i];
-                c0[(size_t)(bstart[(size_t)k] + pos[(size_t)((int64_t)(pr >> 32) - r0)]++)] = (int32_t)(uint32_t)pr;
-            }
-            for (int64_t r = r0; r < r1; ++r) {  // after the scatter pos[r - r0] is the end of row r
-                const int64_t beg = off0[(size_t)r], end = bstart[(size_t)k] + pos[(size_t)(r - r0)];
-                if (end - beg <= 1) {
-                    deg0[(size_t)r] = (int32_t)(end - beg);
-                    continue;
+        thread_local uint64_t table_of = 0;
+        if (table_of != build) table.clear();
+        table_of = build;
+        const int64_t beg = off0[(size_t)r];
+        if (end - beg <= 1) {
+            deg0[(size_t)r] = (int32_t)(end - beg);
+            return;
+        }
+        int lg = 1;
+        while (((int64_t)1 << lg) < 2 * (end - beg)) ++lg;
+        if (table.size() < ((size_t)1 << lg)) table.assign((size_t)1 << lg, 0);  // stamp 0: empty
+        const uint64_t stamp = (uint64_t)(r + 1) << 32, mask = ((uint64_t)1 << lg) - 1;
+        int64_t w = beg;
+        for (int64_t i = beg; i < end; ++i) {
+            const uint32_t v = (uint32_t)c0[(size_t)i];
+            uint64_t h = ((uint64_t)v * 0x9E3779B97F4A7C15ull) >> (64 - lg);
+            for (;;) {
+                const uint64_t e = table[(size_t)h];
+                if ((e & ~0xffffffffull) != stamp) {  // a slot of another row: free here
+                    table[(size_t)h] = stamp | v;
+                    c0[(size_t)w++] = (int32_t)v;
+                    break;
                 }
-                int lg = 1;
-                while (((int64_t)1 << lg) < 2 * (end - beg)) ++lg;
-                if (table.size() < ((size_t)1 << lg)) table.assign((size_t)1 << lg, 0);  // stamp 0: empty
-                const uint64_t stamp = (uint64_t)(r + 1) << 32, mask = ((uint64_t)1 << lg) - 1;
-                int64_t w = beg;
-                for (int64_t i = beg; i < end; ++i) {
-                    const uint32_t v = (uint32_t)c0[(size_t)i];
-                    uint64_t h = ((uint64_t)v * 0x9E3779B97F4A7C15ull) >> (64 - lg);
-                    for (;;) {
-                        const uint64_t e = table[(size_t)h];
-                        if ((e & ~0xffffffffull) != stamp) {  // a slot of another row: free here
-                            table[(size_t)h] = stamp | v;
-                            c0[(size_t)w++] = (int32_t)v;
-                            break;
-                        }
-                        if ((uint32_t)e == v) break;  // a duplicate
-                        h = (h + 1) & mask;
-                    }
-                }
-                deg0[(size_t)r] = (int32_t)(w - beg);
+                if ((uint32_t)e == v) break;  // a duplicate
+                h = (h + 1) & mask;
             }
         }
+        deg0[(size_t)r] = (int32_t)(w - beg);
+    };
+    // A bucket of more than a quarter of a thread's arcs (hubs of close ids) is taken by all threads, the others by
+    // one each: left to one thread, the hubs' bucket of a Chung-Lu graph of 23,157,049 edges took 70 ms.
+    const int64_t heavy = std::max<int64_t>(A / (4 * (int64_t)nt), 1 << 16);
+    for (int64_t k = 0; k < nb; ++k) {
+        const int64_t e0 = bstart[(size_t)k], len = bstart[(size_t)k + 1] - e0;
+        if (len <= heavy || nt == 1) continue;
+        const int64_t r0 = k << sh, rows = std::min<int64_t>((k + 1) << sh, n) - r0;
+        std::vector<std::vector<int64_t>> pos(nt, std::vector<int64_t>((size_t)rows, 0));
+        parallel_for(len, [&](int64_t lo, int64_t hi, unsigned t) {
+            for (int64_t i = e0 + lo; i < e0 + hi; ++i) pos[t][(size_t)((int64_t)(pairs[(size_t)i] >> 32) - r0)]++;
+        });
+        int64_t run = e0;
+        for (int64_t r = 0; r < rows; ++r) {  // thread t's part of a row after those of threads < t
+            off0[(size_t)(r0 + r)] = run;
+            for (unsigned t = 0; t < nt; ++t) {
+                const int64_t c = pos[t][(size_t)r];
+                pos[t][(size_t)r] = run;
+                run += c;
+            }
+        }
+        parallel_for(len, [&](int64_t lo, int64_t hi, unsigned t) {
+            for (int64_t i = e0 + lo; i < e0 + hi; ++i) {
+                const uint64_t pr = pairs[(size_t)i];
+                c0[(size_t)pos[t][(size_t)((int64_t)(pr >> 32) - r0)]++] = (int32_t)(uint32_t)pr;
+            }
+        });
+        parallel_dynamic(rows, 1, [&](int64_t a, int64_t b) {  // the last thread's place is the end of the row
+            for (int64_t r = a; r < b; ++r) dedupe(r0 + r, pos[nt - 1][(size_t)r]);
+        });
+    }
+    parallel_dynamic(nb, 1, [&](int64_t k0, int64_t k1) {
+        for (int64_t k = k0; k < k1; ++k) {
+            const int64_t r0 = k << sh, r1 = std::min<int64_t>((k + 1) << sh, n);
+            const int64_t e0 = bstart[(size_t)k], e1 = bstart[(size_t)k + 1];
+            if (r0 >= r1 || (e1 - e0 > heavy && nt > 1)) continue;
+            std::vector<int64_t> pos((size_t)(r1 - r0 + 1), 0);
+            for (int64_t i = e0; i < e1; ++i) pos[(size_t)((int64_t)(pairs[(size_t)i] >> 32) - r0) + 1]++;
+            for (int64_t r = 0; r < r1 - r0; ++r) pos[(size_t)r + 1] += pos[(size_t)r];
+            for (int64_t r = r0; r < r1; ++r) off0[(size_t)r] = e0 + pos[(size_t)(r - r0)];
+            for (int64_t i = e0; i < e1; ++i) {
+                const uint64_t pr = pairs[(size_t)i];
+                c0[(size_t)(e0 + pos[(size_t)((int64_t)(pr >> 32) - r0)]++)] = (int32_t)(uint32_t)pr;
+            }
+            for (int64_t r = r0; r < r1; ++r) dedupe(r, e0 + pos[(size_t)(r - r0)]);  // pos: now the rows' ends
+        }
     });
-    off0[(size_t)n] = A;
     // rank = (degree, id): counting sort by degree, ids ascending inside a degree
     int32_t maxd = 0;
     for (int32_t d : deg0) maxd = d > maxd ? d : maxd;
@@ -317,28 +355,33 @@ harp_status build_rank_graph(int64_t n, int64_t m_in, const int32_t* src, const 
     }
     g.n = n;
     g.off.assign((size_t)n + 1, 0);
-    for (int64_t r = 0; r < n; ++r) g.off[(size_t)r + 1] = g.off[(size_t)r] + deg0[(size_t)order[(size_t)r]];
-    g.m = g.off[(size_t)n] / 2;
     g.deg.resize((size_t)n);
+    buf<int64_t> from((size_t)n);  // where the row of rank r begins
+    parallel_for(n, [&](int64_t lo, int64_t hi, unsigned) {
+        for (int64_t r = lo; r < hi; ++r) {
+            const size_t v = (size_t)order[(size_t)r];
+            from[(size_t)r] = off0[v];
+            g.deg[(size_t)r] = deg0[v];
+        }
+    });
+    for (int64_t r = 0; r < n; ++r) g.off[(size_t)r + 1] = g.off[(size_t)r] + g.deg[(size_t)r];
+    g.m = g.off[(size_t)n] / 2;
     g.dplus.resize((size_t)n);
-    // rows by rank, sorted: the other endpoints relabelled in place (one gather each), then vertices
-    // visited in rank order
-    parallel_dynamic(n, 4096, [&](int64_t lo, int64_t hi) {
-        for (int64_t v = lo; v < hi; ++v)
-            for (int64_t k = off0[(size_t)v]; k < off0[(size_t)v] + deg0[(size_t)v]; ++k)
-                c0[(size_t)k] = rank[(size_t)c0[(size_t)k]];
+    // rows by rank, sorted: the other endpoints relabelled in place (one gather each; what the dropped repeats left
+    // between the rows is relabelled too and never read), then vertices visited in rank order
+    parallel_dynamic(A, 1 << 16, [&](int64_t lo, int64_t hi) {
+        for (int64_t k = lo; k < hi; ++k) c0[(size_t)k] = rank[(size_t)c0[(size_t)k]];
     });
     regroup_by_destination(
         n,
         [&](int64_t r) {
-            const int32_t v = order[(size_t)r];
-            return std::make_pair(c0.data() + off0[(size_t)v], c0.data() + off0[(size_t)v] + deg0[(size_t)v]);
+            const int32_t* p = c0.data() + from[(size_t)r];
+            return std::make_pair(p, p + g.deg[(size_t)r]);
         },
         [](int32_t c) { return (int64_t)c; }, n, g.off.data(), c0.data(), pairs.data(),
-        [&](int64_t r0, int64_t r1) {  // degree and out-degree (entries above r) of the rows just filled
+        [&](int64_t r0, int64_t r1) {  // out-degree (entries above r) of the rows just filled
             for (int64_t r = r0; r < r1; ++r) {
                 const int64_t a = g.off[(size_t)r], z = g.off[(size_t)r + 1];
-                g.deg[(size_t)r] = (int32_t)(z - a);
                 const int64_t split = std::upper_bound(c0.begin() + a, c0.begin() + z, (int32_t)r) - (c0.begin() + a);
                 g.dplus[(size_t)r] = (int32_t)(z - a - split);
             }
@@ -352,6 +395,7 @@ harp_status build_rank_graph(int64_t n, int64_t m_in, const int32_t* src, const 
     for (int64_t r = 0; r < n; ++r) {
         if (g.n1 == n && g.deg[(size_t)r] >= 2) g.n1 = r;
         g.offp[(size_t)r + 1] = g.offp[(size_t)r] + g.dplus[(size_t)r];
+        g.max_dplus = std::max(g.max_dplus, g.dplus[(size_t)r]);
     }
     return HARP_OK;
 }
@@ -578,10 +622,17 @@ harp_status cut_wedge_blocks(const RankGraph& g, uint64_t budget, int32_t parts,
     while ((n >> bs) >= 65536) ++bs;
     const int64_t nbk = (n >> bs) + 1;
     const unsigned nt = host_threads();
-    std::vector<std::vector<int64_t>> hist(nt, std::vector<int64_t>((size_t)nbk, 0));
+    std::vector<std::vector<int64_t>> hist(nt);
     std::vector<int64_t> hsum((size_t)nbk, 0);
     std::vector<std::vector<int32_t>> lower(nt);
     std::vector<int32_t> all;
+    auto on_threads = [&](auto&& f) {  // f(thread, take): take(k) reserves the next k items
+        std::atomic<int64_t> next{0};
+        auto take = [&](int64_t k) { return next.fetch_add(k); };
+        std::vector<std::thread> th;
+        for (unsigned t = 0; t < nt; ++t) th.emplace_back([&, t] { f(t, take); });
+        for (auto& x : th) x.join();
+    };
     for (const auto& r : ranges) {
         const int64_t lo = r.first, hi = r.second;
         if (lo >= hi) continue;
@@ -589,51 +640,50 @@ harp_status cut_wedge_blocks(const RankGraph& g, uint64_t budget, int32_t parts,
         for (int64_t u = lo; u < hi; ++u) la += list_arcs_of(g, u);
         // the block's rows are those of every w < hi with a root u in N+(w) n [lo, hi) that has two or
         // more lower neighbours; one pass over w (chunks taken dynamically: hub rows sit at the top)
-        // finds them and counts their elements x in [n1, hi) per x-bucket
+        // finds them and counts their elements x in [n1, hi)
         for (auto& l : lower) l.clear();
         const int64_t xa = g.n1, xb = hi;  // opposite vertices of degree >= 2, below the range's end
         auto seg = [&](int32_t w, int64_t x0, int64_t x1, auto&& visit) {  // row w's elements in [x0, x1)
             const auto b = g.cols.begin() + g.off[(size_t)w], e = g.cols.begin() + g.off[(size_t)w + 1];
             for (auto it = std::lower_bound(b, e, (int32_t)x0); it != e && *it < x1; ++it) visit(*it);
         };
-        {
-            std::atomic<int64_t> next{0};
-            std::vector<std::thread> th;
-            for (unsigned t = 0; t < nt; ++t)
-                th.emplace_back([&, t] {
-                    std::vector<int64_t>& h = hist[t];
-                    std::fill(h.begin(), h.end(), 0);
-                    for (;;) {
-                        const int64_t w0 = next.fetch_add(256);
-                        if (w0 >= hi) break;
-                        for (int64_t w = w0; w < std::min<int64_t>(w0 + 256, hi); ++w) {
-                            const auto e = g.cols.begin() + g.off[(size_t)w + 1];
-                            bool root = false;
-                            for (auto it = std::lower_bound(g.cols.begin() + g.off[(size_t)w], e,
-                                                            (int32_t)std::max<int64_t>(lo, w + 1));
-                                 it != e && *it < hi && !root; ++it)
-                                root = list_arcs_of(g, *it) > 0;
-                            if (!root) continue;
-                            lower[t].push_back((int32_t)w);
-                            seg((int32_t)w, xa, xb, [&](int32_t x) { h[(size_t)(x >> bs)]++; });
-                        }
-                    }
-                });
-            for (auto& x : th) x.join();
-        }
-        all.clear();
-        for (auto& l : lower) all.insert(all.end(), l.begin(), l.end());
-        for (int64_t k = 0; k < nbk; ++k) {
-            int64_t c = 0;
-            for (unsigned t = 0; t < nt; ++t) c += hist[t][(size_t)k];
-            hsum[(size_t)k] = c;
-        }
-        int64_t rows_total = 0;
-        for (int64_t k = 0; k < nbk; ++k) rows_total += hsum[(size_t)k];
+        std::atomic<int64_t> elements{0};
+        on_threads([&](unsigned t, auto&& take) {
+            int64_t count = 0;
+            for (int64_t w0; (w0 = take(256)) < hi;)
+                for (int64_t w = w0; w < std::min<int64_t>(w0 + 256, hi); ++w) {
+                    const auto b = g.cols.begin() + g.off[(size_t)w], e = g.cols.begin() + g.off[(size_t)w + 1];
+                    bool root = false;
+                    for (auto it = std::lower_bound(b, e, (int32_t)std::max<int64_t>(lo, w + 1)); it != e && *it < hi && !root;
+                         ++it)
+                        root = list_arcs_of(g, *it) > 0;
+                    if (!root) continue;
+                    lower[t].push_back((int32_t)w);
+                    const auto p = std::lower_bound(b, e, (int32_t)xa);
+                    if (xa < xb) count += std::lower_bound(p, e, (int32_t)xb) - p;
+                }
+            elements += count;
+        });
+        const int64_t rows_total = elements;
         if (parts > 0 || xa >= xb || wedge_block_bytes(n, rows_total, la) <= budget) {
             peak = std::max<uint64_t>(peak, wedge_block_bytes(n, rows_total, la));
             out.push_back({lo, hi, 0, n});
             continue;
+        }
+        // slices: the elements per x-bucket
+        all.clear();
+        for (auto& l : lower) all.insert(all.end(), l.begin(), l.end());
+        on_threads([&](unsigned t, auto&& take) {
+            std::vector<int64_t>& h = hist[t];
+            h.assign((size_t)nbk, 0);
+            for (int64_t k0; (k0 = take(256)) < (int64_t)all.size();)
+                for (int64_t k = k0; k < std::min<int64_t>(k0 + 256, (int64_t)all.size()); ++k)
+                    seg(all[(size_t)k], xa, xb, [&](int32_t x) { h[(size_t)(x >> bs)]++; });
+        });
+        for (int64_t k = 0; k < nbk; ++k) {
+            int64_t c = 0;
+            for (unsigned t = 0; t < nt; ++t) c += hist[t][(size_t)k];
+            hsum[(size_t)k] = c;
         }
         int64_t x0 = xa, rows = 0;
         auto close = [&](int64_t x) {  // the slice [x0, x) holds `rows` row elements
@@ -672,19 +722,19 @@ harp_status cut_wedge_blocks(const RankGraph& g, uint64_t budget, int32_t parts,
 }
 
 // Scratch the triangle kernels of a block allocate: the fallback's per-warp frontier buffers (sized
-// for the largest out-degree a graph of m edges can have, sqrt(2m)) and the global-staged tier's rows
-// (4096 x 4096 bits per block, one block per SM).
-int64_t tri_scratch_bytes(int64_t m) {
-    int64_t dmax = 1;
-    while (dmax * dmax < 2 * m) ++dmax;
-    const int64_t sms = num_sms();
+// for the largest out-degree) and the global-staged tier's rows (4096 x 4096 bits per block, one block
+// per SM).  The out-degrees are known here: sized for the largest that m edges allow (sqrt(2m)), a
+// Chung-Lu graph of 2,000,000 vertices and 23,157,049 edges set 348 MB of a 512 MiB budget aside and
+// took five triangle blocks instead of one.
+int64_t tri_scratch_bytes(const RankGraph& g) {
+    const int64_t dmax = std::max<int64_t>(1, g.max_dplus), sms = num_sms();
     return sms * 8 * (dmax + 32) * 4 + (dmax > 1024 ? sms * 4096 * 128 * 4 : 0);
 }
 
 // The device results of all blocks, and where the time went.
 struct PartSums {
     uint64_t T = 0, K4 = 0, C4 = 0, PAWSUM = 0;
-    std::vector<uint32_t> te;  // global out-arc numbering
+    buf<uint32_t> te;  // global out-arc numbering
     double transfer_ms = 0, device_ms = 0, tri_ms = 0, wedge_ms = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // copies in | kernels | copies out | end
 };
@@ -711,19 +761,21 @@ harp_status run_triangle_block(const RankGraph& g, const TriBlock& blk, int dev,
                                PartSums& sum, uint64_t& h2d, uint64_t& halo_arcs) {
     const int64_t n = g.n;
     // halo: out-lists of R and N+(R), local numbering in rank order (flags set on all host cores)
-    std::vector<uint8_t> in((size_t)n, 0);
-    parallel_for(blk.hi - blk.lo, [&](int64_t a, int64_t b, unsigned) {
-        for (int64_t u = blk.lo + a; u < blk.lo + b; ++u) {
-            __atomic_store_n(&in[(size_t)u], (uint8_t)1, __ATOMIC_RELAXED);
-            for (int64_t k = 0; k < g.dplus[(size_t)u]; ++k)
-                __atomic_store_n(&in[(size_t)out_nbr(g, u, k)], (uint8_t)1, __ATOMIC_RELAXED);
-        }
-    });
+    const bool whole = blk.lo == 0 && blk.hi == n;  // every vertex is in the halo
+    std::vector<uint8_t> in((size_t)n, (uint8_t)whole);
+    if (!whole)
+        parallel_dynamic(blk.hi - blk.lo, kRowChunk, [&](int64_t a, int64_t b) {
+            for (int64_t u = blk.lo + a; u < blk.lo + b; ++u) {
+                __atomic_store_n(&in[(size_t)u], (uint8_t)1, __ATOMIC_RELAXED);
+                for (int64_t k = 0; k < g.dplus[(size_t)u]; ++k)
+                    __atomic_store_n(&in[(size_t)out_nbr(g, u, k)], (uint8_t)1, __ATOMIC_RELAXED);
+            }
+        });
     std::vector<int64_t> offp((size_t)n + 1, 0);
     for (int64_t v = 0; v < n; ++v) offp[(size_t)v + 1] = offp[(size_t)v] + (in[(size_t)v] ? g.dplus[(size_t)v] : 0);
     const int64_t outs = offp[(size_t)n];
     buf<int32_t> colsp((size_t)(outs > 0 ? outs : 1));
-    parallel_for(n, [&](int64_t lo, int64_t hi, unsigned) {
+    parallel_dynamic(n, kRowChunk, [&](int64_t lo, int64_t hi) {
         for (int64_t v = lo; v < hi; ++v) {
             const int64_t len = offp[(size_t)v + 1] - offp[(size_t)v];
             if (len)
@@ -759,23 +811,24 @@ harp_status run_triangle_block(const RankGraph& g, const TriBlock& blk, int dev,
     if (e == cudaSuccess) e = cudaMemsetAsync(ws.acc, 0, sizeof(uint64_t) * kOutLen, s);
     harp_status st = check_cuda(e);
     h2d += 8 * (uint64_t)(n + 1) + 4 * (uint64_t)outs + 8 * (uint64_t)n;
-    harp_csr view;  // the kernels' view: global n, m and maximum degree
+    harp_csr view;  // the kernels' view: global n and m; the triangle kernels bound out-degrees by max_deg
     view.device = dev;
     view.stream = s;
     view.n = n;
     view.m = g.m;
-    view.max_deg = n ? *std::max_element(g.deg.begin(), g.deg.end()) : 0;
+    view.max_deg = g.max_dplus;
     harp_plan plan;
     normalise_plan(nullptr, &plan);
     cudaEventRecord(sum.ev[1], s);
     if (st == HARP_OK && n > 0) st = count_triangles_k4(&view, ws, plan, s);
     cudaEventRecord(sum.ev[2], s);
-    buf<uint32_t> te_local((size_t)outs);
+    buf<uint32_t> te_local;
+    if (!whole) te_local.resize((size_t)outs);  // a whole block's out-arcs are the global ones
     uint64_t acc[kOutLen] = {0};
     if (st == HARP_OK) {
         e = cudaMemcpyAsync(acc, ws.acc, sizeof(acc), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess && outs)
-            e = cudaMemcpyAsync(te_local.data(), ws.te, sizeof(uint32_t) * (size_t)outs, cudaMemcpyDeviceToHost, s);
+            e = cudaMemcpyAsync(whole ? sum.te.data() : te_local.data(), ws.te, sizeof(uint32_t) * (size_t)outs, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaEventRecord(sum.ev[3], s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         st = check_cuda(e);
@@ -787,7 +840,8 @@ harp_status run_triangle_block(const RankGraph& g, const TriBlock& blk, int dev,
     sum.T += acc[ACC_T];
     sum.K4 += acc[ACC_K4];
     sum.PAWSUM += acc[ACC_PAWSUM];
-    parallel_for(n, [&](int64_t lo, int64_t hi, unsigned) {  // local out-arcs -> global out-arc ids
+    if (whole) return HARP_OK;
+    parallel_dynamic(n, kRowChunk, [&](int64_t lo, int64_t hi) {  // local out-arcs -> global out-arc ids
         for (int64_t v = lo; v < hi; ++v) {
             const int64_t lb = offp[(size_t)v], len = offp[(size_t)v + 1] - lb, gb = g.offp[(size_t)v];
             for (int64_t k = 0; k < len; ++k) sum.te[(size_t)(gb + k)] += te_local[(size_t)(lb + k)];
@@ -806,20 +860,21 @@ harp_status run_wedge_block(const RankGraph& g, const WedgeBlock& blk, int dev, 
     const int64_t la = loff[(size_t)n];
     buf<int32_t> lcols((size_t)(la > 0 ? la : 1));
     std::vector<uint8_t> in((size_t)n, 0);
-    parallel_for(blk.hi - blk.lo, [&](int64_t a0, int64_t b0, unsigned) {  // on all host cores
+    parallel_dynamic(blk.hi - blk.lo, kRowChunk, [&](int64_t a0, int64_t b0) {
         for (int64_t u = blk.lo + a0; u < blk.lo + b0; ++u) {
             const int64_t len = loff[(size_t)u + 1] - loff[(size_t)u];
             for (int64_t a = 0; a < len; ++a) {
                 const int32_t w = g.cols[(size_t)(g.off[(size_t)u] + a)];
                 lcols[(size_t)(loff[(size_t)u] + a)] = w;
-                __atomic_store_n(&in[(size_t)w], (uint8_t)1, __ATOMIC_RELAXED);
+                if (!__atomic_load_n(&in[(size_t)w], __ATOMIC_RELAXED))  // mostly set: the line stays shared
+                    __atomic_store_n(&in[(size_t)w], (uint8_t)1, __ATOMIC_RELAXED);
             }
         }
     });
     // rows of the lower neighbours, restricted to the slice [xa, xb) of opposite vertices
     const int64_t xa = std::max<int64_t>(blk.xlo, g.n1), xb = std::min<int64_t>(blk.xhi, blk.hi);
     std::vector<int64_t> off((size_t)n + 1, 0), rb((size_t)n, 0);
-    parallel_for(n, [&](int64_t lo, int64_t hi, unsigned) {  // slice lengths, then a prefix sum
+    parallel_dynamic(n, kRowChunk, [&](int64_t lo, int64_t hi) {  // slice lengths, then a prefix sum
         for (int64_t w = lo; w < hi; ++w) {
             int64_t len = 0;
             if (in[(size_t)w] && xa < xb) {
@@ -835,7 +890,7 @@ harp_status run_wedge_block(const RankGraph& g, const WedgeBlock& blk, int dev, 
     const int64_t ra = off[(size_t)n];
     if (la == 0 || ra == 0) return HARP_OK;  // no root or no opposite vertex: nothing to count here
     buf<int32_t> cols((size_t)ra);
-    parallel_for(n, [&](int64_t lo, int64_t hi, unsigned) {
+    parallel_dynamic(n, kRowChunk, [&](int64_t lo, int64_t hi) {
         for (int64_t w = lo; w < hi; ++w) {
             const int64_t len = off[(size_t)w + 1] - off[(size_t)w];
             if (len)
@@ -933,7 +988,7 @@ extern "C" harp_status harp_count4_partitioned(int64_t n, int64_t m_in, const in
         HARP_CK(cudaMemGetInfo(&fr, &tot));
         budget_bytes = fr / 2;
     }
-    const int64_t fb = tri_scratch_bytes(g.m);
+    const int64_t fb = tri_scratch_bytes(g);
     std::vector<TriBlock> tri;
     std::vector<WedgeBlock> wedge;
     uint64_t device_peak = 0, h2d = 0, halo_arcs = 0;
@@ -941,7 +996,8 @@ extern "C" harp_status harp_count4_partitioned(int64_t n, int64_t m_in, const in
     HARP_TRY(cut_wedge_blocks(g, budget_bytes, parts, wedge, device_peak));
     const auto t2 = std::chrono::steady_clock::now();
     PartSums sum;
-    sum.te.assign((size_t)g.offp[(size_t)n], 0);
+    sum.te.resize((size_t)g.offp[(size_t)n]);
+    if (tri.size() != 1 || tri[0].lo != 0 || tri[0].hi != n) std::fill(sum.te.begin(), sum.te.end(), 0u);
     cudaStream_t s = nullptr;
     HARP_CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     harp_status st = HARP_OK;
@@ -961,8 +1017,9 @@ extern "C" harp_status harp_count4_partitioned(int64_t n, int64_t m_in, const in
         if (ev) cudaEventDestroy(ev);
     if (st != HARP_OK) return st;
     // degree sums by owner (every vertex / edge once) and the global sum_e C(t_e, 2)
-    std::vector<uint64_t> pS(host_threads(), 0), pPW(host_threads(), 0), pD(host_threads(), 0);
-    parallel_for(n, [&](int64_t lo, int64_t hi, unsigned t) {
+    std::vector<uint64_t> pD(host_threads(), 0);
+    std::atomic<uint64_t> aS{0}, aPW{0};
+    parallel_dynamic(n, kRowChunk, [&](int64_t lo, int64_t hi) {
         uint64_t s3 = 0, pw = 0;
         for (int64_t r = lo; r < hi; ++r) {
             const uint64_t dr = (uint64_t)g.deg[(size_t)r];
@@ -970,20 +1027,17 @@ extern "C" harp_status harp_count4_partitioned(int64_t n, int64_t m_in, const in
             for (int64_t k = 0; k < g.dplus[(size_t)r]; ++k)
                 pw += (dr - 1) * ((uint64_t)g.deg[(size_t)out_nbr(g, r, k)] - 1);
         }
-        pS[t] += s3;
-        pPW[t] += pw;
+        aS += s3;
+        aPW += pw;
     });
     parallel_for((int64_t)sum.te.size(), [&](int64_t lo, int64_t hi, unsigned t) {
         uint64_t d = 0;
         for (int64_t i = lo; i < hi; ++i) d += choose2_h(sum.te[(size_t)i]);
         pD[t] += d;
     });
-    uint64_t S = 0, PW = 0, D = 0;
-    for (size_t t = 0; t < pS.size(); ++t) {
-        S += pS[t];
-        PW += pPW[t];
-        D += pD[t];
-    }
+    const uint64_t S = aS, PW = aPW;
+    uint64_t D = 0;
+    for (uint64_t d : pD) D += d;
     const uint64_t T = sum.T, K4 = sum.K4;
     const uint64_t P = PW - 3 * T, pawn = sum.PAWSUM - 6 * T;
     const uint64_t diamond = D - 6 * K4;
@@ -1038,7 +1092,7 @@ extern "C" harp_status harp_partition_plan(int64_t n, int64_t m_in, const int32_
     std::vector<TriBlock> tri;
     std::vector<WedgeBlock> wedge;
     uint64_t device_peak = 0;
-    HARP_TRY(cut_triangle_ranges(g, budget_bytes, parts, tri_scratch_bytes(g.m), tri, device_peak));
+    HARP_TRY(cut_triangle_ranges(g, budget_bytes, parts, tri_scratch_bytes(g), tri, device_peak));
     HARP_TRY(cut_wedge_blocks(g, budget_bytes, parts, wedge, device_peak));
     const auto t2 = std::chrono::steady_clock::now();
     *stats = harp_partition_stats{};
