@@ -40,6 +40,7 @@ int64_t union_blocks(int64_t n, int64_t arcs) {
 __global__ void __launch_bounds__(256) k_union_build(const MemberDesc* __restrict__ desc, int64_t G,
                                                      int64_t* __restrict__ off_u, int32_t* __restrict__ cols_u,
                                                      int32_t* __restrict__ gid_u, int64_t N, int64_t A) {
+    grid_begin();
     int64_t lo = 0, hi = G;  // member: last g with desc[g].bstart <= blockIdx.x
     while (hi - lo > 1) {
         const int64_t mid = (lo + hi) >> 1;
@@ -230,7 +231,7 @@ harp_status harp_batch_create(const harp_csr* const* graphs, int64_t G, harp_bat
     if (e == cudaSuccess && blocks > 2147483647LL) e = cudaErrorInvalidValue;
     if (e == cudaSuccess && G == 0) e = cudaMemsetAsync(b->u.off, 0, sizeof(int64_t), s);  // off[0] = 0
     if (e == cudaSuccess && G > 0) {
-        k_union_build<<<(unsigned)blocks, 256, 0, s>>>(b->d_desc, G, b->u.off, b->u.cols, b->d_gid_in, N, 2 * M);
+        launch(k_union_build, (unsigned)blocks, 256, 0, s, b->d_desc, G, b->u.off, b->u.cols, b->d_gid_in, N, 2 * M);
         note_launch();
         e = cudaGetLastError();
     }

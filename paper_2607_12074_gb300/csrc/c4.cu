@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kGinfoThreads) k_c4_ginfo(const int32_t* __res
                                                             const int64_t* __restrict__ gbase, int64_t G, int64_t x_lo,
                                                             int64_t x_hi, bool merge, const int64_t* __restrict__ off,
                                                             int64_t* __restrict__ ginfo, uint64_t* __restrict__ acc) {
+    grid_begin();
     __shared__ uint64_t s_score[kGinfoWarps][kMergeMasks];
     __shared__ int64_t s_rank[kBands + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -309,6 +310,7 @@ __global__ void __launch_bounds__(256) k_c4_fpos(const int64_t* __restrict__ off
                                                  const int64_t* __restrict__ offp, const int32_t* __restrict__ gid,
                                                  const int64_t* __restrict__ ginfo, int64_t n,
                                                  int32_t* __restrict__ fpos, uint4* __restrict__ vinfo) {
+    grid_begin();
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (int64_t)gridDim.x * blockDim.x) {
         const int64_t wb = off[w], we = off[w + 1];
         int32_t f = 0;
@@ -342,6 +344,7 @@ __global__ void __launch_bounds__(256) k_c4_seglen(const int64_t* __restrict__ o
                                                    const uint4* __restrict__ vinfo, const int32_t* __restrict__ gid,
                                                    const int64_t* __restrict__ ginfo, int64_t n, int run,
                                                    int32_t* __restrict__ rev) {
+    grid_begin();
     const int l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     // one graph: the arcs of its core rows come last and are left out
@@ -410,6 +413,7 @@ __global__ void __launch_bounds__(256) k_c4_seglen_rows(const int64_t* __restric
                                                         const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
                                                         const int32_t* __restrict__ fpos, int64_t n, int64_t arcs,
                                                         int32_t* __restrict__ rev) {
+    grid_begin();
     const int64_t runs = (arcs + kRevRun - 1) / kRevRun;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < runs; r += (int64_t)gridDim.x * blockDim.x) {
         const int64_t a0 = r * kRevRun;
@@ -492,6 +496,7 @@ template <int WORDS>
 __global__ void k_c4_bpos(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
                           const int32_t* __restrict__ gid, const int64_t* __restrict__ ginfo, int64_t n,
                           const int32_t* __restrict__ fpos, const uint64_t* __restrict__ acc, int32_t* __restrict__ bpos) {
+    grid_begin();
     if (!table_pays(acc, n)) return;
     const int64_t total = n * kGridCap;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
@@ -639,6 +644,7 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
                                                      int64_t own_hi, uint32_t warp_max, uint32_t mid_max,
                                                      int32_t* __restrict__ q_small, int32_t* __restrict__ q_win,
                                                      int32_t* __restrict__ wcount, uint64_t* __restrict__ acc) {
+    grid_begin();
     const int l = lane_id();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -819,6 +825,7 @@ __global__ void __launch_bounds__(kSmallThreads, PACKED ? 5 : 3) k_c4_light(cons
                                                                             const int32_t* __restrict__ q_small,
                                                                             int64_t n, uint64_t* __restrict__ acc,
                                                                             Sink sink) {
+    grid_begin();
     using Table = HashTable<kSmallSlots, kLightBits, PACKED>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t s_rel[kSmallWarps][32];
@@ -926,6 +933,7 @@ __global__ void __launch_bounds__(kMidThreads) k_c4_mid(const int64_t* __restric
                                                         const uint4* __restrict__ vinfo, const int64_t* __restrict__ ginfo,
                                                         const int32_t* __restrict__ q_small, int64_t n,
                                                         uint64_t* __restrict__ acc, Sink sink) {
+    grid_begin();
     using Table = HashTable<kMidSlots, kMidBits, PACKED>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t s_rel[kMidWarps][32];
@@ -1171,6 +1179,7 @@ __global__ void __launch_bounds__(win_threads(MINB), MINB) k_c4_window(const int
                                                               const int32_t* __restrict__ q_win,
                                                               const int64_t* __restrict__ win_prefix, int64_t n,
                                                               uint64_t* __restrict__ acc, Sink sink) {
+    grid_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t* cw = reinterpret_cast<uint32_t*>(smem_raw);
     constexpr int WORDS = win_words(MINB);
@@ -1253,8 +1262,8 @@ harp_status segment_lengths(const harp_csr* g, Workspace& ws, const uint4* vinfo
     const int64_t warps = (int64_t)num_sms() * 64;
     int64_t run = ((g->m + g->n) / warps + 31) / 32 * 32;
     run = run < 32 ? 32 : (run > 256 ? 256 : run);
-    k_c4_seglen<<<grid_cap((g->m + g->n + run - 1) / run * 32, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(
-        ws.off, ws.cols, ws.offp, ws.colsp, vinfo, ginfo ? ws.gid : nullptr, ginfo, g->n, (int)run, ws.rev);
+    launch(k_c4_seglen, grid_cap((g->m + g->n + run - 1) / run * 32, 256, (int64_t)num_sms() * 64), 256, 0, s, ws.off,
+           ws.cols, ws.offp, ws.colsp, vinfo, ginfo ? ws.gid : nullptr, ginfo, g->n, (int)run, ws.rev);
     HARP_LAUNCHED();
     return HARP_OK;
 }
@@ -1274,18 +1283,18 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     const int64_t* loff = lists ? ws.loff : ws.off;
     const int32_t* lcols = lists ? ws.lcols : ws.cols;
     uint4* vinfo = lists ? nullptr : reinterpret_cast<uint4*>(ws.vkeys);  // the sort keys' two arrays are done with
-    k_c4_fpos<<<grid_cap(n, 256, (int64_t)sms * 64), 256, 0, s>>>(ws.off, ws.cols, ws.offp, ws.gid, ws.ginfo, n, ws.fpos,
-                                                                 vinfo);
+    launch(k_c4_fpos, grid_cap(n, 256, (int64_t)sms * 64), 256, 0, s, ws.off, ws.cols, ws.offp, ws.gid, ws.ginfo, n,
+           ws.fpos, vinfo);
     HARP_LAUNCHED();
     if (lists) {
         const int64_t la = ws.lower_arcs;  // == loff[n]
-        k_c4_seglen_rows<<<grid_cap((la + kRevRun - 1) / kRevRun, 256, (int64_t)sms * 64), 256, 0, s>>>(
-            ws.loff, ws.lcols, ws.off, ws.cols, ws.fpos, n, la, ws.rev);
+        launch(k_c4_seglen_rows, grid_cap((la + kRevRun - 1) / kRevRun, 256, (int64_t)sms * 64), 256, 0, s, ws.loff,
+               ws.lcols, ws.off, ws.cols, ws.fpos, n, la, ws.rev);
         HARP_LAUNCHED();
     } else {
         HARP_TRY(segment_lengths(g, ws, vinfo, ws.ginfo, s));
     }
-    k_c4_classify<WORDS><<<grid_cap(n, 256, (int64_t)sms * 32), 256, 0, s>>>(  // a lane per root
+    launch(k_c4_classify<WORDS>, grid_cap(n, 256, (int64_t)sms * 32), 256, 0, s, // a lane per root
         loff, ws.deg, ws.dplus, ws.rev, ws.gid, ws.ginfo, n, ws.own_lo, ws.own_hi, warp_max, mid_max, ws.q_mid, ws.q_win,
         wcount, ws.acc);
     HARP_LAUNCHED();
@@ -1295,34 +1304,30 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     const size_t light_smem = (size_t)kSmallWarps * kSmallSlots * (packed_light ? 4 : 8);
     auto light = packed_light ? k_c4_light<true> : k_c4_light<false>;
     HARP_CK(cudaFuncSetAttribute(light, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)light_smem));
-    light<<<sms * (packed_light ? 5 : 3), kSmallThreads, light_smem, s>>>(ws.off, ws.cols, loff, lcols, ws.deg, ws.dplus,
-                                                                          ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc,
-                                                                          sink);
+    launch(light, sms * (packed_light ? 5 : 3), kSmallThreads, light_smem, s, ws.off, ws.cols, loff, lcols, ws.deg,
+           ws.dplus, ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc, sink);
     HARP_LAUNCHED();
     HARP_CK(prof_mark(s, SEG_C4_SMALL));
     if (mid_max > warp_max) {
         const size_t mid_smem = (size_t)kMidSlots * (packed_mid ? 4 : 8);
         auto mid = packed_mid ? k_c4_mid<true> : k_c4_mid<false>;
         HARP_CK(cudaFuncSetAttribute(mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem));
-        mid<<<sms * (packed_mid ? 12 : 6), kMidThreads, mid_smem, s>>>(ws.off, ws.cols, loff, lcols, ws.deg, ws.dplus,
-                                                                       ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc,
-                                                                       sink);
+        launch(mid, sms * (packed_mid ? 12 : 6), kMidThreads, mid_smem, s, ws.off, ws.cols, loff, lcols, ws.deg,
+               ws.dplus, ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc, sink);
         HARP_LAUNCHED();
     }
     HARP_CK(prof_mark(s, SEG_C4_MID));
     // only the queued roots' counts matter (and are set); what follows them in the scan is never read
     HARP_TRY(exclusive_scan_i32_to_i64(wcount, ws.win_prefix, n, ws.scan_tmp, ws.scan_tmp_len, s));
     if (ws.bpos) {
-        k_c4_bpos<WORDS><<<grid_cap(n * kGridCap, 256, (int64_t)sms * 64), 256, 0, s>>>(ws.off, ws.cols, ws.gid, ws.ginfo,
-                                                                                       n, ws.fpos, ws.acc, ws.bpos);
+        launch(k_c4_bpos<WORDS>, grid_cap(n * kGridCap, 256, (int64_t)sms * 64), 256, 0, s, ws.off, ws.cols, ws.gid,
+               ws.ginfo, n, ws.fpos, ws.acc, ws.bpos);
         HARP_LAUNCHED();
     }
     const size_t win_smem = (size_t)WORDS * sizeof(uint32_t);
     HARP_CK(cudaFuncSetAttribute(k_c4_window<MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_smem));
-    k_c4_window<MINB><<<sms * MINB, win_threads(MINB), win_smem, s>>>(ws.off, ws.cols, loff, lcols, ws.deg, ws.dplus,
-                                                                ws.fpos, ws.rev,
-                                                                ws.bpos, ws.gid, ws.ginfo, ws.q_win, ws.win_prefix, n,
-                                                                ws.acc, sink);
+    launch(k_c4_window<MINB>, sms * MINB, win_threads(MINB), win_smem, s, ws.off, ws.cols, loff, lcols, ws.deg,
+           ws.dplus, ws.fpos, ws.rev, ws.bpos, ws.gid, ws.ginfo, ws.q_win, ws.win_prefix, n, ws.acc, sink);
     HARP_LAUNCHED();
     HARP_CK(prof_mark(s, SEG_C4_WINDOW));
     return HARP_OK;
@@ -1332,8 +1337,8 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
 
 harp_status wedge_positions(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     uint4* vinfo = reinterpret_cast<uint4*>(ws.vkeys);
-    k_c4_fpos<<<grid_cap(g->n, 256, (int64_t)num_sms() * 64), 256, 0, s>>>(ws.off, ws.cols, ws.offp, nullptr, nullptr, g->n,
-                                                                          nullptr, vinfo);
+    launch(k_c4_fpos, grid_cap(g->n, 256, (int64_t)num_sms() * 64), 256, 0, s, ws.off, ws.cols, ws.offp, nullptr,
+           nullptr, g->n, nullptr, vinfo);
     HARP_LAUNCHED();
     return segment_lengths(g, ws, vinfo, nullptr, s);
 }
@@ -1357,8 +1362,8 @@ int window_blocks(const harp_csr* g, const Workspace& ws, const harp_plan& plan)
 template <int MINB>
 harp_status launch_ginfo(const harp_csr* g, Workspace& ws, bool merge, bool core, cudaStream_t s) {
     const int64_t G = ws.G > 0 ? ws.G : 1;
-    k_c4_ginfo<win_words(MINB)><<<(unsigned)(G < 8192 ? G : 8192), kGinfoThreads, 0, s>>>(
-        ws.deg, g->n, ws.gbase, G, ws.x_lo, ws.x_hi, merge, core ? ws.off : nullptr, ws.ginfo, ws.acc);
+    launch(k_c4_ginfo<win_words(MINB)>, (unsigned)(G < 8192 ? G : 8192), kGinfoThreads, 0, s, ws.deg, g->n, ws.gbase,
+           G, ws.x_lo, ws.x_hi, merge, core ? ws.off : nullptr, ws.ginfo, ws.acc);
     HARP_LAUNCHED();
     return HARP_OK;
 }

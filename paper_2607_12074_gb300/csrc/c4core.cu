@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(256) k_core_queue(const int64_t* __restrict__ 
                                                     uint2* __restrict__ cseg, int32_t* __restrict__ below,
                                                     int32_t* __restrict__ q_s, int32_t* __restrict__ q_m,
                                                     int32_t* __restrict__ q_l, uint64_t* __restrict__ acc) {
+    grid_begin();
     if (acc[A_CORE_ANY] == 0) return;
     const int l = lane_id();
     for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - l; base < n;
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_core_bits(const int64_t* __r
                                                               const int64_t* __restrict__ ginfo,
                                                               const uint64_t* __restrict__ acc,
                                                               uint32_t* __restrict__ region) {
+    grid_begin();
     __shared__ __align__(16) uint32_t sbuf[kRowWarps][kKWordsMax];
     if (acc[A_CORE_ANY] == 0) return;
     uint32_t* buf = sbuf[threadIdx.x >> 5];
@@ -443,6 +445,7 @@ __global__ void __launch_bounds__(kWarpsS * 32, 6) k_core_warp(const int64_t* __
                                                                const int32_t* __restrict__ below,
                                                                const uint32_t* __restrict__ bits,
                                                                const int32_t* __restrict__ q, Sink sink) {
+    grid_begin();
     extern __shared__ __align__(16) uint32_t smem_ctr[];
     __shared__ uint64_t red[32];
     uint32_t* ctr = smem_ctr + (threadIdx.x >> 5) * (kBitsS * kKWordsMax);
@@ -541,6 +544,7 @@ __global__ void __launch_bounds__(NT, MINB) k_core_block(const int64_t* __restri
                                                    const int32_t* __restrict__ below, const uint32_t* __restrict__ bits,
                                                    const int32_t* __restrict__ q,
                                                    int qslot, int tslot, Sink sink) {
+    grid_begin();
     // the parts' planes of block_words fit the counters' bytes
     static_assert((NT / 32) * 32 * VEC <= kKWordsMax, "scratch of the row parts");
     extern __shared__ __align__(16) uint32_t ctr[];
@@ -579,8 +583,8 @@ harp_status launch_block(const Workspace& ws, const uint32_t* bits, const uint2*
                          int tslot, const Sink& sink, cudaStream_t s) {
     const size_t smem = (size_t)CB * kKWordsMax * sizeof(uint32_t);
     HARP_CK(cudaFuncSetAttribute(k_core_block<CB, NT, VEC, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_core_block<CB, NT, VEC, MINB><<<num_sms() * MINB, NT, smem, s>>>(ws.off, ws.cols, ws.colsp, cseg, ws.gid, ws.ginfo,
-                                                                       ws.fpos, bits, q, qslot, tslot, sink);
+    launch(k_core_block<CB, NT, VEC, MINB>, num_sms() * MINB, NT, smem, s, ws.off, ws.cols, ws.colsp, cseg, ws.gid,
+           ws.ginfo, ws.fpos, bits, q, qslot, tslot, sink);
     HARP_LAUNCHED();
     return HARP_OK;
 }
@@ -594,8 +598,8 @@ bool wedge_core_applies(const harp_csr* g, const Workspace& ws) {
 }
 
 harp_status build_core_bits(Workspace& ws, cudaStream_t s) {
-    k_core_bits<<<num_sms() * 4, kRowWarps * 32, 0, s>>>(ws.offp, ws.colsp, ws.G > 0 ? ws.G : 1, ws.ginfo, ws.acc,
-                                                         reinterpret_cast<uint32_t*>(ws.rev));
+    launch(k_core_bits, num_sms() * 4, kRowWarps * 32, 0, s, ws.offp, ws.colsp, ws.G > 0 ? ws.G : 1, ws.ginfo, ws.acc,
+           reinterpret_cast<uint32_t*>(ws.rev));
     HARP_LAUNCHED();
     return HARP_OK;
 }
@@ -609,8 +613,8 @@ harp_status count_wedge_core(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     int32_t *q_s = ws.q_mid, *q_m = ws.q_mid + n, *q_l = ws.q_win;
     int64_t blocks = (n + 255) / 256;
     if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
-    k_core_queue<<<(unsigned)blocks, 256, 0, s>>>(ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.gid, ws.ginfo, n, cseg,
-                                                  ws.fpos, q_s, q_m, q_l, ws.acc);
+    launch(k_core_queue, (unsigned)blocks, 256, 0, s, ws.off, ws.cols, ws.offp, ws.colsp, ws.deg, ws.gid, ws.ginfo, n,
+           cseg, ws.fpos, q_s, q_m, q_l, ws.acc);
     HARP_LAUNCHED();
     if (g->max_deg >= (1 << kBitsL))
         HARP_TRY((launch_block<kBitsXL, 512, 1, 1>(ws, bits, cseg, q_l + n - 1, Q_CORE_XL, T_CORE_XL, sink, s)));
@@ -618,7 +622,8 @@ harp_status count_wedge_core(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     HARP_TRY((launch_block<kBitsM, 64, 4, 12>(ws, bits, cseg, q_m, Q_CORE_M, T_CORE_M, sink, s)));
     const size_t smem = (size_t)kWarpsS * kBitsS * kKWordsMax * sizeof(uint32_t);
     HARP_CK(cudaFuncSetAttribute(k_core_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_core_warp<<<sms * 6, kWarpsS * 32, smem, s>>>(ws.off, ws.cols, ws.colsp, cseg, ws.gid, ws.ginfo, ws.fpos, bits, q_s, sink);
+    launch(k_core_warp, sms * 6, kWarpsS * 32, smem, s, ws.off, ws.cols, ws.colsp, cseg, ws.gid, ws.ginfo, ws.fpos,
+           bits, q_s, sink);
     HARP_LAUNCHED();
     return HARP_OK;
 }

@@ -38,6 +38,7 @@ __device__ __forceinline__ Pair load_pair(const int32_t* __restrict__ src, const
 __global__ void __launch_bounds__(256) k_build_degrees(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
                                                        int64_t m_in, int64_t n, int32_t* __restrict__ deg,
                                                        unsigned long long* __restrict__ summary) {
+    grid_begin();
     const int l = lane_id();
     bool bad = false;
     for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - l; base < m_in;
@@ -57,6 +58,7 @@ __global__ void __launch_bounds__(256) k_build_degrees(const int32_t* __restrict
 __global__ void __launch_bounds__(256) k_build_scatter(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
                                                        int64_t m_in, int64_t n, const int64_t* __restrict__ roff,
                                                        int32_t* __restrict__ deg, int32_t* __restrict__ out) {
+    grid_begin();
     const int l = lane_id();
     bool bad = false;
     for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - l; base < m_in;
@@ -95,6 +97,7 @@ __global__ void __launch_bounds__(256) k_build_rows_small(const int64_t* __restr
                                                           int32_t* __restrict__ ndeg, int32_t* __restrict__ q,
                                                           int32_t* __restrict__ q_block,
                                                           unsigned long long* __restrict__ summary) {
+    grid_begin();
     const int l = lane_id();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -201,6 +204,7 @@ __global__ void __launch_bounds__(kMidWarps * 32) k_build_rows_mid(const int64_t
                                                                     int32_t* __restrict__ out, int32_t* __restrict__ ndeg,
                                                                     const int32_t* __restrict__ q,
                                                                     const unsigned long long* __restrict__ summary) {
+    grid_begin();
     const int64_t nq = (int64_t)summary[B_Q_WARP];
     for (int64_t k = (int64_t)blockIdx.x * kMidWarps + (threadIdx.x >> 5); k < nq; k += (int64_t)gridDim.x * kMidWarps) {
         const int64_t i = q[k], b = roff[i];
@@ -221,6 +225,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32) k_build_rows_block(const int
                                                                        int32_t* __restrict__ ndeg,
                                                                        const int32_t* __restrict__ q_block,
                                                                        const unsigned long long* __restrict__ summary) {
+    grid_begin();
     constexpr int E = kBlockE, RUN = 32 * E;
     __shared__ int32_t buf[kTierB];
     __shared__ int32_t s_last[kBlockWarps];
@@ -262,6 +267,7 @@ __global__ void __launch_bounds__(kBitmapThreads) k_build_rows_bitmap(const int6
                                                                       int32_t* __restrict__ ndeg,
                                                                       const int32_t* __restrict__ q,
                                                                       const unsigned long long* __restrict__ summary) {
+    grid_begin();
     extern __shared__ uint32_t bm[];
     __shared__ int s_count[kBitmapWarps];
     const int64_t nq = (int64_t)summary[B_Q_HUB];
@@ -296,6 +302,7 @@ __global__ void __launch_bounds__(kBitmapThreads) k_build_rows_bitmap(const int6
 __global__ void __launch_bounds__(256) k_build_summary(const int32_t* __restrict__ ndeg, const int64_t* __restrict__ off,
                                                        const int64_t* __restrict__ roff, int64_t n,
                                                        unsigned long long* __restrict__ summary) {
+    grid_begin();
     int32_t best = 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
         best = max(best, ndeg[v]);
@@ -311,6 +318,7 @@ __global__ void __launch_bounds__(256) k_build_summary(const int32_t* __restrict
 __global__ void __launch_bounds__(256) k_build_compact(const int64_t* __restrict__ roff, const int64_t* __restrict__ off,
                                                        int64_t n, const int32_t* __restrict__ in,
                                                        int32_t* __restrict__ cols) {
+    grid_begin();
     const int l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; i0 < n; i0 += nw * 32) {
@@ -408,30 +416,30 @@ harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t
     BCK(cudaMallocAsync((void**)&raw, 2 * (size_t)m_in * sizeof(int32_t), s));
     BCK(cudaMallocAsync((void**)&sorted, 2 * (size_t)m_in * sizeof(int32_t), s));
     BCK(cudaMemsetAsync(slab, 0, head + per_n, s));  // summary and degrees
-    k_build_degrees<<<grid_for(m_in, 256), 256, 0, s>>>(d_src, d_dst, m_in, n, deg, summary);
+    launch(k_build_degrees, grid_for(m_in, 256), 256, 0, s, d_src, d_dst, m_in, n, deg, summary);
     BLAUNCHED();
     BTRY(exclusive_scan_i32_to_i64(deg, roff, n, tmp, tmp_len, s));
-    k_build_scatter<<<grid_for(m_in, 256), 256, 0, s>>>(d_src, d_dst, m_in, n, roff, deg, raw);
+    launch(k_build_scatter, grid_for(m_in, 256), 256, 0, s, d_src, d_dst, m_in, n, roff, deg, raw);
     BLAUNCHED();
-    k_build_rows_small<<<grid_for(n, 256), 256, 0, s>>>(roff, n, raw, sorted, ndeg, q, q_block, summary);
+    launch(k_build_rows_small, grid_for(n, 256), 256, 0, s, roff, n, raw, sorted, ndeg, q, q_block, summary);
     BLAUNCHED();
     // a row has at most m_in entries: tiers above that are empty
     if (m_in > kTierA) {
-        k_build_rows_mid<<<num_sms() * 8, kMidWarps * 32, 0, s>>>(roff, raw, sorted, ndeg, q, summary);
+        launch(k_build_rows_mid, num_sms() * 8, kMidWarps * 32, 0, s, roff, raw, sorted, ndeg, q, summary);
         BLAUNCHED();
     }
     if (m_in > kTierB1) {
-        k_build_rows_block<<<num_sms() * 4, kBlockWarps * 32, 0, s>>>(roff, raw, sorted, ndeg, q_block, summary);
+        launch(k_build_rows_block, num_sms() * 4, kBlockWarps * 32, 0, s, roff, raw, sorted, ndeg, q_block, summary);
         BLAUNCHED();
     }
     if (m_in > kTierB) {
         const size_t smem = sizeof(uint32_t) * (size_t)kBitmapWords;
         BCK(cudaFuncSetAttribute(k_build_rows_bitmap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_build_rows_bitmap<<<num_sms(), kBitmapThreads, smem, s>>>(roff, n, raw, sorted, ndeg, q, summary);
+        launch(k_build_rows_bitmap, num_sms(), kBitmapThreads, smem, s, roff, n, raw, sorted, ndeg, q, summary);
         BLAUNCHED();
     }
     BTRY(exclusive_scan_i32_to_i64(ndeg, g->off, n, tmp, tmp_len, s));
-    k_build_summary<<<grid_for(n, 256), 256, 0, s>>>(ndeg, g->off, roff, n, summary);
+    launch(k_build_summary, grid_for(n, 256), 256, 0, s, ndeg, g->off, roff, n, summary);
     BLAUNCHED();
     unsigned long long host[B_WORDS] = {0};
     BCK(cudaMemcpyAsync(host, summary, sizeof(host), cudaMemcpyDeviceToHost, s));
@@ -451,7 +459,7 @@ harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t
     } else {
         BCK(cudaMallocAsync((void**)&g->cols, (size_t)(M > 0 ? M : 1) * sizeof(int32_t), s));
         if (M > 0) {
-            k_build_compact<<<grid_for(n, 256), 256, 0, s>>>(roff, g->off, n, sorted, g->cols);
+            launch(k_build_compact, grid_for(n, 256), 256, 0, s, roff, g->off, n, sorted, g->cols);
             BLAUNCHED();
         }
         BCK(cudaStreamSynchronize(s));

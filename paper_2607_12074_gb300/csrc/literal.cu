@@ -261,6 +261,7 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_tri(Graph G, const int64_t*
                                                          const int32_t* __restrict__ colsp, int64_t n, int64_t m,
                                                          SigCache cache, uint64_t* __restrict__ tau3,
                                                          uint64_t* __restrict__ acc) {
+    grid_begin();
     __shared__ int32_t sbuf[kLitWarps][kStageCap];
     __shared__ uint64_t red[32];
     const int w = threadIdx.x >> 5, l = lane_id();
@@ -344,6 +345,7 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_tri(Graph G, const int64_t*
 __global__ void __launch_bounds__(kLitThreads) k_lit_edge(Graph G, const int64_t* __restrict__ offp,
                                                           const int32_t* __restrict__ colsp, int64_t n, int64_t m,
                                                           SigCache cache, uint64_t* __restrict__ acc) {
+    grid_begin();
     __shared__ int32_t sbuf[kLitWarps][kStageCap];
     __shared__ uint64_t red[32];
     const int w = threadIdx.x >> 5, l = lane_id();
@@ -422,6 +424,7 @@ struct StagedShape {
 
 __global__ void __launch_bounds__(kStagedThreads) k_lit_edge_staged(Graph G, const int64_t* __restrict__ offp, int64_t n,
                                                                     SigCache cache, uint64_t* __restrict__ acc) {
+    grid_begin();
     extern __shared__ uint32_t smem[];
     __shared__ uint64_t red[32];
     __shared__ int64_t s_item;
@@ -518,6 +521,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_lit_edge_staged(Graph G, con
 __global__ void __launch_bounds__(kLitThreads) k_lit_star(Graph G, int64_t n, SigCache cache,
                                                           const uint64_t* __restrict__ tau3,
                                                           uint64_t* __restrict__ acc) {
+    grid_begin();
     __shared__ uint64_t red[32];
     const int l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -553,6 +557,7 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_star(Graph G, int64_t n, Si
 // ---------------------------------------------------------------------------------------------
 // staged: the edge sum lacks its correction
 __global__ void k_lit_close(int64_t m, bool staged, uint64_t* __restrict__ acc) {
+    grid_begin();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const unsigned __int128 X2 = (unsigned __int128)acc[ACC_LIT_X2] | ((unsigned __int128)acc[ACC_LIT_X2 + 1] << 64);
     const unsigned __int128 X3 = (unsigned __int128)acc[ACC_LIT_X3] | ((unsigned __int128)acc[ACC_LIT_X3 + 1] << 64);
@@ -620,7 +625,7 @@ harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& pla
     if (e == cudaSuccess && slots) e = cudaMemsetAsync(cache.vals, 0, 8 * slots, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(tau3, 0, 8 * (size_t)(n > 0 ? n : 1), s);
     if (e == cudaSuccess && m > 0) {
-        k_lit_tri<<<lit_grid(m), kLitThreads, 0, s>>>(G, ws.offp, ws.colsp, n, m, cache, tau3, ws.acc);
+        launch(k_lit_tri, lit_grid(m), kLitThreads, 0, s, G, ws.offp, ws.colsp, n, m, cache, tau3, ws.acc);
         note_launch();
         e = cudaGetLastError();
         if (e == cudaSuccess) e = prof_mark(s, SEG_TRI_WARP);
@@ -631,22 +636,22 @@ harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& pla
                 const int per_sm = smem <= 50 * 1024 ? 4 : (smem <= 100 * 1024 ? 2 : 1);
                 const int64_t blocks = n < (int64_t)num_sms() * per_sm ? n : (int64_t)num_sms() * per_sm;
                 if (e == cudaSuccess)
-                    k_lit_edge_staged<<<(unsigned)blocks, kStagedThreads, smem, s>>>(G, ws.offp, n, cache, ws.acc);
+                    launch(k_lit_edge_staged, (unsigned)blocks, kStagedThreads, smem, s, G, ws.offp, n, cache, ws.acc);
             } else {
-                k_lit_edge<<<lit_grid(m), kLitThreads, 0, s>>>(G, ws.offp, ws.colsp, n, m, cache, ws.acc);
+                launch(k_lit_edge, lit_grid(m), kLitThreads, 0, s, G, ws.offp, ws.colsp, n, m, cache, ws.acc);
             }
             note_launch();
             if (e == cudaSuccess) e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = prof_mark(s, SEG_C4_SMALL);
         if (e == cudaSuccess) {
-            k_lit_star<<<lit_grid(n), kLitThreads, 0, s>>>(G, n, cache, tau3, ws.acc);
+            launch(k_lit_star, lit_grid(n), kLitThreads, 0, s, G, n, cache, tau3, ws.acc);
             note_launch();
             e = cudaGetLastError();
         }
     }
     if (e == cudaSuccess) {
-        k_lit_close<<<1, 32, 0, s>>>(m, staged, ws.acc);
+        launch(k_lit_close, 1, 32, 0, s, m, staged, ws.acc);
         note_launch();
         e = cudaGetLastError();
     }

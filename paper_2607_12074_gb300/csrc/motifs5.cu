@@ -134,6 +134,7 @@ __device__ __forceinline__ int extend(const int64_t* __restrict__ off, const int
 __global__ void __launch_bounds__(kM5Threads) k_m5_esu(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
                                                        int64_t n, M5Table table, int32_t* __restrict__ scratch,
                                                        int64_t D, unsigned long long* __restrict__ out) {
+    grid_begin();
     __shared__ unsigned long long hist[kM5Warps][kM5Classes];
     __shared__ uint8_t cls[1024];
     for (int i = threadIdx.x; i < 1024; i += kM5Threads) cls[i] = table.cls[i];
@@ -233,7 +234,7 @@ extern "C" harp_status harp_count5(const harp_csr* gc, uint64_t counts_out[21]) 
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&d_out, sizeof(unsigned long long) * kM5Classes, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_out, 0, sizeof(unsigned long long) * kM5Classes, s);
     if (e == cudaSuccess) {
-        k_m5_esu<<<(unsigned)blocks, kM5Threads, 0, s>>>(ws.off, ws.cols, g->n, h.table, scratch, D, d_out);
+        launch(k_m5_esu, (unsigned)blocks, kM5Threads, 0, s, ws.off, ws.cols, g->n, h.table, scratch, D, d_out);
         note_launch();
         e = cudaGetLastError();
     }

@@ -34,6 +34,7 @@ void* g_noalloc_ptr[64] = {nullptr};  // device address of g_noalloc_scratch, pe
 // sets kErrBadCsr in acc[ACC_ERR]; the orientation pass then treats the graph as edgeless, so no
 // kernel indexes past the scratch laid out for (n, m).
 __global__ void k_check_offsets(const int64_t* __restrict__ off, int64_t n, int64_t m, uint64_t* __restrict__ acc) {
+    grid_begin();
     bool bad = false;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v <= n; v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = off[v];
@@ -48,6 +49,7 @@ __global__ void k_check_offsets(const int64_t* __restrict__ off, int64_t n, int6
 }
 
 __global__ void k_check_cols(const int32_t* __restrict__ cols, int64_t n, int64_t m, uint64_t* __restrict__ acc) {
+    grid_begin();
     // offsets failed: off[n] may not bound the columns.  Lane 0 reads the flag for its warp, so the
     // warp leaves (or stays) as a whole even while other warps set the same bit.
     const uint64_t flag = __shfl_sync(kFull, lane_id() == 0 ? acc[ACC_ERR] : 0ull, 0);
@@ -126,10 +128,10 @@ extern "C" harp_status harp_count4_noalloc(int64_t n, int64_t m, const int64_t* 
     // a CSR that fails its check has none
     HARP_CK(cudaMemsetAsync(ws.acc, 0, sizeof(uint64_t) * kOutLen, s));
     HARP_CK(cudaMemsetAsync(ws.te, 0, sizeof(uint32_t) * (size_t)(m > 0 ? m : 1), s));
-    k_check_offsets<<<check_grid(n + 1), 256, 0, s>>>(d_offsets, n, m, ws.acc);
+    launch(k_check_offsets, check_grid(n + 1), 256, 0, s, d_offsets, n, m, ws.acc);
     HARP_LAUNCHED();
     if (m > 0) {
-        k_check_cols<<<check_grid(2 * m), 256, 0, s>>>(d_cols, n, m, ws.acc);
+        launch(k_check_cols, check_grid(2 * m), 256, 0, s, d_cols, n, m, ws.acc);
         HARP_LAUNCHED();
     }
     if (n > 0) {

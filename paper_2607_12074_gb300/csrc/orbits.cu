@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_tri_big(OrbGraph G, const i
                                                              const uint64_t* __restrict__ qcnt,
                                                              unsigned long long* __restrict__ n9,
                                                              unsigned long long* __restrict__ tau6, EdgeRoute er) {
+    grid_begin();
     __shared__ int32_t sbuf[kOrbWarps][kOrbStage];
     const int w = threadIdx.x >> 5, l = lane_id();
     for (int64_t i = blockIdx.x; i < (int64_t)*qcnt; i += gridDim.x)
@@ -248,6 +249,7 @@ constexpr int kRowLane = 64, kRowWarp = 256;
 __global__ void __launch_bounds__(kOrbThreads) k_orb_vertex(OrbGraph G, const int32_t* __restrict__ rev, int64_t n,
                                                             uint64_t* __restrict__ tsum, uint64_t* __restrict__ s1,
                                                             uint64_t* __restrict__ N) {
+    grid_begin();
     const int l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     auto store = [&](int64_t v, const VertexSums& x) {
@@ -288,6 +290,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_vertex_hub(OrbGraph G, cons
                                                                 unsigned long long* __restrict__ tsum,
                                                                 unsigned long long* __restrict__ s1,
                                                                 unsigned long long* __restrict__ N) {
+    grid_begin();
     const int l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     int64_t lo = 0, hi = n;  // first rank of degree above kRowWarp
@@ -339,6 +342,7 @@ enum : int { QO_LIGHT = 0, QO_MID, QO_HUGE, QO_HEAVY, QO_TICKET };
 __global__ void k_orb_classify(OrbGraph G, const int32_t* __restrict__ rev, int64_t n, int32_t* __restrict__ q_light,
                                int32_t* __restrict__ w_light, int32_t* __restrict__ q_heavy,
                                unsigned long long* __restrict__ qcnt) {
+    grid_begin();
     const int l = lane_id();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -454,6 +458,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_orb_c4w(OrbGraph G, const int32_
                                                         unsigned long long* __restrict__ n7,
                                                         unsigned long long* __restrict__ n7x2,
                                                         unsigned long long* __restrict__ e6a) {
+    grid_begin();
     constexpr int TEAMS = MID ? 1 : WARPS, TW = MID ? WARPS : 1;  // roots per block, warps per root
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ uint32_t s_sw[WARPS][32];
@@ -536,6 +541,7 @@ __global__ void __launch_bounds__(kWinThreads, 2) k_orb_c4win(OrbGraph G, const 
                                                               unsigned long long* __restrict__ n7,
                                                               unsigned long long* __restrict__ n7x2,
                                                               unsigned long long* __restrict__ e6a) {
+    grid_begin();
     constexpr int PER = 32 / BITS;
     constexpr int64_t X = (int64_t)kWinWords * PER;
     extern __shared__ uint32_t ctr[];
@@ -673,6 +679,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_c4b(OrbGraph G, int64_t n, 
                                                          unsigned long long* __restrict__ n7,
                                                          unsigned long long* __restrict__ n7x2,
                                                          unsigned long long* __restrict__ e6a) {
+    grid_begin();
     __shared__ uint64_t red[32];
     uint32_t* cntv = dense + (size_t)blockIdx.x * (size_t)n;
     const int64_t nq = (int64_t)(qcnt[QO_HUGE] + qcnt[QO_HEAVY]);
@@ -730,6 +737,7 @@ __global__ void __launch_bounds__(kOrbThreads) k_orb_close(OrbGraph G, int64_t n
                                                            const int32_t* __restrict__ order,
                                                            uint64_t* __restrict__ N, uint64_t* __restrict__ out,
                                                            uint64_t* __restrict__ acc) {
+    grid_begin();
     const int l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += nw) {
@@ -788,6 +796,7 @@ __constant__ uint8_t c_econtain[kEdgeOrbits][kEdgeOrbits] = {
 // up[x] = neighbours of input vertex x above x (its row's suffix in the input CSR)
 __global__ void k_eorb_up(const int64_t* __restrict__ off_in, const int32_t* __restrict__ cols_in, int64_t n,
                           int32_t* __restrict__ up) {
+    grid_begin();
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
         const int64_t b = off_in[x], e = off_in[x + 1];
         up[x] = (int32_t)(e - b - lower_bound_i32(cols_in + b, e - b, (int32_t)x + 1));
@@ -804,6 +813,7 @@ __global__ void k_eorb_close(OrbGraph G, int64_t n, int64_t m, const int32_t* __
                              const int32_t* __restrict__ cols_in, const int32_t* __restrict__ up,
                              const int64_t* __restrict__ ebase, uint64_t* __restrict__ out,
                              uint64_t* __restrict__ acc) {
+    grid_begin();
     for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < m; a += (int64_t)gridDim.x * blockDim.x) {
         const int32_t u = arc_row(G.offp, n, a);
         const int32_t v = G.colsp[a];
@@ -889,37 +899,40 @@ harp_status orbit_passes(const harp_csr* g, Workspace& ws, const OrbScratch& o, 
     HARP_TRY(orbit_triangles(g, ws, OrbTri{o.n9, o.tau6, o.e5, o.e8, o.e9}, s));
     if (max_out_degree(g) > 1024) {
         const EdgeRoute er{o.e5, o.e8, o.e9};
-        k_orb_tri_big<<<num_sms() * 4, kOrbThreads, 0, s>>>(G, ws.q_mid + n, ws.acc + Q_TRI_BIG, o.n9, o.tau6, er);
+        launch(k_orb_tri_big, num_sms() * 4, kOrbThreads, 0, s, G, ws.q_mid + n, ws.acc + Q_TRI_BIG, o.n9, o.tau6, er);
         HARP_LAUNCHED();
-        k_orb_tri_big<<<num_sms() * 4, kOrbThreads, 0, s>>>(G, ws.q_mid, ws.acc + Q_TRI_FB, o.n9, o.tau6, er);
+        launch(k_orb_tri_big, num_sms() * 4, kOrbThreads, 0, s, G, ws.q_mid, ws.acc + Q_TRI_FB, o.n9, o.tau6, er);
         HARP_LAUNCHED();
     }
     HARP_TRY(wedge_positions(g, ws, s));
-    k_orb_vertex<<<orb_grid((n + 3) / 4), kOrbThreads, 0, s>>>(G, ws.rev, n, o.tsum, o.s1, o.N);
+    launch(k_orb_vertex, orb_grid((n + 3) / 4), kOrbThreads, 0, s, G, ws.rev, n, o.tsum, o.s1, o.N);
     HARP_LAUNCHED();
     if (g->max_deg > kRowWarp) {
-        k_orb_vertex_hub<<<num_sms() * 4, kOrbThreads, 0, s>>>(G, ws.rev, n, (unsigned long long*)o.tsum,
-                                                               (unsigned long long*)o.s1, (unsigned long long*)o.N);
+        launch(k_orb_vertex_hub, num_sms() * 4, kOrbThreads, 0, s, G, ws.rev, n, (unsigned long long*)o.tsum,
+               (unsigned long long*)o.s1, (unsigned long long*)o.N);
         HARP_LAUNCHED();
     }
-    k_orb_classify<<<orb_grid((n + 31) / 32), kOrbThreads, 0, s>>>(G, ws.rev, n, o.q_light, o.w_light, o.q_heavy, o.qcnt);
+    launch(k_orb_classify, orb_grid((n + 31) / 32), kOrbThreads, 0, s, G, ws.rev, n, o.q_light, o.w_light, o.q_heavy,
+           o.qcnt);
     HARP_LAUNCHED();
     const size_t light_smem = (size_t)kOrbWarps * kHashSlots * 8, mid_smem = (size_t)kMidSlots * 8;
     auto light = k_orb_c4w<kHashSlots, kOrbWarps, false>;
     auto mid = k_orb_c4w<kMidSlots, kMidWarps, true>;
     HARP_CK(cudaFuncSetAttribute(light, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)light_smem));
     HARP_CK(cudaFuncSetAttribute(mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem));
-    light<<<orb_grid(n), kOrbThreads, light_smem, s>>>(G, ws.rev, n, o.q_light, o.w_light, o.qcnt, o.n7, o.n7x2, o.e6a);
+    launch(light, orb_grid(n), kOrbThreads, light_smem, s, G, ws.rev, n, o.q_light, o.w_light, o.qcnt, o.n7, o.n7x2,
+           o.e6a);
     HARP_LAUNCHED();
-    mid<<<num_sms() * 6, kMidWarps * 32, mid_smem, s>>>(G, ws.rev, n, o.q_light, o.w_light, o.qcnt, o.n7, o.n7x2, o.e6a);
+    launch(mid, num_sms() * 6, kMidWarps * 32, mid_smem, s, G, ws.rev, n, o.q_light, o.w_light, o.qcnt, o.n7, o.n7x2,
+           o.e6a);
     HARP_LAUNCHED();
     if (o.dense) {
-        k_orb_c4b<<<o.heavy_blocks, kOrbThreads, 0, s>>>(G, n, o.q_heavy, o.qcnt, o.dense, o.n7, o.n7x2, o.e6a);
+        launch(k_orb_c4b, o.heavy_blocks, kOrbThreads, 0, s, G, n, o.q_heavy, o.qcnt, o.dense, o.n7, o.n7x2, o.e6a);
     } else {
         const size_t smem = (size_t)kWinWords * sizeof(uint32_t);
         auto kernel = g->max_deg < 65536 ? k_orb_c4win<16> : k_orb_c4win<32>;
         HARP_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kernel<<<num_sms() * 2, kWinThreads, smem, s>>>(G, ws.rev, n, o.q_heavy, o.qcnt, o.n7, o.n7x2, o.e6a);
+        launch(kernel, num_sms() * 2, kWinThreads, smem, s, G, ws.rev, n, o.q_heavy, o.qcnt, o.n7, o.n7x2, o.e6a);
     }
     HARP_LAUNCHED();
     return HARP_OK;
@@ -956,8 +969,8 @@ harp_status count_orbits(const harp_csr* g, Workspace& ws, uint64_t* d_out, cuda
     if (e == cudaSuccess) st = orbit_passes(g, ws, o, s);
     if (e == cudaSuccess && st == HARP_OK) {
         const OrbGraph G{ws.off, ws.cols, ws.deg, ws.offp, ws.colsp, ws.te};
-        k_orb_close<<<orb_grid(n), kOrbThreads, 0, s>>>(G, n, o.tsum, o.s1, o.n9, o.tau6, o.n7, o.n7x2, ws.order, o.N,
-                                                         d_out, ws.acc);
+        launch(k_orb_close, orb_grid(n), kOrbThreads, 0, s, G, n, o.tsum, o.s1, o.n9, o.tau6, o.n7, o.n7x2, ws.order,
+               o.N, d_out, ws.acc);
         note_launch();
         e = cudaGetLastError();
     }
@@ -1000,7 +1013,7 @@ harp_status count_edge_orbits(const harp_csr* g, Workspace& ws, uint64_t* d_out,
     if (e == cudaSuccess) st = orbit_passes(g, ws, o, s);
     if (e == cudaSuccess && st == HARP_OK) {
         const int64_t blocks = (n + 255) / 256;
-        k_eorb_up<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(g->off, g->cols, n, up);
+        launch(k_eorb_up, (unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s, g->off, g->cols, n, up);
         note_launch();
         e = cudaGetLastError();
     }
@@ -1008,8 +1021,9 @@ harp_status count_edge_orbits(const harp_csr* g, Workspace& ws, uint64_t* d_out,
     if (e == cudaSuccess && st == HARP_OK) {
         const OrbGraph G{ws.off, ws.cols, ws.deg, ws.offp, ws.colsp, ws.te};
         const int64_t blocks = (m + 255) / 256;
-        k_eorb_close<<<(unsigned)(blocks < (int64_t)num_sms() * 16 ? blocks : (int64_t)num_sms() * 16), 256, 0, s>>>(
-            G, n, m, ws.dplus, o.tsum, o.s1, o.e5, o.e8, o.e9, o.e6a, ws.order, g->off, g->cols, up, ebase, d_out, ws.acc);
+        launch(k_eorb_close, (unsigned)(blocks < (int64_t)num_sms() * 16 ? blocks : (int64_t)num_sms() * 16), 256, 0,
+               s, G, n, m, ws.dplus, o.tsum, o.s1, o.e5, o.e8, o.e9, o.e6a, ws.order, g->off, g->cols, up, ebase,
+               d_out, ws.acc);
         note_launch();
         e = cudaGetLastError();
     }

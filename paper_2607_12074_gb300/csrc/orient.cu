@@ -38,6 +38,7 @@ unsigned grid_for(int64_t work, int threads, int64_t cap = -1) {
 __global__ void k_vertex_keys(const int64_t* __restrict__ off, int64_t n, int b, int bd,
                               uint64_t* __restrict__ keys, uint64_t* __restrict__ acc,
                               const int32_t* __restrict__ gid_in, uint64_t* __restrict__ accG) {
+    grid_begin();
     uint64_t s3 = 0;
     // a caller-built CSR that failed its check (harp_count4_noalloc) is counted as edgeless: every
     // later kernel then stays inside the arrays sized for its (n, m)
@@ -68,6 +69,7 @@ __global__ void k_relabel(const uint64_t* __restrict__ keys, int64_t n, int b, i
                           int32_t* __restrict__ perm, int32_t* __restrict__ deg,
                           const int32_t* __restrict__ gid_in, int32_t* __restrict__ gid,
                           int32_t* __restrict__ q, int32_t* __restrict__ q_block, uint64_t* __restrict__ acc) {
+    grid_begin();
     const uint64_t mask = ((uint64_t)1 << b) - 1;
     const uint64_t dmask = ((uint64_t)1 << bd) - 1;
     const int l = lane_id();
@@ -138,6 +140,7 @@ __global__ void __launch_bounds__(256) k_sort_rows_warp(const int64_t* __restric
                                                         const int64_t* __restrict__ off, int64_t n,
                                                         int32_t* __restrict__ cols,
                                                         int32_t* __restrict__ dplus) {
+    grid_begin();
     const int l = lane_id();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -226,6 +229,7 @@ __global__ void __launch_bounds__(kMidWarps * 32) k_sort_rows_mid(const int64_t*
                                                                    int32_t* __restrict__ dplus,
                                                                    const int32_t* __restrict__ q,
                                                                    const uint64_t* __restrict__ acc) {
+    grid_begin();
     const int64_t nq = (int64_t)acc[Q_SORT_WARP];
     for (int64_t qi = (int64_t)blockIdx.x * kMidWarps + (threadIdx.x >> 5); qi < nq; qi += (int64_t)gridDim.x * kMidWarps) {
         const int64_t i = q[qi];
@@ -251,6 +255,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32) k_sort_rows_block(const int6
                                                                       int32_t* __restrict__ dplus,
                                                                       const int32_t* __restrict__ q,
                                                                       const uint64_t* __restrict__ acc) {
+    grid_begin();
     constexpr int E = kBlockE, RUN = 32 * E;
     __shared__ int32_t buf[kTierB];
     __shared__ int s_above[kBlockWarps];
@@ -304,6 +309,7 @@ __global__ void __launch_bounds__(kBitmapThreads) k_sort_rows_bitmap(const int64
                                                                      int32_t* __restrict__ dplus,
                                                                      const int32_t* __restrict__ q,
                                                                      const uint64_t* __restrict__ acc) {
+    grid_begin();
     extern __shared__ uint32_t bm[];
     __shared__ int s_count[kBitmapWarps];
     __shared__ int s_above;
@@ -363,6 +369,7 @@ __global__ void __launch_bounds__(kHubThreads) k_sort_rows_hub(const int64_t* __
                                                                int32_t* __restrict__ dplus,
                                                                const int32_t* __restrict__ q,
                                                                const unsigned long long* __restrict__ qcnt) {
+    grid_begin();
     __shared__ uint32_t base[256];
     __shared__ uint32_t wcnt[kHubWarps][256];
     __shared__ int cnt_below;
@@ -453,6 +460,7 @@ __global__ void __launch_bounds__(256) k_out_csr(const int64_t* __restrict__ off
                                                  const int32_t* __restrict__ deg,
                                                  const int64_t* __restrict__ offp, int64_t n,
                                                  int32_t* __restrict__ colsp, uint32_t* __restrict__ te, Sink sink) {
+    grid_begin();
     __shared__ uint64_t red[32];
     const int l = lane_id();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -535,45 +543,43 @@ harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s) {
 
     // rank = (graph, degree, id): each graph's vertices form one contiguous rank range, sorted by
     // degree (a single graph is graph 0)
-    k_vertex_keys<<<grid_for(n, 256), 256, 0, s>>>(g->off, n, b, bd, ws.vkeys, ws.acc, ws.gid_in, ws.accG);
+    launch(k_vertex_keys, grid_for(n, 256), 256, 0, s, g->off, n, b, bd, ws.vkeys, ws.acc, ws.gid_in, ws.accG);
     HARP_LAUNCHED();
     uint64_t* k0 = ws.vkeys;
     uint64_t* k1 = ws.vkeys_alt;
     // the keys are written in id order and every pass is stable, so only the graph and degree bits
     // need sorting: equal (graph, degree) keep ascending ids
     HARP_TRY(radix_sort_u64(&k0, &k1, n, b, b + bd + bg, ws.hist, ws.scan_tmp, ws.scan_tmp_len, s));
-    k_relabel<<<grid_for(n, 256), 256, 0, s>>>(k0, n, b, bd, ws.order, ws.perm, ws.deg, ws.gid_in, ws.gid, ws.q_tri,
-                                               ws.q_mid, ws.acc);
+    launch(k_relabel, grid_for(n, 256), 256, 0, s, k0, n, b, bd, ws.order, ws.perm, ws.deg, ws.gid_in, ws.gid,
+           ws.q_tri, ws.q_mid, ws.acc);
     HARP_LAUNCHED();
     HARP_TRY(exclusive_scan_i32_to_i64(ws.deg, ws.off, n, ws.scan_tmp, ws.scan_tmp_len, s));
     if (m > 0) {
         // 32 rows per warp
-        k_sort_rows_warp<<<grid_for(n, 256), 256, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg,
-                                                                ws.off, n, ws.cols, ws.dplus);
+        launch(k_sort_rows_warp, grid_for(n, 256), 256, 0, s, g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off, n,
+               ws.cols, ws.dplus);
         HARP_LAUNCHED();
         if (g->max_deg > kTierA) {
-            k_sort_rows_mid<<<num_sms() * 8, kMidWarps * 32, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off,
-                                                                     ws.cols, ws.dplus, ws.q_tri, ws.acc);
+            launch(k_sort_rows_mid, num_sms() * 8, kMidWarps * 32, 0, s, g->off, g->cols, ws.order, ws.perm, ws.deg,
+                   ws.off, ws.cols, ws.dplus, ws.q_tri, ws.acc);
             HARP_LAUNCHED();
         }
         if (g->max_deg > kTierB1) {
-            k_sort_rows_block<<<num_sms() * 4, kBlockWarps * 32, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg,
-                                                                         ws.off, ws.cols, ws.dplus, ws.q_mid, ws.acc);
+            launch(k_sort_rows_block, num_sms() * 4, kBlockWarps * 32, 0, s, g->off, g->cols, ws.order, ws.perm,
+                   ws.deg, ws.off, ws.cols, ws.dplus, ws.q_mid, ws.acc);
             HARP_LAUNCHED();
         }
         const int64_t most_n = ws.G > 1 ? ws.max_member_n : n;  // ranks of the largest graph
         if (g->max_deg > kTierB && most_n <= kBitmapRanks) {
             const size_t smem = sizeof(uint32_t) * (size_t)kBitmapWords;
             HARP_CK(cudaFuncSetAttribute(k_sort_rows_bitmap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            k_sort_rows_bitmap<<<num_sms(), kBitmapThreads, smem, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off,
-                                                                       n, ws.G > 1 ? ws.gid : nullptr, ws.gbase, ws.cols,
-                                                                       ws.dplus, ws.q_tri, ws.acc);
+            launch(k_sort_rows_bitmap, num_sms(), kBitmapThreads, smem, s, g->off, g->cols, ws.order, ws.perm, ws.deg,
+                   ws.off, n, ws.G > 1 ? ws.gid : nullptr, ws.gbase, ws.cols, ws.dplus, ws.q_tri, ws.acc);
             HARP_LAUNCHED();
         } else if (g->max_deg > kTierB) {
             // the out-CSR columns + t_e region (2m int32) is free until k_out_csr: hub sort ping-pong
-            k_sort_rows_hub<<<num_sms(), kHubThreads, 0, s>>>(g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off, n, b,
-                                                              ws.cols, ws.colsp, ws.dplus, ws.q_tri,
-                                                              (const unsigned long long*)&ws.acc[Q_SORT_WARP]);
+            launch(k_sort_rows_hub, num_sms(), kHubThreads, 0, s, g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off,
+                   n, b, ws.cols, ws.colsp, ws.dplus, ws.q_tri, (const unsigned long long*)&ws.acc[Q_SORT_WARP]);
             HARP_LAUNCHED();
         }
     } else {
@@ -583,8 +589,8 @@ harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     if (m > 0) {
         const Sink sink{ws.acc, ws.gid, ws.accG};
         // 32 rows per warp
-        k_out_csr<<<grid_for(n, 256), 256, 0, s>>>(ws.off, ws.cols, ws.dplus, ws.deg, ws.offp, n, ws.colsp,
-                                                   ws.te, sink);
+        launch(k_out_csr, grid_for(n, 256), 256, 0, s, ws.off, ws.cols, ws.dplus, ws.deg, ws.offp, n, ws.colsp, ws.te,
+               sink);
         HARP_LAUNCHED();
     }
     return HARP_OK;

@@ -45,6 +45,7 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 // out[3 * i + 0] = d_u, [+1] = d_v, [+2] = t_uv.
 __global__ void k_plan_sample(const int64_t* __restrict__ off, const int32_t* __restrict__ cols, int64_t n,
                               int64_t arcs, uint64_t samples, uint64_t seed, uint32_t* __restrict__ out) {
+    grid_begin();
     const int l = lane_id();
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < samples; i += nw) {
@@ -155,8 +156,8 @@ extern "C" harp_status harp_select_anchors(const harp_csr* g, const harp_select_
         cudaError_t e = cudaMallocAsync((void**)&d_smp, 3 * samples * sizeof(uint32_t), g->stream);
         if (e == cudaSuccess) {
             const uint64_t blocks = (samples * 32 + 255) / 256;
-            k_plan_sample<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, g->stream>>>(
-                g->off, g->cols, g->n, 2 * g->m, samples, seed, d_smp);
+            launch(k_plan_sample, (unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, g->stream, g->off, g->cols, g->n,
+                   2 * g->m, samples, seed, d_smp);
             note_launch();
             e = cudaGetLastError();
             if (e == cudaSuccess)

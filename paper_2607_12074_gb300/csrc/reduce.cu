@@ -21,6 +21,7 @@ namespace {
 
 __global__ void __launch_bounds__(256) k_reduce_close(const uint32_t* __restrict__ te, int64_t m,
                                                       uint64_t* __restrict__ acc) {
+    grid_begin();
     __shared__ uint64_t red[32];
     __shared__ bool last;
     uint64_t dsum = 0;
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(256) k_reduce_close(const uint32_t* __restrict
 // rows almost always share one) instead of one per row.
 __global__ void __launch_bounds__(256) k_reduce_rows_batch(const int64_t* __restrict__ offp,
                                                            const uint32_t* __restrict__ te, int64_t n, Sink sink) {
+    grid_begin();
     const int l = lane_id();
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -99,6 +101,7 @@ __global__ void __launch_bounds__(256) k_reduce_rows_batch(const int64_t* __rest
 
 // Batch mode: the closure of every graph (one thread per graph); out holds 16 uint64 per graph.
 __global__ void k_close_batch(const uint64_t* __restrict__ accG, int64_t G, uint64_t* __restrict__ out) {
+    grid_begin();
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < G; g += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t* a = accG + g * kGStride;
         const uint64_t T = a[G_T], K4 = a[G_K4], C4n = a[G_C4], S = a[G_S];
@@ -138,12 +141,12 @@ harp_status reduce_and_close_batch(const harp_csr* g, Workspace& ws, int64_t G, 
     if (blocks < 1) blocks = 1;
     if (blocks > (int64_t)num_sms() * 16) blocks = (int64_t)num_sms() * 16;
     if (g->m > 0) {
-        k_reduce_rows_batch<<<(unsigned)blocks, 256, 0, s>>>(ws.offp, ws.te, g->n, sink);
+        launch(k_reduce_rows_batch, (unsigned)blocks, 256, 0, s, ws.offp, ws.te, g->n, sink);
         HARP_LAUNCHED();
     }
     int64_t cb = (G + 255) / 256;
     if (cb < 1) cb = 1;
-    k_close_batch<<<(unsigned)cb, 256, 0, s>>>(ws.accG, G, d_out);
+    launch(k_close_batch, (unsigned)cb, 256, 0, s, ws.accG, G, d_out);
     HARP_LAUNCHED();
     return HARP_OK;
 }
@@ -152,7 +155,7 @@ harp_status reduce_and_close(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     int64_t blocks = (g->m + 255) / 256;
     if (blocks < 1) blocks = 1;
     if (blocks > (int64_t)num_sms() * 8) blocks = (int64_t)num_sms() * 8;
-    k_reduce_close<<<(unsigned)blocks, 256, 0, s>>>(ws.te, g->m, ws.acc);
+    launch(k_reduce_close, (unsigned)blocks, 256, 0, s, ws.te, g->m, ws.acc);
     HARP_LAUNCHED();
     return HARP_OK;
 }

@@ -40,6 +40,7 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T* warp_tot, T* total) {
 template <typename Tin>
 __global__ void __launch_bounds__(kScanThreads) k_tile_reduce(const Tin* __restrict__ in, int64_t n,
                                                               int64_t* __restrict__ partial) {
+    grid_begin();
     const int64_t base = (int64_t)blockIdx.x * kScanTile;
     int64_t s = 0;
 #pragma unroll
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_reduce(const Tin* __restr
 template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(kScanThreads) k_tile_scan(const Tin* in, Tout* out, int64_t n,
                                                             const int64_t* __restrict__ partial) {
+    grid_begin();
     __shared__ int64_t tile[kScanTile];
     __shared__ int64_t warp_tot[32];
     __shared__ int64_t tot;
@@ -96,15 +98,15 @@ int64_t ntiles(int64_t n) { return (n + kScanTile - 1) / kScanTile; }
 harp_status scan_i64_inplace(int64_t* data, int64_t n, int64_t* tmp, size_t tmp_len, cudaStream_t s) {
     const int64_t nb = ntiles(n);
     if (nb <= 1) {
-        k_tile_scan<int64_t, int64_t><<<1, kScanThreads, 0, s>>>(data, data, n, nullptr);
+        launch(k_tile_scan<int64_t, int64_t>, 1, kScanThreads, 0, s, data, data, n, nullptr);
         HARP_LAUNCHED();
         return HARP_OK;
     }
     if ((size_t)(nb + 1) > tmp_len) return HARP_ENOMEM;
-    k_tile_reduce<int64_t><<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, tmp);
+    launch(k_tile_reduce<int64_t>, (unsigned)nb, kScanThreads, 0, s, data, n, tmp);
     HARP_LAUNCHED();
     HARP_TRY(scan_i64_inplace(tmp, nb, tmp + nb + 1, tmp_len - (size_t)(nb + 1), s));
-    k_tile_scan<int64_t, int64_t><<<(unsigned)nb, kScanThreads, 0, s>>>(data, data, n, tmp);
+    launch(k_tile_scan<int64_t, int64_t>, (unsigned)nb, kScanThreads, 0, s, data, data, n, tmp);
     HARP_LAUNCHED();
     return HARP_OK;
 }
@@ -127,15 +129,15 @@ harp_status exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n
                                       size_t tmp_len, cudaStream_t s) {
     const int64_t nb = ntiles(n);
     if (nb <= 1) {
-        k_tile_scan<int32_t, int64_t><<<1, kScanThreads, 0, s>>>(in, out, n, nullptr);
+        launch(k_tile_scan<int32_t, int64_t>, 1, kScanThreads, 0, s, in, out, n, nullptr);
         HARP_LAUNCHED();
         return HARP_OK;
     }
     if ((size_t)(nb + 1) > tmp_len) return HARP_ENOMEM;
-    k_tile_reduce<int32_t><<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, tmp);
+    launch(k_tile_reduce<int32_t>, (unsigned)nb, kScanThreads, 0, s, in, n, tmp);
     HARP_LAUNCHED();
     HARP_TRY(scan_i64_inplace(tmp, nb, tmp + nb + 1, tmp_len - (size_t)(nb + 1), s));
-    k_tile_scan<int32_t, int64_t><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, tmp);
+    launch(k_tile_scan<int32_t, int64_t>, (unsigned)nb, kScanThreads, 0, s, in, out, n, tmp);
     HARP_LAUNCHED();
     return HARP_OK;
 }
@@ -149,15 +151,15 @@ harp_status exclusive_scan_u32_inplace(uint32_t* data, int64_t n, int64_t* tmp, 
     if (nb <= 1) {
         // single tile; write the total into a scratch slot instead of data[n]
         if (tmp_len < 2) return HARP_ENOMEM;
-        k_tile_scan<uint32_t, uint32_t><<<1, kScanThreads, 0, s>>>(data, data, n - 1, nullptr);
+        launch(k_tile_scan<uint32_t, uint32_t>, 1, kScanThreads, 0, s, data, data, n - 1, nullptr);
         HARP_LAUNCHED();
         return HARP_OK;
     }
     if ((size_t)(nb + 1) > tmp_len) return HARP_ENOMEM;
-    k_tile_reduce<uint32_t><<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, tmp);
+    launch(k_tile_reduce<uint32_t>, (unsigned)nb, kScanThreads, 0, s, data, n, tmp);
     HARP_LAUNCHED();
     HARP_TRY(scan_i64_inplace(tmp, nb, tmp + nb + 1, tmp_len - (size_t)(nb + 1), s));
-    k_tile_scan<uint32_t, uint32_t><<<(unsigned)nb, kScanThreads, 0, s>>>(data, data, n - 1, tmp);
+    launch(k_tile_scan<uint32_t, uint32_t>, (unsigned)nb, kScanThreads, 0, s, data, data, n - 1, tmp);
     HARP_LAUNCHED();
     return HARP_OK;
 }

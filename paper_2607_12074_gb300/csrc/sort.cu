@@ -19,6 +19,7 @@ constexpr int kRadix = 256;
 __global__ void __launch_bounds__(kRsThreads) k_radix_upsweep(const uint64_t* __restrict__ keys, int64_t n,
                                                               int shift, uint32_t mask,
                                                               uint32_t* __restrict__ hist, int64_t nb) {
+    grid_begin();
     __shared__ uint32_t cnt[kRadix];
     cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -37,6 +38,7 @@ __global__ void __launch_bounds__(kRsThreads) k_radix_downsweep(const uint64_t* 
                                                                 int shift, uint32_t mask,
                                                                 const uint32_t* __restrict__ hist,
                                                                 int64_t nb) {
+    grid_begin();
     __shared__ uint32_t wcnt[kRsWarps][kRadix];
     __shared__ uint32_t gbase[kRadix];
     const int w = threadIdx.x >> 5, l = lane_id();
@@ -101,10 +103,10 @@ harp_status radix_sort_u64(uint64_t** keys, uint64_t** alt, int64_t n, int begin
     for (int shift = begin_bit; shift < end_bit; shift += 8) {
         const int bits = (end_bit - shift) < 8 ? (end_bit - shift) : 8;
         const uint32_t mask = (1u << bits) - 1u;
-        k_radix_upsweep<<<(unsigned)nb, kRsThreads, 0, s>>>(*keys, n, shift, mask, hist, nb);
+        launch(k_radix_upsweep, (unsigned)nb, kRsThreads, 0, s, *keys, n, shift, mask, hist, nb);
         HARP_LAUNCHED();
         HARP_TRY(exclusive_scan_u32_inplace(hist, nb * kRadix, tmp, tmp_len, s));
-        k_radix_downsweep<<<(unsigned)nb, kRsThreads, 0, s>>>(*keys, *alt, n, shift, mask, hist, nb);
+        launch(k_radix_downsweep, (unsigned)nb, kRsThreads, 0, s, *keys, *alt, n, shift, mask, hist, nb);
         HARP_LAUNCHED();
         uint64_t* t = *keys;
         *keys = *alt;

@@ -20,8 +20,8 @@
 // of L remain after L[i], searches each of those keys in N+(L[i]) (row_searches).
 // Warp-local mode: d <= tri_warp_max (<= 32), rows are single words, one warp per anchor.
 // CTA mode: up to tri_cta_max (<= 1024) in three sizes (256 / 512 / 1024), rows in shared memory, one
-// block per anchor; the 4-clique sum is dealt to the block as (word, row) units of the bitmap.  Global-staged mode (up to tri_big_max <= 4096, hubs of very large skewed
-// graphs): the same rows in a per-block scratch that stays in L2 (d^2 / 8 bytes), each row built in
+// block per anchor; the 4-clique sum is dealt to the block as (word, row) units of the bitmap.  Global-staged
+// mode (up to tri_big_max <= 4096, hubs of very large skewed graphs): the same rows in a per-block scratch that stays in L2 (d^2 / 8 bytes), each row built in
 // a per-warp shared buffer and written out once.  Fallback (larger d): per out-arc ordered
 // intersections through global memory with binary-searched membership; 4-cliques by binary search
 // in N+(w).  Membership of y in L is a hash lookup (HARP_PROBE_HASH) or a binary search of the
@@ -53,8 +53,8 @@ constexpr int32_t kNoKey = -1;
 
 // Anchor queues: in ws.q_tri (n entries) warp-mode anchors (2 <= d <= tri_warp_max) from the front
 // and CTA-mode anchors from the back; fallback anchors in ws.q_mid[0, n) and global-staged anchors in
-// ws.q_mid[n, 2n) (q_mid is free until the wedge pass).  Vertices are scanned in descending rank, so high-degree anchors tend to be queued
-// (and taken) first.
+// ws.q_mid[n, 2n) (q_mid is free until the wedge pass).  Vertices are scanned in descending rank, so
+// high-degree anchors tend to be queued (and taken) first.
 //
 // Tier of an anchor of out-degree d: -1 none, 0 warp, 1/2/3 CTA 256/512/1024, 4 global-staged,
 // 5 fallback.  wmax <= 32, cmax <= kCtaMax, bmax <= kBigMax (tri_warp_max / tri_cta_max / tri_big_max).
@@ -70,6 +70,7 @@ __global__ void k_tri_classify(const int32_t* __restrict__ dplus, int64_t n, int
                                int wmax, int cmax, int bmax, int32_t* __restrict__ q, int32_t* __restrict__ q_fb,
                                unsigned long long* __restrict__ cnt, unsigned long long* __restrict__ cnt_fb,
                                unsigned long long* __restrict__ cnt_big) {
+    grid_begin();
     const int l = lane_id();
     for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - l; base < n;
          base += (int64_t)gridDim.x * blockDim.x) {
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(kWarpThreads, 4) k_tri_warp(const int64_t* __r
                                                            const int32_t* __restrict__ q,
                                                            const unsigned long long* __restrict__ cnt,
                                                            bool reuse, uint32_t* __restrict__ te, Sink sink) {
+    grid_begin();
     __shared__ int32_t sL[kWarpsPerBlock][32];
     __shared__ uint32_t sRow[kWarpsPerBlock][32];  // row i: bit j (j > i) iff L[j] in N+(L[i])
     __shared__ uint32_t sCol[kWarpsPerBlock][32];  // its transpose
@@ -762,6 +764,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tri_cta(const int64_t* __rest
                                                      const int64_t* __restrict__ ginfo,
                                                      const uint32_t* __restrict__ region,
                                                      uint32_t* __restrict__ te, Sink sink) {
+    grid_begin();
     using S = CtaSmem<DMAX>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S& s = *reinterpret_cast<S*>(smem_raw);
@@ -892,6 +895,7 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_tri_big(const int64_t* __res
                                                             unsigned long long* __restrict__ ticket, bool reuse,
                                                             uint32_t* __restrict__ scratch,
                                                             uint32_t* __restrict__ te, Sink sink) {
+    grid_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BigSmem& s = *reinterpret_cast<BigSmem*>(smem_raw);
     __shared__ int64_t s_item;
@@ -1044,6 +1048,7 @@ __global__ void __launch_bounds__(256) k_tri_fallback(const int64_t* __restrict_
                                                       const unsigned long long* __restrict__ cnt_fb,
                                                       int32_t* __restrict__ scratch, int64_t scratch_per_warp,
                                                       uint32_t* __restrict__ te, Sink sink) {
+    grid_begin();
     __shared__ uint64_t red[32];
     const int w = threadIdx.x >> 5, l = lane_id();
     const int nw = blockDim.x >> 5;
@@ -1148,6 +1153,7 @@ __global__ void __launch_bounds__(kOrbWarps * 32) k_orb_tri_warp(const int64_t* 
                                                                  const uint32_t* __restrict__ te,
                                                                  const int32_t* __restrict__ q,
                                                                  const unsigned long long* __restrict__ cnt, OrbTri o) {
+    grid_begin();
     __shared__ int32_t s_L[kOrbWarps][32], s_pos[kOrbWarps][32 * 31 / 2];
     __shared__ uint32_t s_row[kOrbWarps][32], s_k[kOrbWarps][32], s_t[kOrbWarps][32], s_d[kOrbWarps][32];
     __shared__ uint32_t s_lo[kOrbWarps][32], s_hi[kOrbWarps][32], s_lo2[kOrbWarps][32], s_hi2[kOrbWarps][32];
@@ -1268,6 +1274,7 @@ __global__ void __launch_bounds__(THREADS) k_orb_tri_cta(const int64_t* __restri
                                                          const int32_t* __restrict__ q, int64_t n, int cls,
                                                          const unsigned long long* __restrict__ cnt,
                                                          unsigned long long* __restrict__ ticket, OrbTri o) {
+    grid_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     OrbSmem<DMAX>& s = *reinterpret_cast<OrbSmem<DMAX>*>(smem_raw);
     __shared__ int64_t s_item;
@@ -1370,17 +1377,17 @@ harp_status launch_orb_cta(const harp_csr* g, Workspace& ws, int cls, int ticket
                            cudaStream_t s) {
     const size_t smem = sizeof(OrbSmem<DMAX>);
     HARP_CK(cudaFuncSetAttribute(k_orb_tri_cta<DMAX, THREADS, EDGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_orb_tri_cta<DMAX, THREADS, EDGE><<<num_sms() * per_sm, THREADS, smem, s>>>(
-        ws.offp, ws.colsp, ws.deg, ws.te, ws.q_tri, g->n, cls, (const unsigned long long*)&ws.acc[Q_TRI_WARP],
-        (unsigned long long*)&ws.acc[ticket_slot], o);
+    launch(k_orb_tri_cta<DMAX, THREADS, EDGE>, num_sms() * per_sm, THREADS, smem, s, ws.offp, ws.colsp, ws.deg, ws.te,
+           ws.q_tri, g->n, cls, (const unsigned long long*)&ws.acc[Q_TRI_WARP],
+           (unsigned long long*)&ws.acc[ticket_slot], o);
     HARP_LAUNCHED();
     return HARP_OK;
 }
 
 template <bool EDGE>
 harp_status orbit_tiers(const harp_csr* g, Workspace& ws, const OrbTri& o, int64_t dmax, cudaStream_t s) {
-    k_orb_tri_warp<EDGE><<<num_sms() * 8, kOrbWarps * 32, 0, s>>>(ws.offp, ws.colsp, ws.deg, ws.te, ws.q_tri,
-                                                                  (const unsigned long long*)&ws.acc[Q_TRI_WARP], o);
+    launch(k_orb_tri_warp<EDGE>, num_sms() * 8, kOrbWarps * 32, 0, s, ws.offp, ws.colsp, ws.deg, ws.te, ws.q_tri,
+           (const unsigned long long*)&ws.acc[Q_TRI_WARP], o);
     HARP_LAUNCHED();
     if (dmax > 32) HARP_TRY((launch_orb_cta<kCta1, 256, EDGE>(g, ws, 1, T_TRI_S, 5, o, s)));
     if (dmax > kCta1) HARP_TRY((launch_orb_cta<kCta2, 256, EDGE>(g, ws, 2, T_TRI_M, 3, o, s)));
@@ -1394,10 +1401,11 @@ harp_status launch_cta(const harp_csr* g, Workspace& ws, int cls, int ticket_slo
     const size_t smem = sizeof(CtaSmem<DMAX>);
     HARP_CK(cudaFuncSetAttribute(k_tri_cta<DMAX, THREADS, MINB, BS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
-    k_tri_cta<DMAX, THREADS, MINB, BS><<<num_sms() * MINB, THREADS, smem, s>>>(
-        ws.offp, ws.colsp, ws.deg, ws.q_tri, g->n, cls, wmax, cmax, bmax, reuse,
-        (const unsigned long long*)&ws.acc[Q_TRI_WARP], (unsigned long long*)&ws.acc[ticket_slot], ws.ginfo,
-        ws.core && reuse ? reinterpret_cast<const uint32_t*>(ws.rev) : nullptr, ws.te, Sink{ws.acc, ws.gid, ws.accG});
+    launch(k_tri_cta<DMAX, THREADS, MINB, BS>, num_sms() * MINB, THREADS, smem, s, ws.offp, ws.colsp, ws.deg, ws.q_tri,
+           g->n, cls, wmax, cmax, bmax, reuse, (const unsigned long long*)&ws.acc[Q_TRI_WARP],
+           (unsigned long long*)&ws.acc[ticket_slot], ws.ginfo,
+           ws.core && reuse ? reinterpret_cast<const uint32_t*>(ws.rev) : nullptr, ws.te, Sink{ws.acc, ws.gid,
+           ws.accG});
     HARP_LAUNCHED();
     return HARP_OK;
 }
@@ -1410,8 +1418,10 @@ harp_status launch_tiers(const harp_csr* g, Workspace& ws, int wmax, int cmax, i
     const bool bs2 = probe_bin[2] == HARP_PROBE_BSEARCH, bs3 = probe_bin[3] == HARP_PROBE_BSEARCH;
     const unsigned wgrid = (unsigned)num_sms() * 4;
     const unsigned long long* qcnt = (const unsigned long long*)&ws.acc[Q_TRI_WARP];
-    if (bs0) k_tri_warp<true><<<wgrid, kWarpThreads, 0, s>>>(ws.offp, ws.colsp, ws.deg, ws.q_tri, qcnt, reuse, ws.te, sink);
-    else k_tri_warp<false><<<wgrid, kWarpThreads, 0, s>>>(ws.offp, ws.colsp, ws.deg, ws.q_tri, qcnt, reuse, ws.te, sink);
+    if (bs0) launch(k_tri_warp<true>, wgrid, kWarpThreads, 0, s, ws.offp, ws.colsp, ws.deg, ws.q_tri, qcnt, reuse,
+                    ws.te, sink);
+    else launch(k_tri_warp<false>, wgrid, kWarpThreads, 0, s, ws.offp, ws.colsp, ws.deg, ws.q_tri, qcnt, reuse, ws.te,
+                sink);
     HARP_LAUNCHED();
     HARP_CK(prof_mark(s, SEG_TRI_WARP));
     // tiers that the largest possible out-degree does not reach have no anchors
@@ -1461,8 +1471,8 @@ harp_status count_triangles_k4(const harp_csr* g, Workspace& ws, const harp_plan
     if (blocks > (int64_t)num_sms() * 16) blocks = (int64_t)num_sms() * 16;
     unsigned long long* cnt_fb = (unsigned long long*)&ws.acc[Q_TRI_FB];
     unsigned long long* cnt_big = (unsigned long long*)&ws.acc[Q_TRI_BIG];
-    k_tri_classify<<<(unsigned)blocks, 256, 0, s>>>(ws.dplus, n, ws.own_lo, ws.own_hi, wmax, cmax, bmax, ws.q_tri,
-                                                    ws.q_mid, cnt, cnt_fb, cnt_big);
+    launch(k_tri_classify, (unsigned)blocks, 256, 0, s, ws.dplus, n, ws.own_lo, ws.own_hi, wmax, cmax, bmax, ws.q_tri,
+           ws.q_mid, cnt, cnt_fb, cnt_big);
     HARP_LAUNCHED();
     const Sink sink{ws.acc, ws.gid, ws.accG};
     const int64_t dmax = max_out_degree(g);
@@ -1475,9 +1485,8 @@ harp_status count_triangles_k4(const harp_csr* g, Workspace& ws, const harp_plan
         const size_t smem = sizeof(BigSmem);
         cudaError_t e = cudaFuncSetAttribute(k_tri_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess) {
-            k_tri_big<<<num_sms(), kBigThreads, smem, s>>>(ws.offp, ws.colsp, ws.deg, ws.q_mid + n, cnt_big,
-                                                      (unsigned long long*)&ws.acc[T_TRI_BIG], reuse, scratch, ws.te,
-                                                      sink);
+            launch(k_tri_big, num_sms(), kBigThreads, smem, s, ws.offp, ws.colsp, ws.deg, ws.q_mid + n, cnt_big,
+                   (unsigned long long*)&ws.acc[T_TRI_BIG], reuse, scratch, ws.te, sink);
             note_launch();
             e = cudaGetLastError();
         }
@@ -1494,8 +1503,8 @@ harp_status count_triangles_k4(const harp_csr* g, Workspace& ws, const harp_plan
         const size_t bytes = (size_t)fb_blocks * 8 * (size_t)per_warp * sizeof(int32_t);
         int32_t* scratch = nullptr;
         HARP_CK(cudaMallocAsync((void**)&scratch, bytes, s));
-        k_tri_fallback<<<fb_blocks, 256, 0, s>>>(ws.offp, ws.colsp, ws.deg, ws.q_mid, cnt_fb, scratch, per_warp,
-                                                 ws.te, sink);
+        launch(k_tri_fallback, fb_blocks, 256, 0, s, ws.offp, ws.colsp, ws.deg, ws.q_mid, cnt_fb, scratch, per_warp,
+               ws.te, sink);
         note_launch();
         cudaError_t e = cudaGetLastError();
         cudaFreeAsync(scratch, s);
