@@ -144,14 +144,12 @@ harp_status batch_release(harp_batch* b) {
 }
 
 // Enqueue the whole batched count on stream s (also used while capturing).
-harp_status enqueue_batch(harp_batch* b, const harp_plan& plan, cudaStream_t s) {
+harp_status enqueue_batch(harp_batch* b, const harp_plan& plan, Fork* fork, cudaStream_t s) {
     Workspace& ws = b->u.ws;
     HARP_CK(cudaMemsetAsync(ws.acc, 0, sizeof(uint64_t) * kOutLen, s));
     HARP_CK(cudaMemsetAsync(b->d_accG, 0, sizeof(uint64_t) * kGStride * (size_t)b->G, s));
     HARP_TRY(orient(&b->u, ws, s));
-    HARP_TRY(wedge_geometry(&b->u, ws, plan, s));
-    HARP_TRY(count_triangles_k4(&b->u, ws, plan, s));
-    HARP_TRY(count_wedge_c4(&b->u, ws, plan, s));
+    HARP_TRY(count_passes(&b->u, ws, plan, fork, s));
     HARP_TRY(reduce_and_close_batch(&b->u, ws, b->G, b->d_out, s));
     HARP_CK(cudaMemcpyAsync(b->h_out, b->d_out, sizeof(uint64_t) * 16 * (size_t)b->G, cudaMemcpyDeviceToHost, s));
     HARP_CK(cudaMemcpyAsync(b->h_out + 16 * b->G, ws.acc + ACC_ERR, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
@@ -271,8 +269,9 @@ harp_status batch_prepare(harp_batch* b, const harp_plan& plan) {
         HARP_CK(cudaStreamSynchronize(b->capture_stream));
         cudaGraph_t graph = nullptr;
         const int64_t l0 = harp_launch_count();
+        Fork* fork = thread_fork();  // branches of the graph
         HARP_CK(cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeRelaxed));
-        harp_status st = enqueue_batch(b, plan, b->capture_stream);
+        harp_status st = enqueue_batch(b, plan, fork, b->capture_stream);
         cudaError_t e = cudaStreamEndCapture(b->capture_stream, &graph);
         if (st != HARP_OK) {
             if (graph) cudaGraphDestroy(graph);
@@ -315,7 +314,7 @@ harp_status harp_batch_count(harp_batch* b, const harp_plan* user_plan, uint64_t
         HARP_CK(cudaStreamSynchronize(s));
     } else {
         HARP_CK(cudaStreamSynchronize(b->capture_stream));
-        HARP_TRY(enqueue_batch(b, plan, s));
+        HARP_TRY(enqueue_batch(b, plan, nullptr, s));
         HARP_CK(cudaStreamSynchronize(s));
     }
     if (b->h_out[16 * b->G]) return HARP_EDEVICE;  // a kernel's self-check skipped an out-of-range access

@@ -1294,17 +1294,24 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     } else {
         HARP_TRY(segment_lengths(g, ws, vinfo, ws.ginfo, s));
     }
-    launch(k_c4_classify<WORDS>, grid_cap(n, 256, (int64_t)sms * 32), 256, 0, s, // a lane per root
-        loff, ws.deg, ws.dplus, ws.rev, ws.gid, ws.ginfo, n, ws.own_lo, ws.own_hi, warp_max, mid_max, ws.q_mid, ws.q_win,
-        wcount, ws.acc);
+    launch(k_c4_classify<WORDS>, grid_cap(n, 256, (int64_t)sms * 32), 256, 0, s, loff, ws.deg, ws.dplus, ws.rev, ws.gid,
+           ws.ginfo, n, ws.own_lo, ws.own_hi, warp_max, mid_max, ws.q_mid, ws.q_win, wcount, ws.acc);  // a lane per root
     HARP_LAUNCHED();
+    // the three tiers read the same arrays and meet only in the accumulators
+    cudaStream_t s_light = s, s_mid = s;
+    if (ws.fork) {
+        HARP_TRY(ws.fork->go(1, s));
+        HARP_TRY(ws.fork->go(2, s));
+        s_light = ws.fork->side[1];
+        s_mid = ws.fork->side[2];
+    }
     // one word per hash slot where every graph's ranks fit beside the count
     const bool packed_light = most_n < ((int64_t)1 << (32 - kLightBits)) - 1;
     const bool packed_mid = most_n < ((int64_t)1 << (32 - kMidBits)) - 1;
     const size_t light_smem = (size_t)kSmallWarps * kSmallSlots * (packed_light ? 4 : 8);
     auto light = packed_light ? k_c4_light<true> : k_c4_light<false>;
     HARP_CK(cudaFuncSetAttribute(light, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)light_smem));
-    launch(light, sms * (packed_light ? 5 : 3), kSmallThreads, light_smem, s, ws.off, ws.cols, loff, lcols, ws.deg,
+    launch(light, sms * (packed_light ? 5 : 3), kSmallThreads, light_smem, s_light, ws.off, ws.cols, loff, lcols, ws.deg,
            ws.dplus, ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc, sink);
     HARP_LAUNCHED();
     HARP_CK(prof_mark(s, SEG_C4_SMALL));
@@ -1312,7 +1319,7 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
         const size_t mid_smem = (size_t)kMidSlots * (packed_mid ? 4 : 8);
         auto mid = packed_mid ? k_c4_mid<true> : k_c4_mid<false>;
         HARP_CK(cudaFuncSetAttribute(mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem));
-        launch(mid, sms * (packed_mid ? 12 : 6), kMidThreads, mid_smem, s, ws.off, ws.cols, loff, lcols, ws.deg,
+        launch(mid, sms * (packed_mid ? 12 : 6), kMidThreads, mid_smem, s_mid, ws.off, ws.cols, loff, lcols, ws.deg,
                ws.dplus, ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc, sink);
         HARP_LAUNCHED();
     }
@@ -1329,6 +1336,10 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     launch(k_c4_window<MINB>, sms * MINB, win_threads(MINB), win_smem, s, ws.off, ws.cols, loff, lcols, ws.deg,
            ws.dplus, ws.fpos, ws.rev, ws.bpos, ws.gid, ws.ginfo, ws.q_win, ws.win_prefix, n, ws.acc, sink);
     HARP_LAUNCHED();
+    if (ws.fork) {
+        HARP_TRY(ws.fork->back(1, s));
+        HARP_TRY(ws.fork->back(2, s));
+    }
     HARP_CK(prof_mark(s, SEG_C4_WINDOW));
     return HARP_OK;
 }

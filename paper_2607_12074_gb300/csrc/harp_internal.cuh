@@ -182,6 +182,18 @@ enum : int { G_T = 0, G_K4, G_C4, G_S, G_PW, G_PAWSUM, G_D };
 // ---------------------------------------------------------------------------------------------
 // Workspace for one counting pass, sized for (n, m) and cached in the graph handle.
 // ---------------------------------------------------------------------------------------------
+// Streams and events of the calling thread for work that can go beside a count's own stream, where the thread waits for
+// the count before it returns, or captures it.  Made at the thread's first use on a device, given back at its end.  go(k, s): side k starts after what s holds; back(k, s): s goes on
+// after what side k holds.
+struct Fork {
+    static constexpr int kSides = 3;
+    cudaStream_t side[kSides] = {};
+    cudaEvent_t start = nullptr, done[kSides] = {};
+    harp_status go(int k, cudaStream_t s);
+    harp_status back(int k, cudaStream_t s);
+};
+Fork* thread_fork();  // nullptr while profiling and where they cannot be made
+
 struct Workspace {
     void* base = nullptr;
     size_t bytes = 0;
@@ -211,6 +223,7 @@ struct Workspace {
     size_t scan_tmp_len = 0;
     uint64_t* acc = nullptr;       // [kOutLen]
     bool core = false;             // wedge_geometry built core bitmaps (in rev and bpos)
+    Fork* fork = nullptr;          // count_passes: the streams its independent kernels go to
     // batch mode only (the union of many graphs); nullptr for a single graph
     int64_t G = 1;                    // graphs
     int64_t max_member_m = 0;         // most edges and vertices of one graph
@@ -303,6 +316,10 @@ harp_status wedge_positions(const harp_csr* g, Workspace& ws, cudaStream_t s);
 // c4.cu: the grid of the wedge windows and the graphs' cores (ginfo), and the cores' row bitmaps where one can
 // apply (ws.core); before the triangle pass, which reads the bitmaps, and the wedge pass
 harp_status wedge_geometry(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s);
+
+// api.cu: wedge_geometry, count_triangles_k4 and count_wedge_c4, side by side on fork's streams where the passes use
+// different parts of the workspace (fork may be nullptr)
+harp_status count_passes(const harp_csr* g, Workspace& ws, const harp_plan& plan, Fork* fork, cudaStream_t s);
 
 // c4.cu: wedge anchor, non-induced 4-cycles (step a5), after wedge_geometry
 harp_status count_wedge_c4(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s);
