@@ -5,8 +5,9 @@
 // are skipped; out-of-range ids are skipped and raise a flag that turns into HARP_EINVAL.  Rows are then sorted by
 // the tiers of rowsort.cuh, equal neighbours dropped while they are written, and, where any were, the rows
 // closed up.  The rows' order makes the result independent of the order in which slots were taken.
-// (A radix sort of all arcs as 64-bit keys moved every arc 2 * bits(n) / 8 times: R-MAT scale 18, 4.1 M pairs:
-// 0.66 ms of kernels against 0.22.)
+// (A radix sort of all arcs as 64-bit keys moved every arc 2 * bits(n) / 8 times.)  Kernels of a build, with the sort and
+// now: R-MAT scale 20 2.8 and 1.6 ms, Chung-Lu of 1,347,423 vertices (hubs of close ids) 2.2 and 1.4 ms, random
+// geometric of 1,000,003 vertices 1.24 and 0.30 ms.
 #include "harp_internal.cuh"
 #include "rowsort.cuh"
 
@@ -15,6 +16,9 @@ namespace {
 
 // Words of the build's summary, read back by the host.
 enum : int { B_BAD = 0, B_MAXDEG, B_ARCS, B_RAW, B_Q_WARP, B_Q_BLOCK, B_Q_HUB, B_WORDS = 8 };
+
+// Fewer vertices keep their counters by id: the copy back costs a launch and there is little to contend for.
+constexpr int64_t kSpreadMinN = 1 << 14;
 
 // An input pair's endpoints; valid: in range and not a self-loop.
 struct Pair {
@@ -35,8 +39,24 @@ __device__ __forceinline__ Pair load_pair(const int32_t* __restrict__ src, const
     return p;
 }
 
+// Where a vertex's counter lies: ids 32 apart are neighbours, so that hubs of close ids (weights or arrival times that
+// fall with the id) are counted in different L2 slices; stride 0: by id.  Chung-Lu of 1,347,423 vertices: degrees 1.07
+// -> 0.36 ms, scatter 1.14 -> 0.48 ms.
+struct Spread {
+    int64_t stride;
+    __device__ __forceinline__ int64_t at(int64_t v) const { return stride ? (v & 31) * stride + (v >> 5) : v; }
+};
+
+// the counters by id
+__global__ void __launch_bounds__(256) k_build_gather(const int32_t* __restrict__ deg, Spread at, int64_t n,
+                                                      int32_t* __restrict__ by_id) {
+    grid_begin();
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+        by_id[v] = deg[at.at(v)];
+}
+
 __global__ void __launch_bounds__(256) k_build_degrees(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                                                       int64_t m_in, int64_t n, int32_t* __restrict__ deg,
+                                                       int64_t m_in, int64_t n, Spread at, int32_t* __restrict__ deg,
                                                        unsigned long long* __restrict__ summary) {
     grid_begin();
     const int l = lane_id();
@@ -48,7 +68,7 @@ __global__ void __launch_bounds__(256) k_build_degrees(const int32_t* __restrict
         for (int h = 0; h < 2; ++h) {
             const int32_t x = p.valid ? (h ? p.v : p.u) : -1 - l;
             const uint32_t same = __match_any_sync(kFull, x);
-            if (p.valid && l == __ffs(same) - 1) atomicAdd(&deg[x], __popc(same));
+            if (p.valid && l == __ffs(same) - 1) atomicAdd(&deg[at.at(x)], __popc(same));
         }
     }
     if (__any_sync(kFull, bad) && l == 0) atomicOr(&summary[B_BAD], 1ull);
@@ -57,7 +77,7 @@ __global__ void __launch_bounds__(256) k_build_degrees(const int32_t* __restrict
 // deg counts down to zero: each pair's slot is the value before.
 __global__ void __launch_bounds__(256) k_build_scatter(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
                                                        int64_t m_in, int64_t n, const int64_t* __restrict__ roff,
-                                                       int32_t* __restrict__ deg, int32_t* __restrict__ out) {
+                                                       Spread at, int32_t* __restrict__ deg, int32_t* __restrict__ out) {
     grid_begin();
     const int l = lane_id();
     bool bad = false;
@@ -70,7 +90,7 @@ __global__ void __launch_bounds__(256) k_build_scatter(const int32_t* __restrict
             const uint32_t same = __match_any_sync(kFull, x);
             const int leader = __ffs(same) - 1;
             int left = 0;
-            if (p.valid && l == leader) left = atomicSub(&deg[x], __popc(same));
+            if (p.valid && l == leader) left = atomicSub(&deg[at.at(x)], __popc(same));
             left = __shfl_sync(kFull, left, leader);
             if (p.valid) out[roff[x] + left - 1 - __popc(same & lanemask_lt())] = y;
         }
@@ -314,39 +334,50 @@ __global__ void __launch_bounds__(256) k_build_summary(const int32_t* __restrict
     }
 }
 
-// Closes up the rows: cols[off[i] + k] = in[roff[i] + k], 32 consecutive rows per warp (a lane copies a short row).
+// Rows closed up: a warp per `run` consecutive columns of the result.  The row of the first is searched (32 probes a
+// round), then the lanes hold the bounds of 32 rows and each column looks its row up among them.  (A warp per 32 rows
+// copied a graph's hubs by itself where their ids are close: Chung-Lu of 1,347,423 vertices, 2.0 ms of the build.)
 __global__ void __launch_bounds__(256) k_build_compact(const int64_t* __restrict__ roff, const int64_t* __restrict__ off,
-                                                       int64_t n, const int32_t* __restrict__ in,
+                                                       int64_t n, const int32_t* __restrict__ in, int run,
                                                        int32_t* __restrict__ cols) {
     grid_begin();
     const int l = lane_id();
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; i0 < n; i0 += nw * 32) {
-        const int64_t i = i0 + l;
-        const int64_t s = i < n ? roff[i] : 0, o = i < n ? off[i] : 0;
-        const int d = i < n ? (int)(off[i + 1] - o) : 0;
-        if (d <= 16) {  // all loads first
-            int32_t x[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) x[k] = k < d ? in[s + k] : 0;
-#pragma unroll
-            for (int k = 0; k < 16; ++k)
-                if (k < d) cols[o + k] = x[k];
+    const int64_t M = off[n], nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t t0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * run; t0 < M; t0 += nw * run) {
+        const int64_t t1 = t0 + run < M ? t0 + run : M;
+        int64_t r0 = 0, hi = n;  // the last row that begins at or before t0: off[r0] <= t0 < off[hi]
+        while (hi - r0 > 1) {
+            const int64_t step = (hi - r0 + 31) >> 5, p = r0 + (int64_t)(l + 1) * step;
+            const uint32_t m = __ballot_sync(kFull, p >= hi || off[p] > t0);
+            r0 += (int64_t)(__ffs(m) - 1) * step;
+            hi = r0 + step < hi ? r0 + step : hi;
         }
-        uint32_t rest = __ballot_sync(kFull, d > 16);
-        while (rest) {
-            const int src = __ffs(rest) - 1;
-            rest &= rest - 1;
-            const int64_t rs = __shfl_sync(kFull, s, src), ro = __shfl_sync(kFull, o, src);
-            const int rd = __shfl_sync(kFull, d, src);
-            for (int k = l; k < rd; k += 128) {
+        for (int64_t cur = t0; cur < t1; r0 += 32) {
+            const int64_t r = r0 + l < n ? r0 + l : n;
+            const int64_t o = off[r];
+            const int64_t next = off[r0 + 32 < n ? r0 + 32 : n];
+            if (next <= cur) continue;  // these rows are empty
+            const int64_t shift = roff[r] - o;
+            const int64_t end = next < t1 ? next : t1;
+            for (int64_t b = cur; b < end; b += 128) {  // four loads in flight
                 int32_t x[4];
 #pragma unroll
-                for (int t = 0; t < 4; ++t) x[t] = k + 32 * t < rd ? in[rs + k + 32 * t] : 0;
+                for (int h = 0; h < 4; ++h) {
+                    const int64_t t = b + 32 * h + l;
+                    int k = 0;  // last row with o <= t
 #pragma unroll
-                for (int t = 0; t < 4; ++t)
-                    if (k + 32 * t < rd) cols[ro + k + 32 * t] = x[t];
+                    for (int sft = 16; sft >= 1; sft >>= 1) {
+                        const int64_t v = __shfl_sync(kFull, o, k + sft);
+                        if (v <= t) k += sft;
+                    }
+                    const int64_t at = t + __shfl_sync(kFull, shift, k);
+                    x[h] = t < end ? in[at] : 0;
+                }
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    if (b + 32 * h + l < end) cols[b + 32 * h + l] = x[h];
             }
+            cur = end;
         }
     }
 }
@@ -403,7 +434,7 @@ harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t
         return HARP_OK;
     }
     const size_t tmp_len = scan_tmp_needed(nn) + 64;
-    const size_t head = align256(B_WORDS * sizeof(unsigned long long)), per_n = align256((size_t)nn * sizeof(int32_t));
+    const size_t head = align256(B_WORDS * sizeof(unsigned long long)), per_n = align256((size_t)(nn + 32) * sizeof(int32_t));
     const size_t offs = align256((size_t)(nn + 1) * sizeof(int64_t));
     BCK(cudaMallocAsync((void**)&slab, head + 4 * per_n + offs + tmp_len * sizeof(int64_t), s));
     unsigned long long* summary = reinterpret_cast<unsigned long long*>(slab);
@@ -416,10 +447,15 @@ harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t
     BCK(cudaMallocAsync((void**)&raw, 2 * (size_t)m_in * sizeof(int32_t), s));
     BCK(cudaMallocAsync((void**)&sorted, 2 * (size_t)m_in * sizeof(int32_t), s));
     BCK(cudaMemsetAsync(slab, 0, head + per_n, s));  // summary and degrees
-    launch(k_build_degrees, grid_for(m_in, 256), 256, 0, s, d_src, d_dst, m_in, n, deg, summary);
+    const Spread at{n >= kSpreadMinN ? (n + 31) >> 5 : 0};
+    launch(k_build_degrees, grid_for(m_in, 256), 256, 0, s, d_src, d_dst, m_in, n, at, deg, summary);
     BLAUNCHED();
-    BTRY(exclusive_scan_i32_to_i64(deg, roff, n, tmp, tmp_len, s));
-    launch(k_build_scatter, grid_for(m_in, 256), 256, 0, s, d_src, d_dst, m_in, n, roff, deg, raw);
+    if (at.stride) {
+        launch(k_build_gather, grid_for(n, 256), 256, 0, s, deg, at, n, ndeg);
+        BLAUNCHED();
+    }
+    BTRY(exclusive_scan_i32_to_i64(at.stride ? ndeg : deg, roff, n, tmp, tmp_len, s));
+    launch(k_build_scatter, grid_for(m_in, 256), 256, 0, s, d_src, d_dst, m_in, n, roff, at, deg, raw);
     BLAUNCHED();
     launch(k_build_rows_small, grid_for(n, 256), 256, 0, s, roff, n, raw, sorted, ndeg, q, q_block, summary);
     BLAUNCHED();
@@ -459,7 +495,8 @@ harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t
     } else {
         BCK(cudaMallocAsync((void**)&g->cols, (size_t)(M > 0 ? M : 1) * sizeof(int32_t), s));
         if (M > 0) {
-            launch(k_build_compact, grid_for(n, 256), 256, 0, s, roff, g->off, n, sorted, g->cols);
+            const int run = M >= (1 << 20) ? 1024 : (M >= (1 << 17) ? 256 : 32);  // small: enough warps
+            launch(k_build_compact, grid_for((M + run - 1) / run * 32, 256), 256, 0, s, roff, g->off, n, sorted, run, g->cols);
             BLAUNCHED();
         }
         BCK(cudaStreamSynchronize(s));
