@@ -24,8 +24,10 @@
 //
 // Work per root W(u) = sum_{w in N-(u)} (pos_w(u) - fpos[w]) picks the execution mode:
 //   W <= warp_max   one warp, hash table of 1024 slots in shared memory (warp-local mode)
-//   W <= mid_max    one warp, hash table of 4096 slots (the middle tier: roots with few wedges spread
-//                   over many windows would otherwise cost a whole window pass per window)
+//   W <= mid_max    a block of four warps, hash table of 4096 slots (the middle tier: roots with few wedges
+//                   spread over many windows would otherwise cost a whole window pass per window)
+//   W <= 16384      the wide tier, where two or more windows lie below the root: hash tables of 16384 and 32768
+//                   slots
 //   larger          one block per (root, grid window): dense packed counters in shared memory
 //                   (CTA mode); lower neighbours are handed to warps in groups of 32, heaviest first,
 //                   and segments of 2048+ elements are split across all warps of the block.  The
@@ -56,6 +58,11 @@ constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallSlots = 1024;            // per-warp hash table of the light roots (W <= 512)
 constexpr int kMidSlots = 4096;              // hash table of the middle tier (W <= 2048)
 constexpr int kMidWarps = 4;                 // warps of the block that takes a middle root
+constexpr int kWideSlots = 16384;            // hash tables of the wide tier: W <= 8192,
+constexpr int kWideWarps = 16;
+constexpr int kWide2Slots = 32768;           // and W <= 16384
+constexpr int kWide2Warps = 32;
+constexpr int kWideBits = 10;                // its counts: at most 1,024 lower neighbours
 constexpr int kLong = 32;                    // segments this long are read warp-coalesced
 constexpr int kSplit = 2048;                 // segments this long are split across the block
 constexpr int kSplitQ = 128;                 // split-queue capacity per window item
@@ -642,6 +649,7 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
                                                      const int32_t* __restrict__ gid,
                                                      const int64_t* __restrict__ ginfo, int64_t n, int64_t own_lo,
                                                      int64_t own_hi, uint32_t warp_max, uint32_t mid_max,
+                                                     uint32_t wide_max,
                                                      int32_t* __restrict__ q_small, int32_t* __restrict__ q_win,
                                                      int32_t* __restrict__ wcount, uint64_t* __restrict__ acc) {
     grid_begin();
@@ -651,6 +659,7 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
     unsigned long long* qcnt_small = (unsigned long long*)&acc[Q_C4_MID];
     unsigned long long* qcnt_mid = (unsigned long long*)&acc[Q_C4_MIDW];
     unsigned long long* qcnt_win = (unsigned long long*)&acc[Q_C4_WIN];
+    unsigned long long* qcnt_wide = (unsigned long long*)&acc[Q_C4_WIDE];
     // a warp takes 32 ranks, one root per lane, spaced by the number of warps (so the hubs at the top
     // ranks fall to different warps): a lane sums W(u) itself when u has at most 32 lower neighbours,
     // the warp sums the larger roots together; queue slots are taken in lane order (descending rank).
@@ -678,14 +687,19 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
             bw = warp_sum(bw);
             if (l == src) W = bw;
         }
-        const int cls = W == 0 ? -1 : (W <= warp_max ? 0 : (W <= mid_max ? 1 : 2));
+        int cls = W == 0 ? -1 : (W <= warp_max ? 0 : (W <= mid_max ? 1 : 2));
+        int64_t windows = 0;
+        if (cls == 2) {
+            windows = windows_below<WORDS>(ginfo + (gid ? (int64_t)gid[u] : 0) * kGInfo, u);
+            if (W <= wide_max && windows >= 2 && dm <= (1 << kWideBits)) cls = 3;
+        }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int c = 0; c < 4; ++c) {
             const uint32_t mask = __ballot_sync(kFull, cls == c);
             if (!mask) continue;
             unsigned long long base = 0;
             const int leader = __ffs(mask) - 1;
-            unsigned long long* ctr = c == 0 ? qcnt_small : (c == 1 ? qcnt_mid : qcnt_win);
+            unsigned long long* ctr = c == 0 ? qcnt_small : (c == 1 ? qcnt_mid : (c == 2 ? qcnt_win : qcnt_wide));
             if (l == leader) base = atomicAdd(ctr, (unsigned long long)__popc(mask));
             base = __shfl_sync(kFull, base, leader);
             if (cls == c) {
@@ -696,12 +710,13 @@ __global__ void __launch_bounds__(256) k_c4_classify(const int64_t* __restrict__
                 } else if (c == 1) {  // the middle tier fills the same queue from the back
                     q_small[n - 1 - slot] = u;
                     q_small[2 * n - 1 - slot] = (int32_t)W;
-                } else {
-                    const int64_t* gi = ginfo + (gid ? (int64_t)gid[u] : 0) * kGInfo;
-                    const int64_t windows = windows_below<WORDS>(gi, u);
+                } else if (c == 2) {
                     q_win[slot] = u;
                     wcount[slot] = (int32_t)windows;
                     visits += (uint64_t)(windows * dm);
+                } else {
+                    q_win[n - 1 - slot] = u;
+                    wcount[n - 1 - slot] = (int32_t)W;
                 }
             }
         }
@@ -919,39 +934,52 @@ __global__ void __launch_bounds__(kSmallThreads, PACKED ? 5 : 3) k_c4_light(cons
     if (threadIdx.x == 0 && c4) atomicAdd((unsigned long long*)&acc[ACC_C4], (unsigned long long)c4);
 }
 
-// Middle roots (512 < W <= 2048, the back of q_small): a block of kMidWarps warps each, the lower neighbours dealt
-// to the warps.
+// Middle roots (512 < W <= 2048, the back of q_mid) and wide ones (2048 < W <= 16384, the back of q_win): a block each,
+// the lower neighbours dealt to its warps.  A wide root would else cost a pass over its lower neighbours and a scan of
+// the counters for every window of ranks below it: Chung-Lu of 2,000,000 vertices, 40,000 such roots over up to 40
+// windows, 10.4 ms of window passes against 2.3 ms (its whole count 50.6 -> 42.4 ms); R-MAT scale 20 0.72 and 0.28 ms.
+// One table size of 32,768 slots for both halves took 3.1 ms, blocks of 8 warps for the lower half 1.33 instead of 0.99.
 constexpr int kMidThreads = kMidWarps * 32;
 constexpr int kMidBits = 11;  // counts of at most 2048
 
-template <bool PACKED>
-__global__ void __launch_bounds__(kMidThreads) k_c4_mid(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
+template <int SLOTS, int WARPS, int BITS, bool PACKED>
+__global__ void __launch_bounds__(WARPS * 32) k_c4_mid(const int64_t* __restrict__ off, const int32_t* __restrict__ cols,
                                                         const int64_t* __restrict__ loff,
                                                         const int32_t* __restrict__ lcols,
                                                         const int32_t* __restrict__ deg, const int32_t* __restrict__ dplus,
                                                         const int32_t* __restrict__ fpos, const int32_t* __restrict__ rev,
                                                         const uint4* __restrict__ vinfo, const int64_t* __restrict__ ginfo,
-                                                        const int32_t* __restrict__ q_small, int64_t n,
+                                                        const int32_t* __restrict__ q, int64_t n, uint32_t wlo,
+                                                        uint32_t whi, int qslot, int tslot,
                                                         uint64_t* __restrict__ acc, Sink sink) {
     grid_begin();
-    using Table = HashTable<kMidSlots, kMidBits, PACKED>;
+    using Table = HashTable<SLOTS, BITS, PACKED>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint32_t s_rel[kMidWarps][32];
+    __shared__ uint32_t s_rel[WARPS][32];
     __shared__ uint64_t red[32];
     __shared__ int64_t s_item;
     const int w = threadIdx.x >> 5, l = lane_id();
     Table table;
     table.t = reinterpret_cast<uint32_t*>(smem_raw);
-    const int64_t nq = (int64_t)acc[Q_C4_MIDW];
-    unsigned long long* ticket = (unsigned long long*)&acc[T_C4_MID];
+    const int64_t nq = (int64_t)acc[qslot];
+    unsigned long long* ticket = (unsigned long long*)&acc[tslot];
     GraphSum sum;
-    if (threadIdx.x == 0) s_item = (int64_t)atomicAdd(ticket, 1ull);
+    auto take = [&] {  // the next root with wlo < W <= whi
+        int64_t k;
+        uint32_t W = 0;
+        do {
+            k = (int64_t)atomicAdd(ticket, 1ull);
+            if (k < nq) W = (uint32_t)q[2 * n - 1 - k];
+        } while (k < nq && (W <= wlo || W > whi));
+        s_item = k;
+    };
+    if (threadIdx.x == 0) take();
     __syncthreads();
     for (;;) {
         const int64_t k = s_item;
         if (k >= nq) break;
-        const int32_t u = q_small[n - 1 - k];
-        const uint32_t W = (uint32_t)q_small[2 * n - 1 - k];
+        const int32_t u = q[n - 1 - k];
+        const uint32_t W = (uint32_t)q[2 * n - 1 - k];
         const int64_t dm = (int64_t)deg[u] - dplus[u];
         const int64_t ub = loff[u];
         const int32_t g = sink.batch() ? sink.gid[u] : 0;
@@ -960,12 +988,12 @@ __global__ void __launch_bounds__(kMidThreads) k_c4_mid(const int64_t* __restric
         uint32_t P = 64;
         while (P < 2 * W) P <<= 1;
         table.mask = P - 1;
-        table.clear(threadIdx.x, kMidThreads);
+        table.clear(threadIdx.x, WARPS * 32);
         __syncthreads();  // the table is clear, every thread has read s_item
-        if (threadIdx.x == 0) s_item = (int64_t)atomicAdd(ticket, 1ull);
+        if (threadIdx.x == 0) take();
         uint64_t part = 0;
-        for (int64_t a0 = 0; a0 < dm; a0 += kMidThreads) {
-            const int64_t a = a0 + l * kMidWarps + w;
+        for (int64_t a0 = 0; a0 < dm; a0 += WARPS * 32) {
+            const int64_t a = a0 + l * WARPS + w;
             uint32_t base = 0;
             int len = 0;
             if (a < dm) {
@@ -1277,6 +1305,10 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     const int sms = num_sms();
     const int64_t most_n = ws.G > 1 ? ws.max_member_n : n;  // vertices of the largest graph
     int32_t* wcount = ws.q_win + n;
+    // the wide tier: where a graph can have several windows (fewer vertices than a window has words fit one at any
+    // width but the last) and its ranks fit beside the counts; a middle tier set lower turns it off
+    const bool wide_on = mid_max == kMidSlots / 2 && most_n >= WORDS && most_n < ((int64_t)1 << (32 - kWideBits)) - 1;
+    const uint32_t wide_max = wide_on ? kWide2Slots / 2 : 0;
     if (ws.core) HARP_TRY(count_wedge_core(g, ws, s));  // uses rev, bpos and the queues before they are filled below
     // the roots' lower lists: row prefixes of a whole graph, or their own CSR in a partitioned block
     const bool lists = ws.loff != nullptr;
@@ -1295,7 +1327,8 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
         HARP_TRY(segment_lengths(g, ws, vinfo, ws.ginfo, s));
     }
     launch(k_c4_classify<WORDS>, grid_cap(n, 256, (int64_t)sms * 32), 256, 0, s, loff, ws.deg, ws.dplus, ws.rev, ws.gid,
-           ws.ginfo, n, ws.own_lo, ws.own_hi, warp_max, mid_max, ws.q_mid, ws.q_win, wcount, ws.acc);  // a lane per root
+           ws.ginfo, n, ws.own_lo, ws.own_hi, warp_max, mid_max, wide_max, ws.q_mid, ws.q_win, wcount,
+           ws.acc);  // a lane per root
     HARP_LAUNCHED();
     // the three tiers read the same arrays and meet only in the accumulators
     cudaStream_t s_light = s, s_mid = s;
@@ -1317,10 +1350,26 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     HARP_CK(prof_mark(s, SEG_C4_SMALL));
     if (mid_max > warp_max) {
         const size_t mid_smem = (size_t)kMidSlots * (packed_mid ? 4 : 8);
-        auto mid = packed_mid ? k_c4_mid<true> : k_c4_mid<false>;
+        auto mid = packed_mid ? k_c4_mid<kMidSlots, kMidWarps, kMidBits, true>
+                              : k_c4_mid<kMidSlots, kMidWarps, kMidBits, false>;
         HARP_CK(cudaFuncSetAttribute(mid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem));
         launch(mid, sms * (packed_mid ? 12 : 6), kMidThreads, mid_smem, s_mid, ws.off, ws.cols, loff, lcols, ws.deg,
-               ws.dplus, ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, ws.acc, sink);
+               ws.dplus, ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_mid, n, 0u, (uint32_t)kMidSlots / 2, (int)Q_C4_MIDW,
+               (int)T_C4_MID, ws.acc, sink);
+        HARP_LAUNCHED();
+    }
+    if (wide_on) {
+        auto wide2 = k_c4_mid<kWide2Slots, kWide2Warps, kWideBits, true>;
+        HARP_CK(cudaFuncSetAttribute(wide2, cudaFuncAttributeMaxDynamicSharedMemorySize, kWide2Slots * 4));
+        launch(wide2, sms, kWide2Warps * 32, (size_t)kWide2Slots * 4, s_mid, ws.off, ws.cols, loff, lcols, ws.deg,
+               ws.dplus, ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_win, n, (uint32_t)kWideSlots / 2,
+               (uint32_t)kWide2Slots / 2, (int)Q_C4_WIDE, (int)T_C4_WIDE2, ws.acc, sink);
+        HARP_LAUNCHED();
+        auto wide = k_c4_mid<kWideSlots, kWideWarps, kWideBits, true>;
+        HARP_CK(cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSlots * 4));
+        launch(wide, sms * 3, kWideWarps * 32, (size_t)kWideSlots * 4, s_mid, ws.off, ws.cols, loff, lcols, ws.deg,
+               ws.dplus, ws.fpos, ws.rev, vinfo, ws.ginfo, ws.q_win, n, 0u, (uint32_t)kWideSlots / 2, (int)Q_C4_WIDE,
+               (int)T_C4_WIDE, ws.acc, sink);
         HARP_LAUNCHED();
     }
     HARP_CK(prof_mark(s, SEG_C4_MID));

@@ -127,6 +127,9 @@ enum : int {
     T_CORE_M = 60,         // its tickets
     T_CORE_L = 61,
     T_CORE_XL = 62,
+    Q_C4_WIDE = 69,        // length of the wedge wide tier's queue (from the back of q_win)
+    T_C4_WIDE = 70,        // its tickets: W <= 8192, above
+    T_C4_WIDE2 = 71,
     A_CORE_ANY = 63,       // graphs that have a wedge core
     ACC_LIT_CORR = 64,     // 64 lo, 65 hi: what the staged edge pass counts too much (literal.cu)
     T_LIT_EDGE = 66,       // its ticket
