@@ -9,7 +9,7 @@ reduction and closure, counts copied to the host.  L2 is flushed (256 MiB write)
 `value` = m / (device time per step).  `e2e` = the same metric through the public API from pinned
 host edge lists: harp_build_csr (H2D + device CSR build) + harp_count4 (D2H of the counts) per step.
 `roofline` = the dominant kernel's algorithmic bytes (host work meter) / its CUDA-event time, against
-the measured HBM copy bandwidth (`segment_rooflines`: the same for every segment).  `cpu_baseline` =
+the measured HBM copy bandwidth (`segment_rooflines`: the same for every pass).  `cpu_baseline` =
 the CPU oracle (OpenMP, all host cores) on the bench graph itself.
 
 `batched`: the batched workload (4,096 graphs: ER / BA / RGG, n log-uniform in [50, 20000], mean degree
@@ -616,22 +616,23 @@ def main():
     segment_rooflines = None
     if not args.no_meter:
         meter = workmeter.meter(g.n, g.src, g.dst)
-        # every segment against the HBM roofline: its algorithmic bytes (work meter) over its CUDA-event
-        # time; the windowed wedge kernel's per-window re-reads are listed apart as overhead
+        # every pass against the HBM roofline: its algorithmic bytes (work meter) over its CUDA-event time.
+        # The wedge segments are one pass: the meter deals roots to tiers by their work alone, while the
+        # library counts the roots of the highest ranks in the core pass (timed with the light tier)
+        passes = {k: (k,) for k in SEGMENTS if not k.startswith("c4_")}
+        passes["wedges"] = tuple(k for k in SEGMENTS if k.startswith("c4_"))
+        pass_ms = {p: sum(seg_avg[k] for k in ks) for p, ks in passes.items()}
+        pass_bytes = {p: sum(meter[k]["bytes"] for k in ks if k in meter) for p, ks in passes.items()}
         segment_rooflines = {}
-        for k in SEGMENTS:
-            t_ms = seg_avg[k]
-            alg_k = meter[k]["bytes"] if k in meter else 0
-            if t_ms <= 0 or alg_k <= 0:
+        for p, t_ms in pass_ms.items():
+            if t_ms <= 0 or pass_bytes[p] <= 0:
                 continue
-            ach = alg_k / (t_ms / 1000) / 1e9
-            segment_rooflines[k] = {"ms": t_ms, "algorithmic_bytes": alg_k, "achieved_gbs": ach, "frac": ach / peak}
-            if meter[k].get("overhead_bytes"):
-                segment_rooflines[k]["overhead_bytes"] = meter[k]["overhead_bytes"]
-        kernel_segments = [k for k in SEGMENTS if k != "orient"]
-        dom = max(kernel_segments, key=lambda k: seg_avg[k])
-        alg = meter[dom]["bytes"]
-        achieved = alg / (seg_avg[dom] / 1000) / 1e9
+            ach = pass_bytes[p] / (t_ms / 1000) / 1e9
+            segment_rooflines[p] = {"ms": t_ms, "algorithmic_bytes": pass_bytes[p], "achieved_gbs": ach,
+                                    "frac": ach / peak}
+        dom = max((p for p in passes if p != "orient"), key=lambda p: pass_ms[p])
+        alg = pass_bytes[dom]
+        achieved = alg / (pass_ms[dom] / 1000) / 1e9
         traffic = None
         tfile = os.path.join(ROOT, "profiles", "traffic.json")
         if os.path.exists(tfile):  # DRAM bytes of one ncu capture, valid while the kernel is unchanged
@@ -645,8 +646,7 @@ def main():
                         traffic = rec[dom]
         roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
                     "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
-                    "algorithmic_bytes": alg, "kernel_ms": seg_avg[dom],
-                    "overhead_bytes": meter[dom].get("overhead_bytes", 0)}
+                    "algorithmic_bytes": alg, "kernel_ms": pass_ms[dom]}
     cpu = None
     if not args.no_cpu_baseline:
         # the oracle on the bench graph itself (R-MAT scale 20, the same generator call), all host cores

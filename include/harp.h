@@ -144,9 +144,10 @@ typedef struct harp_plan {
                                  /* staged in an L2-resident global scratch; above: unstaged        */
                                  /* fallback, every extension a miss                                */
     uint32_t c4_warp_max_work;   /* wedge work W(u) <= this: warp-local hash table                 */
-    uint32_t c4_cta_max_work;    /* W(u) <= this (at most 2048): the middle tier, a warp-local hash */
-                                 /* table of 4096 slots; above: windowed counters (<= c4_warp_max_ */
-                                 /* work turns the middle tier off)                                */
+    uint32_t c4_cta_max_work;    /* W(u) <= this (at most 2048): the middle tier, a hash table of  */
+                                 /* 4096 slots per root; above: windowed counters, and at 2048     */
+                                 /* larger tables up to W(u) = 16384 where x spans two windows     */
+                                 /* (<= c4_warp_max_work turns these tiers off)                    */
     uint32_t c4_window_bytes;    /* shared-memory bytes of one dense counter window: 200, 100, 64   */
                                  /* or 48 KiB (the largest that fits); 0 = by graph: 200 KiB for a */
                                  /* single graph of more than 2^22 vertices, else 100 KiB          */
