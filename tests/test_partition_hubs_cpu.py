@@ -12,7 +12,7 @@ H = pytest.importorskip("paper_2607_12074_gb300.harp")
 @pytest.mark.parametrize("first", (0, 30_000))
 @pytest.mark.parametrize("hubs", (1, 40))
 def test_hubs_of_close_ids(hubs, first):
-    n, m = 50_000, 400_000
+    n, m = 50_000, 900_000
     rng = np.random.default_rng(hubs)
     src = rng.integers(first, first + hubs, m).astype(np.int32)  # every edge at a hub, many of them repeated
     dst = rng.integers(0, n, m).astype(np.int32)
