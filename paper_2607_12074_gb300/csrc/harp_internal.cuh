@@ -120,7 +120,7 @@ enum : int {
     ACC_LIT_T = 52,        // triangles enumerated by the literal triangle pass
     ACC_SIG_LOOKUPS = 53,  // literal basis: frontier requests to the signature cache
     Q_C4_MIDW = 54,        // length of the wedge middle tier's queue (from the back of q_mid)
-    Q_CORE_S = 55,         // wedge core pass: queue lengths by degree class, and of the core rows
+    Q_CORE_S = 55,         // wedge core pass: queue lengths by degree class
     Q_CORE_M = 56,
     Q_CORE_L = 57,
     Q_CORE_XL = 58,
