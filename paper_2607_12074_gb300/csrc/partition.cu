@@ -87,8 +87,8 @@ constexpr int64_t kRowChunk = 512;  // rows of a chunk where the work is the row
 template <typename F>
 void parallel_dynamic(int64_t n, int64_t chunk, F&& f);
 template <typename F>
-void parallel_rows(int64_t n, F&& f) {  // inline when n is small
-    if (n < (1 << 16)) f((int64_t)0, n);
+void parallel_rows(int64_t n, int64_t arcs, F&& f) {  // inline when there is little to do (a few rows may be all hubs)
+    if (n + arcs < (1 << 18)) f((int64_t)0, n);
     else parallel_dynamic(n, kRowChunk, f);
 }
 template <typename F>
@@ -772,7 +772,7 @@ harp_status run_triangle_block(const RankGraph& g, const TriBlock& blk, int dev,
     const bool whole = blk.lo == 0 && blk.hi == n;  // every vertex is in the halo
     std::vector<uint8_t> in((size_t)n, (uint8_t)whole);
     if (!whole)
-        parallel_rows(blk.hi - blk.lo, [&](int64_t a, int64_t b) {
+        parallel_rows(blk.hi - blk.lo, 2 * g.m, [&](int64_t a, int64_t b) {
             for (int64_t u = blk.lo + a; u < blk.lo + b; ++u) {
                 __atomic_store_n(&in[(size_t)u], (uint8_t)1, __ATOMIC_RELAXED);
                 for (int64_t k = 0; k < g.dplus[(size_t)u]; ++k)
@@ -783,7 +783,7 @@ harp_status run_triangle_block(const RankGraph& g, const TriBlock& blk, int dev,
     for (int64_t v = 0; v < n; ++v) offp[(size_t)v + 1] = offp[(size_t)v] + (in[(size_t)v] ? g.dplus[(size_t)v] : 0);
     const int64_t outs = offp[(size_t)n];
     buf<int32_t> colsp((size_t)(outs > 0 ? outs : 1));
-    parallel_rows(n, [&](int64_t lo, int64_t hi) {
+    parallel_rows(n, 2 * g.m, [&](int64_t lo, int64_t hi) {
         for (int64_t v = lo; v < hi; ++v) {
             const int64_t len = offp[(size_t)v + 1] - offp[(size_t)v];
             if (len)
@@ -849,7 +849,7 @@ harp_status run_triangle_block(const RankGraph& g, const TriBlock& blk, int dev,
     sum.K4 += acc[ACC_K4];
     sum.PAWSUM += acc[ACC_PAWSUM];
     if (whole) return HARP_OK;
-    parallel_rows(n, [&](int64_t lo, int64_t hi) {  // local out-arcs -> global out-arc ids
+    parallel_rows(n, 2 * g.m, [&](int64_t lo, int64_t hi) {  // local out-arcs -> global out-arc ids
         for (int64_t v = lo; v < hi; ++v) {
             const int64_t lb = offp[(size_t)v], len = offp[(size_t)v + 1] - lb, gb = g.offp[(size_t)v];
             for (int64_t k = 0; k < len; ++k) sum.te[(size_t)(gb + k)] += te_local[(size_t)(lb + k)];
@@ -868,7 +868,7 @@ harp_status run_wedge_block(const RankGraph& g, const WedgeBlock& blk, int dev, 
     const int64_t la = loff[(size_t)n];
     buf<int32_t> lcols((size_t)(la > 0 ? la : 1));
     std::vector<uint8_t> in((size_t)n, 0);
-    parallel_rows(blk.hi - blk.lo, [&](int64_t a0, int64_t b0) {
+    parallel_rows(blk.hi - blk.lo, 2 * g.m, [&](int64_t a0, int64_t b0) {
         for (int64_t u = blk.lo + a0; u < blk.lo + b0; ++u) {
             const int64_t len = loff[(size_t)u + 1] - loff[(size_t)u];
             for (int64_t a = 0; a < len; ++a) {
@@ -882,7 +882,7 @@ harp_status run_wedge_block(const RankGraph& g, const WedgeBlock& blk, int dev, 
     // rows of the lower neighbours, restricted to the slice [xa, xb) of opposite vertices
     const int64_t xa = std::max<int64_t>(blk.xlo, g.n1), xb = std::min<int64_t>(blk.xhi, blk.hi);
     std::vector<int64_t> off((size_t)n + 1, 0), rb((size_t)n, 0);
-    parallel_rows(n, [&](int64_t lo, int64_t hi) {  // slice lengths, then a prefix sum
+    parallel_rows(n, 2 * g.m, [&](int64_t lo, int64_t hi) {  // slice lengths, then a prefix sum
         for (int64_t w = lo; w < hi; ++w) {
             int64_t len = 0;
             if (in[(size_t)w] && xa < xb) {
@@ -898,7 +898,7 @@ harp_status run_wedge_block(const RankGraph& g, const WedgeBlock& blk, int dev, 
     const int64_t ra = off[(size_t)n];
     if (la == 0 || ra == 0) return HARP_OK;  // no root or no opposite vertex: nothing to count here
     buf<int32_t> cols((size_t)ra);
-    parallel_rows(n, [&](int64_t lo, int64_t hi) {
+    parallel_rows(n, 2 * g.m, [&](int64_t lo, int64_t hi) {
         for (int64_t w = lo; w < hi; ++w) {
             const int64_t len = off[(size_t)w + 1] - off[(size_t)w];
             if (len)
@@ -1027,7 +1027,7 @@ extern "C" harp_status harp_count4_partitioned(int64_t n, int64_t m_in, const in
     // degree sums by owner (every vertex / edge once) and the global sum_e C(t_e, 2)
     std::vector<uint64_t> pD(host_threads(), 0);
     std::atomic<uint64_t> aS{0}, aPW{0};
-    parallel_rows(n, [&](int64_t lo, int64_t hi) {
+    parallel_rows(n, 2 * g.m, [&](int64_t lo, int64_t hi) {
         uint64_t s3 = 0, pw = 0;
         for (int64_t r = lo; r < hi; ++r) {
             const uint64_t dr = (uint64_t)g.deg[(size_t)r];
