@@ -124,7 +124,8 @@ enum : int {
     Q_CORE_M = 56,
     Q_CORE_L = 57,
     Q_CORE_XL = 58,
-    T_CORE_M = 60,         // its tickets
+    T_LIT_STAR = 59,       // blocks of the literal basis's last pass that are done
+    T_CORE_M = 60,         // tickets of the wedge core pass
     T_CORE_L = 61,
     T_CORE_XL = 62,
     Q_C4_WIDE = 69,        // length of the wedge wide tier's queue (from the back of q_win)

@@ -51,7 +51,7 @@ constexpr int kLitThreads = 256;
 constexpr int kLitWarps = kLitThreads / 32;
 constexpr int kStageCap = 512;        // C_uv members staged per warp (shared memory); larger: unstaged
 constexpr int kProbeWindow = 16;      // cache slots probed per lookup / insertion
-constexpr unsigned long long kSigEmpty = ~0ull;
+constexpr unsigned long long kSigEmpty = 0;  // no key: a key's code is not 0
 constexpr unsigned long long kValid = 1ull << 32;
 enum : uint64_t { SIG_C = 1, SIG_W = 2 };
 
@@ -189,13 +189,15 @@ __device__ uint32_t frontier_warp(const SigCache& c, const Graph& G, uint64_t co
     return v;
 }
 
-// Row of the out-arc a (offp[u] <= a < offp[u + 1]).
+// Row of the out-arc a (offp[u] <= a < offp[u + 1]), by the whole warp: 32 probes a round (a graph of 300 vertices takes
+// two dependent loads where halving takes nine).
 __device__ __forceinline__ int32_t arc_source(const int64_t* __restrict__ offp, int64_t n, int64_t a) {
     int64_t lo = 0, hi = n;
     while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (offp[mid] <= a) lo = mid;
-        else hi = mid;
+        const int64_t step = (hi - lo + 31) >> 5, p = lo + (int64_t)(lane_id() + 1) * step;
+        const uint32_t m = __ballot_sync(kFull, p >= hi || offp[p] > a);  // lane 31 probes at or past hi
+        lo += (int64_t)(__ffs(m) - 1) * step;
+        hi = lo + step < hi ? lo + step : hi;
     }
     return (int32_t)lo;
 }
@@ -228,30 +230,53 @@ __device__ __forceinline__ void add128(uint64_t* acc_lo, unsigned __int128 v) {
     if (hi + carry) atomicAdd((unsigned long long*)(acc_lo + 1), hi + carry);
 }
 
-__device__ __forceinline__ void flush_u64(uint64_t* dst, uint64_t v, uint64_t* red) {
-    v = block_sum_u64(v, red);
-    if (threadIdx.x == 0 && v) atomicAdd((unsigned long long*)dst, (unsigned long long)v);
-}
+// The block's sums of N64 64-bit and N128 128-bit values (a 128-bit one as its two low 32-bit parts and its high word,
+// whose sums over a block cannot overflow) added to acc at their places, behind one barrier.  With a barrier pair per sum,
+// a halving search per arc and a memset per table the literal basis had lost its lead on the smallest graphs (Barabasi-Albert
+// of 300 vertices, 894 edges: 94 to 102 us, the triangle-wedge basis 94 to 100; now 84 to 87).
+template <int N64, int N128>
+struct Sums {
+    uint64_t v[N64];
+    int at[N64];
+    unsigned __int128 x[N128 > 0 ? N128 : 1];
+    int xat[N128 > 0 ? N128 : 1];
+};
 
-// per-thread 128-bit partial -> one 128-bit atomic per block (low and high words reduced apart; the
-// low words' carries are counted by summing them as 128-bit through two 32-bit halves)
-__device__ __forceinline__ void flush_u128(uint64_t* dst_lo, unsigned __int128 v, uint64_t* red) {
-    const uint64_t lo32 = (uint64_t)v & 0xffffffffull;
-    const uint64_t hi32 = (uint64_t)(v >> 32) & 0xffffffffull;
-    const uint64_t top = (uint64_t)(v >> 64);
-    const uint64_t s_lo32 = block_sum_u64(lo32, red);  // < 2^32 * threads: no overflow
-    const uint64_t s_hi32 = block_sum_u64(hi32, red);
-    const uint64_t s_top = block_sum_u64(top, red);
-    if (threadIdx.x == 0) {
-        const unsigned __int128 total = (unsigned __int128)s_lo32 + ((unsigned __int128)s_hi32 << 32) +
-                                        ((unsigned __int128)s_top << 64);
-        if (total) add128(dst_lo, total);
+template <int N64, int N128, int THREADS>
+__device__ __forceinline__ void flush(uint64_t* acc, const Sums<N64, N128>& f) {
+    constexpr int K = N64 + 3 * N128, NW = THREADS / 32;
+    static_assert(N64 <= 32 && 32 + N128 <= THREADS, "a thread per sum");
+    __shared__ uint64_t part[K][NW];
+    const int w = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int j = k < N64 ? 0 : (k - N64) / 3, piece = k < N64 ? 0 : (k - N64) % 3;
+        uint64_t y;
+        if (k < N64) y = f.v[k < N64 ? k : 0];
+        else y = piece == 2 ? (uint64_t)(f.x[j] >> 64) : (uint64_t)(f.x[j] >> (32 * piece)) & 0xffffffffull;
+        y = warp_sum(y);
+        if (lane_id() == 0) part[k][w] = y;
     }
-}
-
-__device__ __forceinline__ void flush_stats(uint64_t* acc, const SigStats& st, uint64_t* red) {
-    flush_u64(&acc[ACC_SIG_LOOKUPS], st.lookups, red);
-    flush_u64(&acc[ACC_SIG_HITS], st.hits, red);
+    __syncthreads();
+    auto total = [&](int k) {
+        uint64_t t = 0;
+        for (int i = 0; i < NW; ++i) t += part[k][i];
+        return t;
+    };
+#pragma unroll
+    for (int k = 0; k < N64; ++k)
+        if (threadIdx.x == k) {
+            const uint64_t t = total(k);
+            if (t) atomicAdd((unsigned long long*)&acc[f.at[k]], (unsigned long long)t);
+        }
+#pragma unroll
+    for (int j = 0; j < N128; ++j)
+        if (threadIdx.x == 32 + j) {
+            const int k = N64 + 3 * j;
+            const unsigned __int128 t = (unsigned __int128)total(k) + ((unsigned __int128)total(k + 1) << 32) +
+                                        ((unsigned __int128)total(k + 2) << 64);
+            if (t) add128(&acc[f.xat[j]], t);
+        }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -263,7 +288,6 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_tri(Graph G, const int64_t*
                                                          uint64_t* __restrict__ acc) {
     grid_begin();
     __shared__ int32_t sbuf[kLitWarps][kStageCap];
-    __shared__ uint64_t red[32];
     const int w = threadIdx.x >> 5, l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     SigStats st;
@@ -331,12 +355,10 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_tri(Graph G, const int64_t*
         }
         __syncwarp();
     }
-    flush_u64(&acc[ACC_LIT_X1], x1, red);
-    flush_u64(&acc[ACC_LIT_T], tri, red);
-    flush_u128(&acc[ACC_LIT_X2], x2, red);
-    flush_u128(&acc[ACC_LIT_X3], x3, red);
-    flush_u128(&acc[ACC_LIT_CORR], corr, red);
-    flush_stats(acc, st, red);
+    flush<4, 3, kLitThreads>(acc, {{x1, tri, st.lookups, st.hits},
+                                   {ACC_LIT_X1, ACC_LIT_T, ACC_SIG_LOOKUPS, ACC_SIG_HITS},
+                                   {x2, x3, corr},
+                                   {ACC_LIT_X2, ACC_LIT_X3, ACC_LIT_CORR}});
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -347,7 +369,6 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_edge(Graph G, const int64_t
                                                           SigCache cache, uint64_t* __restrict__ acc) {
     grid_begin();
     __shared__ int32_t sbuf[kLitWarps][kStageCap];
-    __shared__ uint64_t red[32];
     const int w = threadIdx.x >> 5, l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     SigStats st;
@@ -398,9 +419,10 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_edge(Graph G, const int64_t
         if (l != 0) e_sum = 0;
         __syncwarp();
     }
-    flush_u64(&acc[ACC_LIT_AB], ab_sum, red);
-    flush_u128(&acc[ACC_LIT_E], e_sum, red);
-    flush_stats(acc, st, red);
+    flush<3, 1, kLitThreads>(acc, {{ab_sum, st.lookups, st.hits},
+                                   {ACC_LIT_AB, ACC_SIG_LOOKUPS, ACC_SIG_HITS},
+                                   {e_sum},
+                                   {ACC_LIT_E}});
 }
 
 // The edge pass with staged frontiers: a block per v.  For one v every frontier cnt(x) = |N(x) n N(v)| it can be
@@ -426,7 +448,6 @@ __global__ void __launch_bounds__(kStagedThreads) k_lit_edge_staged(Graph G, con
                                                                     SigCache cache, uint64_t* __restrict__ acc) {
     grid_begin();
     extern __shared__ uint32_t smem[];
-    __shared__ uint64_t red[32];
     __shared__ int64_t s_item;
     __shared__ unsigned int s_walked;
     const StagedShape sh(n);
@@ -510,19 +531,55 @@ __global__ void __launch_bounds__(kStagedThreads) k_lit_edge_staged(Graph G, con
         }
         __syncthreads();
     }
-    flush_u64(&acc[ACC_LIT_AB], ab_sum, red);
-    flush_u128(&acc[ACC_LIT_E], e_sum, red);
-    flush_stats(acc, st, red);
+    flush<3, 1, kStagedThreads>(acc, {{ab_sum, st.lookups, st.hits},
+                                   {ACC_LIT_AB, ACC_SIG_LOOKUPS, ACC_SIG_HITS},
+                                   {e_sum},
+                                   {ACC_LIT_E}});
 }
 
 // ---------------------------------------------------------------------------------------------
-// 3. Vertices: the star form on H_u.
+// 3. The closure as printed, and the non-induced statistics it implies (by one thread, once every sum is in acc).
+// ---------------------------------------------------------------------------------------------
+// staged: the edge sum lacks its correction
+__device__ __forceinline__ void lit_close(int64_t m, bool staged, volatile uint64_t* acc) {
+    const unsigned __int128 X2 = (unsigned __int128)acc[ACC_LIT_X2] | ((unsigned __int128)acc[ACC_LIT_X2 + 1] << 64);
+    const unsigned __int128 X3 = (unsigned __int128)acc[ACC_LIT_X3] | ((unsigned __int128)acc[ACC_LIT_X3 + 1] << 64);
+    unsigned __int128 E = (unsigned __int128)acc[ACC_LIT_E] | ((unsigned __int128)acc[ACC_LIT_E + 1] << 64);
+    if (staged) E -= (unsigned __int128)acc[ACC_LIT_CORR] | ((unsigned __int128)acc[ACC_LIT_CORR + 1] << 64);
+    if ((X2 & 1) || (X3 & 3) || (E & 3))
+        atomicOr((unsigned long long*)acc + ACC_ERR, (unsigned long long)kErrLitDiv);
+    const uint64_t paw = acc[ACC_LIT_X1];
+    const uint64_t diamond = (uint64_t)(X2 >> 1);
+    const uint64_t k4 = (uint64_t)(X3 >> 2);
+    const uint64_t cycle = (uint64_t)(E >> 2);
+    const uint64_t path = acc[ACC_LIT_AB] - (uint64_t)E;
+    const uint64_t star = acc[ACC_LIT_STAR];
+    acc[OUT_COUNTS + HARP_STAR3] = star;
+    acc[OUT_COUNTS + HARP_PATH4] = path;
+    acc[OUT_COUNTS + HARP_PAW] = paw;
+    acc[OUT_COUNTS + HARP_CYCLE4] = cycle;
+    acc[OUT_COUNTS + HARP_DIAMOND] = diamond;
+    acc[OUT_COUNTS + HARP_CLIQUE4] = k4;
+    // the non-induced statistics, by the containment of each pattern in the induced classes (the
+    // forward direction of the system the triangle-wedge basis inverts); T as enumerated
+    acc[OUT_STATS + HARP_STAT_TRIANGLES] = acc[ACC_LIT_T];
+    acc[OUT_STATS + HARP_STAT_K4] = k4;
+    acc[OUT_STATS + HARP_STAT_C4] = cycle + diamond + 3 * k4;
+    acc[OUT_STATS + HARP_STAT_STARS] = star + paw + 2 * diamond + 4 * k4;
+    acc[OUT_STATS + HARP_STAT_PATHS] = path + 2 * paw + 4 * cycle + 6 * diamond + 12 * k4;
+    acc[OUT_STATS + HARP_STAT_PAWS] = paw + 4 * diamond + 12 * k4;
+    acc[OUT_STATS + HARP_STAT_DIAMONDS] = diamond + 6 * k4;
+    acc[OUT_STATS + HARP_STAT_EDGES] = (uint64_t)m;
+}
+
+// ---------------------------------------------------------------------------------------------
+// 4. Vertices: the star form on H_u; the last block closes.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kLitThreads) k_lit_star(Graph G, int64_t n, SigCache cache,
-                                                          const uint64_t* __restrict__ tau3,
+                                                          const uint64_t* __restrict__ tau3, int64_t m, bool staged,
                                                           uint64_t* __restrict__ acc) {
     grid_begin();
-    __shared__ uint64_t red[32];
+    __shared__ bool last;
     const int l = lane_id();
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     SigStats st;
@@ -546,47 +603,16 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_star(Graph G, int64_t n, Si
             star += choose3_u64(d) - mH * (d >= 2 ? d - 2 : 0) + s2 - tau;
         }
     }
-    flush_u64(&acc[ACC_LIT_STAR], star, red);
-    bad = block_sum_u64(bad, red);
-    if (threadIdx.x == 0 && bad) atomicOr((unsigned long long*)&acc[ACC_ERR], (unsigned long long)kErrLitDiv);
-    flush_stats(acc, st, red);
-}
-
-// ---------------------------------------------------------------------------------------------
-// 4. The closure as printed, and the non-induced statistics it implies.
-// ---------------------------------------------------------------------------------------------
-// staged: the edge sum lacks its correction
-__global__ void k_lit_close(int64_t m, bool staged, uint64_t* __restrict__ acc) {
-    grid_begin();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const unsigned __int128 X2 = (unsigned __int128)acc[ACC_LIT_X2] | ((unsigned __int128)acc[ACC_LIT_X2 + 1] << 64);
-    const unsigned __int128 X3 = (unsigned __int128)acc[ACC_LIT_X3] | ((unsigned __int128)acc[ACC_LIT_X3 + 1] << 64);
-    unsigned __int128 E = (unsigned __int128)acc[ACC_LIT_E] | ((unsigned __int128)acc[ACC_LIT_E + 1] << 64);
-    if (staged) E -= (unsigned __int128)acc[ACC_LIT_CORR] | ((unsigned __int128)acc[ACC_LIT_CORR + 1] << 64);
-    if ((X2 & 1) || (X3 & 3) || (E & 3))
-        atomicOr((unsigned long long*)&acc[ACC_ERR], (unsigned long long)kErrLitDiv);
-    const uint64_t paw = acc[ACC_LIT_X1];
-    const uint64_t diamond = (uint64_t)(X2 >> 1);
-    const uint64_t k4 = (uint64_t)(X3 >> 2);
-    const uint64_t cycle = (uint64_t)(E >> 2);
-    const uint64_t path = acc[ACC_LIT_AB] - (uint64_t)E;
-    const uint64_t star = acc[ACC_LIT_STAR];
-    acc[OUT_COUNTS + HARP_STAR3] = star;
-    acc[OUT_COUNTS + HARP_PATH4] = path;
-    acc[OUT_COUNTS + HARP_PAW] = paw;
-    acc[OUT_COUNTS + HARP_CYCLE4] = cycle;
-    acc[OUT_COUNTS + HARP_DIAMOND] = diamond;
-    acc[OUT_COUNTS + HARP_CLIQUE4] = k4;
-    // the non-induced statistics, by the containment of each pattern in the induced classes (the
-    // forward direction of the system the triangle-wedge basis inverts); T as enumerated
-    acc[OUT_STATS + HARP_STAT_TRIANGLES] = acc[ACC_LIT_T];
-    acc[OUT_STATS + HARP_STAT_K4] = k4;
-    acc[OUT_STATS + HARP_STAT_C4] = cycle + diamond + 3 * k4;
-    acc[OUT_STATS + HARP_STAT_STARS] = star + paw + 2 * diamond + 4 * k4;
-    acc[OUT_STATS + HARP_STAT_PATHS] = path + 2 * paw + 4 * cycle + 6 * diamond + 12 * k4;
-    acc[OUT_STATS + HARP_STAT_PAWS] = paw + 4 * diamond + 12 * k4;
-    acc[OUT_STATS + HARP_STAT_DIAMONDS] = diamond + 6 * k4;
-    acc[OUT_STATS + HARP_STAT_EDGES] = (uint64_t)m;
+    if (bad) atomicOr((unsigned long long*)&acc[ACC_ERR], (unsigned long long)kErrLitDiv);  // lane 0's
+    flush<3, 0, kLitThreads>(acc, {{star, st.lookups, st.hits}, {ACC_LIT_STAR, ACC_SIG_LOOKUPS, ACC_SIG_HITS}, {}, {}});
+    __threadfence();  // each adding thread's sums are visible before its block counts as done
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd((unsigned long long*)&acc[T_LIT_STAR], 1ull) == gridDim.x - 1;
+    __syncthreads();
+    if (last && threadIdx.x == 0) {
+        __threadfence();
+        lit_close(m, staged, acc);
+    }
 }
 
 unsigned lit_grid(int64_t warps) {
@@ -621,9 +647,7 @@ harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& pla
     const Graph G{ws.off, ws.cols, ws.deg};
     const bool staged = use_cache && n <= kStagedMaxN && g->max_deg < 65536;
     cudaError_t e = cudaSuccess;
-    if (slots) e = cudaMemsetAsync(cache.keys, 0xff, 8 * slots, s);
-    if (e == cudaSuccess && slots) e = cudaMemsetAsync(cache.vals, 0, 8 * slots, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(tau3, 0, 8 * (size_t)(n > 0 ? n : 1), s);
+    e = cudaMemsetAsync(scratch, 0, bytes, s);  // free keys, values and tau3 are all zero
     if (e == cudaSuccess && m > 0) {
         launch(k_lit_tri, lit_grid(m), kLitThreads, 0, s, G, ws.offp, ws.colsp, n, m, cache, tau3, ws.acc);
         note_launch();
@@ -645,15 +669,10 @@ harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& pla
         }
         if (e == cudaSuccess) e = prof_mark(s, SEG_C4_SMALL);
         if (e == cudaSuccess) {
-            launch(k_lit_star, lit_grid(n), kLitThreads, 0, s, G, n, cache, tau3, ws.acc);
+            launch(k_lit_star, lit_grid(n), kLitThreads, 0, s, G, n, cache, tau3, m, staged, ws.acc);
             note_launch();
             e = cudaGetLastError();
         }
-    }
-    if (e == cudaSuccess) {
-        launch(k_lit_close, 1, 32, 0, s, m, staged, ws.acc);
-        note_launch();
-        e = cudaGetLastError();
     }
     cudaFreeAsync(scratch, s);
     if (e != cudaSuccess) {
