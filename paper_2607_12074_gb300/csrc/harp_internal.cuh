@@ -337,6 +337,8 @@ harp_status count_wedge_core(const harp_csr* g, Workspace& ws, cudaStream_t s);
 // literal.cu: the literal basis (per-triangle X_j, per-edge A_e x B_e, per-vertex H_u stars) and its
 // closure, after orient(); writes acc[OUT_COUNTS..], acc[OUT_STATS..]
 harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s);
+// literal.cu: whether its edge pass is the staged one (where reuse is on)
+bool literal_stages(const harp_csr* g);
 
 // orbits.cu: per-vertex orbit counts (11 roles) after orient() and count_triangles_k4(); d_out is
 // device uint64[n][11] indexed by input vertex id

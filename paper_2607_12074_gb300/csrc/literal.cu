@@ -622,7 +622,24 @@ unsigned lit_grid(int64_t warps) {
     return (unsigned)(b > cap ? cap : b);
 }
 
+// Resident blocks of the staged pass per SM (registers allow two).
+int staged_blocks(int64_t n) { return StagedShape(n).bytes() <= 100 * 1024 ? 2 : 1; }
+
 }  // namespace
+
+// The staged pass costs a block's turn per vertex (5 ns of the device with two blocks to an SM, 9 with one), the pass by
+// edges the intersections of each edge's frontiers, which grow with the degrees' square and with hubs.  Whole counts,
+// staged and by edges: Erdos-Renyi of 40,000 vertices, mean degree 4 0.43 and 0.32 ms, 8 0.57 and 0.76; of 80,000
+// vertices, 8 1.61 and 1.34, 16 2.35 and 4.14; random geometric of 22,000 vertices, 6 0.42 and 0.35, 10 0.59 and 0.68;
+// Barabasi-Albert of 40,000 vertices, 4 (largest degree 497) 0.44 and 0.63; of 80,000, 4 (691) 1.21 and 0.91, 8 (867)
+// 1.76 and 3.05.  Up to 2,048 vertices the blocks have a few turns each: staged 0.084 and 0.102 on Barabasi-Albert
+// of 300 vertices, 0.077 and 0.084 on Erdos-Renyi of 1,000 with mean degree 3.
+bool literal_stages(const harp_csr* g) {
+    if (g->n > kStagedMaxN || g->max_deg >= 65536) return false;
+    if (g->n <= 2048) return true;
+    const double mean = 2.0 * (double)g->m / (double)g->n, top = (double)g->max_deg;
+    return staged_blocks(g->n) == 2 ? mean * mean + 0.3 * top >= 45.0 : mean * mean + 0.15 * top >= 150.0;
+}
 
 harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s) {
     const int64_t n = g->n, m = g->m;
@@ -645,7 +662,7 @@ harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& pla
     }
     uint64_t* tau3 = reinterpret_cast<uint64_t*>(scratch + 16 * slots);
     const Graph G{ws.off, ws.cols, ws.deg};
-    const bool staged = use_cache && n <= kStagedMaxN && g->max_deg < 65536;
+    const bool staged = use_cache && literal_stages(g);
     cudaError_t e = cudaSuccess;
     e = cudaMemsetAsync(scratch, 0, bytes, s);  // free keys, values and tau3 are all zero
     if (e == cudaSuccess && m > 0) {
@@ -657,8 +674,7 @@ harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& pla
             if (staged) {
                 const size_t smem = StagedShape(n).bytes();
                 e = cudaFuncSetAttribute(k_lit_edge_staged, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                const int per_sm = smem <= 50 * 1024 ? 4 : (smem <= 100 * 1024 ? 2 : 1);
-                const int64_t blocks = n < (int64_t)num_sms() * per_sm ? n : (int64_t)num_sms() * per_sm;
+                const int64_t most = (int64_t)num_sms() * staged_blocks(n), blocks = n < most ? n : most;
                 if (e == cudaSuccess)
                     launch(k_lit_edge_staged, (unsigned)blocks, kStagedThreads, smem, s, G, ws.offp, n, cache, ws.acc);
             } else {
