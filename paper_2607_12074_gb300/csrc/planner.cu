@@ -12,10 +12,17 @@
 //   * LIT (the closure equations as printed, Section III-F: per-triangle X_j, per-edge A_e x B_e,
 //         per-vertex H_u): C_enum = the row intersections of every arc plus, per triangle, the
 //         three-way intersection for X_3, and per edge one frontier per x in A_e; C_inter = the
-//         signature-cache probes; R_reuse = frontier requests expected to hit the cache.
-// Both also pay a fixed cost per kernel launch after the shared orientation pass (15 for TW, 4 for
-// LIT), expressed in element operations: kLaunchOps, about the element operations one dependent
-// launch costs at the measured rate of the wedge kernel (~4e11 elements/s, ~2.5 us a launch).  Both
+//         signature-cache probes; R_reuse = frontier requests expected to hit the cache.  Where the edge
+//         pass is staged (literal_stages) the frontiers cost one walk over the rows of N(v) per v and a
+//         counter read per x, and nothing is left to reuse.
+// Element operations are charged at the wedge kernel's rate (kOpsPerUs).  Graphs small enough for the choice
+// to be close are bound by latency instead, charged at what it takes beside that rate: the passes' fixed
+// cost after the shared orientation (TW 40 us: some ten dependent launches, those of the two passes side by
+// side; LIT 25 us: three), and in LIT a warp's turn per arc (2.5 ns of the device), the two cache requests of a
+// triangle (1 ns) and the longest chain of triangles that one arc's warp takes one after the other (0.5 us
+// each).  Measured with both bases: Barabasi-Albert of 300 vertices (894 edges) TW 98 us, LIT 84; of 3,000 (11,990) 132
+// and 143; random geometric of 1,000 (3,779) 90 and 98; Erdos-Renyi of 1,000 (4,974) 103 and 96, of 80,000
+// (160,193) 202 and 547.  (A term for launches alone named LIT up to 160,000 edges, up to 6 times slower.)  Both
 // recover all six counts (Y = 6).  The lambda weights normalise the terms to element operations (the
 // paper leaves their values open): l_I = 1, l_H = 1/4 per replicated byte, l_R = 1 (reuse is counted
 // in the element operations it saves), l_Y = 0 (equal yield decides nothing between these bases).
@@ -32,7 +39,8 @@
 namespace harp {
 namespace {
 
-constexpr int kSampleThreads = 256;
+constexpr double kOpsPerUs = 4.0e5;  // element operations (wedge kernel: about 4e11 a second)
+constexpr double kTwFixedUs = 40.0, kLitFixedUs = 25.0, kLitArcUs = 2.5e-3, kLitTriangleUs = 1.0e-3, kLitChainUs = 0.5;
 
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
@@ -175,6 +183,8 @@ extern "C" harp_status harp_select_anchors(const harp_csr* g, const harp_select_
     const double mean_deg = g->n > 0 ? 2.0 * m / (double)g->n : 0.0;
     // per-arc means of the cost terms (element operations); lg = binary-search depth in the longer row
     double tw_enum = 0, tw_inter = 0, tw_reuse = 0, lit_enum = 0, lit_inter = 0, lit_reuse = 0;
+    double triangles = 0, t_max = 0;
+    const bool staged = literal_stages(g);
     for (uint64_t i = 0; i < got; ++i) {
         const double du = host[3 * i], dv = host[3 * i + 1], t = host[3 * i + 2];
         const double dl = du < dv ? du : dv, dh = du < dv ? dv : du;
@@ -185,10 +195,14 @@ extern "C" harp_status harp_select_anchors(const harp_csr* g, const harp_select_
         tw_reuse += (t / 3.0) * dl;     // one staged 4-clique extension per triangle (t/3 per edge)
         // literal: the arc's intersection (tri pass and edge pass), the X_3 walks of its t/3
         // triangles, and per x in A_e the correction |C_e n N(x)| plus a frontier (half of them
-        // computed on a miss, at min(d_x, d_v) with d_x ~ the mean degree)
-        lit_enum += 2.0 * dl * lg + (t / 3.0) * t * lg + A * (t * lg + 0.5 * std::fmin(mean_deg, dh) * lg);
+        // computed on a miss, at min(d_x, d_v) with d_x ~ the mean degree); staged: the walks of the edge's
+        // two rows, for the counters, in place of its second intersection
+        lit_enum += dl * lg + (t / 3.0) * t * lg;
+        lit_enum += staged ? du + dv + A : dl * lg + A * (t * lg + 0.5 * std::fmin(mean_deg, dh) * lg);
         lit_inter += 2.0 * (t / 3.0) + A + 2.0;  // cache probes: two per triangle, one per x, two per edge
-        lit_reuse += 0.5 * A * std::fmin(mean_deg, dh) * lg;  // frontier hits save their recompute
+        if (!staged) lit_reuse += 0.5 * A * std::fmin(mean_deg, dh) * lg;  // frontier hits save their recompute
+        triangles += t / 3.0;
+        t_max = t > t_max ? t : t_max;
     }
     delete[] host;
     const double inv = got > 0 ? 1.0 / (double)got : 0.0;
@@ -198,10 +212,8 @@ extern "C" harp_status harp_select_anchors(const harp_csr* g, const harp_select_
     lit_enum *= m * inv;
     lit_inter *= m * inv;
     lit_reuse *= m * inv;
-    // fixed cost of the kernel launches after the shared orientation pass
-    constexpr double kLaunchOps = 1.0e6;
-    tw_enum += 15.0 * kLaunchOps;
-    lit_enum += 4.0 * kLaunchOps;
+    tw_enum += kOpsPerUs * kTwFixedUs;
+    lit_enum += kOpsPerUs * (kLitFixedUs + kLitArcUs * m + kLitTriangleUs * triangles * m * inv + kLitChainUs * t_max);
     // Halo term: replication factor if the CSR plus workspace exceed the memory budget.
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
