@@ -167,9 +167,7 @@ bool same_plan(const harp_plan& a, const harp_plan& b) {
 
 }  // namespace
 
-extern "C" {
-
-harp_status harp_batch_create(const harp_csr* const* graphs, int64_t G, harp_batch** out) {
+harp_status harp::batch_create(const harp_csr* const* graphs, int64_t G, int priority, harp_batch** out) {
     if (!out || G < 0 || (G > 0 && !graphs)) return HARP_EINVAL;
     int dev = 0;
     HARP_CK(cudaGetDevice(&dev));
@@ -187,7 +185,7 @@ harp_status harp_batch_create(const harp_csr* const* graphs, int64_t G, harp_bat
     b->device = dev;
     b->G = G;
     b->m_of.resize((size_t)G);
-    cudaError_t e = cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking);
+    cudaError_t e = cudaStreamCreateWithPriority(&b->capture_stream, cudaStreamNonBlocking, priority);
     cudaStream_t s = b->capture_stream;
     std::vector<MemberDesc> desc((size_t)G);
     std::vector<int64_t> gbase((size_t)G + 1);
@@ -244,7 +242,9 @@ harp_status harp_batch_create(const harp_csr* const* graphs, int64_t G, harp_bat
     return HARP_OK;
 }
 
-}  // extern "C"
+extern "C" harp_status harp_batch_create(const harp_csr* const* graphs, int64_t G, harp_batch** out) {
+    return batch_create(graphs, G, 0, out);
+}
 
 namespace {
 

@@ -3,12 +3,13 @@
 // Requests (host edge lists, copied at submit into a page-locked staging arena when it has room)
 // wait in a FIFO.  Two builder threads admit them in order while the device memory held by admitted
 // requests stays within the HBM budget and a slot is free, copy each edge list to the device and
-// build its CSR, each on its own copy stream.  Built requests go to one of two lanes by size: small
+// build its CSR, each on copy streams of its own.  Requests go to one of two lanes by size: small
 // requests (at most small_edges input pairs) and the rest.  Each lane has an executor thread that
 // takes every built request of its lane as the next batch and counts it with the batched pipeline
-// (the disjoint union of the batch, one launch per kernel) on the lane's compute stream; the small
-// lane's stream has the higher priority, so when a large batch's kernel finishes its blocks the small
-// batch's kernels are scheduled first and a small request does not wait for a whole large batch.
+// (the disjoint union of the batch, one launch per kernel) on the lane's compute stream.  All streams
+// of the small lane (CSR build, union, count) have the higher priority, so when a large batch's kernel
+// finishes its blocks the small requests' kernels are scheduled first and a small request does not wait
+// for a whole large batch.
 // With a batching window an executor first waits, up to the window, while requests are still queued
 // for admission or being built.  Requests that arrive while batches are on the GPU are admitted,
 // copied and built meanwhile (their copies and CSR builds overlap the running counts) and form their
@@ -128,7 +129,8 @@ struct harp_server {
     int64_t building = 0;               // requests between admission and a built CSR
     bool stop = false;
     static constexpr int kBuilders = 2;
-    cudaStream_t copy_stream[kBuilders] = {nullptr, nullptr};
+    int priority[kLanes] = {0, 0};      // lane 1 the greatest the device offers, lane 0 the least
+    cudaStream_t copy_stream[kBuilders][kLanes] = {};
     cudaStream_t compute_stream[kLanes] = {nullptr, nullptr};
     std::thread builder[kBuilders], executor[kLanes];
     StagingArena staging;
@@ -180,7 +182,6 @@ void drop_host_copy(harp_server* s, Request* r) {  // caller holds the lock
 
 void builder_loop(harp_server* s, int which) {
     cudaSetDevice(s->device);
-    cudaStream_t stream = s->copy_stream[which];
     std::unique_lock<std::mutex> lk(s->mu);
     while (true) {
         s->cv_build.wait(lk, [&] { return s->stop || can_admit(s); });
@@ -210,6 +211,7 @@ void builder_loop(harp_server* s, int which) {
             continue;
         }
         s->building++;
+        cudaStream_t stream = s->copy_stream[which][lane_of(s, r)];
         lk.unlock();
         st = harp_build_csr(r->n, r->m_in, r->hsrc, r->hdst, HARP_PTR_HOST, stream, &r->csr);
         lk.lock();
@@ -257,7 +259,7 @@ void executor_loop(harp_server* s, int lane) {
         for (size_t k = 0; k < batch.size(); ++k) hs[k] = batch[k]->csr;
         std::vector<uint64_t> counts(6 * batch.size());
         harp_batch* b = nullptr;
-        harp_status st = harp_batch_create(hs.data(), (int64_t)hs.size(), &b);
+        harp_status st = harp::batch_create(hs.data(), (int64_t)hs.size(), s->priority[lane], &b);
         if (st == HARP_OK) {
             harp_plan p;
             std::memset(&p, 0, sizeof(p));
@@ -302,23 +304,20 @@ harp_status harp_server_create(const harp_server_opts* opts, harp_server** out) 
         delete s;
         return HARP_ECUDA;
     }
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < harp_server::kBuilders && e == cudaSuccess; ++k)
-        e = cudaStreamCreateWithFlags(&s->copy_stream[k], cudaStreamNonBlocking);
-    // lane 1 (small requests) gets the greatest priority the device offers, lane 0 the least
-    int prio_least = 0, prio_greatest = 0;
-    if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
-    if (e == cudaSuccess)
-        e = cudaStreamCreateWithPriority(&s->compute_stream[0], cudaStreamNonBlocking, prio_least);
-    if (e == cudaSuccess)
-        e = cudaStreamCreateWithPriority(&s->compute_stream[1], cudaStreamNonBlocking, prio_greatest);
+    cudaError_t e = cudaDeviceGetStreamPriorityRange(&s->priority[0], &s->priority[1]);
+    for (int l = 0; l < harp_server::kLanes && e == cudaSuccess; ++l) {
+        e = cudaStreamCreateWithPriority(&s->compute_stream[l], cudaStreamNonBlocking, s->priority[l]);
+        for (int k = 0; k < harp_server::kBuilders && e == cudaSuccess; ++k)
+            e = cudaStreamCreateWithPriority(&s->copy_stream[k][l], cudaStreamNonBlocking, s->priority[l]);
+    }
     void* arena = nullptr;
     const size_t arena_bytes = (size_t)s->opts.staging_mib << 20;
     if (e == cudaSuccess) e = cudaMallocHost(&arena, arena_bytes);
     if (e != cudaSuccess) {
         harp::record_cuda_error(e);
-        for (cudaStream_t c : s->copy_stream)
-            if (c) cudaStreamDestroy(c);
+        for (auto& lanes : s->copy_stream)
+            for (cudaStream_t c : lanes)
+                if (c) cudaStreamDestroy(c);
         for (cudaStream_t c : s->compute_stream)
             if (c) cudaStreamDestroy(c);
         delete s;
@@ -454,10 +453,11 @@ void harp_server_destroy(harp_server* s) {
         if (kv.second->csr) harp_csr_free(kv.second->csr);
         delete kv.second;
     }
-    for (cudaStream_t c : s->copy_stream) {
-        cudaStreamSynchronize(c);
-        cudaStreamDestroy(c);
-    }
+    for (auto& lanes : s->copy_stream)
+        for (cudaStream_t c : lanes) {
+            cudaStreamSynchronize(c);
+            cudaStreamDestroy(c);
+        }
     for (cudaStream_t c : s->compute_stream) {
         cudaStreamSynchronize(c);
         cudaStreamDestroy(c);

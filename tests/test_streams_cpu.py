@@ -1,0 +1,61 @@
+"""The streams that host code uses, without a GPU: the library's objects linked with a fake CUDA runtime
+(fake_cudart.c) in which kernels do nothing and every enqueued operation is recorded."""
+import ctypes
+import glob
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+GREATEST = -5  # the fake's priorities: 0 .. -5
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_2607_12074_gb300 import _build
+    nvcc = shutil.which(_build.nvcc())
+    if not nvcc or not shutil.which("gcc"):
+        pytest.skip("needs nvcc and gcc to link the library with the fake runtime")
+    _build.build()
+    out = tmp_path_factory.mktemp("fake")
+    obj, lib = str(out / "fake_cudart.o"), str(out / "libharp_fake.so")
+    include = os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include")
+    subprocess.run(["gcc", "-O1", "-fPIC", "-I", include, "-c", os.path.join(HERE, "fake_cudart.c"), "-o", obj], check=True)
+    subprocess.run([nvcc, *_build.ARCH, "-shared", "-cudart", "none", "-o", lib, *glob.glob(os.path.join(_build.BUILD, "*.cu.o")),
+                    obj], check=True)
+    L = ctypes.CDLL(lib)
+    L.fake_launches.restype = L.fake_calls.restype = ctypes.c_long
+    L.harp_status_str.restype = ctypes.c_char_p
+    return L
+
+
+def submit(L, server, edges):
+    n = edges + 1
+    src, dst = np.arange(edges, dtype=np.int32), np.arange(1, n, dtype=np.int32)
+    ticket = ctypes.c_uint64()
+    ptr = ctypes.POINTER(ctypes.c_int32)
+    assert L.harp_submit(server, ctypes.c_int64(n), ctypes.c_int64(edges), src.ctypes.data_as(ptr), dst.ctypes.data_as(ptr),
+                         ctypes.byref(ticket)) == 0
+    counts = (ctypes.c_uint64 * 6)()
+    assert L.harp_wait(server, ticket, counts, ctypes.c_double(20_000)) == 0
+
+
+def test_server_lanes_keep_to_their_priority(fake):
+    """CSR build, union and count of a small request run at the small lane's priority, those of a large one at the
+    lowest."""
+    L = fake
+    server = ctypes.c_void_p()
+    assert L.harp_server_create(None, ctypes.byref(server)) == 0
+    try:
+        before = {p: L.fake_launches(p) for p in (0, GREATEST)}
+        submit(L, server, 1000)
+        small = {p: L.fake_launches(p) for p in (0, GREATEST)}
+        assert small[0] == before[0] and small[GREATEST] > before[GREATEST]
+        submit(L, server, 65_537)
+        large = {p: L.fake_launches(p) for p in (0, GREATEST)}
+        assert large[0] > small[0] and large[GREATEST] == small[GREATEST]
+    finally:
+        L.harp_server_destroy(server)
