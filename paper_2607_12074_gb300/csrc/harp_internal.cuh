@@ -136,7 +136,8 @@ enum : int {
     T_LIT_EDGE = 66,       // its ticket
     Q_SORT_BLOCK = 67,     // rows for the block row sort
     C4_VISITS = 68,        // (root, lower neighbour, window) visits of the windowed wedge mode
-    kOutLen = 72
+    Q_SORT_AGAIN = 72,     // hub rows whose bitmap came out short of entries (unchecked rows only)
+    kOutLen = 73
 };
 
 // Bits of acc[ACC_ERR].  Any set bit makes a blocking count return HARP_EDEVICE; the asynchronous
@@ -267,6 +268,7 @@ struct harp_csr {
     int64_t* off = nullptr;   // [n+1]
     int32_t* cols = nullptr;  // [2m]
     size_t csr_bytes = 0;
+    bool simple = true;       // built here: no repeats in a row, every edge in both rows (a caller's CSR may break either)
     harp::Workspace ws;
     // signature-reuse counters of the last blocking count (valid once have_reuse is set)
     uint64_t sig_lookups = 0, sig_hits = 0;

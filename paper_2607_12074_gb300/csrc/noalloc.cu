@@ -118,6 +118,7 @@ extern "C" harp_status harp_count4_noalloc(int64_t n, int64_t m, const int64_t* 
     g.n = n;
     g.m = m;
     g.max_deg = n > 0 ? n - 1 : 0;  // an upper bound suffices (it only sizes the degree sort key)
+    g.simple = false;
     g.off = const_cast<int64_t*>(d_offsets);
     g.cols = const_cast<int32_t*>(d_cols);
     Workspace ws;

@@ -297,6 +297,9 @@ __global__ void __launch_bounds__(kBlockWarps * 32) k_sort_rows_block(const int6
 
 // Tier C: hubs (d > 4096) of graphs of at most kBitmapRanks ranks: a block per row sets the row's ranks in a bitmap
 // in shared memory and writes them out in order, a window of ranks at a time (one for up to 1.6 M ranks).
+// again (rows of a caller's CSR, which may hold a rank more than once; nullptr: such rows cannot occur): a row that
+// comes out short is queued from the back for the radix sort below, which keeps repeats, so that all of
+// its deg entries are written.
 __global__ void __launch_bounds__(kBitmapThreads) k_sort_rows_bitmap(const int64_t* __restrict__ goff,
                                                                      const int32_t* __restrict__ gcols,
                                                                      const int32_t* __restrict__ order,
@@ -308,7 +311,8 @@ __global__ void __launch_bounds__(kBitmapThreads) k_sort_rows_bitmap(const int64
                                                                      int32_t* __restrict__ cols,
                                                                      int32_t* __restrict__ dplus,
                                                                      const int32_t* __restrict__ q,
-                                                                     const uint64_t* __restrict__ acc) {
+                                                                     int32_t* __restrict__ again,
+                                                                     uint64_t* __restrict__ acc) {
     grid_begin();
     extern __shared__ uint32_t bm[];
     __shared__ int s_count[kBitmapWarps];
@@ -348,11 +352,16 @@ __global__ void __launch_bounds__(kBitmapThreads) k_sort_rows_bitmap(const int64
         above = warp_sum(above);
         if (l == 0 && above) atomicAdd(&s_above, above);
         __syncthreads();
-        if (threadIdx.x == 0) dplus[i] = s_above;
+        if (threadIdx.x == 0) {
+            dplus[i] = s_above;
+            if (again && dst - off[i] != d)
+                again[n - 1 - (int64_t)atomicAdd((unsigned long long*)&acc[Q_SORT_AGAIN], 1ull)] = (int32_t)i;
+        }
         __syncthreads();
     }
 }
-// Tier C, graphs of more ranks: one block per hub row, LSD radix sort (8-bit digits) through global memory.
+
+// Tier C, graphs of more ranks (and rows with repeats): one block per hub row, LSD radix sort (8-bit digits) through global memory.
 // Pass p reads the previous pass's output; pass 0 reads the old row through perm.  The pass count
 // decides which buffer each pass writes so that the last one lands in `cols`.
 constexpr int kHubThreads = 512;
@@ -368,7 +377,7 @@ __global__ void __launch_bounds__(kHubThreads) k_sort_rows_hub(const int64_t* __
                                                                int32_t* __restrict__ tmp,
                                                                int32_t* __restrict__ dplus,
                                                                const int32_t* __restrict__ q,
-                                                               const unsigned long long* __restrict__ qcnt) {
+                                                               const uint64_t* __restrict__ qcnt) {
     grid_begin();
     __shared__ uint32_t base[256];
     __shared__ uint32_t wcnt[kHubWarps][256];
@@ -376,7 +385,7 @@ __global__ void __launch_bounds__(kHubThreads) k_sort_rows_hub(const int64_t* __
     const int npass = (nbits + 7) / 8;
     const int w = threadIdx.x >> 5, l = lane_id();
     const uint32_t lt = lanemask_lt();
-    const int64_t nq = (int64_t)qcnt[1];
+    const int64_t nq = (int64_t)*qcnt;
     for (int64_t qi = blockIdx.x; qi < nq; qi += gridDim.x) {
         const int64_t i = q[n - 1 - qi];
         const int64_t d = deg[i];
@@ -582,16 +591,20 @@ harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s) {
             HARP_LAUNCHED();
         }
         const int64_t most_n = ws.G > 1 ? ws.max_member_n : n;  // ranks of the largest graph
-        if (g->max_deg > kTierB && most_n <= kBitmapRanks) {
+        const bool bitmap = most_n <= kBitmapRanks;
+        int32_t* again = g->simple ? nullptr : ws.q_mid + n;
+        if (g->max_deg > kTierB && bitmap) {
             const size_t smem = sizeof(uint32_t) * (size_t)kBitmapWords;
             HARP_CK(cudaFuncSetAttribute(k_sort_rows_bitmap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             launch(k_sort_rows_bitmap, num_sms(), kBitmapThreads, smem, s, g->off, g->cols, ws.order, ws.perm, ws.deg,
-                   ws.off, n, ws.G > 1 ? ws.gid : nullptr, ws.gbase, ws.cols, ws.dplus, ws.q_tri, ws.acc);
+                   ws.off, n, ws.G > 1 ? ws.gid : nullptr, ws.gbase, ws.cols, ws.dplus, ws.q_tri, again, ws.acc);
             HARP_LAUNCHED();
-        } else if (g->max_deg > kTierB) {
+        }
+        if (g->max_deg > kTierB && (!bitmap || again)) {
             // the out-CSR columns + t_e region (2m int32) is free until k_out_csr: hub sort ping-pong
             launch(k_sort_rows_hub, num_sms(), kHubThreads, 0, s, g->off, g->cols, ws.order, ws.perm, ws.deg, ws.off,
-                   n, b, ws.cols, ws.colsp, ws.dplus, ws.q_tri, (const unsigned long long*)&ws.acc[Q_SORT_WARP]);
+                   n, b, ws.cols, ws.colsp, ws.dplus, bitmap ? again : ws.q_tri,
+                   &ws.acc[bitmap ? Q_SORT_AGAIN : Q_SORT_WARP + 1]);
             HARP_LAUNCHED();
         }
     } else {
