@@ -467,8 +467,9 @@ void harp_server_destroy(harp_server* srv);
  *              ascending, no self-loops, no duplicates (e.g. the arrays of harp_csr_arrays);
  *              read only.  The device checks d_offsets[0] = 0, d_offsets[n] = 2m, non-decreasing
  *              offsets with degrees <= n - 1 and column ids in [0, n) before anything else; a CSR
- *              that fails is counted as edgeless and d_out[6] is nonzero.  Self-loops, duplicates
- *              or an asymmetric CSR pass that check and give wrong counts.
+ *              that fails is counted as edgeless and d_out[6] is nonzero; so is an asymmetric CSR in
+ *              which more than m entries name a vertex of larger (degree, id).  Self-loops,
+ *              duplicates or any other asymmetric CSR pass that check and give wrong counts.
  *   d_out      device uint64[16]: [0..5] counts, [6] the device self-check word (0 = fine; nonzero =
  *              the CSR check or a kernel's consistency check fired and the counts are not valid),
  *              [7] reserved, [8..15] statistics (HARP_STAT_* order), written when `stream` reaches

@@ -32,7 +32,8 @@ void* g_noalloc_ptr[64] = {nullptr};  // device address of g_noalloc_scratch, pe
 // with every degree at most n - 1, and every column id in [0, n).  The offsets are checked first;
 // the columns are read only when the offsets passed (so no read goes past off[n] = 2m).  A failure
 // sets kErrBadCsr in acc[ACC_ERR]; the orientation pass then treats the graph as edgeless, so no
-// kernel indexes past the scratch laid out for (n, m).
+// kernel indexes past the scratch laid out for (n, m).  It does the same when the rows are not symmetric and
+// more than m of their entries point upwards in rank (k_check_out_arcs).
 __global__ void k_check_offsets(const int64_t* __restrict__ off, int64_t n, int64_t m, uint64_t* __restrict__ acc) {
     grid_begin();
     bool bad = false;

@@ -552,6 +552,26 @@ __global__ void __launch_bounds__(256) k_out_csr(const int64_t* __restrict__ off
     if (threadIdx.x == 0 && pw) atomicAdd((unsigned long long*)&sink.acc[ACC_PW], (unsigned long long)pw);
 }
 
+// A caller's CSR need not list every edge in both rows: then more than m arcs may point upwards in rank, and what is laid
+// out for m of them (t_e above all) would be written past its end.  Such a graph is counted as edgeless
+// and flagged.  One block: the rest of the device has nothing to do here.
+__global__ void __launch_bounds__(1024) k_check_out_arcs(int64_t n, int64_t m, int32_t* __restrict__ deg,
+                                                         int32_t* __restrict__ dplus, int64_t* __restrict__ off,
+                                                         int64_t* __restrict__ offp, uint64_t* __restrict__ acc) {
+    grid_begin();
+    const bool bad = offp[n] > m;
+    __syncthreads();  // every thread has read offp[n]
+    if (!bad) return;
+    for (int64_t v = threadIdx.x; v <= n; v += 1024) {
+        off[v] = offp[v] = 0;
+        if (v < n) deg[v] = dplus[v] = 0;
+    }
+    if (threadIdx.x == 0) {
+        acc[ACC_S] = 0;
+        acc[ACC_ERR] |= kErrBadCsr;
+    }
+}
+
 }  // namespace
 
 harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s) {
@@ -611,6 +631,10 @@ harp_status orient(const harp_csr* g, Workspace& ws, cudaStream_t s) {
         HARP_CK(cudaMemsetAsync(ws.dplus, 0, (size_t)n * sizeof(int32_t), s));
     }
     HARP_TRY(exclusive_scan_i32_to_i64(ws.dplus, ws.offp, n, ws.scan_tmp, ws.scan_tmp_len, s));
+    if (!g->simple) {
+        launch(k_check_out_arcs, 1, 1024, 0, s, n, m, ws.deg, ws.dplus, ws.off, ws.offp, ws.acc);
+        HARP_LAUNCHED();
+    }
     if (m > 0) {
         const Sink sink{ws.acc, ws.gid, ws.accG};
         const int run = m >= (1 << 20) ? 1024 : (m >= (1 << 17) ? 256 : 32);  // small graphs: enough warps

@@ -1,5 +1,6 @@
 """harp_count4_noalloc on a caller's CSR that is not simple: repeats in hub rows (longer than the block sort takes)
-are kept, as in shorter rows, so every array holds as many entries as the degrees say."""
+are kept, as in shorter rows, so every array holds as many entries as the degrees say; rows that are not symmetric are
+refused where more than m of their entries point upwards in rank, the most that the arrays have room for."""
 from math import comb
 
 import numpy as np
@@ -69,4 +70,28 @@ def test_repeated_leaf_of_a_hub(harp):
     hub = np.zeros(leaves.size, np.int64)
     out = count(harp, n, *csr_of(n, np.concatenate([hub, leaves]), np.concatenate([leaves, hub])))
     assert out[:7] == [comb(5001, 3), 2 * 5000, 0, 0, 0, 0, 0]
+    counts_normally(harp)
+
+
+def one_sided(k, heads):
+    """k vertices list vertex 0, which lists others instead, so many that they sort below it."""
+    n = 1 + k + heads
+    src = np.concatenate([np.arange(1, k + 1), np.zeros(heads, np.int64)])
+    dst = np.concatenate([np.zeros(k, np.int64), np.arange(k + 1, n)])
+    return n, src, dst
+
+
+@pytest.mark.parametrize("k,heads", [(4, 2), (1000, 2), (20_002, 20_000), (200_000, 40)])
+def test_more_upward_entries_than_edges(harp, k, heads):
+    n, s, d = one_sided(k, heads)
+    out = count(harp, n, *csr_of(n, s, d))
+    assert out[:6] == [0] * 6 and out[6] != 0
+    counts_normally(harp)
+
+
+@pytest.mark.parametrize("k,heads", [(0, 6), (20, 20), (1000, 9000)])
+def test_other_one_sided_rows_pass(harp, k, heads):
+    n, s, d = one_sided(k, heads)
+    out = count(harp, n, *csr_of(n, s, d))
+    assert out[:7] == [comb(heads, 3), 0, 0, 0, 0, 0, 0]
     counts_normally(harp)
