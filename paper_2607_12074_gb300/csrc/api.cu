@@ -206,13 +206,23 @@ namespace harp {
 harp_status Fork::go(int k, cudaStream_t s) {
     HARP_CK(cudaEventRecord(start, s));
     HARP_CK(cudaStreamWaitEvent(side[k], start, 0));
+    started[k] = true;
     return HARP_OK;
 }
 
-harp_status Fork::back(int k, cudaStream_t s) {
-    HARP_CK(cudaEventRecord(done[k], side[k]));
-    HARP_CK(cudaStreamWaitEvent(s, done[k], 0));
-    return HARP_OK;
+harp_status Fork::join(cudaStream_t s) {
+    harp_status st = HARP_OK;
+    for (int k = 0; k < kSides; ++k) {
+        if (!started[k]) continue;
+        started[k] = false;
+        cudaError_t e = cudaEventRecord(done[k], side[k]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, done[k], 0);
+        if (e == cudaSuccess) continue;
+        record_cuda_error(e);
+        st = HARP_ECUDA;
+        cudaStreamSynchronize(side[k]);  // the order could not be given: wait here
+    }
+    return st;
 }
 
 namespace {
@@ -265,12 +275,12 @@ harp_status count_passes(const harp_csr* g, Workspace& ws, const harp_plan& plan
     HARP_TRY(wedge_geometry(g, ws, plan, s));
     const bool apart = fork && !ws.core && max_out_degree(g) <= (int64_t)plan.tri_cta_max;
     ws.fork = apart ? fork : nullptr;
-    if (apart) HARP_TRY(fork->go(0, s));
-    harp_status st = count_triangles_k4(g, ws, plan, apart ? fork->side[0] : s);
+    harp_status st = apart ? fork->go(0, s) : HARP_OK;
+    if (st == HARP_OK) st = count_triangles_k4(g, ws, plan, apart ? fork->side[0] : s);
     if (st == HARP_OK) st = count_wedge_c4(g, ws, plan, s);
     ws.fork = nullptr;
-    if (apart) HARP_TRY(fork->back(0, s));
-    return st;
+    const harp_status joined = apart ? fork->join(s) : HARP_OK;
+    return st == HARP_OK ? joined : st;
 }
 
 }  // namespace harp

@@ -1330,7 +1330,7 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
            ws.ginfo, n, ws.own_lo, ws.own_hi, warp_max, mid_max, wide_max, ws.q_mid, ws.q_win, wcount,
            ws.acc);  // a lane per root
     HARP_LAUNCHED();
-    // the three tiers read the same arrays and meet only in the accumulators
+    // the three tiers read the same arrays and meet only in the accumulators (count_passes joins the sides)
     cudaStream_t s_light = s, s_mid = s;
     if (ws.fork) {
         HARP_TRY(ws.fork->go(1, s));
@@ -1385,10 +1385,6 @@ harp_status wedge_pass(const harp_csr* g, Workspace& ws, uint32_t warp_max, uint
     launch(k_c4_window<MINB>, sms * MINB, win_threads(MINB), win_smem, s, ws.off, ws.cols, loff, lcols, ws.deg,
            ws.dplus, ws.fpos, ws.rev, ws.bpos, ws.gid, ws.ginfo, ws.q_win, ws.win_prefix, n, ws.acc, sink);
     HARP_LAUNCHED();
-    if (ws.fork) {
-        HARP_TRY(ws.fork->back(1, s));
-        HARP_TRY(ws.fork->back(2, s));
-    }
     HARP_CK(prof_mark(s, SEG_C4_WINDOW));
     return HARP_OK;
 }

@@ -188,14 +188,16 @@ enum : int { G_T = 0, G_K4, G_C4, G_S, G_PW, G_PAWSUM, G_D };
 // Workspace for one counting pass, sized for (n, m) and cached in the graph handle.
 // ---------------------------------------------------------------------------------------------
 // Streams and events of the calling thread for work that can go beside a count's own stream, where the thread waits for
-// the count before it returns, or captures it.  Made at the thread's first use on a device, given back at its end.  go(k, s): side k starts after what s holds; back(k, s): s goes on
-// after what side k holds.
+// the count before it returns, or captures it.  Made at the thread's first use on a device, given back at its end.
+// go(k, s): side k starts after what s holds.  join(s): s goes on after what every started side holds; on every path,
+// errors too, or a side would still be at work in memory that the caller gives back.
 struct Fork {
     static constexpr int kSides = 3;
     cudaStream_t side[kSides] = {};
     cudaEvent_t start = nullptr, done[kSides] = {};
+    bool started[kSides] = {};
     harp_status go(int k, cudaStream_t s);
-    harp_status back(int k, cudaStream_t s);
+    harp_status join(cudaStream_t s);
 };
 Fork* thread_fork();  // nullptr while profiling and where they cannot be made
 

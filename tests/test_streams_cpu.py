@@ -59,3 +59,35 @@ def test_server_lanes_keep_to_their_priority(fake):
         assert large[0] > small[0] and large[GREATEST] == small[GREATEST]
     finally:
         L.harp_server_destroy(server)
+
+
+def build(L, n, m, stream):
+    """A handle of n vertices and m edges, all in the fake's word: no repeats, largest degree 40."""
+    L.fake_answer((ctypes.c_uint64 * 8)(0, 40, 2 * m, 2 * m, 0, 0, 0, 0), ctypes.c_size_t(64))
+    src = np.zeros(m, np.int32)
+    ptr = src.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
+    g = ctypes.c_void_p()
+    assert L.harp_build_csr(ctypes.c_int64(n), ctypes.c_int64(m), ptr, ptr, 0, stream, ctypes.byref(g)) == 0
+    return g
+
+
+def test_side_streams_are_joined_where_a_call_fails(fake):
+    """Whichever runtime call of a count fails, the handle's stream waits for all work given to the side streams, so
+    that freeing the handle (ordered on its stream) cannot overtake it."""
+    L = fake
+    g = build(L, 3000, 9000, None)
+    counts = (ctypes.c_uint64 * 6)()
+    assert L.harp_count4(g, None, counts) == 0
+    open_before = L.fake_unjoined(None)
+    L.fake_fail_at(ctypes.c_long(-1))
+    assert L.harp_count4(g, None, counts) == 0
+    calls = L.fake_calls()
+    assert calls > 40
+    for k in range(calls):
+        L.fake_fail_at(ctypes.c_long(k))
+        status = L.harp_count4(g, None, counts)
+        assert status != 0, k
+        assert L.fake_unjoined(None) == open_before, k
+    L.fake_fail_at(ctypes.c_long(-1))
+    assert L.harp_count4(g, None, counts) == 0
+    L.harp_csr_free(g)
