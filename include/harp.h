@@ -161,7 +161,8 @@ typedef struct harp_plan {
     double objective;            /* value of the Eq. 1 objective for the chosen basis              */
     /* version >= 2 only (a version-1 plan ends at `objective` and gets the defaults below) */
     uint32_t lit_cache_log2;     /* literal basis: signature-cache slots = 2^this (0 = sized from m, */
-                                 /* at most 2^25; 16 bytes a slot)                                  */
+                                 /* at most 2^25; 16 bytes a slot); the requests of a staged edge   */
+                                 /* pass do not use it (harp_reuse_stats)                           */
     uint32_t lit_cache_min_deg;  /* literal basis: degree bin admitted to the cache: a frontier is   */
                                  /* cached only if both generating vertices have degree >= this     */
                                  /* (smaller ones are recomputed; 0 = all)                          */
@@ -197,8 +198,12 @@ harp_status harp_count4(const harp_csr* g, const harp_plan* plan, uint64_t count
 
 /* Signature-reuse counters of the last blocking count on g (harp_count4 / harp_count4_stats)
  * (Section III-C).  Triangle-wedge basis: lookups = 4-clique extensions (one per triangle), hits =
- * those answered by a staged frontier.  Literal basis: lookups = frontier requests to the signature
- * cache (common neighbours of an edge or of a non-adjacent pair), hits = those found in it.
+ * those answered by a staged frontier.  Literal basis: lookups = frontier requests (common neighbours
+ * of an edge or of a non-adjacent pair), hits = those answered without an intersection.  Requests go to
+ * the signature cache, except in the edge pass of graphs of up to 90,000 vertices that are small, dense or
+ * have hubs: there one walk per vertex counts all its frontiers in shared memory, whatever the cache's size,
+ * and a hit is an edge's request (the triangle pass has computed it) or a pair's second and later one for
+ * the same vertex; pairs that lit_cache_min_deg does not admit count as no hit.
  * HARP_ENOTFOUND before the first blocking count. */
 harp_status harp_reuse_stats(const harp_csr* g, uint64_t* lookups, uint64_t* hits);
 

@@ -118,7 +118,7 @@ enum : int {
     ACC_LIT_E = 49,        // 49 lo, 50 hi: sum over edges of the A_e x B_e pairs that are edges
     ACC_LIT_STAR = 51,     // sum over vertices of the H_u star form (mod 2^64)
     ACC_LIT_T = 52,        // triangles enumerated by the literal triangle pass
-    ACC_SIG_LOOKUPS = 53,  // literal basis: frontier requests to the signature cache
+    ACC_SIG_LOOKUPS = 53,  // literal basis: frontier requests (cache or staged counters)
     Q_C4_MIDW = 54,        // length of the wedge middle tier's queue (from the back of q_mid)
     Q_CORE_S = 55,         // wedge core pass: queue lengths by degree class
     Q_CORE_M = 56,

@@ -25,7 +25,8 @@
 //      (u is a common neighbour of x and v; the rest of N(x) n N(v) n N[u] lies in C_uv).  The
 //      frontier N(x) n N(v) of the non-adjacent pair (x, v) recurs for every common neighbour of x
 //      and v that anchors an edge, so it is read through the cache; the correction probes the staged
-//      C_uv.  path4 terms |A_e||B_e| - E_e, cycle4 terms E_e.
+//      C_uv.  path4 terms |A_e||B_e| - E_e, cycle4 terms E_e.  Where a vertex has enough edges
+//      (literal_stages) a block per v counts all its frontiers in shared memory instead (k_lit_edge_staged).
 //   3. k_lit_star, one warp per vertex u: deg_H(v) = t_uv for every v in N(u) through the cache,
 //      m(H_u) = (1/2) sum t_uv, tau(H_u) = tau3[u] / 3.
 // The sums divided by 2 and 4 are accumulated in 128 bits, so the divisions are exact (a sum that is
@@ -41,7 +42,8 @@
 // (key, value) with a bounded probe window; insertion claims an empty slot with a CAS and publishes
 // the value with a valid bit, so a reader that sees the key before its value treats it as a miss.
 // Frontiers of pairs below the degree bin lit_cache_min_deg are recomputed instead of cached.  With
-// the cache off (HARP_PLAN_NO_REUSE) every frontier is recomputed; the counts are the same.
+// the cache off (HARP_PLAN_NO_REUSE) every frontier is recomputed; the counts are the same.  SIG_W states
+// reach the cache only from the edge pass that is not staged.
 #include "harp_internal.cuh"
 
 namespace harp {
@@ -432,9 +434,10 @@ __global__ void __launch_bounds__(kLitThreads) k_lit_edge(Graph G, const int64_t
 // cnt(x) - 1 over x in A_e = N(u) \ N[v], one counter read each.  The correction, summed over x in A_e, is
 //   sum_x |C_uv n N(x)| = sum over w in C_uv of |N(w) n A_e| = sum over w in C_uv of (t_uw - 1 - X_3(u, v, w)),
 // which the triangle pass has at hand for the three edges of every triangle (acc[ACC_LIT_CORR]).
-// A frontier's first request counts as computed and the later ones, answered by the staged counter, as hits
-// (where the admission by degree caches it at all).  Computing each missing frontier by its own intersection, in the
-// lane that asked for it, took 10.7 ms on R-MAT scale 13 (130,000 edges).
+// The counters answer every request: an edge's frontier, which the triangle pass has computed, counts as a hit, and
+// so does a non-adjacent pair's from its second request for the same v on (both where the admission by degree
+// would cache it).  The cache itself is neither read nor filled.  Computing each missing frontier by its own
+// intersection, in the lane that asked for it, took 10.7 ms on R-MAT scale 13 (130,000 edges).
 constexpr int kStagedThreads = 512;
 constexpr int64_t kStagedMaxN = 90000;
 
@@ -490,10 +493,7 @@ __global__ void __launch_bounds__(kStagedThreads) k_lit_edge_staged(Graph G, con
                 const uint64_t A = (uint64_t)(e - b) - 1 - t, B = (uint64_t)(ve - vb) - 1 - t;
                 if (l == 0) {
                     ++st.lookups;
-                    const bool cached = cacheable(cache, G, u, (int32_t)v);
-                    uint32_t found = 0;
-                    if (cached && sig_find(cache, sig_key(SIG_C, u, (int32_t)v), found)) ++st.hits;
-                    else if (cached) sig_put(cache, sig_key(SIG_C, u, (int32_t)v), t);
+                    if (cacheable(cache, G, u, (int32_t)v)) ++st.hits;
                     ab_sum += A * B;
                 }
                 if (A == 0 || B == 0) continue;  // no pair

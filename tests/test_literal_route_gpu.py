@@ -1,7 +1,8 @@
 """Which edge pass a literal count takes: staged frontiers where a vertex has enough edges to pay for a block's turn, the
-pass by edges on sparse graphs, on both sides of each line of the rule.  Copies of K_{2,3} beside a star: in the staged
-pass, whose repeats are answered by its counters, 4 of a copy's 6 requests for the two hubs' frontier repeat whatever the
-signature cache holds; the pass by edges has nothing but the cache."""
+pass by edges on sparse graphs, on both sides of each line of the rule; and what harp_reuse_stats counts in either.
+Copies of K_{2,3} beside a star: in the staged pass an edge's request and 4 of a copy's 6 requests for the two hubs'
+frontier are answered by its counters, whatever the signature cache holds; the pass by edges has nothing but the
+cache."""
 from math import comb
 
 import numpy as np
@@ -44,16 +45,22 @@ def test_route(harp, n, leaves, staged):
     want = [2 * copies + comb(leaves, 3), 0, 0, 3 * copies, 0, 0]
     seen = {}
     g = harp.harp_build_csr(n, src, dst)
-    for slots in (0, 6):
+    for slots, min_deg in ((0, 0), (6, 0), (0, 3)):
         plan = harp.harp_plan()
         plan.version, plan.basis, plan.lit_cache_log2 = harp.HARP_ABI_VERSION, harp.HARP_BASIS_LITERAL, slots
+        plan.lit_cache_min_deg = min_deg
         assert harp.harp_count4(g, plan).tolist() == want
-        seen[slots] = harp.harp_reuse_stats(g)
+        seen[slots, min_deg] = harp.harp_reuse_stats(g)
     g.close()
     # requests: one per edge in the first pass, one per edge and 6 per copy in the second, two per edge in the third
-    assert seen[0][0] == seen[6][0] == 30 * copies + 4 * leaves
-    assert (seen[6][1] >= 4 * copies) == staged
+    edges = 6 * copies + leaves
+    assert {lookups for lookups, _ in seen.values()} == {4 * edges + 6 * copies}
+    full, tiny, hubs = (seen[k][1] for k in ((0, 0), (6, 0), (0, 3)))
     if staged:
-        assert seen[0][1] == 22 * copies + 3 * leaves
+        assert full == 3 * edges + 4 * copies
+        assert edges + 4 * copies <= tiny <= edges + 4 * copies + 128  # the third pass finds at most 64 edges kept
+        assert hubs == 4 * copies
     else:  # of the 6, those made before the first is kept miss
-        assert 18 * copies + 3 * leaves <= seen[0][1] <= 23 * copies + 3 * leaves
+        assert 3 * edges <= full <= 3 * edges + 5 * copies
+        assert tiny <= 1000  # what 64 slots can answer
+        assert hubs <= 5 * copies
