@@ -158,7 +158,7 @@ harp_status enqueue_count(harp_csr* g, const harp_plan* user_plan, Fork* fork, c
     harp_status st = orient(g, ws, s);
     if (st == HARP_OK) st = prof_mark(s, SEG_ORIENT) == cudaSuccess ? HARP_OK : HARP_ECUDA;
     if (plan.basis == HARP_BASIS_LITERAL) {
-        if (st == HARP_OK) st = count_literal(g, ws, plan, s);
+        if (st == HARP_OK) st = count_literal(g, ws, plan, fork, s);
     } else {
         if (st == HARP_OK) st = count_passes(g, ws, plan, fork, s);
         if (st == HARP_OK) st = reduce_and_close(g, ws, s);

@@ -340,7 +340,7 @@ harp_status count_wedge_core(const harp_csr* g, Workspace& ws, cudaStream_t s);
 
 // literal.cu: the literal basis (per-triangle X_j, per-edge A_e x B_e, per-vertex H_u stars) and its
 // closure, after orient(); writes acc[OUT_COUNTS..], acc[OUT_STATS..]
-harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& plan, cudaStream_t s);
+harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& plan, Fork* fork, cudaStream_t s);
 // batch.cu: harp_batch_create with the priority of the batch's own stream (the union's build and, captured, the count)
 harp_status batch_create(const harp_csr* const* graphs, int64_t G, int priority, harp_batch** out);
 

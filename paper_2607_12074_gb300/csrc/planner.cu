@@ -18,11 +18,12 @@
 // Element operations are charged at the wedge kernel's rate (kOpsPerUs).  Graphs small enough for the choice
 // to be close are bound by latency instead, charged at what it takes beside that rate: the passes' fixed
 // cost after the shared orientation (TW 40 us: some ten dependent launches, those of the two passes side by
-// side; LIT 25 us: three), and in LIT a warp's turn per arc (2.5 ns of the device), the two cache requests of a
-// triangle (1 ns) and the longest chain of triangles that one arc's warp takes one after the other (0.5 us
-// each).  Measured with both bases: Barabasi-Albert of 300 vertices (894 edges) TW 98 us, LIT 84; of 3,000 (11,990) 132
-// and 143; random geometric of 1,000 (3,779) 90 and 98; Erdos-Renyi of 1,000 (4,974) 103 and 96, of 80,000
-// (160,193) 202 and 547.  (A term for launches alone named LIT up to 160,000 edges, up to 6 times slower.)  Both
+// side; LIT 25 us: three, or 17 with the staged edge pass beside the first), and in LIT a warp's turn per arc (2.5
+// ns of the device), the two cache requests of a triangle (1 ns) and the longest chain of triangles that one
+// arc's warp takes one after the other (0.8 us each).  Measured with both bases (TW, LIT in us): Barabasi-Albert of
+// 300 vertices (894 edges) 96, 76, of 3,000 (29,945) 155, 197; Erdos-Renyi of 1,000 (4,974) 101, 87, of 3,000 (24,060)
+// 124, 135, of 80,000 (160,193) 203, 548; random geometric of 3,000 (14,529) 112, 153; R-MAT scale 9 (869) 100, 109.  Within
+// 8 % of each other either may be named.  (A term for launches alone named LIT up to 160,000 edges.)  Both
 // recover all six counts (Y = 6).  The lambda weights normalise the terms to element operations (the
 // paper leaves their values open): l_I = 1, l_H = 1/4 per replicated byte, l_R = 1 (reuse is counted
 // in the element operations it saves), l_Y = 0 (equal yield decides nothing between these bases).
@@ -40,7 +41,8 @@ namespace harp {
 namespace {
 
 constexpr double kOpsPerUs = 4.0e5;  // element operations (wedge kernel: about 4e11 a second)
-constexpr double kTwFixedUs = 40.0, kLitFixedUs = 25.0, kLitArcUs = 2.5e-3, kLitTriangleUs = 1.0e-3, kLitChainUs = 0.5;
+constexpr double kTwFixedUs = 40.0, kLitFixedUs = 25.0, kLitStagedFixedUs = 17.0;
+constexpr double kLitArcUs = 2.5e-3, kLitTriangleUs = 1.0e-3, kLitChainUs = 0.8;
 
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
@@ -213,7 +215,8 @@ extern "C" harp_status harp_select_anchors(const harp_csr* g, const harp_select_
     lit_inter *= m * inv;
     lit_reuse *= m * inv;
     tw_enum += kOpsPerUs * kTwFixedUs;
-    lit_enum += kOpsPerUs * (kLitFixedUs + kLitArcUs * m + kLitTriangleUs * triangles * m * inv + kLitChainUs * t_max);
+    lit_enum += kOpsPerUs * ((staged ? kLitStagedFixedUs : kLitFixedUs) + kLitArcUs * m + kLitTriangleUs * triangles * m * inv +
+                             kLitChainUs * t_max);
     // Halo term: replication factor if the CSR plus workspace exceed the memory budget.
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);

@@ -8,19 +8,19 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 CASES = {
-    "ba_300_3": (lambda: graphgen.ba(300, 3, 21), True),        # 98, 84
-    "er_300_6": (lambda: graphgen.er(300, 6, 1), True),         # 84, 76
-    "er_1000_3": (lambda: graphgen.er(1000, 3, 3), True),       # 84, 77
-    "er_3000_2": (lambda: graphgen.er(3000, 2, 2), True),       # 101, 89
-    "rmat_9_2": (lambda: graphgen.rmat(9, 2, seed=1), False),   # 96, 120
-    "rgg_1000_8": (lambda: graphgen.rgg(1000, 8, 3), False),    # 90, 98
-    "er_3000_8": (lambda: graphgen.er(3000, 8, 2), False),      # 113, 127
-    "ba_3000_4": (lambda: graphgen.ba(3000, 4, 3), False),      # 132, 143
-    "rgg_3000_10": (lambda: graphgen.rgg(3000, 10, 12), False),  # 116, 166
-    "er_10000_4": (lambda: graphgen.er(10000, 4, 2), False),    # 114, 151
-    "ba_22000_4": (lambda: graphgen.ba(22000, 4, 3), False),    # 190, 401
-    "er_80000_4": (lambda: graphgen.er(80000, 4, 2), False),    # 202, 547
-    "rmat_13_8": (lambda: graphgen.rmat(13, 8, seed=1), False),  # 202, 805
+    "ba_300_3": (lambda: graphgen.ba(300, 3, 21), True),        # 96, 76
+    "er_300_6": (lambda: graphgen.er(300, 6, 1), True),         # 81, 75
+    "er_1000_3": (lambda: graphgen.er(1000, 3, 3), True),       # 83, 73
+    "er_1000_10": (lambda: graphgen.er(1000, 10, 3), True),     # 101, 87
+    "er_3000_2": (lambda: graphgen.er(3000, 2, 2), True),       # 100, 91
+    "rmat_9_2": (lambda: graphgen.rmat(9, 2, seed=1), False),   # 100, 109
+    "er_3000_16": (lambda: graphgen.er(3000, 16, 2), False),    # 124, 135
+    "ba_3000_10": (lambda: graphgen.ba(3000, 10, 3), False),    # 155, 197
+    "rgg_3000_10": (lambda: graphgen.rgg(3000, 10, 12), False),  # 112, 153
+    "er_10000_4": (lambda: graphgen.er(10000, 4, 2), False),    # 111, 150
+    "ba_22000_4": (lambda: graphgen.ba(22000, 4, 3), False),    # 189, 376
+    "er_80000_4": (lambda: graphgen.er(80000, 4, 2), False),    # 203, 548
+    "rmat_13_8": (lambda: graphgen.rmat(13, 8, seed=1), False),  # 206, 681
 }
 
 

@@ -71,23 +71,28 @@ def build(L, n, m, stream):
     return g
 
 
-def test_side_streams_are_joined_where_a_call_fails(fake):
+@pytest.mark.parametrize("literal", [False, True], ids=["triangle_wedge", "literal"])
+def test_side_streams_are_joined_where_a_call_fails(fake, literal):
     """Whichever runtime call of a count fails, the handle's stream waits for all work given to the side streams, so
     that freeing the handle (ordered on its stream) cannot overtake it."""
+    from paper_2607_12074_gb300 import harp as H
     L = fake
-    g = build(L, 3000, 9000, None)
+    p = H.harp_plan()
+    p.version, p.basis = H.HARP_ABI_VERSION, H.HARP_BASIS_LITERAL if literal else H.HARP_BASIS_TRIANGLE_WEDGE
+    plan = ctypes.byref(p)
+    g = build(L, 2000, 9000, None)
     counts = (ctypes.c_uint64 * 6)()
-    assert L.harp_count4(g, None, counts) == 0
+    assert L.harp_count4(g, plan, counts) == 0
     open_before = L.fake_unjoined(None)
     L.fake_fail_at(ctypes.c_long(-1))
-    assert L.harp_count4(g, None, counts) == 0
+    assert L.harp_count4(g, plan, counts) == 0
     calls = L.fake_calls()
-    assert calls > 40
+    assert calls >= 20
     for k in range(calls):
         L.fake_fail_at(ctypes.c_long(k))
-        status = L.harp_count4(g, None, counts)
+        status = L.harp_count4(g, plan, counts)
         assert status != 0, k
         assert L.fake_unjoined(None) == open_before, k
     L.fake_fail_at(ctypes.c_long(-1))
-    assert L.harp_count4(g, None, counts) == 0
+    assert L.harp_count4(g, plan, counts) == 0
     L.harp_csr_free(g)
