@@ -184,7 +184,7 @@ harp_status count_to_host(const harp_csr* gc, const harp_plan* plan, uint64_t* c
     if (!gc || !counts_out) return HARP_EINVAL;
     harp_csr* g = const_cast<harp_csr*>(gc);
     HARP_CK(cudaSetDevice(g->device));
-    HARP_TRY(enqueue_count(g, plan, thread_fork(), g->stream));
+    HARP_TRY(enqueue_count(g, plan, thread_fork(g->stream), g->stream));
     uint64_t host[kOutLen];
     HARP_CK(cudaMemcpyAsync(host, g->ws.acc, sizeof(host), cudaMemcpyDeviceToHost, g->stream));
     HARP_CK(cudaStreamSynchronize(g->stream));
@@ -227,9 +227,9 @@ harp_status Fork::join(cudaStream_t s) {
 
 namespace {
 struct ThreadForks {
-    static constexpr int kDevices = 16;
-    Fork of[kDevices];
-    bool tried[kDevices] = {};
+    static constexpr int kDevices = 16, kPriorities = 8;  // stream priorities are 0, -1, ..
+    Fork of[kDevices][kPriorities];
+    bool tried[kDevices][kPriorities] = {};
     static void release(Fork& f) {
         for (int k = 0; k < Fork::kSides; ++k) {
             if (f.side[k]) cudaStreamDestroy(f.side[k]);
@@ -239,23 +239,29 @@ struct ThreadForks {
         f = Fork();
     }
     ~ThreadForks() {
-        for (Fork& f : of)
-            if (f.start) release(f);
+        for (auto& device : of)
+            for (Fork& f : device)
+                if (f.start) release(f);
     }
 };
 }  // namespace
 
-Fork* thread_fork() {
+Fork* thread_fork(cudaStream_t s) {
     if (g_profiling.load(std::memory_order_relaxed)) return nullptr;  // profiled segments follow one another
     static thread_local ThreadForks forks;
-    int dev = 0;
+    int dev = 0, priority = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev >= ThreadForks::kDevices) return nullptr;
-    Fork& f = forks.of[dev];
-    if (!forks.tried[dev]) {
-        forks.tried[dev] = true;
+    if (cudaStreamGetPriority(s, &priority) != cudaSuccess || priority > 0 || -priority >= ThreadForks::kPriorities) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    Fork& f = forks.of[dev][-priority];
+    bool& tried = forks.tried[dev][-priority];
+    if (!tried) {
+        tried = true;
         cudaError_t e = cudaEventCreateWithFlags(&f.start, cudaEventDisableTiming);
         for (int k = 0; k < Fork::kSides && e == cudaSuccess; ++k) {
-            e = cudaStreamCreateWithFlags(&f.side[k], cudaStreamNonBlocking);
+            e = cudaStreamCreateWithPriority(&f.side[k], cudaStreamNonBlocking, priority);
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f.done[k], cudaEventDisableTiming);
         }
         if (e != cudaSuccess) {  // counts keep to one stream

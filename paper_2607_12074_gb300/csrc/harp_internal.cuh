@@ -188,7 +188,8 @@ enum : int { G_T = 0, G_K4, G_C4, G_S, G_PW, G_PAWSUM, G_D };
 // Workspace for one counting pass, sized for (n, m) and cached in the graph handle.
 // ---------------------------------------------------------------------------------------------
 // Streams and events of the calling thread for work that can go beside a count's own stream, where the thread waits for
-// the count before it returns, or captures it.  Made at the thread's first use on a device, given back at its end.
+// the count before it returns, or captures it; of the priority of that stream.  Made at the thread's first use on a
+// device and of a priority, given back at its end.
 // go(k, s): side k starts after what s holds.  join(s): s goes on after what every started side holds; on every path,
 // errors too, or a side would still be at work in memory that the caller gives back.
 struct Fork {
@@ -199,7 +200,7 @@ struct Fork {
     harp_status go(int k, cudaStream_t s);
     harp_status join(cudaStream_t s);
 };
-Fork* thread_fork();  // nullptr while profiling and where they cannot be made
+Fork* thread_fork(cudaStream_t s);  // beside s; nullptr while profiling and where they cannot be made
 
 struct Workspace {
     void* base = nullptr;

@@ -96,3 +96,21 @@ def test_side_streams_are_joined_where_a_call_fails(fake, literal):
     L.fake_fail_at(ctypes.c_long(-1))
     assert L.harp_count4(g, plan, counts) == 0
     L.harp_csr_free(g)
+
+
+@pytest.mark.parametrize("literal", [False, True], ids=["triangle_wedge", "literal"])
+@pytest.mark.parametrize("priority", [0, -2, GREATEST])
+def test_side_streams_have_the_priority_of_the_handles_stream(fake, priority, literal):
+    from paper_2607_12074_gb300 import harp as H
+    L = fake
+    p = H.harp_plan()
+    p.version, p.basis = H.HARP_ABI_VERSION, H.HARP_BASIS_LITERAL if literal else H.HARP_BASIS_TRIANGLE_WEDGE
+    stream = ctypes.c_void_p()
+    assert L.cudaStreamCreateWithPriority(ctypes.byref(stream), 1, priority) == 0
+    before = [L.fake_launches(q) for q in range(0, GREATEST - 1, -1)]
+    g = build(L, 2000, 9000, stream)
+    counts = (ctypes.c_uint64 * 6)()
+    assert L.harp_count4(g, ctypes.byref(p), counts) == 0
+    L.harp_csr_free(g)
+    after = [L.fake_launches(q) for q in range(0, GREATEST - 1, -1)]
+    assert [q for q in range(6) if after[q] > before[q]] == [-priority]
