@@ -3,8 +3,8 @@
 // Every input pair (u, v), u != v, counts towards both degrees and is scattered into both rows at slots taken by
 // atomics (equal endpoints within a warp take theirs together: edge lists often run along one vertex).  Self-loops
 // are skipped; out-of-range ids are skipped and raise a flag that turns into HARP_EINVAL.  Rows are then sorted by
-// the tiers of rowsort.cuh, equal neighbours dropped while they are written, and, where any were, the rows
-// closed up.  The rows' order makes the result independent of the order in which slots were taken.
+// the tiers of rowsort.cuh (very long ones, and hubs among very many ids, by one radix sort of them all), equal
+// neighbours dropped while they are written, and, where any were, the rows closed up.  The rows' order makes the result independent of the order in which slots were taken.
 // (A radix sort of all arcs as 64-bit keys moved every arc 2 * bits(n) / 8 times.)  Kernels of a build, with the sort and
 // now: R-MAT scale 20 2.8 and 1.6 ms, Chung-Lu of 1,347,423 vertices (hubs of close ids) 2.2 and 1.4 ms, random
 // geometric of 1,000,003 vertices 1.24 and 0.30 ms.
@@ -15,7 +15,7 @@ namespace harp {
 namespace {
 
 // Words of the build's summary, read back by the host.
-enum : int { B_BAD = 0, B_MAXDEG, B_ARCS, B_RAW, B_Q_WARP, B_Q_BLOCK, B_Q_HUB, B_WORDS = 8 };
+enum : int { B_BAD = 0, B_MAXDEG, B_ARCS, B_Q_WARP, B_Q_BLOCK, B_Q_HUB, B_Q_LONG, B_LONG_LEN, B_WORDS = 8 };
 
 // Fewer vertices keep their counters by id: the copy back costs a launch and there is little to contend for.
 constexpr int64_t kSpreadMinN = 1 << 14;
@@ -97,8 +97,32 @@ __global__ void __launch_bounds__(256) k_build_scatter(const int32_t* __restrict
     }
 }
 
+// Hub rows whose bitmap sort may not pay: a block reads its row once for each window of ids, about 1 ns an entry, while
+// the rest of the device may have nothing to do, and every window is cleared and searched (5 us) whatever the row
+// holds.  Rows of more than 2^18 entry reads, and all hub rows where the ids take more than four windows (the
+// bound of the orientation's rows too), wait for the host, which knows their number and length then and takes a
+// radix sort of all of them over the device (0.15 ns an entry) where that is estimated to be faster.  Whole builds by
+// bitmaps alone and now, the radix sort of all arcs that the build once was in brackets: a star of 5,900,000 leaves
+// 10.0 and 1.3 ms [1.5], of 99,000,000 1,134 and 25 [23]; 20,000 rows of 5,000 among 100,000,000 ids 130 and 28 [23], among
+// 500,000,000 585 and 45 [26: the other passes here go over the ids]; Chung-Lu of 20,000,000 vertices 28 and 25 [48].  300
+// rows of 300,000 among 20,000,000 ids keep to bitmaps: 11 ms, by the radix sort 17 [19].
+constexpr int64_t kLongReads = 1 << 18;
+__host__ __device__ __forceinline__ int64_t bitmap_windows(int64_t n) {
+    return (n + 32 * (int64_t)kBitmapWords - 1) / (32 * (int64_t)kBitmapWords);
+}
+__device__ __forceinline__ bool long_row(int64_t n, int64_t d) {
+    return n > kBitmapRanks || d * bitmap_windows(n) > kLongReads;
+}
+// nr long rows of H entries
+bool long_by_bitmap(int64_t n, int64_t nr, int64_t H) {
+    const double turns = (double)((nr + num_sms() - 1) / num_sms());
+    const double bitmap_us = turns * (double)bitmap_windows(n) * (5.0 + 1.0e-3 * (double)H / (double)nr);
+    return bitmap_us < 100.0 + 0.15e-3 * (double)H;
+}
+
 // Rows of at most kTierA entries, 32 consecutive rows per warp (a lane's network up to 16, the warp's above); longer
-// ones are queued: the warp sort's from the front of q, hubs from its back, the block sort's in q_block.
+// ones are queued: the warp sort's from the front of q, hubs from its back, the block sort's from the front of
+// q_block, long rows (long_row) from its back, with their entries added up.
 template <int P>
 __device__ __forceinline__ int lane_unique_row(const int32_t* __restrict__ in, int32_t* __restrict__ out, int d) {
     int32_t a[P];
@@ -125,12 +149,12 @@ __global__ void __launch_bounds__(256) k_build_rows_small(const int64_t* __restr
         const int64_t i = i0 + l;
         const int64_t b = i < n ? roff[i] : 0;
         const int d = i < n ? (int)(roff[i + 1] - b) : -1;
-        if (d == 0) ndeg[i] = 0;
+        const int cls = d > kTierB ? (long_row(n, d) ? 3 : 2) : (d > kTierB1 ? 1 : (d > kTierA ? 0 : -1));
+        if (d == 0 || cls == 3) ndeg[i] = 0;
         else if (d >= 1 && d <= 8) ndeg[i] = lane_unique_row<8>(in + b, out + b, d);
         else if (d > 8 && d <= 16) ndeg[i] = lane_unique_row<16>(in + b, out + b, d);
-        const int cls = d > kTierB ? 2 : (d > kTierB1 ? 1 : (d > kTierA ? 0 : -1));
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int c = 0; c < 4; ++c) {
             const uint32_t m = __ballot_sync(kFull, cls == c);
             if (!m) continue;
             unsigned long long start = 0;
@@ -141,7 +165,9 @@ __global__ void __launch_bounds__(256) k_build_rows_small(const int64_t* __restr
             const int64_t k = (int64_t)start + __popc(m & lanemask_lt());
             if (c == 0) q[k] = (int32_t)i;
             else if (c == 1) q_block[k] = (int32_t)i;
-            else q[n - 1 - k] = (int32_t)i;
+            else if (c == 2) q[n - 1 - k] = (int32_t)i;
+            else q_block[n - 1 - k] = (int32_t)i;
+            if (c == 3) atomicAdd(&summary[B_LONG_LEN], (unsigned long long)d);
         }
         uint32_t rest = __ballot_sync(kFull, d > 16 && d <= kTierA);
         while (rest) {  // four rows at a time: their loads overlap
@@ -286,11 +312,11 @@ __global__ void __launch_bounds__(kBitmapThreads) k_build_rows_bitmap(const int6
                                                                       int32_t* __restrict__ out,
                                                                       int32_t* __restrict__ ndeg,
                                                                       const int32_t* __restrict__ q,
-                                                                      const unsigned long long* __restrict__ summary) {
+                                                                      const unsigned long long* __restrict__ count) {
     grid_begin();
     extern __shared__ uint32_t bm[];
     __shared__ int s_count[kBitmapWarps];
-    const int64_t nq = (int64_t)summary[B_Q_HUB];
+    const int64_t nq = (int64_t)*count;
     for (int64_t k = blockIdx.x; k < nq; k += gridDim.x) {
         const int64_t i = q[n - 1 - k], b = roff[i], e = roff[i + 1];
         int64_t dst = b;
@@ -318,20 +344,70 @@ __global__ void __launch_bounds__(kBitmapThreads) k_build_rows_bitmap(const int6
     }
 }
 
-// Largest degree, and the arc counts before and after dropping repeats.
+// Long rows by radix sort, nr of them in q_block from the back: their entries as keys (row's place in the queue, id), radix-sorted,
+// the first of each value written to its row.
+__global__ void __launch_bounds__(256) k_long_lengths(const int64_t* __restrict__ roff, int64_t n,
+                                                      const int32_t* __restrict__ q_block, int64_t nr,
+                                                      int32_t* __restrict__ len) {
+    grid_begin();
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nr; k += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = q_block[n - 1 - k];
+        len[k] = (int32_t)(roff[i + 1] - roff[i]);
+    }
+}
+
+constexpr int kLongRun = 1024;  // entries per warp and search of the first one's row
+
+__global__ void __launch_bounds__(256) k_long_gather(const int64_t* __restrict__ roff, int64_t n,
+                                                     const int32_t* __restrict__ q_block, int64_t nr,
+                                                     const int64_t* __restrict__ loff, int b,
+                                                     const int32_t* __restrict__ in, uint64_t* __restrict__ keys) {
+    grid_begin();
+    const int64_t H = loff[nr], nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t e0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kLongRun; e0 < H; e0 += nw * kLongRun) {
+        int64_t k = 0, hi = nr;  // the last row that begins at or before e0
+        while (hi - k > 1) {
+            const int64_t mid = (k + hi) >> 1;
+            if (loff[mid] <= e0) k = mid;
+            else hi = mid;
+        }
+        const int64_t e1 = e0 + kLongRun < H ? e0 + kLongRun : H;
+        for (int64_t e = e0 + lane_id(); e < e1; e += 32) {
+            while (loff[k + 1] <= e) ++k;  // e < H = loff[nr]
+            keys[e] = ((uint64_t)k << b) | (uint64_t)(uint32_t)in[roff[q_block[n - 1 - k]] + (e - loff[k])];
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) k_long_first(const uint64_t* __restrict__ keys, int64_t H, int32_t* __restrict__ first) {
+    grid_begin();
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < H; e += (int64_t)gridDim.x * blockDim.x)
+        first[e] = e == 0 || keys[e] != keys[e - 1];
+}
+
+__global__ void __launch_bounds__(256) k_long_write(const uint64_t* __restrict__ keys, const int64_t* __restrict__ pos,
+                                                    int64_t H, const int64_t* __restrict__ loff, int b,
+                                                    const int64_t* __restrict__ roff, int64_t n,
+                                                    const int32_t* __restrict__ q_block, int32_t* __restrict__ out,
+                                                    int32_t* __restrict__ ndeg) {
+    grid_begin();
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < H; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = (int64_t)(keys[e] >> b), i = q_block[n - 1 - k], before = pos[loff[k]];
+        if (pos[e + 1] != pos[e]) out[roff[i] + (pos[e] - before)] = (int32_t)(keys[e] & (((uint64_t)1 << b) - 1));
+        if (e == loff[k]) ndeg[i] = (int32_t)(pos[loff[k + 1]] - before);
+    }
+}
+
+// Largest degree, and the arcs after dropping repeats.
 __global__ void __launch_bounds__(256) k_build_summary(const int32_t* __restrict__ ndeg, const int64_t* __restrict__ off,
-                                                       const int64_t* __restrict__ roff, int64_t n,
-                                                       unsigned long long* __restrict__ summary) {
+                                                       int64_t n, unsigned long long* __restrict__ summary) {
     grid_begin();
     int32_t best = 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
         best = max(best, ndeg[v]);
     best = __reduce_max_sync(kFull, best);
     if (lane_id() == 0 && best > 0) atomicMax(&summary[B_MAXDEG], (unsigned long long)best);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        summary[B_ARCS] = (unsigned long long)off[n];
-        summary[B_RAW] = (unsigned long long)roff[n];
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) summary[B_ARCS] = (unsigned long long)off[n];
 }
 
 // Rows closed up: a warp per `run` consecutive columns of the result.  The row of the first is searched (32 probes a
@@ -390,6 +466,50 @@ unsigned grid_for(int64_t work, int threads) {
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// The long rows of a build: raw holds the scattered rows (and, gathered, is scratch), sorted receives them.
+harp_status sort_long_rows(int64_t n, int64_t nr, int64_t H, const int64_t* roff, const int32_t* q_block, int32_t* raw,
+                           int32_t* sorted, int32_t* ndeg, cudaStream_t s) {
+    auto bits_for = [](int64_t x) {  // to hold values up to x
+        int b = 1;
+        while (b < 62 && ((int64_t)1 << b) <= x) ++b;
+        return b;
+    };
+    const int b = bits_for(n - 1), br = bits_for(nr - 1);
+    const size_t hist_len = radix_hist_len(H), tmp_len = scan_tmp_needed(H) + scan_tmp_needed((int64_t)hist_len) + 64;
+    const size_t keys_b = align256(sizeof(uint64_t) * (size_t)(H + 1)), hist_b = align256(sizeof(uint32_t) * hist_len);
+    const size_t tmp_b = align256(sizeof(int64_t) * tmp_len), loff_b = align256(sizeof(int64_t) * (size_t)(nr + 1));
+    unsigned char* slab = nullptr;
+    cudaError_t e = cudaMallocAsync((void**)&slab, 2 * keys_b + hist_b + tmp_b + loff_b + sizeof(int32_t) * (size_t)nr, s);
+    if (e != cudaSuccess) {
+        record_cuda_error(e);
+        return e == cudaErrorMemoryAllocation ? HARP_ENOMEM : HARP_ECUDA;
+    }
+    uint64_t *keys = reinterpret_cast<uint64_t*>(slab), *alt = reinterpret_cast<uint64_t*>(slab + keys_b);
+    uint32_t* hist = reinterpret_cast<uint32_t*>(slab + 2 * keys_b);
+    int64_t* tmp = reinterpret_cast<int64_t*>(slab + 2 * keys_b + hist_b);
+    int64_t* loff = reinterpret_cast<int64_t*>(slab + 2 * keys_b + hist_b + tmp_b);
+    int32_t* len = reinterpret_cast<int32_t*>(slab + 2 * keys_b + hist_b + tmp_b + loff_b);
+    auto run = [&]() -> harp_status {
+        launch(k_long_lengths, grid_for(nr, 256), 256, 0, s, roff, n, q_block, nr, len);
+        HARP_LAUNCHED();
+        HARP_TRY(exclusive_scan_i32_to_i64(len, loff, nr, tmp, tmp_len, s));
+        launch(k_long_gather, grid_for((H + kLongRun - 1) / kLongRun * 32, 256), 256, 0, s, roff, n, q_block, nr, loff, b,
+               raw, keys);
+        HARP_LAUNCHED();
+        HARP_TRY(radix_sort_u64(&keys, &alt, H, 0, b + br, hist, tmp, tmp_len, s));
+        launch(k_long_first, grid_for(H, 256), 256, 0, s, keys, H, raw);
+        HARP_LAUNCHED();
+        int64_t* pos = reinterpret_cast<int64_t*>(alt);
+        HARP_TRY(exclusive_scan_i32_to_i64(raw, pos, H, tmp, tmp_len, s));
+        launch(k_long_write, grid_for(H, 256), 256, 0, s, keys, pos, H, loff, b, roff, n, q_block, sorted, ndeg);
+        HARP_LAUNCHED();
+        return HARP_OK;
+    };
+    const harp_status st = run();
+    cudaFreeAsync(slab, s);
+    return st;
+}
 
 }  // namespace
 
@@ -468,18 +588,27 @@ harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t
         launch(k_build_rows_block, num_sms() * 4, kBlockWarps * 32, 0, s, roff, raw, sorted, ndeg, q_block, summary);
         BLAUNCHED();
     }
-    if (m_in > kTierB) {
+    auto bitmap_rows = [&](const int32_t* queue, int count) -> harp_status {  // from the back of the queue
         const size_t smem = sizeof(uint32_t) * (size_t)kBitmapWords;
-        BCK(cudaFuncSetAttribute(k_build_rows_bitmap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        launch(k_build_rows_bitmap, num_sms(), kBitmapThreads, smem, s, roff, n, raw, sorted, ndeg, q, summary);
-        BLAUNCHED();
-    }
-    BTRY(exclusive_scan_i32_to_i64(ndeg, g->off, n, tmp, tmp_len, s));
-    launch(k_build_summary, grid_for(n, 256), 256, 0, s, ndeg, g->off, roff, n, summary);
-    BLAUNCHED();
+        HARP_CK(cudaFuncSetAttribute(k_build_rows_bitmap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        launch(k_build_rows_bitmap, num_sms(), kBitmapThreads, smem, s, roff, n, raw, sorted, ndeg, queue, summary + count);
+        HARP_LAUNCHED();
+        return HARP_OK;
+    };
+    if (m_in > kTierB && n <= kBitmapRanks) BTRY(bitmap_rows(q, B_Q_HUB));
     unsigned long long host[B_WORDS] = {0};
-    BCK(cudaMemcpyAsync(host, summary, sizeof(host), cudaMemcpyDeviceToHost, s));
-    BCK(cudaStreamSynchronize(s));
+    for (;;) {
+        BTRY(exclusive_scan_i32_to_i64(ndeg, g->off, n, tmp, tmp_len, s));
+        launch(k_build_summary, grid_for(n, 256), 256, 0, s, ndeg, g->off, n, summary);
+        BLAUNCHED();
+        const bool again = host[B_LONG_LEN] > 0;
+        BCK(cudaMemcpyAsync(host, summary, sizeof(host), cudaMemcpyDeviceToHost, s));
+        BCK(cudaStreamSynchronize(s));
+        if (again || host[B_BAD] || host[B_LONG_LEN] == 0) break;
+        const int64_t nr = (int64_t)host[B_Q_LONG], H = (int64_t)host[B_LONG_LEN];
+        if (long_by_bitmap(n, nr, H)) BTRY(bitmap_rows(q_block, B_Q_LONG));
+        else BTRY(sort_long_rows(n, nr, H, roff, q_block, raw, sorted, ndeg, s));
+    }
     if (host[B_BAD]) {
         cleanup();
         return HARP_EINVAL;

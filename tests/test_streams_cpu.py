@@ -63,7 +63,7 @@ def test_server_lanes_keep_to_their_priority(fake):
 
 def build(L, n, m, stream):
     """A handle of n vertices and m edges, all in the fake's word: no repeats, largest degree 40."""
-    L.fake_answer((ctypes.c_uint64 * 8)(0, 40, 2 * m, 2 * m, 0, 0, 0, 0), ctypes.c_size_t(64))
+    L.fake_answer((ctypes.c_uint64 * 8)(0, 40, 2 * m, 0, 0, 0, 0, 0), ctypes.c_size_t(64))
     src = np.zeros(m, np.int32)
     ptr = src.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
     g = ctypes.c_void_p()
