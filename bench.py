@@ -617,12 +617,12 @@ def main():
     if not args.no_meter:
         meter = workmeter.meter(g.n, g.src, g.dst)
         # every pass against the HBM roofline: its algorithmic bytes (work meter) over its CUDA-event time.
-        # The wedge segments are one pass: the meter deals roots to tiers by their work alone, while the
-        # library counts the roots of the highest ranks in the core pass (timed with the light tier)
+        # The wedge segments are one pass (the core pass is timed with the light tier)
         passes = {k: (k,) for k in SEGMENTS if not k.startswith("c4_")}
         passes["wedges"] = tuple(k for k in SEGMENTS if k.startswith("c4_"))
         pass_ms = {p: sum(seg_avg[k] for k in ks) for p, ks in passes.items()}
         pass_bytes = {p: sum(meter[k]["bytes"] for k in ks if k in meter) for p, ks in passes.items()}
+        pass_bytes["wedges"] += meter["c4_core"]["bytes"]
         segment_rooflines = {}
         for p, t_ms in pass_ms.items():
             if t_ms <= 0 or pass_bytes[p] <= 0:
@@ -633,19 +633,8 @@ def main():
         dom = max((p for p in passes if p != "orient"), key=lambda p: pass_ms[p])
         alg = pass_bytes[dom]
         achieved = alg / (pass_ms[dom] / 1000) / 1e9
-        traffic = None
-        tfile = os.path.join(ROOT, "profiles", "traffic.json")
-        if os.path.exists(tfile):  # DRAM bytes of one ncu capture, valid while the kernel is unchanged
-            import hashlib
-            with open(tfile) as f:
-                rec = json.load(f)
-            src = os.path.join(ROOT, rec.get("source", ""))
-            if dom in rec and os.path.isfile(src):
-                with open(src, "rb") as f:
-                    if hashlib.sha256(f.read()).hexdigest()[:16] == rec.get("source_sha256_16"):
-                        traffic = rec[dom]
         roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
-                    "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
+                    "frac": achieved / peak, "peak_kind": peak_kind,
                     "algorithmic_bytes": alg, "kernel_ms": pass_ms[dom]}
     cpu = None
     if not args.no_cpu_baseline:
@@ -686,7 +675,7 @@ def main():
         "served": served,
         "partitioned": partitioned,
         "counts": [int(x) for x in counts],
-        "hbm_pct_alg": (100.0 * sum(meter[k]["bytes"] for k in SEGMENTS) / (t_step / 1000) / 1e9 / peak)
+        "hbm_pct_alg": (100.0 * sum(pass_bytes.values()) / (t_step / 1000) / 1e9 / peak)
         if meter else None,
     }
     print(json.dumps(line), flush=True)

@@ -608,7 +608,8 @@ harp_status count_wedge_core(const harp_csr* g, Workspace& ws, cudaStream_t s) {
     const int64_t n = g->n;
     const int sms = num_sms();
     const Sink sink{ws.acc, ws.gid, ws.accG};
-    uint32_t* bits = reinterpret_cast<uint32_t*>(ws.rev);  // rev and bpos are adjacent (ws_layout) and still unused
+    // the bitmaps that build_core_bits wrote; rev and bpos are adjacent (ws_layout) and filled after this pass
+    uint32_t* bits = reinterpret_cast<uint32_t*>(ws.rev);
     uint2* cseg = reinterpret_cast<uint2*>(ws.vkeys);      // the sort keys are done with
     int32_t *q_s = ws.q_mid, *q_m = ws.q_mid + n, *q_l = ws.q_win;
     int64_t blocks = (n + 255) / 256;

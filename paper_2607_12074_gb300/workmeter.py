@@ -12,10 +12,16 @@ Per unit (int32 ids and counters = 4 B, int64 offsets = 8 B):
   triangle      per anchor u: its list N+(u) (4 d+), per row v in N+(u): offsets (16) and the probed
                 part of N+(v) up to max N+(u) (4 each); per triangle: 3 t_e updates (8 each, RMW);
                 per out-arc: its own t_e update (8)
-  wedge (C4)    per root u: N-(u) read once (4 d-) + the row bounds of each w (16 d-); per wedge
-                element x of degree >= 2: 4.  The windowed kernel re-reads N-(u) and the row
+                Rows v in the graph's core (core_start) of anchors of out-degree 33 to 1024 are read from
+                the core's bitmaps instead: 4 per pair (row, later key of N+(u))
+  wedge (C4)    per root u below the core: N-(u) read once (4 d-) + the row bounds of each w (16 d-); per
+                wedge element x of degree >= 2: 4.  The windowed kernel re-reads N-(u) and the row
                 bounds once per further x-window; those bytes are this design's overhead and are
                 reported apart ("overhead_bytes"), not counted as algorithmic
+  core          the wedges whose root lies in the core, counted per lower end x (core_bytes): the core's rows
+                written as bitmaps with their prefix counts; per x of degree >= 2 its row, 8 per neighbour
+                below the core and 4 per element above x of that neighbour's part of the core, and the
+                words above x of each core neighbour's bitmap row (4 per 32 ranks)
   reduction     t_e read: 4 m
 """
 from __future__ import annotations
@@ -86,13 +92,55 @@ def _merged_windows(bounds, widths, mask, u, words):
     return total
 
 
+CORE_MIN_M, CORE_MIN_MAX_DEG = 1 << 18, 256
+
+
+def core_start(G):
+    """First rank of the graph's wedge core, n without one: the largest K = 2^10 .. 2^14 highest ranks with 2 K <= n, a
+    degree of K / 64 at the first, an eighth of the arcs, and room for its bitmaps."""
+    n, m, deg, indptr = G["n"], G["m"], G["deg"], G["indptr"]
+    if m < CORE_MIN_M or deg[-1] < CORE_MIN_MAX_DEG:
+        return n
+    for lg in range(14, 9, -1):
+        K = 1 << lg
+        if (2 * K <= n and 3 * K * K // 16 <= 8 * m + 64 * n and deg[n - K] >= K // 64
+                and 8 * (2 * m - int(indptr[n - K])) >= 2 * m):
+            return n - K
+    return n
+
+
+def core_bytes(G, c0):
+    """Bytes of the core pass and its bitmaps for the core [c0, n)."""
+    n, deg, indptr, rows, cols, pos = G["n"], G["deg"], G["indptr"], G["rows"], G["cols"], G["pos"]
+    K = n - c0
+    if K == 0:
+        return {"bytes": 0, "elements": 0, "words": 0}
+    KW = K // 32
+    first = (np.arange(K, dtype=np.int64) >> 5) & ~3
+    table = 4 * int(G["dplus"][c0:].sum()) + 6 * int((KW - first).sum())
+    inside = np.zeros(rows.size + 1, np.int64)
+    np.cumsum((cols >= c0) & (cols > rows), out=inside[1:])
+    seg = inside[indptr[1:]] - inside[indptr[:-1]]     # of each row: neighbours in the core, above it
+    active = deg[rows] >= 2                            # arcs (x -> w) of x that can close a cycle
+    low = active & (cols < c0)
+    x, w = rows[low], cols[low]
+    above = deg[w] - 1 - pos[np.searchsorted(rows * n + cols, w * n + x)]  # neighbours of w above x
+    elements = int(np.where(x < c0, seg[w], above).sum())
+    high = active & (cols >= c0)
+    x, r = rows[high], cols[high]
+    words = int((KW - np.maximum(r - c0, np.maximum(x - c0 + 1, 0)) // 32).clip(min=0).sum())
+    return {"bytes": table + 20 * n + 4 * int(active.sum()) + 8 * int(low.sum()) + 4 * elements + 4 * words,
+            "elements": elements, "words": words}
+
+
 def meter(n, src, dst, c4_warp_max=512, c4_window_bytes=0, c4_mid_max=2048):
     """Per-kernel work and algorithmic bytes (dict of dicts) under the given wedge plan fields."""
     G = rank_space(n, src, dst)
     m = G["m"]
     deg, indptr, rows, cols, pos = G["deg"], G["indptr"], G["rows"], G["cols"], G["pos"]
     split, dplus = G["split"], G["dplus"]
-    out = {"n": n, "m": m}
+    c0 = core_start(G)
+    out = {"n": n, "m": m, "core": n - c0}
     out["orient"] = {"bytes": 24 * (n + 1) + 12 * 2 * m + 8 * m}
 
     # ---- triangle anchors: out-arcs (u -> v), u < v
@@ -116,6 +164,8 @@ def meter(n, src, dst, c4_warp_max=512, c4_window_bytes=0, c4_mid_max=2048):
     ends = offp[1:][has] - 1
     is_last[ends] = True
     row_bytes = np.where(is_last, 0, 16 + 4 * probed)
+    gathered = (av >= c0) & ((arc_cls == 1) | (arc_cls == 2))
+    row_bytes = np.where(gathered, 4 * (offp[au + 1] - 1 - np.arange(au.size)), row_bytes)  # later keys of the list
     tri_units = {}
     for c, name in ((0, "tri_warp"), (1, "tri_cta_small"), (2, "tri_cta_large"), (3, "tri_fallback")):
         sel = arc_cls == c
@@ -140,7 +190,7 @@ def meter(n, src, dst, c4_warp_max=512, c4_window_bytes=0, c4_mid_max=2048):
     # slots), windowed counters above
     wmax = min(c4_warp_max, 512)
     mmax = max(min(c4_mid_max, 2048), wmax)
-    tier = np.where((dm < 2) | (W == 0), -1, np.where(W <= wmax, 0, np.where(W <= mmax, 1, 2)))
+    tier = np.where((dm < 2) | (W == 0) | (np.arange(n) >= c0), -1, np.where(W <= wmax, 0, np.where(W <= mmax, 1, 2)))
     words = window_words(c4_window_bytes, n)
     bounds = band_starts + [n]
     # narrow bands may merge into the next wider one: the mask with the fewest degree-weighted windows
@@ -161,6 +211,7 @@ def meter(n, src, dst, c4_warp_max=512, c4_window_bytes=0, c4_mid_max=2048):
                      "items": int(passes.sum()),
                      "bytes": int((20 * dm[sel]).sum() + 4 * W[sel].sum()),
                      "overhead_bytes": int((20 * dm[sel] * (passes - 1)).sum())}
+    out["c4_core"] = core_bytes(G, c0)
     out["c4_wedges_total"] = int(W.sum())
     out["reduce"] = {"bytes": 4 * m}
     return out
