@@ -24,8 +24,9 @@ def fake(tmp_path_factory):
     obj, lib = str(out / "fake_cudart.o"), str(out / "libharp_fake.so")
     include = os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include")
     subprocess.run(["gcc", "-O1", "-fPIC", "-I", include, "-c", os.path.join(HERE, "fake_cudart.c"), "-o", obj], check=True)
-    subprocess.run([nvcc, *_build.ARCH, "-shared", "-cudart", "none", "-o", lib, *glob.glob(os.path.join(_build.BUILD, "*.cu.o")),
-                    obj], check=True)
+    # -Bsymbolic: another CUDA runtime that the process has loaded (torch's) must not take the fake's place
+    subprocess.run([nvcc, *_build.ARCH, "-shared", "-cudart", "none", "-Xlinker", "-Bsymbolic", "-o", lib,
+                    *glob.glob(os.path.join(_build.BUILD, "*.cu.o")), obj], check=True)
     L = ctypes.CDLL(lib)
     L.fake_launches.restype = L.fake_calls.restype = ctypes.c_long
     L.harp_status_str.restype = ctypes.c_char_p
