@@ -288,7 +288,7 @@ def bench_served(harp, graphgen, np, rates=(10.0, 30.0, 100.0, 300.0, 1000.0, 20
         c.close()
     out = {"workload": f"{nreq} requests per rate, Poisson arrivals, edge counts log-uniform [1e3, 1e7], "
                        f"ER/BA/RGG/R-MAT uniform, HBM budget {budget >> 30} GiB", "requests": nreq,
-           "lanes": "small requests (<= 65536 input pairs) on a second, higher-priority compute stream",
+           "lanes": "small requests (<= 65536 input pairs) on a second lane, its streams of a higher priority",
            "generate_s": t_gen, "rates": []}
     for k, rate in enumerate(rates):
         r = served_at_rate(harp, np, gs, rate, seed + k, budget)
