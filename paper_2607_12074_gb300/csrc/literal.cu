@@ -44,6 +44,8 @@
 // Frontiers of pairs below the degree bin lit_cache_min_deg are recomputed instead of cached.  With
 // the cache off (HARP_PLAN_NO_REUSE) every frontier is recomputed; the counts are the same.  SIG_W states
 // reach the cache only from the edge pass that is not staged.
+#include <algorithm>
+
 #include "harp_internal.cuh"
 
 namespace harp {
@@ -627,18 +629,20 @@ int staged_blocks(int64_t n) { return StagedShape(n).bytes() <= 100 * 1024 ? 2 :
 
 }  // namespace
 
-// The staged pass costs a block's turn per vertex (5 ns of the device with two blocks to an SM, 9 with one), the pass by
-// edges the intersections of each edge's frontiers, which grow with the degrees' square and with hubs.  Whole counts,
-// staged and by edges: Erdos-Renyi of 40,000 vertices, mean degree 4 0.43 and 0.32 ms, 8 0.57 and 0.76; of 80,000
-// vertices, 8 1.61 and 1.34, 16 2.35 and 4.14; random geometric of 22,000 vertices, 6 0.42 and 0.35, 10 0.59 and 0.68;
-// Barabasi-Albert of 40,000 vertices, 4 (largest degree 497) 0.44 and 0.63; of 80,000, 4 (691) 1.21 and 0.91, 8 (867)
-// 1.76 and 3.05.  Up to 2,048 vertices the blocks have a few turns each: staged 0.084 and 0.102 on Barabasi-Albert
-// of 300 vertices, 0.077 and 0.084 on Erdos-Renyi of 1,000 with mean degree 3.
+// The staged pass costs a block's turn per vertex (5 ns of the device with two blocks to an SM, 9 with one), beside the
+// triangle pass, the pass by edges the intersections of each edge's frontiers, which grow with the degrees' square and
+// with hubs.  Whole counts in ms, staged and by edges: Erdos-Renyi of 3,000 vertices, mean degree 3 0.102 and 0.099, 4
+// 0.103 and 0.112; of 10,000, 4 0.154 and 0.151, 6 0.168 and 0.214; of 40,000, 4 0.38 and 0.31, 6 0.43 and 0.54; of
+// 80,000, 7 1.17 and 1.07, 10 1.27 and 2.01.  Random geometric of 10,000, 5 0.189 and 0.183, 6 0.207 and 0.224; of 40,000, 6
+// 0.58 and 0.56, 8 0.79 and 0.80; of 80,000, 8 1.71 and 1.42, 10 2.26 and 2.03, 12 2.67 and 2.80.  Barabasi-Albert of 22,000, 2
+// (largest degree 244) 0.214 and 0.221; of 60,000, 4 (598) 0.75 and 0.83.  Up to 2,048 vertices the blocks have a few
+// turns each: Barabasi-Albert of 300 vertices 0.076 and 0.102.
 bool literal_stages(const harp_csr* g) {
     if (g->n > kStagedMaxN || g->max_deg >= 65536) return false;
     if (g->n <= 2048) return true;
     const double mean = 2.0 * (double)g->m / (double)g->n, top = (double)g->max_deg;
-    return staged_blocks(g->n) == 2 ? mean * mean + 0.3 * top >= 45.0 : mean * mean + 0.15 * top >= 150.0;
+    if (staged_blocks(g->n) == 1) return mean * mean + 0.15 * top >= 95.0;
+    return mean * mean + 0.3 * top >= std::min(15.0 + 1.0e-3 * (double)g->n, 41.0);
 }
 
 harp_status count_literal(const harp_csr* g, Workspace& ws, const harp_plan& plan, Fork* fork, cudaStream_t s) {

@@ -33,10 +33,11 @@ def bicliques_and_star(n, leaves):
     return copies, src.astype(np.int32), dst.astype(np.int32)
 
 
-# mean degree about 2.4: staged up to 2,048 vertices; then mean^2 + 0.3 d_max >= 45 while two blocks fit an SM (n <= 45,511),
-# mean^2 + 0.15 d_max >= 150 up to 90,000 vertices
-CASES = [(2048, 0, True), (2049, 0, False), (40_000, 120, False), (40_000, 140, True), (45_500, 140, True), (45_600, 140, False),
-         (80_000, 0, False), (80_000, 900, False), (80_000, 1_000, True), (90_000, 1_000, True), (90_001, 1_000, False)]
+# mean degree about 2.4: staged up to 2,048 vertices; then mean^2 + 0.3 d_max >= min(15 + n / 1000, 41) while two blocks
+# fit an SM (n <= 45,511), mean^2 + 0.15 d_max >= 95 up to 90,000 vertices
+CASES = [(2048, 0, True), (2049, 0, False), (10_000, 55, False), (10_000, 75, True), (40_000, 110, False),
+         (40_000, 125, True), (45_500, 125, True), (45_600, 125, False), (80_000, 0, False), (80_000, 560, False),
+         (80_000, 620, True), (90_000, 620, True), (90_001, 620, False)]
 
 
 @pytest.mark.parametrize("n,leaves,staged", CASES)
