@@ -107,12 +107,9 @@ __global__ void __launch_bounds__(256) k_build_scatter(const int32_t* __restrict
 // 500,000,000 585 and 45 [26: the other passes here go over the ids]; Chung-Lu of 20,000,000 vertices 28 and 25 [48].  300
 // rows of 300,000 among 20,000,000 ids keep to bitmaps: 11 ms, by the radix sort 17 [19].
 constexpr int64_t kLongReads = 1 << 18;
-__host__ __device__ __forceinline__ int64_t bitmap_windows(int64_t n) {
-    return (n + 32 * (int64_t)kBitmapWords - 1) / (32 * (int64_t)kBitmapWords);
-}
-__device__ __forceinline__ bool long_row(int64_t n, int64_t d) {
-    return n > kBitmapRanks || d * bitmap_windows(n) > kLongReads;
-}
+int64_t bitmap_windows(int64_t n) { return (n + 32 * (int64_t)kBitmapWords - 1) / (32 * (int64_t)kBitmapWords); }
+// hub rows of more entries than this are long
+int64_t long_above(int64_t n) { return n > kBitmapRanks ? 0 : kLongReads / bitmap_windows(n); }
 // nr long rows of H entries
 bool long_by_bitmap(int64_t n, int64_t nr, int64_t H) {
     const double turns = (double)((nr + num_sms() - 1) / num_sms());
@@ -122,7 +119,7 @@ bool long_by_bitmap(int64_t n, int64_t nr, int64_t H) {
 
 // Rows of at most kTierA entries, 32 consecutive rows per warp (a lane's network up to 16, the warp's above); longer
 // ones are queued: the warp sort's from the front of q, hubs from its back, the block sort's from the front of
-// q_block, long rows (long_row) from its back, with their entries added up.
+// q_block, long rows from its back, with their entries added up.
 template <int P>
 __device__ __forceinline__ int lane_unique_row(const int32_t* __restrict__ in, int32_t* __restrict__ out, int d) {
     int32_t a[P];
@@ -139,7 +136,7 @@ __device__ __forceinline__ int lane_unique_row(const int32_t* __restrict__ in, i
 __global__ void __launch_bounds__(256) k_build_rows_small(const int64_t* __restrict__ roff, int64_t n,
                                                           const int32_t* __restrict__ in, int32_t* __restrict__ out,
                                                           int32_t* __restrict__ ndeg, int32_t* __restrict__ q,
-                                                          int32_t* __restrict__ q_block,
+                                                          int32_t* __restrict__ q_block, int64_t long_limit,
                                                           unsigned long long* __restrict__ summary) {
     grid_begin();
     const int l = lane_id();
@@ -149,7 +146,7 @@ __global__ void __launch_bounds__(256) k_build_rows_small(const int64_t* __restr
         const int64_t i = i0 + l;
         const int64_t b = i < n ? roff[i] : 0;
         const int d = i < n ? (int)(roff[i + 1] - b) : -1;
-        const int cls = d > kTierB ? (long_row(n, d) ? 3 : 2) : (d > kTierB1 ? 1 : (d > kTierA ? 0 : -1));
+        const int cls = d > kTierB ? (d > long_limit ? 3 : 2) : (d > kTierB1 ? 1 : (d > kTierA ? 0 : -1));
         if (d == 0 || cls == 3) ndeg[i] = 0;
         else if (d >= 1 && d <= 8) ndeg[i] = lane_unique_row<8>(in + b, out + b, d);
         else if (d > 8 && d <= 16) ndeg[i] = lane_unique_row<16>(in + b, out + b, d);
@@ -577,7 +574,8 @@ harp_status build_csr_device(harp_csr* g, int64_t n, int64_t m_in, const int32_t
     BTRY(exclusive_scan_i32_to_i64(at.stride ? ndeg : deg, roff, n, tmp, tmp_len, s));
     launch(k_build_scatter, grid_for(m_in, 256), 256, 0, s, d_src, d_dst, m_in, n, roff, at, deg, raw);
     BLAUNCHED();
-    launch(k_build_rows_small, grid_for(n, 256), 256, 0, s, roff, n, raw, sorted, ndeg, q, q_block, summary);
+    launch(k_build_rows_small, grid_for(n, 256), 256, 0, s, roff, n, raw, sorted, ndeg, q, q_block,
+           long_above(n), summary);
     BLAUNCHED();
     // a row has at most m_in entries: tiers above that are empty
     if (m_in > kTierA) {
