@@ -184,7 +184,7 @@ harp_status count_to_host(const harp_csr* gc, const harp_plan* plan, uint64_t* c
     if (!gc || !counts_out) return HARP_EINVAL;
     harp_csr* g = const_cast<harp_csr*>(gc);
     HARP_CK(cudaSetDevice(g->device));
-    HARP_TRY(enqueue_count(g, plan, thread_fork(g->stream), g->stream));
+    HARP_TRY(enqueue_count(g, plan, thread_fork(g), g->stream));
     uint64_t host[kOutLen];
     HARP_CK(cudaMemcpyAsync(host, g->ws.acc, sizeof(host), cudaMemcpyDeviceToHost, g->stream));
     HARP_CK(cudaStreamSynchronize(g->stream));
@@ -246,15 +246,17 @@ struct ThreadForks {
 };
 }  // namespace
 
-Fork* thread_fork(cudaStream_t s) {
+Fork* thread_fork(harp_csr* g) {
     if (g_profiling.load(std::memory_order_relaxed)) return nullptr;  // profiled segments follow one another
     static thread_local ThreadForks forks;
-    int dev = 0, priority = 0;
+    int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev >= ThreadForks::kDevices) return nullptr;
-    if (cudaStreamGetPriority(s, &priority) != cudaSuccess || priority > 0 || -priority >= ThreadForks::kPriorities) {
+    if (g->priority == harp_csr::kPriorityUnknown && cudaStreamGetPriority(g->stream, &g->priority) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        g->priority = harp_csr::kPriorityUnknown;
     }
+    const int priority = g->priority;
+    if (priority > 0 || priority <= -ThreadForks::kPriorities) return nullptr;
     Fork& f = forks.of[dev][-priority];
     bool& tried = forks.tried[dev][-priority];
     if (!tried) {

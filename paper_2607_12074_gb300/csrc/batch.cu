@@ -269,7 +269,7 @@ harp_status batch_prepare(harp_batch* b, const harp_plan& plan) {
         HARP_CK(cudaStreamSynchronize(b->capture_stream));
         cudaGraph_t graph = nullptr;
         const int64_t l0 = harp_launch_count();
-        Fork* fork = thread_fork(b->capture_stream);  // branches of the graph
+        Fork* fork = thread_fork(&b->u);  // branches of the graph
         HARP_CK(cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeRelaxed));
         harp_status st = enqueue_batch(b, plan, fork, b->capture_stream);
         cudaError_t e = cudaStreamEndCapture(b->capture_stream, &graph);

@@ -200,7 +200,7 @@ struct Fork {
     harp_status go(int k, cudaStream_t s);
     harp_status join(cudaStream_t s);
 };
-Fork* thread_fork(cudaStream_t s);  // beside s; nullptr while profiling and where they cannot be made
+Fork* thread_fork(harp_csr* g);  // beside g's stream; nullptr while profiling and where they cannot be made
 
 struct Workspace {
     void* base = nullptr;
@@ -267,6 +267,8 @@ void ws_release(Workspace& ws, cudaStream_t s);
 struct harp_csr {
     int device = 0;
     cudaStream_t stream = nullptr;
+    static constexpr int kPriorityUnknown = 1;
+    int priority = kPriorityUnknown;  // of the stream, from the first count that asks (thread_fork)
     int64_t n = 0, m = 0, max_deg = 0;
     int64_t* off = nullptr;   // [n+1]
     int32_t* cols = nullptr;  // [2m]
